@@ -32,7 +32,8 @@ namespace pgb {
 struct CellDesc {
     int N, M, nf, n, nnode, fast_gamma;
     double S, gamma, Wsig;
-    long long pairs;     // unordered node pairs, nnode (nnode + 1) / 2
+    int naxp;            // unordered node-index pairs per axis
+    long long nclass;    // classes of node pairs that share their points, naxp^d (SpreadArgs)
     long long f_off;     // packed modes (f~ and Q)
     long long a_off;     // packed node values (a, h)
     long long grid_off;  // packed folded grids
@@ -42,7 +43,7 @@ struct CellDesc {
     int R_off;           // R (N x (N+1)) and E ((N+1) x N)
     int D_off;           // D ((N+1) x nf)
     int sig_off;         // sphere points (M x d) and weights (M)
-    int chunk;           // node pairs per work item
+    int chunk;           // classes of node pairs per work item
     int item0;           // first work item of the cell
     double corr;         // FP32 plans: exact / FP32 constant factors of the strengths (1 for FP64)
 };
@@ -310,7 +311,8 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.M = cd.M;
     sa.r = b.r;
     sa.nnode = cd.nnode;
-    sa.npairs = cd.pairs;
+    sa.naxp = cd.naxp;
+    sa.nclass = cd.nclass;
     sa.n = cd.n;
     sa.nf = cd.nf;
     sa.rows_per_slab = cd.nf;
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
             // negligible points: FP32 points below 0.1 tile unit add exactly zero; FP64 pairs whose
             // summed bounds stay below 2^-64 B are skipped
             floor_q = F32 ? T(spread_detail::kNegligibleF32)
-                          : T(ldexp(Bc, Eg - 64) * sa.cd.wmax / (double)s_cd.pairs);
+                          : T(ldexp(Bc, Eg - 64) * sa.cd.wmax / (double)s_cd.nclass);
             for (int e = threadIdx.x; e < ncell; e += blockDim.x) {
                 if constexpr (F32) {
                     lo[e] = 0;
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
         }
         // the item's node pairs; lanes of a warp take pairs nwarp apart
         const long long p0 = (long long)(item - s_cd.item0) * s_cd.chunk;
-        const long long p1 = min(p0 + (long long)s_cd.chunk, s_cd.pairs);
+        const long long p1 = min(p0 + (long long)s_cd.chunk, s_cd.nclass);
         const long long first = p0 + (long long)lane * nwarp + warp;
         if constexpr (F32) {
             // the warp's queue compacts the points that add something (FP32 points below 0.1 tile
@@ -621,7 +623,7 @@ long long split_items(std::vector<pgb::CellDesc> &cells, long long item_points, 
         pgb::CellDesc &cd = cells[c];
         cd.chunk = (int)std::max<long long>(64, item_points / cd.M);
         cd.item0 = (int)n;
-        const long long nitem = (cd.pairs + cd.chunk - 1) / cd.chunk;
+        const long long nitem = (cd.nclass + cd.chunk - 1) / cd.chunk;
         if (item_cell) item_cell->insert(item_cell->end(), (size_t)nitem, (int)c);
         n += nitem;
     }
@@ -748,7 +750,8 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         cd.fast_gamma = (gammas[c] == 0.0) ? 0 : (gammas[c] == 1.0) ? 1 : (gammas[c] == 0.5) ? 2 : 3;
         cd.S = Ss[c];
         cd.gamma = gammas[c];
-        cd.pairs = pgb::unordered_pairs(cd.nnode);
+        cd.naxp = (int)pgb::unordered_pairs(N);
+        cd.nclass = (long long)ipow((double)cd.naxp, d);
         auto nk = std::make_pair(N, Ss[c]);
         if (!node_key.count(nk)) {
             NodeTables nt = node_tables(N, Ss[c], B->r);
@@ -796,8 +799,9 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         cd.s_len = std::max<long long>(modes, (long long)(N + 1) * (long long)ipow(cd.nf, d - 1));
         cd.s_off = s_off;
         s_off += 4 * cd.s_len;
-        B->points += cd.pairs * M;
-        B->pairs += cd.pairs;
+        const long long pairs = pgb::unordered_pairs(cd.nnode);
+        B->points += pairs * M;
+        B->pairs += pairs;
     }
     B->offsets[ncell] = f_off;
     // work items: room for the autotuner's smallest item size, the default size to start with

@@ -90,7 +90,7 @@ struct pg_boltz_plan_s {
     int n = 0, nf = 0, w = 0;
     double beta = 0.0;
     int nnode = 0;
-    long long npairs = 0;
+    long long npairs = 0, nclass = 0;  // unordered node pairs; classes that share their points (SpreadArgs)
     int fast_gamma = 0;
     double Bconst = 0.0, Wsig = 0.0;
     int nslab = 1, rows_per_slab = 0, spread_blocks = 0, spread_threads = 256;

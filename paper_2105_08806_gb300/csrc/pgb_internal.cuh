@@ -46,7 +46,8 @@ struct TypedConsts {
 struct SpreadArgs {
     int d, N, M, r;
     int nnode;            // N^d interior nodes
-    long long npairs;     // unordered node pairs, unordered_pairs(nnode)
+    int naxp;             // unordered pairs of node indices per axis, unordered_pairs(N)
+    long long nclass;     // classes of node pairs that share their points, naxp^d
     int n, nf;            // periodic grid size, folded cells per axis (n/2 + 1)
     int rows_per_slab;    // folded-grid rows (axis 0) held in shared memory by one block
     int nslab;            // number of slabs covering axis 0
@@ -117,8 +118,7 @@ __device__ __forceinline__ const TypedConsts<T> &kconst(const SpreadArgs &a)
     else return a.cd;
 }
 
-// Node pairs the spreading kernels walk: each unordered pair {i, j} once (the two orders add the
-// same points with the same strength), nnode (nnode + 1) / 2 in all.
+// Unordered pairs of n things, equal ones included.
 __host__ __device__ inline long long unordered_pairs(long long nnode) { return nnode * (nnode + 1) / 2; }
 
 // Values per queued point of the slabbed spreading kernels: FP32 points keep each coordinate as

@@ -32,6 +32,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     const int d = p->d, N = p->N, M = p->M;
     p->nnode = (d == 2) ? N * N : N * N * N;
     p->npairs = pgb::unordered_pairs(p->nnode);
+    p->nclass = (long long)ipow((double)pgb::unordered_pairs(N), d);
     p->fast_gamma = (p->gamma == 0.0) ? 0 : (p->gamma == 1.0) ? 1 : (p->gamma == 0.5) ? 2 : 3;
     p->Bconst = 1.0 / (d == 2 ? 2.0 * kPi : 4.0 * kPi);
     p->ang.n = o.angular_terms;
@@ -150,6 +151,15 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         p->spread_threads = std::max(128, std::min(max_threads, t));
     }
     if (p->nslab > 1 && o.spread_threads <= 0) p->spread_threads = max_threads;  // the queues were sized for it
+    if (p->nslab == 1 && o.spread_threads <= 0) {
+        // small plans: blocks no larger than it takes for every SM to have one (each thread then
+        // owns one class; 1024-thread blocks would keep 18 of 152 SMs busy for 2D N = 16, whose
+        // spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks of 1024 with a
+        // point set per pair)
+        const long long per_block = (p->nclass + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
+        const int small = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
+        p->spread_threads = std::min(p->spread_threads, small);
+    }
     if (p->spread_threads % 32 || p->spread_threads > max_threads)
         return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", max_threads);
     if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32) > qbytes)
@@ -169,7 +179,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     per_sm = std::max(per_sm, 1);
     long long blocks = (long long)prop.multiProcessorCount * per_sm;
     blocks = std::max<long long>(blocks / p->nslab, 1) * p->nslab;
-    const long long need = ((p->npairs + p->spread_threads - 1) / p->spread_threads) * p->nslab;
+    const long long need = ((p->nclass + p->spread_threads - 1) / p->spread_threads) * p->nslab;
     blocks = std::min(blocks, need);
     p->spread_blocks = (int)blocks;
     // the pair schedule permutes thread starts by a multiplier prime to every smaller count
@@ -194,7 +204,8 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.M = M;
     ka.r = p->r;
     ka.nnode = p->nnode;
-    ka.npairs = p->npairs;
+    ka.naxp = (int)pgb::unordered_pairs(N);
+    ka.nclass = p->nclass;
     ka.n = p->n;
     ka.nf = p->nf;
     ka.rows_per_slab = p->rows_per_slab;

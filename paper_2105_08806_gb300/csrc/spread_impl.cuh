@@ -3,7 +3,7 @@
 // Fused post-collision point generation + exponential-of-semicircle spreading onto
 // the folded cosine grid (Section 4.2, Eq. num_fast_k and Eq. nufft).
 //
-// One thread owns one node pair (i, j) and walks the M sphere points sigma_m:
+// One thread owns one class of node pairs (PairData: the pairs (i, j) that share their points) and walks the M sphere points sigma_m:
 //   v'     = (v_i + v_j)/2 + |v_i - v_j| sigma_m / 2
 //   z_l    = arccos(xi(v'_l))                     angle of the l-th mapped coordinate
 //   q      = a_i a_j B(|v_i - v_j|) w_m prod_l mu(xi(v'_l))^-2
@@ -309,33 +309,44 @@ __device__ __forceinline__ void axis_weights_f32(const SpreadArgs &p, float X, f
     }
 }
 
-// Row shear of the pair numbering (load_pair); t K stays below 2^32 for every node count a plan
-// accepts (t <= nnode/2 <= 2^21).
+// Row shear of the class numbering (PairCursor).
 constexpr unsigned kPairShear = 1597u;
 
+// Node pairs in classes.  A pair (i, j) adds M points around its centre (v_i + v_j)/2 at the radius
+// |v_i - v_j|/2.  Exchanging the two nodes' components along any subset of axes changes neither --
+// per axis the centre and the squared difference are symmetric -- so all 2^d ordered pairs of one
+// class {i_0, j_0} x ... x {i_{d-1}, j_{d-1}} (an unordered pair of node indices per axis) add the
+// same M points (for any sphere set), and each class is spread once with the sum of their strengths:
+//   q = B(|v_i - v_j|) w_m prod mu^-2 . 2 prod_l (i_l == j_l ? 1/2 : 1) . sum_o a_{i(o)} a_{j(o)}
+// over the 2^(d-1) ways o to exchange axes 0..d-2 (exchanging every axis swaps i and j: the factor
+// 2; an axis with i_l == j_l would count its two equal ways twice: the factor 1/2).  That is N^4/4
+// point sets in 2D and N^6/8 in 3D, where one per unordered pair {i, j} is N^4/2 and N^6/2: the
+// spreading, which is all but a few percent of an evaluation, halves in 2D and quarters in 3D, and
+// each strength is rounded once for the class instead of once per pair.
+// Measured, one evaluation, one point set per unordered pair -> per class: 2D hard spheres N = 64,
+// M = 32 FP32 2.39 -> 1.47 ms, FP64 223 -> 117 ms; 3D Maxwell N = 16, M = 32 FP32 21.6 -> 10.7 ms;
+// 3D FP64 N = 11, M = 16 140 -> 46 ms.
 template <typename T, int D>
 struct PairData {
-    T cen[D];  // (v_i + v_j)/2
-    T rad;     // |v_i - v_j|/2
-    T base;    // a_i a_j B(|v_i - v_j|)
-    T mult;    // 2 for i != j (the pair stands for (i, j) and (j, i)), 1 for i == j
-    T dir[D];  // (v_i - v_j)/|v_i - v_j| (0 for i == j): cos theta = dir . sigma_m
+    T cen[D];            // (v_i + v_j)/2
+    T rad;               // |v_i - v_j|/2
+    T base;              // VHS: B sum_o a_{i(o)} a_{j(o)}; angular kernels: 1
+    T sabs;              // B sum_o |a_{i(o)} a_{j(o)}|
+    T mult;              // 2 prod_l (i_l == j_l ? 1/2 : 1)
+    T x[1 << (D - 1)];   // angular kernels: B a_{i(o)} a_{j(o)}, bit l of o: axis l exchanged
+    T dir[D];            // angular kernels: |v_i - v_j|^-1 (v_i - v_j), o = 0 (0 for i == j)
 };
 
-// Unordered node pairs.  Swapping i and j keeps the centre (v_i + v_j)/2, the radius
-// |v_i - v_j|/2 and the strength a_i a_j B(|v_i - v_j|) w_m, so (i, j) and (j, i) add the same
-// M points with the same weights: each unordered pair is spread once with twice the strength.
-// Numbering: pair pr = t nnode + u is (i, (i + t) mod nnode) with i = (u + t K) mod nnode, offsets
-// t = 0..floor(nnode/2); t = 0 is the diagonal (multiplicity 1) and, for even nnode, the row
-// t = nnode/2 stops at u = nnode/2 - 1 (its other half repeats the same pairs) and is not sheared:
-// unordered_pairs(nnode) in all.  The shear by K = kPairShear per row is a bijection of each row; it
-// makes a lane that strides through the pairs by a multiple of nnode (the single-plan launches
-// stride by SMs x threads, often a multiple of N^d) visit every node i instead of one, so the
-// lanes of a warp meet the negligible pairs of the tails of f at the same rate.
+// Numbering: an axis has naxp = N (N + 1)/2 unordered pairs p = t N + u <-> {u, (u + t) mod N}
+// (t = 0 the equal ones; for even N the row t = N/2 stops at u = N/2 - 1), and class pr is
+// (row t, column u) with t = pr / naxp numbering the pairs of the leading axes and the last axis'
+// pair i = (u + t K) mod naxp sheared by K = kPairShear per row.  The shear is a bijection of each
+// row; it makes a lane that strides through the classes by a multiple of naxp visit every pair
+// of the last axis, so the lanes of a warp meet the negligible classes of the tails of f at the
+// same rate.
 
-// A position in the pair numbering, advanced by a fixed stride without divisions: pr = t nnode + u
-// and the sheared first node i = (u + t K) mod nnode.  A stride of dt nnode + du moves i by
-// di = (du + dt K) mod nnode, and by K mod nnode more when u wraps.
+// A position in the numbering, advanced by a fixed stride without divisions: a stride of
+// dt naxp + du moves i by di = (du + dt K) mod naxp, and by K mod naxp more when u wraps.
 struct PairCursor {
     long long pr;
     int t, u, i;
@@ -349,9 +360,9 @@ __device__ __forceinline__ PairCursor pair_cursor(const SpreadArgs &p, long long
 {
     PairCursor c;
     c.pr = pr;
-    c.t = (int)(pr / p.nnode);
-    c.u = (int)(pr - (long long)c.t * p.nnode);
-    c.i = (int)(((long long)c.u + (long long)c.t * kPairShear) % p.nnode);
+    c.t = (int)(pr / p.naxp);
+    c.u = (int)(pr - (long long)c.t * p.naxp);
+    c.i = (int)(((long long)c.u + (long long)c.t * kPairShear) % p.naxp);
     return c;
 }
 
@@ -359,71 +370,83 @@ __device__ __forceinline__ PairStep pair_step(const SpreadArgs &p, long long str
 {
     PairStep s;
     s.d = stride;
-    s.dt = (int)(stride / p.nnode);
-    s.du = (int)(stride - (long long)s.dt * p.nnode);
-    s.di = (int)(((long long)s.du + (long long)s.dt * kPairShear) % p.nnode);
-    s.dk = (int)(kPairShear % p.nnode);
+    s.dt = (int)(stride / p.naxp);
+    s.du = (int)(stride - (long long)s.dt * p.naxp);
+    s.di = (int)(((long long)s.du + (long long)s.dt * kPairShear) % p.naxp);
+    s.dk = (int)(kPairShear % p.naxp);
     return s;
 }
 
 __device__ __forceinline__ void pair_advance(const SpreadArgs &p, PairCursor &c, const PairStep &s)
 {
-    const int nnode = p.nnode;
+    const int naxp = p.naxp;
     c.pr += s.d;
     c.t += s.dt;
     c.u += s.du;
     c.i += s.di;
-    if (c.i >= nnode) c.i -= nnode;
-    if (c.u >= nnode) {
-        c.u -= nnode;
+    if (c.i >= naxp) c.i -= naxp;
+    if (c.u >= naxp) {
+        c.u -= naxp;
         c.t += 1;
         c.i += s.dk;
-        if (c.i >= nnode) c.i -= nnode;
+        if (c.i >= naxp) c.i -= naxp;
     }
 }
 
-// Axis indices of node k (C order, axis D-1 fastest) from float quotients: (k + 1/2)/N lies at
-// least 1/(2N) from an integer and its FP32 value within 2^-23 (k + 1/2)/N < 1/(4N) of it for
-// k < 2^21 (every node count a plan allows), so the truncation is the exact quotient.
-template <int D>
-__device__ __forceinline__ void node_axes(int k, int N, float invN, int (&ax)[D])
-{
-#pragma unroll
-    for (int l = D - 1; l > 0; --l) {
-        const int q = __float2int_rz(((float)k + 0.5f) * invN);
-        ax[l] = k - q * N;
-        k = q;
-    }
-    ax[0] = k;
-}
+// Row t = p / N of axis pair p = t N + u from a float quotient: (p + 1/2)/N lies at least 1/(2N)
+// from an integer and its FP32 value within 2^-23 (p + 1/2)/N < 1/(4N) of it for p < 2^21 (every
+// axis pair of a plan: N <= 512), so the truncation is the exact quotient.
+__device__ __forceinline__ int axis_pair_row(int p, float invN) { return __float2int_rz(((float)p + 0.5f) * invN); }
 
-// Load the pair at cursor c; false when its strength is zero.  ANG: also the unit direction
-// (angular kernels).
+// Load the class at cursor c; false when its strength is zero.  ANG: angular kernels.
 template <typename T, int D, bool ANG = false>
 __device__ __forceinline__ bool load_pair(const SpreadArgs &p, const PairCursor &c, PairData<T, D> &P)
 {
-    const int nnode = p.nnode, N = p.N;
-    const int t = c.t;
-    const int i = (2 * t != nnode) ? c.i : c.u;  // the half row t = nnode/2 is not sheared
-    int j = i + t;
-    if (j >= nnode) j -= nnode;
-    P.mult = t ? T(2) : T(1);
+    constexpr int NO = 1 << (D - 1);
+    const int N = p.N;
+    int ap[D];
+    ap[D - 1] = c.i;
+    if constexpr (D == 2) {
+        ap[0] = c.t;
+    } else {
+        ap[0] = c.t / p.naxp;
+        ap[1] = c.t - ap[0] * p.naxp;
+    }
+    const float invN = 1.0f / (float)N;
+    int ni[D], nj[D];
+    P.mult = T(2);
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+        const int t = axis_pair_row(ap[l], invN);
+        ni[l] = ap[l] - t * N;
+        nj[l] = ni[l] + t;
+        if (nj[l] >= N) nj[l] -= N;
+        if (t == 0) P.mult *= T(0.5);
+    }
     const T *vnode = static_cast<const T *>(p.vnode);
     const T *acoef = static_cast<const T *>(p.a);
-    const T aij = acoef[i] * acoef[j];
-    if (aij == T(0)) return false;
-    const float invN = 1.0f / (float)N;
-    int ai[D], aj[D];
-    node_axes<D>(i, N, invN, ai);
-    node_axes<D>(j, N, invN, aj);
+    T x[NO], sum = T(0), sabs = T(0);
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+        int I = 0, J = 0;
+#pragma unroll
+        for (int l = 0; l < D; ++l) {
+            const bool ex = (o >> l) & 1;
+            I = I * N + (ex ? nj[l] : ni[l]);
+            J = J * N + (ex ? ni[l] : nj[l]);
+        }
+        x[o] = acoef[I] * acoef[J];
+        sum += x[o];
+        sabs += fabs(x[o]);
+    }
+    if (sabs == T(0)) return false;
     T g2 = T(0);
 #pragma unroll
     for (int l = D - 1; l >= 0; --l) {
-        const int ni = ai[l], nj = aj[l];
-        const T vi = vnode[ni], vj = vnode[nj];
+        const T vi = vnode[ni[l]], vj = vnode[nj[l]];
         T dl = vi - vj, sl = vi + vj;
         if constexpr (sizeof(T) == 4) {  // FP32 nodes carry their rounding in a second term
-            const float li = p.vnode_lo[ni], lj = p.vnode_lo[nj];
+            const float li = p.vnode_lo[ni[l]], lj = p.vnode_lo[nj[l]];
             dl += li - lj;
             sl += li + lj;
         }
@@ -445,18 +468,26 @@ __device__ __forceinline__ bool load_pair(const SpreadArgs &p, const PairCursor 
     case 2: B = K.Bconst * Fn<T>::sqrt_(g); break;
     default: B = K.Bconst * Fn<T>::pow_(g, K.gamma); break;
     }
-    P.base = aij * B;
+    P.sabs = sabs * B;
     P.rad = T(0.5) * g;
-    return P.base != T(0);
+    if constexpr (ANG) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o) P.x[o] = x[o] * B;
+        P.base = T(1);
+        return P.sabs != T(0);
+    } else {
+        P.base = sum * B;
+        return P.base != T(0);
+    }
 }
 
-// U >= sum_m |q_m|: |base| W_sigma prod_l mu^-2(|c_l| + rad), since |v'_l| <= |c_l| + rad and
-// mu^-2 grows with |v|.
+// sum_m |q_m| <= (strength) x this, for any share of the class' strength: W_sigma prod_l
+// mu^-2(|c_l| + rad), since |v'_l| <= |c_l| + rad and mu^-2 grows with |v|.
 template <typename T, int D>
 __device__ __forceinline__ T pair_bound(const SpreadArgs &p, const PairData<T, D> &P)
 {
     const TypedConsts<T> &K = kconst<T>(p);
-    T U = fabs(P.base) * K.Wang;
+    T U = K.Wang;
 #pragma unroll
     for (int l = 0; l < D; ++l) {
         const T R = fabs(P.cen[l]) + P.rad;
@@ -617,8 +648,9 @@ struct Point<double, D> {
     double x[D], q;
 };
 
-// Strength of point m of pair P before the map factors: qbase w_m, times the even part of
-// b(cos theta) for angular kernels (Horner in cos^2 theta).
+// Strength of point m of class P before the map factors: qbase w_m, for angular kernels times
+// sum_o x_o b_e(cos theta_o) with the even part b_e of b (Horner in cos^2 theta) and the direction
+// of the exchanged pair o (the components of its exchanged axes change sign).
 template <typename T, int D, bool ANG>
 __device__ __forceinline__ T point_base(const SpreadArgs &p, const PairData<T, D> &P, T qbase, int m)
 {
@@ -627,13 +659,21 @@ __device__ __forceinline__ T point_base(const SpreadArgs &p, const PairData<T, D
     T q = qbase * wsig[m];
     if constexpr (ANG) {
         const TypedConsts<T> &K = kconst<T>(p);
-        T c = T(0);
+        T s = T(0);
 #pragma unroll
-        for (int l = 0; l < D; ++l) c += P.dir[l] * sig[m * D + l];
-        const T c2 = c * c;
-        T be = K.ang_even[p.nang_even - 1];
-        for (int k = p.nang_even - 2; k >= 0; --k) be = be * c2 + K.ang_even[k];
-        q *= be;
+        for (int o = 0; o < (1 << (D - 1)); ++o) {
+            T c = T(0);
+#pragma unroll
+            for (int l = 0; l < D; ++l) {
+                const T t = P.dir[l] * sig[m * D + l];
+                c += ((o >> l) & 1) ? -t : t;
+            }
+            const T c2 = c * c;
+            T be = K.ang_even[p.nang_even - 1];
+            for (int k = p.nang_even - 2; k >= 0; --k) be = be * c2 + K.ang_even[k];
+            s += P.x[o] * be;
+        }
+        q *= s;
     }
     return q;
 }
@@ -943,10 +983,11 @@ __device__ __forceinline__ void spread_point_any(const SpreadArgs &p, const Poin
     else spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
 }
 
-// Advance the cursor c (in steps of st, below `end`) to this lane's next pair that is not negligible:
-// a loaded pair with non-zero strength, a strength bound not below the screening threshold tau
-// (0: no screening), and a bound Ut >= floor_q on every point's |q| in tile units.  On success
-// P.base is multiplied by the pair's multiplicity; false when no pair is left.
+// Advance the cursor c (in steps of st, below `end`) to this lane's next class that is not
+// negligible: non-zero strength, not below the screening threshold tau (0: no screening; the sum
+// of its pairs' bounds is compared, so every pair skipped is below tau), and a bound Ut >= floor_q
+// on every point's |q| in tile units.  On success P.base is multiplied by the class' multiplicity;
+// false when no class is left.
 template <typename T, int D, bool ANG>
 __device__ __forceinline__ bool next_pair(const SpreadArgs &p, PairCursor &c, long long end, const PairStep &st, T sc,
                                           T tau, T floor_q, PairData<T, D> &P)
@@ -954,8 +995,8 @@ __device__ __forceinline__ bool next_pair(const SpreadArgs &p, PairCursor &c, lo
     for (; c.pr < end; pair_advance(p, c, st)) {
         if (!load_pair<T, D, ANG>(p, c, P)) continue;
         const T U = pair_bound<T, D>(p, P);
-        if (tau > T(0) && U < tau) continue;
-        if (U * P.mult * sc * kconst<T>(p).wmax < floor_q) continue;
+        if (tau > T(0) && P.sabs * U < tau) continue;
+        if ((ANG ? P.sabs : fabs(P.base)) * U * P.mult * sc * kconst<T>(p).wmax < floor_q) continue;
         P.base *= P.mult;
         return true;
     }
@@ -971,8 +1012,11 @@ __device__ __forceinline__ void zero_pair(PairData<T, D> &P)
         P.cen[l] = T(0);
         P.dir[l] = T(0);
     }
+#pragma unroll
+    for (int o = 0; o < (1 << (D - 1)); ++o) P.x[o] = T(0);
     P.rad = T(0);
     P.base = T(0);
+    P.sabs = T(0);
     P.mult = T(0);
 }
 
@@ -1256,15 +1300,15 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     if (p.nslab > 1) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes((size_t)p.rows_per_slab * G.plane, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true);
-        spread_pairs_queued<float, D, W, SplitTile, ANG>(p, first, p.npairs, nthr, sc, tau, kNegligibleF32, tile,
+        spread_pairs_queued<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile,
                                                           G.row_lo, G.nrows, G.plane, buf);
     } else if (p.queued) {  // one slab: the queues only compact the points that add something
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes(G.ncell, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true);
-        spread_pairs_queued<float, D, W, SplitTile, ANG, false>(p, first, p.npairs, nthr, sc, tau, kNegligibleF32,
+        spread_pairs_queued<float, D, W, SplitTile, ANG, false>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32,
                                                                  tile, 0, G.nrows, G.plane, buf);
     } else {
-        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.npairs, nthr, sc, tau, kNegligibleF32, tile, G.row_lo,
+        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile, G.row_lo,
                                                    G.nrows, G.plane);
     }
     __syncthreads();
@@ -1298,18 +1342,18 @@ __global__ void __launch_bounds__(max_threads_f64(D), 1) k_spread_f64(const __gr
     const int Eg = global_exponent(Bnd);
     const double tau = *p.tau;
     const double sc = ldexp(1.0, Eg);  // strengths in grid units
-    // pairs whose summed strength bounds stay below 2^-64 B are skipped (per-point bound below
-    // floor_q, and at most npairs pairs): 2^-3 grid units at most in all
-    const double floor_q = ldexp(Bnd, Eg - 64) * p.cd.wmax / (double)p.npairs;
+    // classes whose summed strength bounds stay below 2^-64 B are skipped (per-point bound below
+    // floor_q, and at most nclass classes): 2^-3 grid units at most in all
+    const double floor_q = ldexp(Bnd, Eg - 64) * p.cd.wmax / (double)p.nclass;
     long long first, nthr;
     pair_schedule(p, first, nthr);
     if (p.nslab > 1) {
         double *buf = reinterpret_cast<double *>(smem_raw + tile_bytes(tile_cells, false)) +
                       (threadIdx.x >> 5) * 32 * spread_queue_values(D, false);
-        spread_pairs_queued<double, D, W, WideTile, ANG>(p, first, p.npairs, nthr, sc, tau, floor_q, tile, G.row_lo,
+        spread_pairs_queued<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
                                                           G.nrows, G.plane, buf);
     } else {
-        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.npairs, nthr, sc, tau, floor_q, tile, G.row_lo,
+        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
                                                    G.nrows, G.plane);
     }
     __syncthreads();
