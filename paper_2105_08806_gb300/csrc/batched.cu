@@ -430,11 +430,12 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
         const long long p1 = min(p0 + (long long)s_cd.chunk, s_cd.nclass);
         const long long first = p0 + (long long)lane * nwarp + warp;
         if constexpr (F32) {
-            // the warp's queue compacts the points that add something (FP32 points below 0.1 tile
-            // unit add exactly zero), so that every lane spreads a real point
             float *buf = reinterpret_cast<float *>(smem_raw + b.queue_off) + warp * 32 * spread_queue_values(D, true);
-            spread_pairs_queued<T, D, W, SplitTile, false, false>(sa, first, p1, blockDim.x, sc, tau, floor_q,
-                                                                   SplitTile{lo, carry}, 0, s_cd.nf, plane, buf);
+            if constexpr (D == 2)
+                spread_quads<W, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, s_cd.nf, plane, buf);
+            else  // the queue compacts the points that add something
+                spread_pairs_queued<T, D, W, SplitTile, false, false>(sa, first, p1, blockDim.x, sc, tau, floor_q,
+                                                                       SplitTile{lo, carry}, 0, s_cd.nf, plane, buf);
         } else
             spread_pairs<T, D, W, WideTile, false>(sa, first, p1, blockDim.x, sc, tau, floor_q, wt, 0,
                                                       s_cd.nf, plane);
@@ -888,22 +889,34 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
     B->static_smem =
         sizeof(pgb::CellDesc) + sizeof(pgb::SpreadArgs) + 64 + (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
     const size_t per_block_extra = B->static_smem + 1024 + prop.reservedSharedMemPerBlock;
-    if (batch_smem(*B, 128) + B->static_smem > prop.sharedMemPerBlockOptin) {
+    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::max_threads_f64(B->d);
+    const int accept_threads = f32 ? pgb::kAcceptThreadsF32 : max_threads;
+    // the smallest block the plan makes: 128 threads, fewer where the largest tile leaves less room
+    int min_threads = 128;
+    while (min_threads > 64 && batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
+        min_threads -= 32;
+    if (batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin) {
         set_error(PG_ERR_ARG, "largest cell's folded grid (%d cells) does not fit shared memory", max_cells_tile);
         free_plan(p);
         return nullptr;
     }
-    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::max_threads_f64(B->d);
-    int per_sm = (int)(prop.sharedMemPerMultiprocessor / (batch_smem(*B, 128) + per_block_extra));
+    int per_sm = (int)(prop.sharedMemPerMultiprocessor / (batch_smem(*B, min_threads) + per_block_extra));
     per_sm = std::max(per_sm, 1);
     if (o.spread_blocks_per_sm > 0) per_sm = std::min(per_sm, o.spread_blocks_per_sm);
-    B->spread_threads = (o.spread_threads > 0) ? o.spread_threads
-                                                : std::max(128, std::min(max_threads, (1024 / per_sm) / 32 * 32));
-    if (B->spread_threads % 32 || B->spread_threads > max_threads) {
-        set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", max_threads);
+    if (o.spread_threads > accept_threads || (o.spread_threads > 0 && o.spread_threads % 32)) {
+        set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
         free_plan(p);
         return nullptr;
     }
+    B->spread_threads = (o.spread_threads > 0) ? std::min(o.spread_threads, max_threads)
+                                                : std::max(min_threads, std::min(max_threads, (1024 / per_sm) / 32 * 32));
+    // fewer threads where the queues would not fit beside the tile (a block size that was asked for
+    // shrinks only when 20 bytes of queue per thread fit)
+    if (o.spread_threads <= 0 ||
+        B->tile_smem + (size_t)o.spread_threads * 20 + B->static_smem <= prop.sharedMemPerBlockOptin)
+        while (B->spread_threads > 32 &&
+               batch_smem(*B, B->spread_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
+            B->spread_threads -= 32;
     B->spread_smem = batch_smem(*B, B->spread_threads);
     if (B->spread_smem + B->static_smem > prop.sharedMemPerBlockOptin) {
         set_error(PG_ERR_ARG, "largest cell's folded grid (%d cells) and the queues of %d threads do not fit "

@@ -121,14 +121,18 @@ __device__ __forceinline__ const TypedConsts<T> &kconst(const SpreadArgs &a)
 // Unordered pairs of n things, equal ones included.
 __host__ __device__ inline long long unordered_pairs(long long nnode) { return nnode * (nnode + 1) / 2; }
 
-// Values per queued point of the slabbed spreading kernels: FP32 points keep each coordinate as
-// a cell and a fraction (2d + 1 floats with the strength), FP64 points d + 1 doubles.
-__host__ __device__ inline int spread_queue_values(int d, bool f32) { return f32 ? 2 * d + 1 : d + 1; }
-// Shared memory of the warp point queues of a slabbed spreading block of `threads` threads:
-// 32 points per warp.
-__host__ __device__ inline size_t spread_queue_bytes(int threads, int d, bool f32)
+// Values per slot of the spreading kernels' warp queues.  FP32, one slab: 2D a large quad (6) and a class
+// (4, angular kernels 8), 3D a point's velocity and strength.  FP32 slabs: a point's velocity, strength
+// and axis-0 coordinate (cell and fraction).  FP64: a point, d coordinates and its strength.
+__host__ __device__ constexpr int spread_queue_values(int d, bool f32, bool ang = false, bool slab = false)
 {
-    return (size_t)(threads / 32) * 32 * spread_queue_values(d, f32) * (f32 ? 4 : 8);
+    return !f32 ? d + 1 : slab ? d + 3 : d == 3 ? 4 : ang ? 14 : 10;
+}
+// Shared memory of the warp queues of a spreading block of `threads` threads: 32 slots per warp.
+__host__ __device__ constexpr size_t spread_queue_bytes(int threads, int d, bool f32, bool ang = false,
+                                                        bool slab = false)
+{
+    return (size_t)(threads / 32) * 32 * spread_queue_values(d, f32, ang, slab) * (f32 ? 4 : 8);
 }
 // Shared memory of a block tile of `cells` cells, rounded up to 16 bytes (the queues follow it):
 // FP32 tiles hold one 32-bit word per cell, FP64 tiles three (fraction, low and high words).
@@ -181,14 +185,19 @@ static_assert(kPolyCoefF64 >= ((kMaxWidthF64 + 1) / 2) * kernel_poly_terms(kMaxW
                   kPolyCoefF64 >= 6 * kernel_poly_terms(11),
               "kernel polynomial storage");
 constexpr int kMinWidth = 2;
-// Largest spreading block for each type (the kernels' launch bounds).
-constexpr int kMaxThreadsF32 = 1024;
+// Largest spreading block for each type (the kernels' launch bounds).  FP32: 640 threads with up to 96
+// registers (the 2D quads keep their weights of both columns and a row set in registers; at 1024
+// threads x 64 registers they spill: 768 batched cells 33.2 -> 31.6 ms, RK4 at N = 32 9.6 -> 8.4 ms, 2D
+// Maxwell N = 16 88 -> 84 us, 3D VHS N = 24 63.7 -> 62.4 ms with 640).  Options may ask for up to
+// kAcceptThreadsF32; a launch then has kMaxThreadsF32.
+constexpr int kMaxThreadsF32 = 640;
+constexpr int kAcceptThreadsF32 = 1024;
 // FP64: 2D kernels use up to 255 registers per thread, 3D kernels fit 128 (their per-point
 // spreading is out of line), so 3D blocks hold twice the threads (integer shared atomics whose
 // returned values feed the next step want many resident warps).
 __host__ __device__ constexpr int max_threads_f64(int d) { return d == 3 ? 512 : 256; }
 // Largest block of the batched FP32 spreading kernel.
-constexpr int kBatchThreadsF32 = 1024;
+constexpr int kBatchThreadsF32 = kMaxThreadsF32;
 
 // Three-axis shape of a C-order array; 2D arrays use e0 = 1.
 struct Dims3 {

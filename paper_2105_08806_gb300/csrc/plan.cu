@@ -117,18 +117,22 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     // block tiles: rows of (nf^(d-2) x ncol) cells, the last axis padded with unfolded columns
     const int cpad = pgb::tile_col_pad(p->w), ncol = p->nf + 2 * cpad;
     const size_t plane = (size_t)ipow(p->nf, d - 2) * ncol;
-    const bool f32 = (p->prec == PG_PREC_FP32);
+    const bool f32 = (p->prec == PG_PREC_FP32), ang = p->ang.n > 0;
     // leave room for the kernels' static shared memory (FP64: the kernel polynomial)
     // (and 16 bytes for rounding the tile up to 16 bytes)
     const size_t max_smem = prop.sharedMemPerBlockOptin - 1024 - 16 - (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
     const int max_threads = f32 ? pgb::kMaxThreadsF32 : pgb::max_threads_f64(d);
+    const int accept_threads = f32 ? pgb::kAcceptThreadsF32 : max_threads;
+    if (o.spread_threads > accept_threads || (o.spread_threads > 0 && o.spread_threads % 32))
+        return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
+    const int ask_threads = std::min(o.spread_threads, max_threads);  // <= 0: chosen here
     int rows_fit = (int)std::min<size_t>(p->nf, max_smem / (plane * elem));
     size_t qbytes = 0;
     if (rows_fit < p->nf) {
         // slabbed grid: the warps' point queues (one block per SM, max_threads threads unless
         // set) share the block's shared memory with the slab
-        const int thr = (o.spread_threads > 0) ? o.spread_threads : max_threads;
-        qbytes = pgb::spread_queue_bytes(thr, d, f32);
+        const int thr = (ask_threads > 0) ? ask_threads : max_threads;
+        qbytes = pgb::spread_queue_bytes(thr, d, f32, ang, true);
         rows_fit = (max_smem > qbytes) ? (int)std::min<size_t>(p->nf, (max_smem - qbytes) / (plane * elem)) : 0;
     }
     if (rows_fit < 1) return set_error(PG_ERR_ARG, "folded grid plane of %zu cells does not fit shared memory", plane);
@@ -138,11 +142,11 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     p->spread_smem = pgb::tile_bytes((size_t)p->rows_per_slab * plane, f32) + (p->nslab > 1 ? qbytes : 0);
     int per_sm = (int)(prop.sharedMemPerMultiprocessor / (p->spread_smem + 1024 + prop.reservedSharedMemPerBlock));
     per_sm = std::max(per_sm, 1);
-    if (o.spread_threads > 0) {
-        p->spread_threads = o.spread_threads;
+    if (ask_threads > 0) {
+        p->spread_threads = ask_threads;
     } else if (f32) {
-        // FP32: one block of 1024 threads per SM (measured fastest; more, smaller blocks
-        // multiply the tile clears and flushes)
+        // FP32: one block per SM (measured fastest; more, smaller blocks multiply the tile
+        // clears and flushes)
         p->spread_threads = max_threads;
         per_sm = 1;
     } else {
@@ -150,8 +154,8 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         int t = (1024 / per_sm) / 32 * 32;
         p->spread_threads = std::max(128, std::min(max_threads, t));
     }
-    if (p->nslab > 1 && o.spread_threads <= 0) p->spread_threads = max_threads;  // the queues were sized for it
-    if (p->nslab == 1 && o.spread_threads <= 0) {
+    if (p->nslab > 1 && ask_threads <= 0) p->spread_threads = max_threads;  // the queues were sized for it
+    if (p->nslab == 1 && ask_threads <= 0) {
         // small plans: blocks no larger than it takes for every SM to have one (each thread then
         // owns one class; 1024-thread blocks would keep 18 of 152 SMs busy for 2D N = 16, whose
         // spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks of 1024 with a
@@ -160,15 +164,17 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         const int small = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
         p->spread_threads = std::min(p->spread_threads, small);
     }
-    if (p->spread_threads % 32 || p->spread_threads > max_threads)
-        return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", max_threads);
-    if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32) > qbytes)
+    if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32, ang, true) > qbytes)
         return set_error(PG_ERR_STATE, "internal: point queues larger than reserved");
-    // FP32 one-slab grids: the warps also queue their points that add something and spread full
-    // queues (every lane busy), when the queues fit beside the tile
+    // FP32 one-slab grids: the warps' queues follow the tile (2D: large quads; 3D: the points that add
+    // something) when they fit beside it, with fewer threads if need be
     p->queued = 0;
     if (f32 && p->nslab == 1) {
-        const size_t qq = pgb::spread_queue_bytes(p->spread_threads, d, true);
+        if (ask_threads <= 0)
+            while (p->spread_threads > 128 &&
+                   p->spread_smem + pgb::spread_queue_bytes(p->spread_threads, d, true, ang) > max_smem)
+                p->spread_threads -= 128;
+        const size_t qq = pgb::spread_queue_bytes(p->spread_threads, d, true, ang);
         if (p->spread_smem + qq <= max_smem) {
             p->queued = 1;
             p->spread_smem += qq;

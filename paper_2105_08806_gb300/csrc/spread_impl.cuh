@@ -514,22 +514,15 @@ __device__ __forceinline__ int tile_to_grid_cell(int c, int D, int nf, int ncol,
 // direction is the addend's sign, which is that of the point's strength (every kernel weight is
 // >= 0), so it is one value per point.  Atomic additions on a word are serialised, so every wrap
 // is that of exactly one addition and word + 2^32 carry is the exact sum in any order.
-// Contributions of 2^31 units or more split into a word part and a multiple of 2^32 added to the
-// carry directly.  A block's partial sum in one cell stays below B 2^Et = 2^(61 - bits), so
+// Contributions of larger points are scaled integers v 2^s: their low word goes to the word, the rest
+// to the carry directly.  A block's partial sum in one cell stays below B 2^Et = 2^(61 - bits), so
 // carries are rare (about B 2^Et / 2^32 in a whole evaluation) and a counter stays below
 // 2^(29 - bits) in magnitude (bits = tile_bits(d)).
 
 struct SplitTile {
     int *lo;     // tile words (shared memory)
     int *carry;  // this block's carry counters (global memory, same layout)
-    // v of sign d (or zero)
-    __device__ __forceinline__ void add_int(int c, int v, int d) const
-    {
-        const int o = atomicAdd(lo + c, v);
-        const int r = (int)((unsigned)o + (unsigned)v);
-        if (((o ^ r) & (v ^ r)) < 0) atomicAdd(carry + c, d);
-    }
-    // The same addition for a run of consecutive cells: the wrap of this addition is shifted
+    // One addition of a run of consecutive cells: its wrap is shifted
     // into `mask` (one funnel shift) and the carries of the run are added afterwards, in
     // add_carries, where the mask is rarely non-zero.
     __device__ __forceinline__ unsigned add_int_run(int c, int v, unsigned mask) const
@@ -547,18 +540,15 @@ struct SplitTile {
             mask &= mask - 1;
         }
     }
-    __device__ __forceinline__ void add64(int c, long long x) const
+    // v 2^s for |v| < 2^31, 0 <= s < 32: its low word, signed, to the word, the rest to the carry counter
+    __device__ __forceinline__ void add_scaled(int c, int v, int s) const
     {
-        const int xl = (int)(unsigned)(unsigned long long)x;  // low word, signed
-        const long long xh = (x - xl) >> 32;                   // exact: x - xl is a multiple of 2^32
-        add_int(c, xl, xl < 0 ? -1 : 1);
-        if (xh) atomicAdd(carry + c, (int)xh);
-    }
-    // any x (zero contributions are added too: a branch around them costs more than the atomic)
-    __device__ __forceinline__ void add(int c, float x) const
-    {
-        if (fabsf(x) < 2147483648.0f) add_int(c, __float2int_rn(x), x < 0.0f ? -1 : 1);
-        else add64(c, __float2ll_rn(x));
+        const int l = (int)((unsigned)v << s);
+        const int h = (int)__funnelshift_l((unsigned)v, (unsigned)(v >> 31), s) - (l >> 31);
+        const int o = atomicAdd(lo + c, l);
+        const int r = (int)((unsigned)o + (unsigned)l);
+        const int k = h + ((((o ^ r) & (l ^ r)) < 0) ? (l < 0 ? -1 : 1) : 0);
+        if (k) atomicAdd(carry + c, k);
     }
     // the cell's sum in tile units
     __device__ __forceinline__ long long value(int c) const { return (long long)carry[c] * 4294967296LL + lo[c]; }
@@ -744,11 +734,11 @@ __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T
 
 // ---- FP32 points
 //
-// Kinds of FP32 point: kInt -- |q| < 2^29 tile units (integer products); kLarge -- any q.
+// Kinds of FP32 point: kInt -- |q| < 2^29 tile units; kLarge -- any q.
 constexpr int kInt = 0, kLarge = 1;
-// Points below this many tile units take the integer products; points below kNegligibleF32 add
-// exactly zero (4 q psi rounds to 0 for every row) and are skipped, and so are pairs whose points
-// all stay below it.
+// Points below this many tile units take the integer products as they are; points below
+// kNegligibleF32 add exactly zero (4 q psi rounds to 0 for every row) and are skipped, and so are
+// pairs whose points all stay below it.
 constexpr float kIntLimitF32 = 536870912.0f;  // 2^29
 constexpr float kNegligibleF32 = 0.1f;
 
@@ -758,13 +748,16 @@ __device__ __forceinline__ int mulhi_rn(int a, int b)
     return (int)(((long long)a * (long long)b + 0x80000000LL) >> 32);
 }
 
-// Add the w^d contributions q psi_a psi_b psi_c of one FP32 point to the block tile.  kInt: the
-// column factors 2^30 psi_c and, per row, 4 q psi_a (psi_b) are rounded to integers, and a
-// contribution is mulhi_rn of the two (at most about one tile unit of rounding).  kLarge: the
-// product is formed in FP32 and rounded to the tile unit.  SLAB: the tile holds a slab of the grid's
-// rows and rows outside it are skipped; otherwise it holds every row (row_lo = 0, nrows = n/2 + 1).
-// 3D points loop over their axis-0 rows (computing that row's kernel value in the loop) so that
-// the unrolled code stays small.
+// Add the w^d contributions q psi_a psi_b psi_c of one FP32 point to the block tile: the column
+// factors 2^30 psi_c and, per row, 4 q psi_a (psi_b) are rounded to integers, and a contribution is
+// mulhi_rn of the two (at most about one tile unit of rounding).  kLarge: the same with q 2^-s in
+// [2^28, 2^29) for the point's own s, i.e. rounded to 2^s tile units, 2^-28 of the point's strength
+// (an FP32 product is rounded to 2^-24 of the contribution, which is more over a point's taps; and
+// the float path that formed it took twice the instructions: 768 batched cells, where points of 2^29
+// units are common, 43.9 -> 33.2 ms).
+// SLAB: the tile holds a slab of the grid's rows and rows outside it are skipped; otherwise it holds
+// every row (row_lo = 0, nrows = n/2 + 1).  3D points loop over their axis-0 rows (computing that
+// row's kernel value in the loop) so that the unrolled code stays small.
 template <int D, int W, int KIND, bool SLAB>
 __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Point<float, D> &pt,
                                                  const SplitTile &tile, int row_lo, int nrows, int plane)
@@ -785,84 +778,50 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
 #pragma unroll
         for (int b = 0; b < W; ++b) c1[b] = c1[b] * p.ncol + cb;
     }
-    if constexpr (KIND == kInt) {
-        const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
-        const float q4 = 4.0f * q;
-        const float bias30 = 30.0f - bl;
-        int wi[W];
+    const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
+    float q4 = 4.0f * q;
+    int sc = 0;
+    if constexpr (KIND == kLarge) {
+        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
+        q4 *= __int_as_float((127 - sc) << 23);  // 2^-sc
+    }
+    const float bias30 = 30.0f - bl;
+    int wi[W];
 #pragma unroll
-        for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_f32(fmaf((float)c, h2, tl0), bl, bias30));
-        if constexpr (D == 2) {
+    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_f32(fmaf((float)c, h2, tl0), bl, bias30));
+    auto run = [&](int line, int rq) {
+        if constexpr (KIND == kLarge) {
 #pragma unroll
-            for (int a = 0; a < W; ++a) {
-                int r = fold_cell(s0 + a, p.n, simple);
-                if constexpr (SLAB) {
-                    r -= row_lo;
-                    if ((unsigned)r >= (unsigned)nrows) continue;
-                }
-                const int rq = __float2int_rn(q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl));
-                const int row = r * plane + cb;
-                unsigned wraps = 0u;
-#pragma unroll
-                for (int c = 0; c < W; ++c) wraps = tile.add_int_run(row + c, mulhi_rn(rq, wi[c]), wraps);
-                if (wraps) tile.add_carries(row, W, wraps, sg);
-            }
+            for (int c = 0; c < W; ++c) tile.add_scaled(line + c, mulhi_rn(rq, wi[c]), sc);
         } else {
-#pragma unroll 1
-            for (int a = 0; a < W; ++a) {
-                int r = fold_cell(s0 + a, p.n, simple);
-                if constexpr (SLAB) {
-                    r -= row_lo;
-                    if ((unsigned)r >= (unsigned)nrows) continue;
-                }
-                const float qa = q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl);
-                const int row = r * plane;
+            unsigned wraps = 0u;
 #pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const int rq = __float2int_rn(qa * w1[b]);
-                    const int line = row + c1[b];
-                    unsigned wraps = 0u;
+            for (int c = 0; c < W; ++c) wraps = tile.add_int_run(line + c, mulhi_rn(rq, wi[c]), wraps);
+            if (wraps) tile.add_carries(line, W, wraps, sg);
+        }
+    };
+    if constexpr (D == 2) {
 #pragma unroll
-                    for (int c = 0; c < W; ++c) wraps = tile.add_int_run(line + c, mulhi_rn(rq, wi[c]), wraps);
-                    if (wraps) tile.add_carries(line, W, wraps, sg);
-                }
+        for (int a = 0; a < W; ++a) {
+            int r = fold_cell(s0 + a, p.n, simple);
+            if constexpr (SLAB) {
+                r -= row_lo;
+                if ((unsigned)r >= (unsigned)nrows) continue;
             }
+            run(r * plane + cb, __float2int_rn(q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl)));
         }
     } else {
-        float wl[W];
-#pragma unroll
-        for (int c = 0; c < W; ++c) wl[c] = es_f32(fmaf((float)c, h2, tl0), bl, -bl);
-        if constexpr (D == 2) {
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                int r = fold_cell(s0 + a, p.n, simple);
-                if constexpr (SLAB) {
-                    r -= row_lo;
-                    if ((unsigned)r >= (unsigned)nrows) continue;
-                }
-                const float qa = q * es_f32(fmaf((float)a, h2, t00), bl, -bl);
-                const int row = r * plane + cb;
-#pragma unroll
-                for (int c = 0; c < W; ++c) tile.add(row + c, qa * wl[c]);
-            }
-        } else {
 #pragma unroll 1
-            for (int a = 0; a < W; ++a) {
-                int r = fold_cell(s0 + a, p.n, simple);
-                if constexpr (SLAB) {
-                    r -= row_lo;
-                    if ((unsigned)r >= (unsigned)nrows) continue;
-                }
-                const float qa = q * es_f32(fmaf((float)a, h2, t00), bl, -bl);
-                const int row = r * plane;
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float qab = qa * w1[b];
-                    const int line = row + c1[b];
-#pragma unroll
-                    for (int c = 0; c < W; ++c) tile.add(line + c, qab * wl[c]);
-                }
+        for (int a = 0; a < W; ++a) {
+            int r = fold_cell(s0 + a, p.n, simple);
+            if constexpr (SLAB) {
+                r -= row_lo;
+                if ((unsigned)r >= (unsigned)nrows) continue;
             }
+            const float qa = q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl);
+            const int row = r * plane;
+#pragma unroll
+            for (int b = 0; b < W; ++b) run(row + c1[b], __float2int_rn(qa * w1[b]));
         }
     }
 }
@@ -983,23 +942,30 @@ __device__ __forceinline__ void spread_point_any(const SpreadArgs &p, const Poin
     else spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
 }
 
+// Load the class at cursor c; whether it is not negligible: non-zero strength, not below the
+// screening threshold tau (0: no screening; the sum of its pairs' bounds is compared, so every pair
+// skipped is below tau), and a bound Ut >= floor_q on every point's |q| in tile units.  On success
+// P.base is multiplied by the class' multiplicity.
+template <typename T, int D, bool ANG>
+__device__ __forceinline__ bool class_passes(const SpreadArgs &p, const PairCursor &c, T sc, T tau, T floor_q,
+                                             PairData<T, D> &P)
+{
+    if (!load_pair<T, D, ANG>(p, c, P)) return false;
+    const T U = pair_bound<T, D>(p, P);
+    if (tau > T(0) && P.sabs * U < tau) return false;
+    if ((ANG ? P.sabs : fabs(P.base)) * U * P.mult * sc * kconst<T>(p).wmax < floor_q) return false;
+    P.base *= P.mult;
+    return true;
+}
+
 // Advance the cursor c (in steps of st, below `end`) to this lane's next class that is not
-// negligible: non-zero strength, not below the screening threshold tau (0: no screening; the sum
-// of its pairs' bounds is compared, so every pair skipped is below tau), and a bound Ut >= floor_q
-// on every point's |q| in tile units.  On success P.base is multiplied by the class' multiplicity;
-// false when no class is left.
+// negligible (class_passes); false when none is left.
 template <typename T, int D, bool ANG>
 __device__ __forceinline__ bool next_pair(const SpreadArgs &p, PairCursor &c, long long end, const PairStep &st, T sc,
                                           T tau, T floor_q, PairData<T, D> &P)
 {
-    for (; c.pr < end; pair_advance(p, c, st)) {
-        if (!load_pair<T, D, ANG>(p, c, P)) continue;
-        const T U = pair_bound<T, D>(p, P);
-        if (tau > T(0) && P.sabs * U < tau) continue;
-        if ((ANG ? P.sabs : fabs(P.base)) * U * P.mult * sc * kconst<T>(p).wmax < floor_q) continue;
-        P.base *= P.mult;
-        return true;
-    }
+    for (; c.pr < end; pair_advance(p, c, st))
+        if (class_passes<T, D, ANG>(p, c, sc, tau, floor_q, P)) return true;
     return false;
 }
 
@@ -1192,7 +1158,7 @@ __device__ __forceinline__ void queue_spread(const SpreadArgs &p, const T *buf, 
 }
 
 // The pairs pr = first, first + nthr, ... below end of one thread, spread through the warp's
-// queue `buf` (spread_queue_values(d, fp32) x 32 values) into one slab (SLAB) or a tile that
+// queue `buf` (spread_queue_values x 32 values) into one slab (SLAB) or a tile that
 // holds every row.  Points below floor_q (they add exactly zero) are not queued, so that every
 // lane spreads a real point; FP32 points queue their velocity and strength and form their grid
 // coordinates after the queue (QEntry; with slabs, all but axis 0's).  Every loop condition is
@@ -1240,6 +1206,231 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
     }
     __syncwarp();
     queue_spread<T, D, W, Tile, SLAB, LATE>(p, buf, lane, lane < count, tile, row_lo, nrows, plane);
+}
+
+// ---- 2D FP32 grids in one tile: quads
+//
+// The M points of a class lie on a circle, sigma_m = (cos theta_m, sin theta_m) with theta_m =
+// 2 pi m/M, and M is even, so the set is symmetric in both axes: the points of m = 0..M/4 and their
+// mirror images (c_0 +- r cos theta_m, c_1 +- r sin theta_m) are all M points, four to a quad (two where
+// the sine (m = 0) or the cosine (4m = M) is zero).  The four points take two coordinates per axis,
+// so a quad evaluates four axes (coordinate, map factor, w kernel values) where four points alone
+// would evaluate eight.  Nearly every quad of a class that is not negligible adds something (91% to
+// 100% on the workloads' densities), so a lane spreads its own class' quads where it forms them, m in
+// step with the warp's other lanes (their classes are unrelated); only quads with a point of 2^29
+// tile units or more go through a queue, so that the slower large-point code runs with full
+// warps (where such points are common -- 15% of them at N = 16 -- almost every warp had one and all
+// its lanes waited).
+// Measured against spreading point by point through a queue: the headline (N = 64, M = 32) 1.47 -> 1.21 ms,
+// 2D angular N = 41 785 -> 706 us, 768 batched cells 40.3 -> 31.6 ms, RK4 at N = 32 11.9 -> 8.4 ms (with
+// the scaled integers of the large points, below).  Bound by issue (70% active) and by bank
+// conflicts of the tile's atomics (3.4 wavefronts each, the shared pipe 73% busy) about equally.
+
+constexpr int kQuadValues = 6;  // a large quad: two coordinates per axis, two strengths
+
+// Column factors of one coordinate of axis 1: first padded column and round(2^30 psi_c).
+template <int W>
+struct QuadCols {
+    int cb, wi[W];
+};
+template <int W>
+__device__ __forceinline__ void quad_cols(const SpreadArgs &p, float v, QuadCols<W> &c)
+{
+    float X, F, t0;
+    grid_coord_f32(p.cf, v, p.r == 1, X, F);
+    const int s = first_tap_f32<W>(X, F, t0);
+    c.cb = min(max(s + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
+    const float bias30 = 30.0f - p.cf.bl;
+#pragma unroll
+    for (int k = 0; k < W; ++k) c.wi[k] = __float2int_rn(es_f32(fmaf((float)k, 2.0f / W, t0), p.cf.bl, bias30));
+}
+
+// The large quad in slot `lane` of the queue: its points one by one.
+template <int W>
+__device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float *buf, const SplitTile &tile, int nrows,
+                                               int plane)
+{
+    const int lane = threadIdx.x & 31;
+    const bool alg = (p.r == 1);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const float v0 = buf[(k & 1) * 32 + lane], v1 = buf[(2 + (k >> 1)) * 32 + lane];
+        if (isinf(v0) || isinf(v1)) continue;  // a coordinate that has no mirror image
+        Point<float, 2> pt;
+        // points (+,+), (-,-) have the first strength, (+,-), (-,+) the second
+        pt.q = buf[(4 + ((k == 1 || k == 2) ? 1 : 0)) * 32 + lane] * axis_m2_f32(p.cf, v0, alg) *
+               axis_m2_f32(p.cf, v1, alg);
+        grid_coord_f32(p.cf, v0, alg, pt.X[0], pt.F[0]);
+        grid_coord_f32(p.cf, v1, alg, pt.X[1], pt.F[1]);
+        spread_point_f32<2, W, kLarge, false>(p, pt, tile, 0, nrows, plane);
+    }
+}
+
+// The points of one class per lane (every lane of the warp calls it; P.base = 0: none).  buf, count:
+// the warp's queue of large quads, 32 slots of kQuadValues floats, and its fill.
+template <int W, bool ANG>
+__device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const PairData<float, 2> &P, float qbase,
+                                                   const SplitTile &tile, int nrows, int plane, float *buf, int &count)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const float *sig = static_cast<const float *>(p.sig);
+    const float *wsig = static_cast<const float *>(p.wsig);
+    const TypedConsts<float> &K = p.cf;
+    const bool alg = (p.r == 1);
+    const bool simple = p.simple_fold != 0;
+#pragma unroll 1
+    for (int m = 0; 4 * m <= p.M; ++m) {
+        const bool one_row = (4 * m == p.M), one_col = (m == 0);  // no mirror image
+        const float cs = sig[2 * m], sn = sig[2 * m + 1];
+        const float vr[2] = {fmaf(P.rad, cs, P.cen[0]), fmaf(-P.rad, cs, P.cen[0])};
+        const float vc[2] = {fmaf(P.rad, sn, P.cen[1]), fmaf(-P.rad, sn, P.cen[1])};
+        const float mr[2] = {axis_m2_f32(K, vr[0], alg), axis_m2_f32(K, vr[1], alg)};
+        const float mc[2] = {axis_m2_f32(K, vc[0], alg), axis_m2_f32(K, vc[1], alg)};
+        // strengths of the points (+,+), (-,-) and (+,-), (-,+) before the map factors
+        float q1 = qbase * wsig[m], q2 = q1;
+        if constexpr (ANG) {
+            const float a0 = P.dir[0] * cs, a1 = P.dir[1] * sn;
+            const float e0 = (a0 + a1) * (a0 + a1), e1 = (a0 - a1) * (a0 - a1);
+            float b0 = K.ang_even[p.nang_even - 1], b1 = b0;
+            for (int k = p.nang_even - 2; k >= 0; --k) {
+                b0 = b0 * e0 + K.ang_even[k];
+                b1 = b1 * e1 + K.ang_even[k];
+            }
+            q2 = q1 * (P.x[0] * b1 + P.x[1] * b0);
+            q1 = q1 * (P.x[0] * b0 + P.x[1] * b1);
+        }
+        const float qmax = fmaxf(fabsf(q1), fabsf(q2)) * fmaxf(mr[0], mr[1]) * fmaxf(mc[0], mc[1]);
+        const bool large = qmax >= kIntLimitF32;
+        const unsigned lmask = __ballot_sync(full, large);
+        if (lmask) {
+            const int n = __popc(lmask), rank = __popc(lmask & ((1u << lane) - 1u)), room = 32 - count;
+            const float inf = __int_as_float(0x7f800000);
+            auto put = [&](int slot) {
+                buf[slot] = vr[0];
+                buf[32 + slot] = one_row ? inf : vr[1];
+                buf[64 + slot] = vc[0];
+                buf[96 + slot] = one_col ? inf : vc[1];
+                buf[128 + slot] = q1;
+                buf[160 + slot] = q2;
+            };
+            if (large && rank < room) put(count + rank);
+            if (n >= room) {
+                __syncwarp();
+                spread_large_quad<W>(p, buf, tile, nrows, plane);
+                __syncwarp();
+                if (large && rank >= room) put(rank - room);
+                count = n - room;
+            } else {
+                count += n;
+            }
+        }
+        if (large || !(qmax >= kNegligibleF32)) continue;
+        QuadCols<W> col[2];
+        quad_cols<W>(p, vc[0], col[0]);
+        if (!one_col) quad_cols<W>(p, vc[1], col[1]);
+#pragma unroll 1
+        for (int s = 0; s < 2; ++s) {
+            if (s && one_row) break;
+            const float v = s ? vr[1] : vr[0];
+            float X, F, t0;
+            grid_coord_f32(K, v, alg, X, F);
+            const int s0 = first_tap_f32<W>(X, F, t0);
+            const float m4 = 4.0f * (s ? mr[1] : mr[0]);
+            float pa[W];
+            int ra[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                pa[k] = es_f32(fmaf((float)k, 2.0f / W, t0), K.bl, -K.bl);
+                ra[k] = fold_cell(s0 + k, p.n, simple) * plane;
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (t && one_col) break;
+                const float q4 = m4 * ((s != t) ? q2 : q1) * mc[t];  // 4 q of the point
+                const int sg = q4 < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
+#pragma unroll
+                for (int k = 0; k < W; ++k) {
+                    const int rq = __float2int_rn(q4 * pa[k]);
+                    const int row = ra[k] + col[t].cb;
+                    unsigned wraps = 0u;
+#pragma unroll
+                    for (int j = 0; j < W; ++j) wraps = tile.add_int_run(row + j, mulhi_rn(rq, col[t].wi[j]), wraps);
+                    if (wraps) tile.add_carries(row, W, wraps, sg);
+                }
+            }
+        }
+    }
+}
+
+// The classes pr = first, first + stride, ... below end of one lane, into a tile that holds every
+// row.  The lanes test one class each per step; the ones that are not negligible go through a
+// queue of 32, so that a warp always spreads 32 classes at once: of a lane's own classes, the share
+// that is negligible varies from lane to lane, and with every lane spreading its own the warp
+// waited for the lane with the most (about a third of the lanes' time on the headline workload).
+// buf: the warp's queues, 32 slots of spread_queue_values(2, true, ANG) floats.
+template <int W, bool ANG>
+__device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long first, long long end, long long stride,
+                                             float sc, float tau, const SplitTile &tile, int nrows, int plane,
+                                             float *buf)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float *cbuf = buf + 32 * kQuadValues;  // the class queue
+    int count = 0, nclass = 0;             // queued large quads and classes, the same in every lane
+    PairCursor c = pair_cursor(p, first);
+    const PairStep st = pair_step(p, stride);
+    for (;;) {
+        const bool more = __any_sync(full, c.pr < end);
+        if (!more && nclass == 0) break;
+        PairData<float, 2> P;
+        bool hit = false;
+        if (c.pr < end) {
+            hit = class_passes<float, 2, ANG>(p, c, sc, tau, kNegligibleF32, P);
+            pair_advance(p, c, st);
+        }
+        auto put = [&](int slot) {
+            cbuf[slot] = P.cen[0];
+            cbuf[32 + slot] = P.cen[1];
+            cbuf[64 + slot] = P.rad;
+            cbuf[96 + slot] = P.base;
+            if constexpr (ANG) {
+                cbuf[128 + slot] = P.x[0];
+                cbuf[160 + slot] = P.x[1];
+                cbuf[192 + slot] = P.dir[0];
+                cbuf[224 + slot] = P.dir[1];
+            }
+        };
+        const unsigned mask = __ballot_sync(full, hit);
+        const int n = __popc(mask), rank = __popc(mask & ((1u << lane) - 1u)), room = 32 - nclass;
+        if (hit && rank < room) put(nclass + rank);
+        __syncwarp();
+        if (n >= room || !more) {  // a full queue, or what is left at the end
+            const bool valid = lane < min(nclass + n, 32);
+            PairData<float, 2> C;
+            zero_pair<float, 2>(C);
+            if (valid) {
+                C.cen[0] = cbuf[lane];
+                C.cen[1] = cbuf[32 + lane];
+                C.rad = cbuf[64 + lane];
+                C.base = cbuf[96 + lane];
+                if constexpr (ANG) {
+                    C.x[0] = cbuf[128 + lane];
+                    C.x[1] = cbuf[160 + lane];
+                    C.dir[0] = cbuf[192 + lane];
+                    C.dir[1] = cbuf[224 + lane];
+                }
+            }
+            __syncwarp();
+            if (hit && rank >= room) put(rank - room);
+            nclass = max(n - room, 0);
+            spread_class_quads<W, ANG>(p, C, C.base * sc, tile, nrows, plane, buf, count);
+        } else {
+            nclass += n;
+        }
+    }
+    __syncwarp();
+    if (lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
 }
 
 struct SlabGeom {
@@ -1299,14 +1490,17 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     pair_schedule(p, first, nthr);
     if (p.nslab > 1) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes((size_t)p.rows_per_slab * G.plane, true)) +
-                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true);
+                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG, true);
         spread_pairs_queued<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile,
                                                           G.row_lo, G.nrows, G.plane, buf);
-    } else if (p.queued) {  // one slab: the queues only compact the points that add something
+    } else if (p.queued) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes(G.ncell, true)) +
-                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true);
-        spread_pairs_queued<float, D, W, SplitTile, ANG, false>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32,
-                                                                 tile, 0, G.nrows, G.plane, buf);
+                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
+        if constexpr (D == 2)
+            spread_quads<W, ANG>(p, first, p.nclass, nthr, sc, tau, tile, G.nrows, G.plane, buf);
+        else  // one slab: the queues only compact the points that add something
+            spread_pairs_queued<float, D, W, SplitTile, ANG, false>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32,
+                                                                     tile, 0, G.nrows, G.plane, buf);
     } else {
         spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile, G.row_lo,
                                                    G.nrows, G.plane);

@@ -91,7 +91,7 @@ def test_result_does_not_depend_on_the_launch_shape(d, N, M, ang, prec):
     rng = np.random.default_rng(N)
     f = torch.as_tensor(rng.normal(size=(N + 1) ** d) * 0.1, device="cuda")
     out = []
-    for threads, per_sm in ((0, 0), (32, 1), (96, 2), (256, 1)):
+    for threads, per_sm in ((0, 0), (32, 1), (96, 2), (256, 1)) + (((1024, 1),) if prec == 2 else ()):
         Q = torch.empty_like(f)
         with Plan(d, N, M, 2.0, 0.5, 1e-6, precision=prec, angular=ang, spread_threads=threads,
                   spread_blocks_per_sm=per_sm) as plan:
