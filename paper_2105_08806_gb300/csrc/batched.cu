@@ -50,7 +50,7 @@ struct CellDesc {
 
 struct BatchArgs {
     int d, r, ncell, nitems, w;
-    double Bconst, beta, screen_eps;
+    double Bconst, beta, screen_eps, trim_q;
     const CellDesc *cells;
     const int *item_cell;
     int *counter;
@@ -340,6 +340,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.ncol = cd.nf + 2 * sa.cpad;
     sa.kpoly = b.kpoly;
     sa.queued = 0;
+    sa.trim_q = b.trim_q;
     fill_spread_consts(sa);
 }
 
@@ -432,10 +433,11 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
         if constexpr (F32) {
             float *buf = reinterpret_cast<float *>(smem_raw + b.queue_off) + warp * 32 * spread_queue_values(D, true);
             if constexpr (D == 2)
-                spread_quads<W, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, s_cd.nf, plane, buf);
-            else  // the queue compacts the points that add something
-                spread_pairs_queued<T, D, W, SplitTile, false, false>(sa, first, p1, blockDim.x, sc, tau, floor_q,
-                                                                       SplitTile{lo, carry}, 0, s_cd.nf, plane, buf);
+                spread_quads<W, false, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
+                                              plane, buf);
+            else
+                spread_points3<W, false, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
+                                                plane, buf);
         } else
             spread_pairs<T, D, W, WideTile, false>(sa, first, p1, blockDim.x, sc, tau, floor_q, wt, 0,
                                                       s_cd.nf, plane);
@@ -829,6 +831,7 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
     a.w = B->w;
     a.Bconst = 1.0 / (d == 2 ? 2.0 * kPi : 4.0 * kPi);
     a.beta = B->beta;
+    a.trim_q = trim_strength(B->w, B->beta);
     a.screen_eps = o.screen ? 0.05 * o.tol : 0.0;
     pgb::CellDesc *d_cells = nullptr;
     int *d_items = nullptr;

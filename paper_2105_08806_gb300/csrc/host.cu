@@ -81,6 +81,13 @@ int grid_size(int N, double sigma)
 
 double kernel_beta(int w, double sigma) { return 0.97 * kPi * (1.0 - 0.5 / sigma) * w; }
 
+double trim_strength(int w, double beta)
+{
+    if (w < 4) return 0.0;
+    const double t = 1.0 - 2.0 / w;
+    return 0.37 / std::exp(beta * (std::sqrt(1.0 - t * t) - 1.0));
+}
+
 int width_for(double tol, double sigma)
 {
     double per_w = 0.9 * std::sqrt(2.0 * (1.0 - 1.0 / sigma));

@@ -51,6 +51,11 @@ void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w);
 // Spreading-kernel width for precision tol at oversampling sigma, and its shape parameter.
 int width_for(double tol, double sigma);
 double kernel_beta(int w, double sigma);
+// Strength in tile units below which an FP32 point's contributions at the first and last taps of every
+// axis (|t| >= 1 - 2/w, so psi <= psi_o = psi(1 - 2/w)) all round to zero: the integer products
+// round(4 q psi_a [psi_b]) round(2^30 psi_c) stay below 2^31 there -- at most 1 x 2^30 when 4 q psi_o < 1.5
+// on axis a (b), and (4 q + 1/2) psi_o 2^30 on axis c.  0 for w < 4.
+double trim_strength(int w, double beta);
 // Even periodic grid size n >= sigma (2N + 1).
 int grid_size(int N, double sigma);
 // Piecewise polynomial form of the kernel for the FP64 spreading kernels: ceil(w/2) blocks of

@@ -36,6 +36,7 @@ struct TypedConsts {
     T Wang;             // Wsig * angmax (pair bound factor)
     T wmax;             // wmax_frac
     T bl;               // beta log2(e): ES kernel values as powers of two
+    T trim_q;
     T ang_even[kMaxAngular / 2];
     // FP32 point coordinates without systematic offsets or scale errors: a grid coordinate is
     // x = xq -+ atan(v/S) gs (r = 1) or 2 atan(exp(-v/S)) gs (r = 0) with xq = n/4 exact and the
@@ -54,6 +55,7 @@ struct SpreadArgs {
     int fast_gamma;       // 0: gamma = 0, 1: gamma = 1, 2: gamma = 1/2, 3: general pow
     double S, gamma, Bconst;
     double beta;          // exponential-of-semicircle shape
+    double trim_q;        // FP32: below this many tile units the first and last taps of every axis add nothing
     double grid_scale;    // n / (2 pi): angle -> grid coordinate
     const void *vnode;    // N node velocities (same on every axis)
     const float *vnode_lo;  // FP32 plans: v - (double)vnode, so that hi + lo carries the node exactly
@@ -88,7 +90,7 @@ struct SpreadArgs {
 };
 
 // Fill a.cf and a.cd from the double fields (call after setting S, grid_scale, Bconst, gamma,
-// Wsig, angmax, wmax_frac, beta and ang_even).
+// Wsig, angmax, wmax_frac, beta, trim_q and ang_even).
 template <typename T>
 __host__ __device__ inline void fill_typed_consts(const SpreadArgs &a, TypedConsts<T> &c)
 {
@@ -101,6 +103,7 @@ __host__ __device__ inline void fill_typed_consts(const SpreadArgs &a, TypedCons
     c.Wang = T(a.Wsig * a.angmax);
     c.wmax = T(a.wmax_frac);
     c.bl = T(a.beta * 1.4426950408889634);
+    c.trim_q = T(a.trim_q);
     for (int k = 0; k < kMaxAngular / 2; ++k) c.ang_even[k] = T(k < a.nang_even ? a.ang_even[k] : 0.0);
     c.invS_lo = T(1.0 / a.S - double(c.invS));
     c.gs_lo = T(a.grid_scale - double(c.gs));
@@ -121,18 +124,17 @@ __device__ __forceinline__ const TypedConsts<T> &kconst(const SpreadArgs &a)
 // Unordered pairs of n things, equal ones included.
 __host__ __device__ inline long long unordered_pairs(long long nnode) { return nnode * (nnode + 1) / 2; }
 
-// Values per slot of the spreading kernels' warp queues.  FP32, one slab: 2D a large quad (6) and a class
-// (4, angular kernels 8), 3D a point's velocity and strength.  FP32 slabs: a point's velocity, strength
-// and axis-0 coordinate (cell and fraction).  FP64: a point, d coordinates and its strength.
-__host__ __device__ constexpr int spread_queue_values(int d, bool f32, bool ang = false, bool slab = false)
+// Values per slot of the spreading kernels' warp queues.  FP32 2D: a large or half quad (6) and a class
+// (4, angular kernels 8); 3D: three points by size (velocity and strength, 4 each) and a class (5,
+// angular kernels 12).  FP64: a point, d coordinates and its strength.
+__host__ __device__ constexpr int spread_queue_values(int d, bool f32, bool ang = false)
 {
-    return !f32 ? d + 1 : slab ? d + 3 : d == 3 ? 4 : ang ? 14 : 10;
+    return !f32 ? d + 1 : d == 2 ? (ang ? 14 : 10) : (ang ? 24 : 17);
 }
 // Shared memory of the warp queues of a spreading block of `threads` threads: 32 slots per warp.
-__host__ __device__ constexpr size_t spread_queue_bytes(int threads, int d, bool f32, bool ang = false,
-                                                        bool slab = false)
+__host__ __device__ constexpr size_t spread_queue_bytes(int threads, int d, bool f32, bool ang = false)
 {
-    return (size_t)(threads / 32) * 32 * spread_queue_values(d, f32, ang, slab) * (f32 ? 4 : 8);
+    return (size_t)(threads / 32) * 32 * spread_queue_values(d, f32, ang) * (f32 ? 4 : 8);
 }
 // Shared memory of a block tile of `cells` cells, rounded up to 16 bytes (the queues follow it):
 // FP32 tiles hold one 32-bit word per cell, FP64 tiles three (fraction, low and high words).

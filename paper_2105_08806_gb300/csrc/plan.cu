@@ -125,21 +125,35 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     const int accept_threads = f32 ? pgb::kAcceptThreadsF32 : max_threads;
     if (o.spread_threads > accept_threads || (o.spread_threads > 0 && o.spread_threads % 32))
         return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
-    const int ask_threads = std::min(o.spread_threads, max_threads);  // <= 0: chosen here
+    int ask_threads = std::min(o.spread_threads, max_threads);  // <= 0: chosen here
     int rows_fit = (int)std::min<size_t>(p->nf, max_smem / (plane * elem));
     size_t qbytes = 0;
     if (rows_fit < p->nf) {
-        // slabbed grid: the warps' point queues (one block per SM, max_threads threads unless
-        // set) share the block's shared memory with the slab
-        const int thr = (ask_threads > 0) ? ask_threads : max_threads;
-        qbytes = pgb::spread_queue_bytes(thr, d, f32, ang, true);
-        rows_fit = (max_smem > qbytes) ? (int)std::min<size_t>(p->nf, (max_smem - qbytes) / (plane * elem)) : 0;
+        // slabbed grid: the warps' queues (one block per SM) share the block's shared memory with the slab.
+        // FP32: at least 384 threads, and as many as the fewest slabs that leave room for those allow
+        // (a point is generated once per slab and its rows straddle two now and then)
+        auto fit = [&](int thr) {
+            qbytes = pgb::spread_queue_bytes(thr, d, f32, ang);
+            return (max_smem > qbytes) ? (int)std::min<size_t>(p->nf, (max_smem - qbytes) / (plane * elem)) : 0;
+        };
+        rows_fit = fit((ask_threads > 0) ? ask_threads : f32 ? 384 : max_threads);
+        if (rows_fit < 1 && f32) {  // a plane that leaves little room
+            ask_threads = (ask_threads > 0) ? std::min(ask_threads, 128) : 128;
+            rows_fit = fit(ask_threads);
+        }
     }
     if (rows_fit < 1) return set_error(PG_ERR_ARG, "folded grid plane of %zu cells does not fit shared memory", plane);
     p->nslab = (p->nf + rows_fit - 1) / rows_fit;
     p->rows_per_slab = (p->nf + p->nslab - 1) / p->nslab;
     p->nslab = (p->nf + p->rows_per_slab - 1) / p->rows_per_slab;  // no empty trailing slab
-    p->spread_smem = pgb::tile_bytes((size_t)p->rows_per_slab * plane, f32) + (p->nslab > 1 ? qbytes : 0);
+    const size_t tile_bytes = pgb::tile_bytes((size_t)p->rows_per_slab * plane, f32);
+    int slab_threads = max_threads;  // threads whose queues fit beside a slab
+    if (p->nslab > 1 && f32 && ask_threads <= 0) {
+        const int warps = (int)((max_smem - tile_bytes) / pgb::spread_queue_bytes(32, d, f32, ang));
+        slab_threads = std::min(max_threads, 32 * warps);
+        qbytes = pgb::spread_queue_bytes(slab_threads, d, f32, ang);
+    }
+    p->spread_smem = tile_bytes + (p->nslab > 1 ? qbytes : 0);
     int per_sm = (int)(prop.sharedMemPerMultiprocessor / (p->spread_smem + 1024 + prop.reservedSharedMemPerBlock));
     per_sm = std::max(per_sm, 1);
     if (ask_threads > 0) {
@@ -154,7 +168,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         int t = (1024 / per_sm) / 32 * 32;
         p->spread_threads = std::max(128, std::min(max_threads, t));
     }
-    if (p->nslab > 1 && ask_threads <= 0) p->spread_threads = max_threads;  // the queues were sized for it
+    if (p->nslab > 1 && ask_threads <= 0) p->spread_threads = slab_threads;  // the queues were sized for it
     if (p->nslab == 1 && ask_threads <= 0) {
         // small plans: blocks no larger than it takes for every SM to have one (each thread then
         // owns one class; 1024-thread blocks would keep 18 of 152 SMs busy for 2D N = 16, whose
@@ -164,7 +178,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         const int small = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
         p->spread_threads = std::min(p->spread_threads, small);
     }
-    if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32, ang, true) > qbytes)
+    if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32, ang) > qbytes)
         return set_error(PG_ERR_STATE, "internal: point queues larger than reserved");
     // FP32 one-slab grids: the warps' queues follow the tile (2D: large quads; 3D: the points that add
     // something) when they fit beside it, with fewer threads if need be
@@ -221,6 +235,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.gamma = p->gamma;
     ka.Bconst = p->Bconst;
     ka.beta = p->beta;
+    ka.trim_q = trim_strength(p->w, p->beta);
     ka.grid_scale = p->n / (2.0 * kPi);
     ka.vnode = f32 ? (const void *)p->v32 : (const void *)p->v64;
     ka.vnode_lo = f32 ? p->v32lo : nullptr;

@@ -734,8 +734,10 @@ __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T
 
 // ---- FP32 points
 //
-// Kinds of FP32 point: kInt -- |q| < 2^29 tile units; kLarge -- any q.
-constexpr int kInt = 0, kLarge = 1;
+// Kinds of FP32 point: kInt -- |q| < 2^29 tile units; kLarge -- any q; kSmall -- |q| < trim_q
+// (SpreadArgs): every contribution of a first or last tap of an axis rounds to zero, so only the inner
+// (w-2)^d taps are added (the same bits).
+constexpr int kInt = 0, kLarge = 1, kSmall = 2;
 // Points below this many tile units take the integer products as they are; points below
 // kNegligibleF32 add exactly zero (4 q psi rounds to 0 for every row) and are skipped, and so are
 // pairs whose points all stay below it.
@@ -1043,9 +1045,9 @@ __device__ __forceinline__ bool rows_hit(const SpreadArgs &p, const Point<T, D> 
 }
 
 // What a warp queue holds for one point.  LATE (FP32): the post-collision velocity v'[D] and the
-// strength q, so that the grid coordinates are formed after the queue and only for the points that
-// go there -- in a slabbed grid (SLAB) with the axis-0 coordinate X0 + F0 formed before, for the
-// slab test; otherwise (FP64) the point itself, x[D] and q.
+// strength q; the grid coordinates are formed after the queue, only for the points that go there (in a
+// slabbed grid axis 0's once more: 45 instructions of the thousand that a 3D point takes, for two
+// words less per slot).  Otherwise (FP64) the point itself, x[D] and q.
 // Slot layout: value k of slot j at buf[32 k + j].
 template <typename T, int D, bool LATE, bool SLAB>
 struct QEntry {
@@ -1091,55 +1093,38 @@ struct QEntry {
 };
 template <int D, bool SLAB>
 struct QEntry<float, D, true, SLAB> {
-    float v[D], qv, X0, F0;
+    float v[D], qv;
     __device__ __forceinline__ float q() const { return qv; }
     __device__ __forceinline__ void put(float *buf, int slot) const
     {
 #pragma unroll
         for (int l = 0; l < D; ++l) buf[l * 32 + slot] = v[l];
         buf[D * 32 + slot] = qv;
-        if constexpr (SLAB) {
-            buf[(D + 1) * 32 + slot] = X0;
-            buf[(D + 2) * 32 + slot] = F0;
-        }
     }
     __device__ __forceinline__ void get(const float *buf, int slot)
     {
 #pragma unroll
         for (int l = 0; l < D; ++l) v[l] = buf[l * 32 + slot];
         qv = buf[D * 32 + slot];
-        if constexpr (SLAB) {
-            X0 = buf[(D + 1) * 32 + slot];
-            F0 = buf[(D + 2) * 32 + slot];
-        }
     }
     template <bool ANG>
     __device__ __forceinline__ void make(const SpreadArgs &p, const PairData<float, D> &P, float qbase, int m)
     {
         qv = point_velocity_f32<D, ANG>(p, P, qbase, m, v);
     }
-    // slabs: the axis-0 coordinate, then whether one of the point's rows lies in the slab
+    // slabs: whether one of the point's rows lies in the slab
     template <int W>
     __device__ __forceinline__ bool in_slab(const SpreadArgs &p, int row_lo, int nrows)
     {
+        float X0, F0, t0;
         grid_coord_f32(kconst<float>(p), v[0], p.r == 1, X0, F0);
-        float t0;
         return rows_hit_from<W>(p, first_tap_f32<W>(X0, F0, t0), row_lo, nrows);
     }
     // the same point make_point forms (same velocity, strength and coordinates)
     __device__ __forceinline__ void point(const SpreadArgs &p, Point<float, D> &out) const
     {
-        const TypedConsts<float> &K = kconst<float>(p);
-        const bool alg = (p.r == 1);
 #pragma unroll
-        for (int l = 0; l < D; ++l) {
-            if (SLAB && l == 0) {
-                out.X[0] = X0;
-                out.F[0] = F0;
-            } else {
-                grid_coord_f32(K, v[l], alg, out.X[l], out.F[l]);
-            }
-        }
+        for (int l = 0; l < D; ++l) grid_coord_f32(kconst<float>(p), v[l], p.r == 1, out.X[l], out.F[l]);
         out.q = qv;
     }
 };
@@ -1228,6 +1213,41 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
 
 constexpr int kQuadValues = 6;  // a large quad: two coordinates per axis, two strengths
 
+// Quad m of a class: the coordinates c +- r cos theta_m of axis 0 and c +- r sin theta_m of axis 1, their map
+// factors mu^-2, and the strengths before them of the points (+,+), (-,-) and (+,-), (-,+).
+struct Quad {
+    float vr[2], vc[2], mr[2], mc[2], q1, q2;
+};
+template <bool ANG>
+__device__ __forceinline__ Quad make_quad(const SpreadArgs &p, const PairData<float, 2> &P, float qbase, int m)
+{
+    const float *sig = static_cast<const float *>(p.sig);
+    const TypedConsts<float> &K = p.cf;
+    const bool alg = (p.r == 1);
+    const float cs = sig[2 * m], sn = sig[2 * m + 1];
+    Quad Q;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        Q.vr[k] = fmaf(P.rad, k ? -cs : cs, P.cen[0]);
+        Q.vc[k] = fmaf(P.rad, k ? -sn : sn, P.cen[1]);
+        Q.mr[k] = axis_m2_f32(K, Q.vr[k], alg);
+        Q.mc[k] = axis_m2_f32(K, Q.vc[k], alg);
+    }
+    Q.q1 = Q.q2 = qbase * static_cast<const float *>(p.wsig)[m];
+    if constexpr (ANG) {
+        const float a0 = P.dir[0] * cs, a1 = P.dir[1] * sn;
+        const float e0 = (a0 + a1) * (a0 + a1), e1 = (a0 - a1) * (a0 - a1);
+        float b0 = K.ang_even[p.nang_even - 1], b1 = b0;
+        for (int k = p.nang_even - 2; k >= 0; --k) {
+            b0 = b0 * e0 + K.ang_even[k];
+            b1 = b1 * e1 + K.ang_even[k];
+        }
+        Q.q2 = Q.q1 * (P.x[0] * b1 + P.x[1] * b0);
+        Q.q1 = Q.q1 * (P.x[0] * b0 + P.x[1] * b1);
+    }
+    return Q;
+}
+
 // Column factors of one coordinate of axis 1: first padded column and round(2^30 psi_c).
 template <int W>
 struct QuadCols {
@@ -1274,45 +1294,26 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const float *sig = static_cast<const float *>(p.sig);
-    const float *wsig = static_cast<const float *>(p.wsig);
     const TypedConsts<float> &K = p.cf;
     const bool alg = (p.r == 1);
     const bool simple = p.simple_fold != 0;
 #pragma unroll 1
     for (int m = 0; 4 * m <= p.M; ++m) {
         const bool one_row = (4 * m == p.M), one_col = (m == 0);  // no mirror image
-        const float cs = sig[2 * m], sn = sig[2 * m + 1];
-        const float vr[2] = {fmaf(P.rad, cs, P.cen[0]), fmaf(-P.rad, cs, P.cen[0])};
-        const float vc[2] = {fmaf(P.rad, sn, P.cen[1]), fmaf(-P.rad, sn, P.cen[1])};
-        const float mr[2] = {axis_m2_f32(K, vr[0], alg), axis_m2_f32(K, vr[1], alg)};
-        const float mc[2] = {axis_m2_f32(K, vc[0], alg), axis_m2_f32(K, vc[1], alg)};
-        // strengths of the points (+,+), (-,-) and (+,-), (-,+) before the map factors
-        float q1 = qbase * wsig[m], q2 = q1;
-        if constexpr (ANG) {
-            const float a0 = P.dir[0] * cs, a1 = P.dir[1] * sn;
-            const float e0 = (a0 + a1) * (a0 + a1), e1 = (a0 - a1) * (a0 - a1);
-            float b0 = K.ang_even[p.nang_even - 1], b1 = b0;
-            for (int k = p.nang_even - 2; k >= 0; --k) {
-                b0 = b0 * e0 + K.ang_even[k];
-                b1 = b1 * e1 + K.ang_even[k];
-            }
-            q2 = q1 * (P.x[0] * b1 + P.x[1] * b0);
-            q1 = q1 * (P.x[0] * b0 + P.x[1] * b1);
-        }
-        const float qmax = fmaxf(fabsf(q1), fabsf(q2)) * fmaxf(mr[0], mr[1]) * fmaxf(mc[0], mc[1]);
+        const Quad Q = make_quad<ANG>(p, P, qbase, m);
+        const float qmax = fmaxf(fabsf(Q.q1), fabsf(Q.q2)) * fmaxf(Q.mr[0], Q.mr[1]) * fmaxf(Q.mc[0], Q.mc[1]);
         const bool large = qmax >= kIntLimitF32;
         const unsigned lmask = __ballot_sync(full, large);
         if (lmask) {
             const int n = __popc(lmask), rank = __popc(lmask & ((1u << lane) - 1u)), room = 32 - count;
             const float inf = __int_as_float(0x7f800000);
             auto put = [&](int slot) {
-                buf[slot] = vr[0];
-                buf[32 + slot] = one_row ? inf : vr[1];
-                buf[64 + slot] = vc[0];
-                buf[96 + slot] = one_col ? inf : vc[1];
-                buf[128 + slot] = q1;
-                buf[160 + slot] = q2;
+                buf[slot] = Q.vr[0];
+                buf[32 + slot] = one_row ? inf : Q.vr[1];
+                buf[64 + slot] = Q.vc[0];
+                buf[96 + slot] = one_col ? inf : Q.vc[1];
+                buf[128 + slot] = Q.q1;
+                buf[160 + slot] = Q.q2;
             };
             if (large && rank < room) put(count + rank);
             if (n >= room) {
@@ -1327,16 +1328,16 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
         }
         if (large || !(qmax >= kNegligibleF32)) continue;
         QuadCols<W> col[2];
-        quad_cols<W>(p, vc[0], col[0]);
-        if (!one_col) quad_cols<W>(p, vc[1], col[1]);
+        quad_cols<W>(p, Q.vc[0], col[0]);
+        if (!one_col) quad_cols<W>(p, Q.vc[1], col[1]);
 #pragma unroll 1
         for (int s = 0; s < 2; ++s) {
             if (s && one_row) break;
-            const float v = s ? vr[1] : vr[0];
+            const float v = s ? Q.vr[1] : Q.vr[0];
             float X, F, t0;
             grid_coord_f32(K, v, alg, X, F);
             const int s0 = first_tap_f32<W>(X, F, t0);
-            const float m4 = 4.0f * (s ? mr[1] : mr[0]);
+            const float m4 = 4.0f * (s ? Q.mr[1] : Q.mr[0]);
             float pa[W];
             int ra[W];
 #pragma unroll
@@ -1347,7 +1348,7 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
                 if (t && one_col) break;
-                const float q4 = m4 * ((s != t) ? q2 : q1) * mc[t];  // 4 q of the point
+                const float q4 = m4 * ((s != t) ? Q.q2 : Q.q1) * Q.mc[t];  // 4 q of the point
                 const int sg = q4 < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
 #pragma unroll
                 for (int k = 0; k < W; ++k) {
@@ -1363,21 +1364,133 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
     }
 }
 
-// The classes pr = first, first + stride, ... below end of one lane, into a tile that holds every
-// row.  The lanes test one class each per step; the ones that are not negligible go through a
+// In a slabbed grid half of a quad's rows or more lie outside a block's slab, so there the quads are
+// queued by halves (N = 120, M = 8: spreading 5.44 -> 4.58 ms against a queue of single points): one
+// coordinate of axis 0 (cell X, fraction F) whose rows reach the slab, and the
+// two of axis 1 with the strengths of their points (0: no such point), kQuadValues values.
+
+// Add one point of a half quad: rows ra (-1: outside the slab) with factors pa, column factors col.
+template <int W, int KIND>
+__device__ __forceinline__ void half_quad_point(const SplitTile &tile, const int (&ra)[W], const float (&pa)[W],
+                                                const QuadCols<W> &col, float q)
+{
+    const int sg = q < 0.0f ? -1 : 1;
+    float q4 = 4.0f * q;
+    int sc = 0;
+    if constexpr (KIND == kLarge) {  // as spread_point_f32
+        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
+        q4 *= __int_as_float((127 - sc) << 23);
+    }
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        if (ra[k] < 0) continue;
+        const int rq = __float2int_rn(q4 * pa[k]);
+        const int row = ra[k] + col.cb;
+        if constexpr (KIND == kLarge) {
+#pragma unroll 1
+            for (int j = 0; j < W; ++j) tile.add_scaled(row + j, mulhi_rn(rq, col.wi[j]), sc);
+        } else {
+            unsigned wraps = 0u;
+#pragma unroll
+            for (int j = 0; j < W; ++j) wraps = tile.add_int_run(row + j, mulhi_rn(rq, col.wi[j]), wraps);
+            if (wraps) tile.add_carries(row, W, wraps, sg);
+        }
+    }
+}
+
+// The half quad in slot `lane` of the queue (valid lanes).
+template <int W>
+__device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const float *buf, bool valid,
+                                                 const SplitTile &tile, int row_lo, int nrows, int plane)
+{
+    if (!valid) return;
+    const int lane = threadIdx.x & 31;
+    const TypedConsts<float> &K = p.cf;
+    const bool simple = p.simple_fold != 0;
+    float t0;
+    const int s0 = first_tap_f32<W>(buf[lane], buf[32 + lane], t0);
+    float pa[W];
+    int ra[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        pa[k] = es_f32(fmaf((float)k, 2.0f / W, t0), K.bl, -K.bl);
+        const int r = fold_cell(s0 + k, p.n, simple) - row_lo;
+        ra[k] = (unsigned)r < (unsigned)nrows ? r * plane : -1;
+    }
+#pragma unroll 1
+    for (int t = 0; t < 2; ++t) {
+        const float q = buf[(4 + t) * 32 + lane];
+        if (!(fabsf(q) >= kNegligibleF32)) continue;
+        QuadCols<W> col;
+        quad_cols<W>(p, buf[(2 + t) * 32 + lane], col);
+        if (fabsf(q) < kIntLimitF32) half_quad_point<W, kInt>(tile, ra, pa, col, q);
+        else half_quad_point<W, kLarge>(tile, ra, pa, col, q);  // rare in grids of this size
+    }
+}
+
+// The points of one class per lane in a slab (every lane of the warp calls it; P.base = 0: none).
+// buf, count: the warp's queue of half quads and its fill.
+template <int W, bool ANG>
+__device__ __forceinline__ void spread_class_halves(const SpreadArgs &p, const PairData<float, 2> &P, float qbase,
+                                                    const SplitTile &tile, int row_lo, int nrows, int plane,
+                                                    float *buf, int &count)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int m = 0; 4 * m <= p.M; ++m) {
+        const Quad Q = make_quad<ANG>(p, P, qbase, m);
+#pragma unroll 1
+        for (int s = 0; s < 2; ++s) {
+            if (s && 4 * m == p.M) break;  // no mirror image
+            const float mr = s ? Q.mr[1] : Q.mr[0];
+            const float qa = (s ? Q.q2 : Q.q1) * mr * Q.mc[0];
+            const float qb = m ? (s ? Q.q1 : Q.q2) * mr * Q.mc[1] : 0.0f;
+            float X = 0.0f, F = 0.0f, t0;
+            bool hit = fmaxf(fabsf(qa), fabsf(qb)) >= kNegligibleF32;
+            if (hit) {
+                grid_coord_f32(p.cf, s ? Q.vr[1] : Q.vr[0], p.r == 1, X, F);
+                hit = rows_hit_from<W>(p, first_tap_f32<W>(X, F, t0), row_lo, nrows);
+            }
+            const unsigned mask = __ballot_sync(full, hit);
+            const int n = __popc(mask), rank = __popc(mask & ((1u << lane) - 1u)), room = 32 - count;
+            auto put = [&](int slot) {
+                buf[slot] = X;
+                buf[32 + slot] = F;
+                buf[64 + slot] = Q.vc[0];
+                buf[96 + slot] = Q.vc[1];
+                buf[128 + slot] = qa;
+                buf[160 + slot] = qb;
+            };
+            if (hit && rank < room) put(count + rank);
+            if (n >= room) {
+                __syncwarp();
+                spread_half_quad<W>(p, buf, true, tile, row_lo, nrows, plane);
+                __syncwarp();
+                if (hit && rank >= room) put(rank - room);
+                count = n - room;
+            } else {
+                count += n;
+            }
+        }
+    }
+}
+
+// The classes pr = first, first + stride, ... below end of one lane, into a slab (SLAB) or a tile
+// that holds every row.  The lanes test one class each per step; the ones that are not negligible go through a
 // queue of 32, so that a warp always spreads 32 classes at once: of a lane's own classes, the share
 // that is negligible varies from lane to lane, and with every lane spreading its own the warp
 // waited for the lane with the most (about a third of the lanes' time on the headline workload).
 // buf: the warp's queues, 32 slots of spread_queue_values(2, true, ANG) floats.
-template <int W, bool ANG>
+template <int W, bool ANG, bool SLAB>
 __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long first, long long end, long long stride,
-                                             float sc, float tau, const SplitTile &tile, int nrows, int plane,
-                                             float *buf)
+                                             float sc, float tau, const SplitTile &tile, int row_lo, int nrows,
+                                             int plane, float *buf)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     float *cbuf = buf + 32 * kQuadValues;  // the class queue
-    int count = 0, nclass = 0;             // queued large quads and classes, the same in every lane
+    int count = 0, nclass = 0;             // queued (large or half) quads and classes, the same in every lane
     PairCursor c = pair_cursor(p, first);
     const PairStep st = pair_step(p, stride);
     for (;;) {
@@ -1424,13 +1537,203 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
             __syncwarp();
             if (hit && rank >= room) put(rank - room);
             nclass = max(n - room, 0);
-            spread_class_quads<W, ANG>(p, C, C.base * sc, tile, nrows, plane, buf, count);
+            if constexpr (SLAB) spread_class_halves<W, ANG>(p, C, C.base * sc, tile, row_lo, nrows, plane, buf, count);
+            else spread_class_quads<W, ANG>(p, C, C.base * sc, tile, nrows, plane, buf, count);
         } else {
             nclass += n;
         }
     }
     __syncwarp();
-    if (lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
+    if constexpr (SLAB) spread_half_quad<W>(p, buf, lane < count, tile, row_lo, nrows, plane);
+    else if (lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
+}
+
+// ---- 3D FP32 grids
+//
+// As in 2D, classes that are not negligible go through a class queue.  Their points are formed 32 at
+// a time and sorted by size into three queues (those that reach the block's slab, with slabs), each
+// spread with full warps: small points, whose first and last taps on every axis add nothing ((w-2)^3
+// of w^3 taps: 64 of 216), points of 2^29 tile units or more (scaled integers), and the others.
+// Measured: 3D Maxwell N = 16, M = 32 9.55 -> 6.4 ms (one point queue, classes spread by the lane that
+// found them -> this), 3D VHS N = 24 67 -> 56 ms.  Bound by the bank conflicts of the tile's atomics
+// (shared pipe 77% busy at N = 16), issue 57%.
+// Spread slot `lane` (valid lanes) of the queue of one kind of point (the same for the whole warp).  One
+// copy of the coordinates and weights serves the three kinds, and only the tap loops differ: with a
+// copy for each the loop outgrew the instruction cache (N = 24: 4.7 of 9.6 warps stalled on instruction fetch, 0.6 with one copy; 67 -> 57 ms).
+template <int W, bool SLAB>
+__device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *buf, int kind, bool valid,
+                                              const SplitTile &tile, int row_lo, int nrows, int plane)
+{
+    if (!valid) return;
+    const int lane = threadIdx.x & 31;
+    const bool alg = (p.r == 1), simple = p.simple_fold != 0;
+    const float bl = p.cf.bl, h2 = 2.0f / W;
+    float X, F, t0, tl0, t1;
+    grid_coord_f32(p.cf, buf[64 + lane], alg, X, F);
+    const int cb = min(max(first_tap_f32<W>(X, F, tl0) + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
+    grid_coord_f32(p.cf, buf[32 + lane], alg, X, F);
+    const int s1 = first_tap_f32<W>(X, F, t1);
+    grid_coord_f32(p.cf, buf[lane], alg, X, F);
+    const int s0 = first_tap_f32<W>(X, F, t0);
+    const float q = buf[96 + lane];
+    int wi[W], c1[W];
+    float w1[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        wi[k] = __float2int_rn(es_f32(fmaf((float)k, h2, tl0), bl, 30.0f - bl));
+        w1[k] = es_f32(fmaf((float)k, h2, t1), bl, -bl);
+        c1[k] = fold_cell(s1 + k, p.n, simple) * p.ncol + cb;
+    }
+    const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
+    float q4 = 4.0f * q;
+    int sc = 0;
+    if (kind == kLarge) {  // as spread_point_f32
+        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
+        q4 *= __int_as_float((127 - sc) << 23);
+    }
+    const int a0 = (kind == kSmall) ? 1 : 0;
+#pragma unroll 1
+    for (int a = a0; a < W - a0; ++a) {
+        int r = fold_cell(s0 + a, p.n, simple);
+        if constexpr (SLAB) {
+            r -= row_lo;
+            if ((unsigned)r >= (unsigned)nrows) continue;
+        }
+        const float qa = q4 * es_f32(fmaf((float)a, h2, t0), bl, -bl);
+        const int row = r * plane;
+        if (kind == kInt) {
+#pragma unroll
+            for (int b = 0; b < W; ++b) {
+                const int rq = __float2int_rn(qa * w1[b]), line = row + c1[b];
+                unsigned wraps = 0u;
+#pragma unroll
+                for (int c = 0; c < W; ++c) wraps = tile.add_int_run(line + c, mulhi_rn(rq, wi[c]), wraps);
+                if (wraps) tile.add_carries(line, W, wraps, sg);
+            }
+        } else if (kind == kSmall) {
+#pragma unroll
+            for (int b = 1; b < W - 1; ++b) {
+                const int rq = __float2int_rn(qa * w1[b]), line = row + c1[b];
+                unsigned wraps = 0u;
+#pragma unroll
+                for (int c = 1; c < W - 1; ++c) wraps = tile.add_int_run(line + c, mulhi_rn(rq, wi[c]), wraps);
+                if (wraps) tile.add_carries(line + 1, W - 2, wraps, sg);
+            }
+        } else {  // rare: small code
+#pragma unroll 1
+            for (int b = 0; b < W; ++b) {
+                float wb = w1[0];
+                int line = c1[0];
+#pragma unroll
+                for (int k = 1; k < W; ++k)
+                    if (b == k) {
+                        wb = w1[k];
+                        line = c1[k];
+                    }
+                const int rq = __float2int_rn(qa * wb);
+#pragma unroll
+                for (int c = 0; c < W; ++c) tile.add_scaled(row + line + c, mulhi_rn(rq, wi[c]), sc);
+            }
+        }
+    }
+}
+
+template <int W, bool ANG, bool SLAB>
+__device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long first, long long end, long long stride,
+                                               float sc, float tau, const SplitTile &tile, int row_lo, int nrows,
+                                               int plane, float *buf)
+{
+    constexpr int PV = 32 * 4;  // values of a point queue: velocity and strength
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    float *cbuf = buf + 3 * PV;  // the class queue
+    int fill = 0;                // of the point queues kInt, kLarge, kSmall, 8 bits each; the same in every lane
+    int nclass = 0;
+    PairCursor c = pair_cursor(p, first);
+    const PairStep st = pair_step(p, stride);
+    for (;;) {
+        const bool more = __any_sync(full, c.pr < end);
+        const bool drain = !more && nclass == 0;  // no class left: spread what is queued, and end
+        PairData<float, 3> C;
+        zero_pair<float, 3>(C);
+        if (!drain) {
+            PairData<float, 3> P;
+            bool hit = false;
+            if (c.pr < end) {
+                hit = class_passes<float, 3, ANG>(p, c, sc, tau, kNegligibleF32, P);
+                pair_advance(p, c, st);
+            }
+            auto put = [&](int slot) {
+#pragma unroll
+                for (int l = 0; l < 3; ++l) cbuf[l * 32 + slot] = P.cen[l];
+                cbuf[96 + slot] = P.rad;
+                cbuf[128 + slot] = P.base;
+                if constexpr (ANG) {
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) cbuf[(5 + o) * 32 + slot] = P.x[o];
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) cbuf[(9 + l) * 32 + slot] = P.dir[l];
+                }
+            };
+            const unsigned mask = __ballot_sync(full, hit);
+            const int n = __popc(mask), rank = __popc(mask & lt), room = 32 - nclass;
+            if (hit && rank < room) put(nclass + rank);
+            __syncwarp();
+            if (n < room && more) {
+                nclass += n;
+                continue;
+            }
+            // a full queue, or what is left at the end
+            if (lane < min(nclass + n, 32)) {
+#pragma unroll
+                for (int l = 0; l < 3; ++l) C.cen[l] = cbuf[l * 32 + lane];
+                C.rad = cbuf[96 + lane];
+                C.base = cbuf[128 + lane];
+                if constexpr (ANG) {
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) C.x[o] = cbuf[(5 + o) * 32 + lane];
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) C.dir[l] = cbuf[(9 + l) * 32 + lane];
+                }
+            }
+            __syncwarp();
+            if (hit && rank >= room) put(rank - room);
+            nclass = max(n - room, 0);
+        }
+        const float qbase = C.base * sc;
+#pragma unroll 1
+        for (int m = 0; m < (drain ? 1 : p.M); ++m) {
+            QEntry<float, 3, true, SLAB> e;
+            int kind = -1;
+            if (!drain) {
+                e.template make<ANG>(p, C, qbase, m);
+                const float qa = fabsf(e.q());
+                if (qa >= kNegligibleF32) kind = qa >= kIntLimitF32 ? kLarge : qa < p.cf.trim_q ? kSmall : kInt;
+                if constexpr (SLAB)
+                    if (kind >= 0 && !e.template in_slab<W>(p, row_lo, nrows)) kind = -1;
+            }
+#pragma unroll 1
+            for (int k = 0; k < 3; ++k) {
+                const unsigned km = __ballot_sync(full, kind == k);
+                const int cnt = (fill >> (8 * k)) & 255;
+                if (!km && !(drain && cnt)) continue;
+                float *q = buf + k * PV;
+                const int kn = __popc(km), kr = __popc(km & lt), kroom = 32 - cnt;
+                if (kind == k && kr < kroom) e.put(q, cnt + kr);
+                int now = cnt + kn;
+                if (kn >= kroom || drain) {
+                    __syncwarp();
+                    queue3_spread<W, SLAB>(p, q, k, !drain || lane < cnt, tile, row_lo, nrows, plane);
+                    __syncwarp();
+                    if (kind == k && kr >= kroom) e.put(q, kr - kroom);
+                    now = max(kn - kroom, 0);
+                }
+                fill += (now - cnt) << (8 * k);
+            }
+        }
+        if (drain) break;
+    }
 }
 
 struct SlabGeom {
@@ -1490,17 +1793,18 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     pair_schedule(p, first, nthr);
     if (p.nslab > 1) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes((size_t)p.rows_per_slab * G.plane, true)) +
-                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG, true);
-        spread_pairs_queued<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile,
-                                                          G.row_lo, G.nrows, G.plane, buf);
+                     (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
+        if constexpr (D == 2)
+            spread_quads<W, ANG, true>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
+        else
+            spread_points3<W, ANG, true>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
     } else if (p.queued) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes(G.ncell, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
         if constexpr (D == 2)
-            spread_quads<W, ANG>(p, first, p.nclass, nthr, sc, tau, tile, G.nrows, G.plane, buf);
-        else  // one slab: the queues only compact the points that add something
-            spread_pairs_queued<float, D, W, SplitTile, ANG, false>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32,
-                                                                     tile, 0, G.nrows, G.plane, buf);
+            spread_quads<W, ANG, false>(p, first, p.nclass, nthr, sc, tau, tile, 0, G.nrows, G.plane, buf);
+        else
+            spread_points3<W, ANG, false>(p, first, p.nclass, nthr, sc, tau, tile, 0, G.nrows, G.plane, buf);
     } else {
         spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile, G.row_lo,
                                                    G.nrows, G.plane);
