@@ -336,7 +336,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.simple_fold = (b.w <= cd.n / 2) ? 1 : 0;
     sa.nang_even = 0;  // batched cells use VHS kernels
     sa.angmax = 1.0;
-    sa.cpad = tile_col_pad(b.w);
+    sa.cpad = tile_col_pad(b.w, b.d, f32);
     sa.ncol = cd.nf + 2 * sa.cpad;
     sa.kpoly = b.kpoly;
     sa.queued = 0;
@@ -345,7 +345,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
 }
 
 template <typename T, int D>
-constexpr int max_threads_of() { return sizeof(T) == 4 ? kBatchThreadsF32 : max_threads_f64(D); }
+constexpr int max_threads_of() { return sizeof(T) == 4 ? kBatchThreadsF32 : kMaxThreadsF64; }
 
 // Add a cell's block tile to the cell's global grid (padding columns folded onto their cells).
 template <bool F32, int D>
@@ -797,7 +797,7 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         cd.grid_off = grid_off;
         grid_off += cells_tile;
         // block tile: the last axis padded with unfolded columns (see spread_impl.cuh)
-        const long long tile_cells = (long long)ipow(cd.nf, d - 1) * (cd.nf + 2 * pgb::tile_col_pad(B->w));
+        const long long tile_cells = (long long)ipow(cd.nf, d - 1) * (cd.nf + 2 * pgb::tile_col_pad(B->w, d, f32));
         max_cells_tile = std::max<int>(max_cells_tile, (int)tile_cells);
         cd.s_len = std::max<long long>(modes, (long long)(N + 1) * (long long)ipow(cd.nf, d - 1));
         cd.s_off = s_off;
@@ -892,8 +892,8 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
     B->static_smem =
         sizeof(pgb::CellDesc) + sizeof(pgb::SpreadArgs) + 64 + (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
     const size_t per_block_extra = B->static_smem + 1024 + prop.reservedSharedMemPerBlock;
-    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::max_threads_f64(B->d);
-    const int accept_threads = f32 ? pgb::kAcceptThreadsF32 : max_threads;
+    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::kMaxThreadsF64;
+    const int accept_threads = pgb::accept_threads(d, f32);
     // the smallest block the plan makes: 128 threads, fewer where the largest tile leaves less room
     int min_threads = 128;
     while (min_threads > 64 && batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
@@ -1094,7 +1094,7 @@ PG_API int pg_boltz_batched_autotune(pg_boltz_plan_t *p, const double *f_dev, do
     int rc = cuda_check(cudaGetDeviceProperties(&prop, p->device), "cudaGetDeviceProperties");
     if (rc) return rc;
     const bool f32 = (B.prec == PG_PREC_FP32);
-    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::max_threads_f64(B.d);
+    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::kMaxThreadsF64;
     const int best0_threads = B.spread_threads, best0_blocks = B.spread_blocks;
     const long long best0_items = B.item_points;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

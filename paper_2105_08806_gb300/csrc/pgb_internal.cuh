@@ -146,7 +146,9 @@ __host__ __device__ inline size_t tile_bytes(size_t cells, bool f32)
 // Padding columns of the block tiles' last axis for kernel width w: the unfolded support of a point
 // at grid coordinate x in [0, n/2] spans floor(x - w/2) + 1 .. floor(x + w/2), i.e. at most w/2
 // columns beyond either end; w/2 + 1 leave a margin for rounding of x.
-__host__ __device__ inline int tile_col_pad(int w) { return w / 2 + 1; }
+// FP64 3D tiles have none (N = 11, w = 14: 24 instead of 40 cells per line of the grid, so that it fits one
+// block instead of two slabs, both of which nearly every point reaches).
+__host__ __device__ inline int tile_col_pad(int w, int d, bool f32) { return (d == 3 && !f32) ? 0 : w / 2 + 1; }
 
 // FP32 block tiles count in units 2^-(Eg - tile_bits(d)), about 2^-47 B (2D) or 2^-53 B (3D) for the
 // strength bound B: each contribution is rounded to the tile unit once, and with w^3 contributions
@@ -194,10 +196,13 @@ constexpr int kMinWidth = 2;
 // kAcceptThreadsF32; a launch then has kMaxThreadsF32.
 constexpr int kMaxThreadsF32 = 640;
 constexpr int kAcceptThreadsF32 = 1024;
-// FP64: 2D kernels use up to 255 registers per thread, 3D kernels fit 128 (their per-point
-// spreading is out of line), so 3D blocks hold twice the threads (integer shared atomics whose
-// returned values feed the next step want many resident warps).
-__host__ __device__ constexpr int max_threads_f64(int d) { return d == 3 ? 512 : 256; }
+// FP64: 512 threads with 128 registers (the axis weights are formed out of line).  Options may ask for
+// up to 512 in 3D and 256 in 2D.
+constexpr int kMaxThreadsF64 = 512;
+__host__ __device__ constexpr int accept_threads(int d, bool f32)
+{
+    return f32 ? kAcceptThreadsF32 : d == 3 ? 512 : 256;
+}
 // Largest block of the batched FP32 spreading kernel.
 constexpr int kBatchThreadsF32 = kMaxThreadsF32;
 

@@ -114,15 +114,15 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     cudaError_t e = cudaGetDeviceProperties(&prop, p->device);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "cudaGetDeviceProperties: %s", cudaGetErrorString(e));
     const size_t elem = (p->prec == PG_PREC_FP32) ? 4 : 12;  // 32-bit words per cell: FP32 one, FP64 three
-    // block tiles: rows of (nf^(d-2) x ncol) cells, the last axis padded with unfolded columns
-    const int cpad = pgb::tile_col_pad(p->w), ncol = p->nf + 2 * cpad;
+    // block tiles: rows of (nf^(d-2) x ncol) cells, the last axis padded with unfolded columns (FP64 3D: not)
+    const int cpad = pgb::tile_col_pad(p->w, d, p->prec == PG_PREC_FP32), ncol = p->nf + 2 * cpad;
     const size_t plane = (size_t)ipow(p->nf, d - 2) * ncol;
     const bool f32 = (p->prec == PG_PREC_FP32), ang = p->ang.n > 0;
     // leave room for the kernels' static shared memory (FP64: the kernel polynomial)
     // (and 16 bytes for rounding the tile up to 16 bytes)
     const size_t max_smem = prop.sharedMemPerBlockOptin - 1024 - 16 - (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
-    const int max_threads = f32 ? pgb::kMaxThreadsF32 : pgb::max_threads_f64(d);
-    const int accept_threads = f32 ? pgb::kAcceptThreadsF32 : max_threads;
+    const int max_threads = f32 ? pgb::kMaxThreadsF32 : pgb::kMaxThreadsF64;
+    const int accept_threads = pgb::accept_threads(d, f32);
     if (o.spread_threads > accept_threads || (o.spread_threads > 0 && o.spread_threads % 32))
         return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
     int ask_threads = std::min(o.spread_threads, max_threads);  // <= 0: chosen here

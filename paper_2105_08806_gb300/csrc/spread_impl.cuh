@@ -151,16 +151,6 @@ __device__ __forceinline__ int kernel_weights_f64(double x, double *wt)
     return s;
 }
 
-// FP64 weights and the folded cells fold(s + a) of one axis.
-template <int W>
-__device__ __forceinline__ void axis_weights_f64(const SpreadArgs &p, double x, double *wt, int *idx)
-{
-    const int s = kernel_weights_f64<W>(x, wt);
-    const bool simple = p.simple_fold != 0;
-#pragma unroll
-    for (int a = 0; a < W; ++a) idx[a] = fold_cell(s + a, p.n, simple);
-}
-
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -566,15 +556,6 @@ struct WideTile {
     unsigned *fr;  // fraction words (shared memory)
     unsigned *lo;  // low words
     int *hi;       // high words
-    __device__ __forceinline__ void add(int c, long long I, unsigned F) const
-    {
-        const unsigned of = atomicAdd(fr + c, F);
-        const long long J = I + ((of + F < of) ? 1 : 0);
-        const unsigned jl = (unsigned)(unsigned long long)J;
-        const unsigned o = atomicAdd(lo + c, jl);
-        const int vh = (int)(J >> 32) + ((o + jl < o) ? 1 : 0);
-        if (vh) atomicAdd(hi + c, vh);
-    }
     // the cell's sum rounded to the grid unit
     __device__ __forceinline__ long long value(int c) const
     {
@@ -583,45 +564,99 @@ struct WideTile {
     }
 };
 
-// Fixed-point kernel weight for the FP64 path: round(w 2^61) = h 2^31 + l with 0 <= l < 2^31
-// (w <= 1 up to the polynomial's rounding, so |h| <= 2^30 + 1).
+// Fixed-point kernel weight for the FP64 path: round(w 2^63) = h 2^32 + l (0 <= w <= 1 up to the
+// polynomial's rounding; what rounds below 0 is 0).
 struct FixW {
-    int h, l;
+    unsigned h, l;
 };
 __device__ __forceinline__ FixW fix_weight(double w)
 {
-    const long long t = __double2ll_rn(w * 2305843009213693952.0);  // 2^61
-    return FixW{(int)(t >> 31), (int)(t & 0x7fffffffll)};
+    const unsigned long long t = __double2ull_rn(w * 9223372036854775808.0);  // 2^63
+    return FixW{(unsigned)(t >> 32), (unsigned)t};
 }
 
-// round(R w) for |R| < 2^62 and a fixed-point weight w: with R = Rh 2^31 + Rl (0 <= Rl < 2^31),
-// R w 2^61 = 2^62 Rh h + 2^31 (Rh l + Rl h) + Rl l, from four 32 x 32-bit integer products; the
-// last one enters truncated to 2^-30 units (error below 2^-30), the result rounds half up.
-// Every intermediate stays below 2^63 in magnitude.
-__device__ __forceinline__ long long fix_mul(long long R, FixW w)
+// The fixed-point weights of one axis of a point at grid coordinate x, into local memory (rows are read
+// one at a time, the last axis' weights loaded into registers once per point); returns the first
+// tap.  One out-of-line copy serves every axis: inlined per axis the tap polynomials fill the
+// registers that the rows need.
+template <int W>
+__device__ __noinline__ int axis_weights_f64(double x, FixW *out)
 {
-    const int Rh = (int)(R >> 31);
-    const int Rl = (int)(R & 0x7fffffffll);
-    const long long X = (long long)Rh * w.l + (long long)Rl * w.h + (((long long)Rl * w.l) >> 31);
-    return 2 * ((long long)Rh * w.h) + ((X + (1ll << 29)) >> 30);
+    double wt[W];
+    const int s = kernel_weights_f64<W>(x, wt);
+#pragma unroll
+    for (int a = 0; a < W; ++a) out[a] = fix_weight(wt[a]);
+    return s;
 }
 
-// A point's contributions in the FP64 path: each tap value v (units 2^-(Eg+s) for the point's
-// scale s) becomes I + F 2^-32 grid units with I = floor(v 2^-s), F the next 32 bits (truncated,
-// below 2^-32 grid units).
-struct TapShift {
-    int sI;    // min(s, 63): |v| < 2^62, so v >> 63 is the sign
-    int sF;    // |s - 32|
-    bool up;   // s < 32: F = v << (32 - s); otherwise F = v >> (s - 32)
+// round(R2 w / 2) for R2 < 2^63 and a fixed-point weight w: the high word of the 128-bit product
+// R2 (w 2^63) plus 2^63, from four 32 x 32-bit products (the low half's low word is dropped after
+// its carry: at most 2^-32 of a unit).
+__device__ __forceinline__ unsigned long long fix_mul(unsigned long long R2, FixW w)
+{
+    const unsigned rh = (unsigned)(R2 >> 32), rl = (unsigned)R2;
+    const unsigned long long t1 = (unsigned long long)rl * w.h + __umulhi(rl, w.l) + 0x80000000ull;
+    const unsigned long long t2 = (unsigned long long)rh * w.l + (unsigned)t1;
+    return (unsigned long long)rh * w.h + (t1 >> 32) + (t2 >> 32);
+}
+
+// The scale of a point of strength q (grid units 2^-Eg): its contributions are formed in units
+// 2^-(Eg+s) with s = 60 - ilogb|q|, at most 32 (the fraction word's resolution) and at least 0, so that
+// |q| 2^s < 2^61.
+struct WideScale {
+    int s;
+    unsigned long long q2;    // round(|q| 2^(s+1))
+    unsigned long long neg;   // all ones for q < 0
 };
-__device__ __forceinline__ TapShift tap_shift(int s)
+__device__ __forceinline__ WideScale wide_scale(double q)
 {
-    return TapShift{min(s, 63), s < 32 ? 32 - s : s - 32, s < 32};
+    const int e = ((__double2hiint(q) >> 20) & 0x7ff) - 1023;
+    WideScale k;
+    k.s = max(0, min(60 - e, 32));
+    k.q2 = __double2ull_rn(fabs(q) * __hiloint2double((1023 + k.s + 1) << 20, 0));
+    k.neg = q < 0.0 ? ~0ull : 0ull;
+    return k;
 }
-__device__ __forceinline__ void tap_split(long long v, const TapShift &t, long long &I, unsigned &F)
+
+// Add the W contributions of one row, round(R2 w_c / 2) in units 2^-(Eg+s) with the point's sign, to
+// the cells at `base + idx[c]`.  A contribution splits into the cell's three words by three funnel
+// shifts.  The fraction words of G taps are added before the first of their returned values is
+// needed, then the low words, so that a warp waits for two atomics per group and not per tap.
+template <int W>
+__device__ __forceinline__ void wide_row(const WideTile &tile, int base, const int (&idx)[W], unsigned long long R2,
+                                         const WideScale &k, const FixW (&fl)[W])
 {
-    I = v >> t.sI;
-    F = (unsigned)(unsigned long long)(t.up ? (v << t.sF) : (v >> t.sF));
+    constexpr int G = W <= 8 ? W : (W + 1) / 2;
+#pragma unroll
+    for (int g = 0; g < W; g += G) {
+        unsigned F[G], of[G], jl[G], ol[G];
+        int jh[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            if (g + j >= W) break;
+            const unsigned long long v = (fix_mul(R2, fl[g + j]) ^ k.neg) - k.neg;
+            const unsigned vl = (unsigned)v, vh = (unsigned)(v >> 32);
+            F[j] = __funnelshift_lc(0u, vl, 32 - k.s);  // v 2^(32-s), its low word
+            jl[j] = __funnelshift_rc(vl, vh, k.s);      // v 2^-s
+            jh[j] = (int)vh >> min(k.s, 31);
+            of[j] = atomicAdd(tile.fr + base + idx[g + j], F[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            if (g + j >= W) break;
+            const unsigned long long J =
+                (((unsigned long long)(unsigned)jh[j] << 32) | jl[j]) + (of[j] + F[j] < F[j] ? 1 : 0);
+            jl[j] = (unsigned)J;
+            jh[j] = (int)(J >> 32);
+            ol[j] = atomicAdd(tile.lo + base + idx[g + j], jl[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            if (g + j >= W) break;
+            const int h = jh[j] + (ol[j] + jl[j] < jl[j] ? 1 : 0);
+            if (h) atomicAdd(tile.hi + base + idx[g + j], h);
+        }
+    }
 }
 
 // One post-collision point: FP32 points carry each grid coordinate (one grid cell = 1,
@@ -726,7 +761,8 @@ __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T
 }
 
 // Tile layout.  A block tile holds rows row_lo..row_lo+nrows-1 of axis 0 of the folded grid, and
-// along the last axis it keeps the UNFOLDED columns u = -cpad..nf-1+cpad at u + cpad (ncol =
+// along the last axis (but for FP64 3D tiles, whose three words per cell leave no room for it: cpad = 0,
+// ncol = nf, and a point's columns are folded once for its w^2 rows) it keeps the UNFOLDED columns u = -cpad..nf-1+cpad at u + cpad (ncol =
 // nf + 2 cpad cells): the w columns of a point are then consecutive, with no folding and no
 // per-contribution index arithmetic.  The padding columns are folded onto their cells when the
 // tile is added to the global grid (tile_to_grid_cell).  2D cell (row, u): row ncol + u + cpad;
@@ -828,82 +864,67 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     }
 }
 
+// Whether any of the w axis-0 rows of a point whose first tap is s lies in the slab.
+template <int W>
+__device__ __forceinline__ bool rows_hit_from(const SpreadArgs &p, int s, int row_lo, int nrows)
+{
+    const bool simple = p.simple_fold != 0;
+    bool hit = false;
+#pragma unroll
+    for (int a = 0; a < W; ++a) hit |= (unsigned)(fold_cell(s + a, p.n, simple) - row_lo) < (unsigned)nrows;
+    return hit;
+}
+
 // ---- FP64 points
 
 // Add the w^d contributions of one FP64 point (q in grid units 2^-Eg) to the block tile.  SLAB:
 // the tile holds a slab of the grid's rows and rows outside it are skipped; otherwise it holds
-// every row (row_lo = 0, nrows = n/2 + 1).  The kernel weights are FP64.  The point works in units
-// 2^-(Eg+s) with s = 60 - ilogb|q| (at most 94), so that |q| 2^s < 2^61: each row takes the
-// integer R = round(q psi_a 2^s) (3D: then round(R psi_b) in integers) and each cell
-// round(R psi_c) from a 61-bit fixed-point psi_c (fix_mul) -- one FP64 product and conversion
-// per row instead of per cell, and about 2^-61 relative rounding -- which goes to the tile as
-// grid units and 32 fraction bits (tap_split).
+// every row (row_lo = 0, nrows = n/2 + 1).  The point works in units 2^-(Eg+s) (wide_scale) with FP64 kernel
+// weights held in 63-bit fixed point: each row takes the integer R = round(q psi_a 2^s) (3D: then
+// round(R psi_b)) and each cell round(R psi_c) -- integer products (fix_mul), about 2^-61 relative
+// rounding -- which goes to the tile as grid units and 32 fraction bits (wide_row).
 template <int D, int W, bool SLAB>
 __device__ __forceinline__ void spread_point_f64(const SpreadArgs &p, const Point<double, D> &pt,
                                                  const WideTile &tile, int row_lo, int nrows, int plane)
 {
-    const double q = pt.q;
-    if (q == 0.0) return;
-    double w0[W];
-    int r0[W];
-    axis_weights_f64<W>(p, pt.x[0], w0, r0);
-    bool hit = !SLAB;
-#pragma unroll
-    for (int a = 0; a < W; ++a) {
-        if constexpr (SLAB) {
-            r0[a] -= row_lo;
-            hit |= ((unsigned)r0[a] < (unsigned)nrows);
-        }
+    if (pt.q == 0.0) return;
+    const bool simple = p.simple_fold != 0;
+    if constexpr (SLAB) {
+        if (!rows_hit_from<W>(p, (int)floor(pt.x[0] - 0.5 * W) + 1, row_lo, nrows)) return;
     }
-    if (!hit) return;
-    const int s = max(0, min(60 - ilogb(q), 94));
-    const double qs = ldexp(q, s);
-    const TapShift ts = tap_shift(s);
-    double wl[W];  // last axis: consecutive padded columns cb..cb+w-1 (clamped: x lies in [0, n/2])
-    const int cb = min(max(kernel_weights_f64<W>(pt.x[D - 1], wl) + p.cpad, 0), p.ncol - W);
-    FixW fl[W];
-#pragma unroll
-    for (int c = 0; c < W; ++c) fl[c] = fix_weight(wl[c]);
+    const WideScale k = wide_scale(pt.q);
+    FixW f0[W], fl[W];
+    int cl[W];
+    const int s0 = axis_weights_f64<W>(pt.x[0], f0);
+    const int sl = axis_weights_f64<W>(pt.x[D - 1], fl);
     if constexpr (D == 2) {
+        // consecutive padded columns (clamped: x lies in [0, n/2])
+        const int cb = min(max(sl + p.cpad, 0), p.ncol - W);
+#pragma unroll
+        for (int c = 0; c < W; ++c) cl[c] = c;
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            if (SLAB && (unsigned)r0[a] >= (unsigned)nrows) continue;
-            const long long R = __double2ll_rn(qs * w0[a]);
-            const int row = r0[a] * plane + cb;
-#pragma unroll
-            for (int c = 0; c < W; ++c) {
-                long long I;
-                unsigned F;
-                tap_split(fix_mul(R, fl[c]), ts, I, F);
-                tile.add(row + c, I, F);
-            }
+            const int r = fold_cell(s0 + a, p.n, simple) - row_lo;
+            if (SLAB && (unsigned)r >= (unsigned)nrows) continue;
+            const unsigned long long R2 = fix_mul(k.q2, f0[a]) << 1;
+            if (R2) wide_row<W>(tile, r * plane + cb, cl, R2, k, fl);
         }
     } else {
-        double w1[W];
-        int c1[W];
-        axis_weights_f64<W>(p, pt.x[1], w1, c1);
-        FixW f1[W];
 #pragma unroll
-        for (int b = 0; b < W; ++b) {
-            f1[b] = fix_weight(w1[b]);
-            c1[b] = c1[b] * p.ncol + cb;
-        }
+        for (int c = 0; c < W; ++c) cl[c] = fold_cell(sl + c, p.n, simple);
+        FixW f1[W];
+        const int s1 = axis_weights_f64<W>(pt.x[1], f1);
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            if (SLAB && (unsigned)r0[a] >= (unsigned)nrows) continue;
-            const long long Ra = __double2ll_rn(qs * w0[a]);
-            const int row = r0[a] * plane;
+            const int r = fold_cell(s0 + a, p.n, simple) - row_lo;
+            if (SLAB && (unsigned)r >= (unsigned)nrows) continue;
+            const unsigned long long Ra2 = fix_mul(k.q2, f0[a]) << 1;
+            if (!Ra2) continue;
+            const int row = r * plane;
 #pragma unroll 1
             for (int b = 0; b < W; ++b) {
-                const long long R = fix_mul(Ra, f1[b]);
-                const int line = row + c1[b];
-#pragma unroll
-                for (int c = 0; c < W; ++c) {
-                    long long I;
-                    unsigned F;
-                    tap_split(fix_mul(R, fl[c]), ts, I, F);
-                    tile.add(line + c, I, F);
-                }
+                const unsigned long long R2 = fix_mul(Ra2, f1[b]) << 1;
+                if (R2) wide_row<W>(tile, row + fold_cell(s1 + b, p.n, simple) * p.ncol, cl, R2, k, fl);
             }
         }
     }
@@ -923,25 +944,6 @@ __device__ __forceinline__ void spread_point_body(const SpreadArgs &p, const Poi
     } else {
         spread_point_f64<D, W, SLAB>(p, pt, tile, row_lo, nrows, plane);
     }
-}
-
-template <typename T, int D, int W, typename Tile, bool SLAB>
-__device__ __noinline__ void spread_point_outlined(const SpreadArgs &p, const Point<T, D> &pt, const Tile &tile,
-                                                   int row_lo, int nrows, int plane)
-{
-    spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
-}
-
-// 3D points (w^3 taps, two integer kinds) are spread by one out-of-line copy per kernel: inlined
-// at each call site the kernel outgrew the instruction cache (stalls on instruction fetch; 13%
-// longer on the 3D bi-Maxwellian, 70% on 3D BKW once the one-slab queue added a third site).
-// 2D points (w^2 taps) stay inline, where the call's register saves cost 5%.
-template <typename T, int D, int W, typename Tile, bool SLAB>
-__device__ __forceinline__ void spread_point_any(const SpreadArgs &p, const Point<T, D> &pt, const Tile &tile,
-                                                 int row_lo, int nrows, int plane)
-{
-    if constexpr (D == 3) spread_point_outlined<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
-    else spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
 }
 
 // Load the class at cursor c; whether it is not negligible: non-zero strength, not below the
@@ -1005,7 +1007,7 @@ __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long firs
         for (int m = 0; m < p.M; ++m) {
             Point<T, D> pt;
             make_point<T, D, ANG>(p, P, qbase, m, pt);
-            spread_point_any<T, D, W, Tile, false>(p, pt, tile, row_lo, nrows, plane);
+            spread_point_body<T, D, W, Tile, false>(p, pt, tile, row_lo, nrows, plane);
         }
         if (ok) pair_advance(p, c, st);
     }
@@ -1018,17 +1020,6 @@ __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long firs
 // spreading them where they are generated would leave most lanes idle while the others add.
 // Instead each warp appends the points that hit its slab to a queue of 32 entries in shared
 // memory (slot-major) and spreads a full queue with all 32 lanes, one point per lane.
-
-// Whether any of the w axis-0 rows of a point whose first tap is s lies in the slab.
-template <int W>
-__device__ __forceinline__ bool rows_hit_from(const SpreadArgs &p, int s, int row_lo, int nrows)
-{
-    const bool simple = p.simple_fold != 0;
-    bool hit = false;
-#pragma unroll
-    for (int a = 0; a < W; ++a) hit |= (unsigned)(fold_cell(s + a, p.n, simple) - row_lo) < (unsigned)nrows;
-    return hit;
-}
 
 // Whether any of the w axis-0 rows of a point lies in the slab (the rows of the point's spreading).
 template <typename T, int D, int W>
@@ -1139,7 +1130,7 @@ __device__ __forceinline__ void queue_spread(const SpreadArgs &p, const T *buf, 
     e.get(buf, lane);
     Point<T, D> pt;
     e.point(p, pt);
-    spread_point_any<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
+    spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
 }
 
 // The pairs pr = first, first + nthr, ... below end of one thread, spread through the warp's
@@ -1820,7 +1811,7 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
 }
 
 template <int D, int W, bool ANG>
-__global__ void __launch_bounds__(max_threads_f64(D), 1) k_spread_f64(const __grid_constant__ SpreadArgs p)
+__global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_constant__ SpreadArgs p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SlabGeom G = slab_geometry(p, D);
