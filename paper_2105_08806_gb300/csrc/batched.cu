@@ -339,7 +339,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.cpad = tile_col_pad(b.w, b.d, f32);
     sa.ncol = cd.nf + 2 * sa.cpad;
     sa.kpoly = b.kpoly;
-    sa.queued = 0;
+    sa.queued = 0;  // (FP64: no orbit items)
     sa.trim_q = b.trim_q;
     fill_spread_consts(sa);
 }

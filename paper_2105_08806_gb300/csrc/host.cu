@@ -196,6 +196,14 @@ void sphere_points(int d, int M, int kind, std::vector<double> &pts, std::vector
     wts.assign(M, 4.0 * kPi / M);
 }
 
+std::vector<unsigned> axis_orbits(int N)
+{
+    std::vector<unsigned> t;
+    for (int i = 0; 2 * i <= N - 1; ++i)
+        for (int j = i; i + j <= N - 1; ++j) t.push_back((unsigned)i | (unsigned)j << 16);
+    return t;
+}
+
 double map_v(double phi, double S, int r)
 {
     // xi = -cos(phi); r = 1: v = S xi / sqrt(1 - xi^2) = -S cot(phi); r = 0: v = S atanh(xi) = S ln tan(phi/2)

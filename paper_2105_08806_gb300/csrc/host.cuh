@@ -65,6 +65,9 @@ void kernel_poly(int w, double beta, double *c);
 std::vector<double> kernel_ft(int N, int w, double beta, int n);
 // Sphere quadrature (points M x d, weights M), Section 4.1.
 void sphere_points(int d, int M, int kind, std::vector<double> &pts, std::vector<double> &wts);
+// One node pair (i <= j, i + j <= N-1, as i + 65536 j) per orbit of an axis' unordered node pairs under
+// the reflection i -> N-1-i.
+std::vector<unsigned> axis_orbits(int N);
 // v(xi) at xi = -cos(phi) for the map with tail parameter r.
 double map_v(double phi, double S, int r);
 
@@ -133,6 +136,7 @@ struct pg_boltz_plan_s {
     float *a32 = nullptr;
     double *h = nullptr, *Qplus = nullptr, *Qlast = nullptr, *mom = nullptr;
     int *carry = nullptr;      // FP32 spreading: per-block carry counters
+    unsigned *orb = nullptr;   // FP64 2D spreading: axis orbits (SpreadArgs::orb)
     double *kpoly = nullptr;   // FP64 spreading: the kernel polynomial (kPolyCoefF64 doubles)
     double *ub = nullptr;      // N^d per-node strength bounds
     double *bound = nullptr;   // scalar B >= sum_p |q_p| (follows the grid in one allocation)

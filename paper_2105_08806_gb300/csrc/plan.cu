@@ -194,12 +194,30 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
             p->spread_smem += qq;
         }
     }
+    // FP64 2D one-slab grids: quads of mirrored classes, numbered in 32 bits
+    const std::vector<unsigned> orbits = (!f32 && d == 2) ? axis_orbits(N) : std::vector<unsigned>();
+    const long long nitem = (long long)orbits.size() * (long long)orbits.size() * (M / 4 + 1);
+    if (!f32 && d == 2 && p->nslab == 1 && nitem < (1ll << 32)) {
+        if (ask_threads <= 0) {
+            const long long per_block = (nitem + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
+            p->spread_threads = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
+            while (p->spread_threads > 128 && p->spread_smem + (size_t)p->spread_threads * 4 > max_smem)
+                p->spread_threads -= 128;
+            per_sm = 1;
+        }
+        const size_t qq = (size_t)p->spread_threads * 4;
+        if (p->spread_smem + qq <= max_smem) {
+            p->queued = 1;
+            p->spread_smem += qq;
+        }
+    }
     per_sm = std::min(per_sm, prop.maxThreadsPerMultiProcessor / p->spread_threads);
     if (o.spread_blocks_per_sm > 0) per_sm = std::min(per_sm, o.spread_blocks_per_sm);
     per_sm = std::max(per_sm, 1);
     long long blocks = (long long)prop.multiProcessorCount * per_sm;
     blocks = std::max<long long>(blocks / p->nslab, 1) * p->nslab;
-    const long long need = ((p->nclass + p->spread_threads - 1) / p->spread_threads) * p->nslab;
+    const long long items = (!f32 && p->queued) ? nitem : p->nclass;
+    const long long need = ((items + p->spread_threads - 1) / p->spread_threads) * p->nslab;
     blocks = std::min(blocks, need);
     p->spread_blocks = (int)blocks;
     // the pair schedule permutes thread starts by a multiplier prime to every smaller count
@@ -214,7 +232,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         std::vector<double> kp(pgb::kPolyCoefF64, 0.0);
         kernel_poly(p->w, p->beta, kp.data());
         int rc2 = upload(p, &p->kpoly, kp);
-        if (rc2) return rc2;
+        if (rc2 || (p->queued && (rc2 = upload(p, &p->orb, orbits)))) return rc2;
     }
 
     // ---- spreading-kernel arguments
@@ -255,6 +273,9 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.tile_cells = (int)tile_cells;
     ka.carry = p->carry;
     ka.queued = p->queued;
+    ka.orb = p->orb;
+    ka.norb = (int)orbits.size();
+    ka.nitem = nitem;
     ka.nang_even = p->ang.n ? (p->ang.n + 1) / 2 : 0;
     for (int k = 0; k < ka.nang_even; ++k) ka.ang_even[k] = p->ang.c[2 * k];
     ka.angmax = p->angmax;

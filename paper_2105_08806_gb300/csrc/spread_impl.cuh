@@ -346,30 +346,29 @@ struct PairStep {
     int dt, du, di, dk;
 };
 
-__device__ __forceinline__ PairCursor pair_cursor(const SpreadArgs &p, long long pr)
+__device__ __forceinline__ PairCursor pair_cursor(int naxp, long long pr)
 {
     PairCursor c;
     c.pr = pr;
-    c.t = (int)(pr / p.naxp);
-    c.u = (int)(pr - (long long)c.t * p.naxp);
-    c.i = (int)(((long long)c.u + (long long)c.t * kPairShear) % p.naxp);
+    c.t = (int)(pr / naxp);
+    c.u = (int)(pr - (long long)c.t * naxp);
+    c.i = (int)(((long long)c.u + (long long)c.t * kPairShear) % naxp);
     return c;
 }
 
-__device__ __forceinline__ PairStep pair_step(const SpreadArgs &p, long long stride)
+__device__ __forceinline__ PairStep pair_step(int naxp, long long stride)
 {
     PairStep s;
     s.d = stride;
-    s.dt = (int)(stride / p.naxp);
-    s.du = (int)(stride - (long long)s.dt * p.naxp);
-    s.di = (int)(((long long)s.du + (long long)s.dt * kPairShear) % p.naxp);
-    s.dk = (int)(kPairShear % p.naxp);
+    s.dt = (int)(stride / naxp);
+    s.du = (int)(stride - (long long)s.dt * naxp);
+    s.di = (int)(((long long)s.du + (long long)s.dt * kPairShear) % naxp);
+    s.dk = (int)(kPairShear % naxp);
     return s;
 }
 
-__device__ __forceinline__ void pair_advance(const SpreadArgs &p, PairCursor &c, const PairStep &s)
+__device__ __forceinline__ void pair_advance(int naxp, PairCursor &c, const PairStep &s)
 {
-    const int naxp = p.naxp;
     c.pr += s.d;
     c.t += s.dt;
     c.u += s.du;
@@ -722,6 +721,22 @@ __device__ __forceinline__ float point_velocity_f32(const SpreadArgs &p, const P
     return q;
 }
 
+// FP64 grid coordinate x = z n/(2 pi) of one mapped coordinate v, and its factor mu^-2.
+__device__ __forceinline__ double grid_coord_f64(const TypedConsts<double> &K, double v, bool alg, double &m2)
+{
+    if (alg) {
+        m2 = (K.SS + v * v) * K.invS;
+        return atan2(K.S, v) * K.gs;
+    }
+    // z = 2 atan(e^-u) and mu^-2 = S cosh u with e = e^-|u| <= 1 (one exp and one atan
+    // instead of sinh, cosh and atan2): for u < 0, 2 atan(e^|u|) = pi - 2 atan(e^-|u|)
+    const double u = v * K.invS;
+    const double e = exp(-fabs(u));
+    const double at2 = 2.0 * atan(e);
+    m2 = 0.5 * K.S * (e + 1.0 / e);
+    return (u >= 0.0 ? at2 : 3.14159265358979323846 - at2) * K.gs;
+}
+
 // Point m of pair P (qbase = a_i a_j B x multiplicity x tile scale).
 template <typename T, int D, bool ANG = false>
 __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T, D> &P, T qbase, int m,
@@ -739,21 +754,8 @@ __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T
         double q = point_base<double, D, ANG>(p, P, qbase, m);
 #pragma unroll
         for (int l = 0; l < D; ++l) {
-            const double vp = P.cen[l] + P.rad * sig[m * D + l];
-            double z, m2;
-            if (alg) {
-                z = Fn<T>::atan2_(K.S, vp);
-                m2 = (K.SS + vp * vp) * K.invS;
-            } else {
-                // z = 2 atan(e^-u) and mu^-2 = S cosh u with e = e^-|u| <= 1 (one exp and one atan
-                // instead of sinh, cosh and atan2): for u < 0, 2 atan(e^|u|) = pi - 2 atan(e^-|u|)
-                const double u = vp * K.invS;
-                const double e = exp(-fabs(u));
-                const double at2 = 2.0 * atan(e);
-                z = u >= 0.0 ? at2 : 3.14159265358979323846 - at2;
-                m2 = 0.5 * K.S * (e + 1.0 / e);
-            }
-            pt.x[l] = z * K.gs;
+            double m2;
+            pt.x[l] = grid_coord_f64(K, P.cen[l] + P.rad * sig[m * D + l], alg, m2);
             q *= m2;
         }
         pt.q = q;
@@ -968,7 +970,7 @@ template <typename T, int D, bool ANG>
 __device__ __forceinline__ bool next_pair(const SpreadArgs &p, PairCursor &c, long long end, const PairStep &st, T sc,
                                           T tau, T floor_q, PairData<T, D> &P)
 {
-    for (; c.pr < end; pair_advance(p, c, st))
+    for (; c.pr < end; pair_advance(p.naxp, c, st))
         if (class_passes<T, D, ANG>(p, c, sc, tau, floor_q, P)) return true;
     return false;
 }
@@ -996,8 +998,8 @@ template <typename T, int D, int W, typename Tile, bool ANG>
 __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long first, long long end, long long stride,
                                              T sc, T tau, T floor_q, const Tile &tile, int row_lo, int nrows, int plane)
 {
-    PairCursor c = pair_cursor(p, first);
-    const PairStep st = pair_step(p, stride);
+    PairCursor c = pair_cursor(p.naxp, first);
+    const PairStep st = pair_step(p.naxp, stride);
     for (;;) {
         PairData<T, D> P;
         const bool ok = next_pair<T, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
@@ -1009,7 +1011,7 @@ __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long firs
             make_point<T, D, ANG>(p, P, qbase, m, pt);
             spread_point_body<T, D, W, Tile, false>(p, pt, tile, row_lo, nrows, plane);
         }
-        if (ok) pair_advance(p, c, st);
+        if (ok) pair_advance(p.naxp, c, st);
     }
 }
 
@@ -1149,8 +1151,8 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     int count = 0;  // queued points, the same in every lane
-    PairCursor c = pair_cursor(p, first);
-    const PairStep st = pair_step(p, nthr);
+    PairCursor c = pair_cursor(p.naxp, first);
+    const PairStep st = pair_step(p.naxp, nthr);
     for (;;) {
         PairData<T, D> P;
         const bool ok = next_pair<T, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
@@ -1178,7 +1180,7 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
                 count += n;
             }
         }
-        if (ok) pair_advance(p, c, st);
+        if (ok) pair_advance(p.naxp, c, st);
     }
     __syncwarp();
     queue_spread<T, D, W, Tile, SLAB, LATE>(p, buf, lane, lane < count, tile, row_lo, nrows, plane);
@@ -1482,8 +1484,8 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
     const int lane = threadIdx.x & 31;
     float *cbuf = buf + 32 * kQuadValues;  // the class queue
     int count = 0, nclass = 0;             // queued (large or half) quads and classes, the same in every lane
-    PairCursor c = pair_cursor(p, first);
-    const PairStep st = pair_step(p, stride);
+    PairCursor c = pair_cursor(p.naxp, first);
+    const PairStep st = pair_step(p.naxp, stride);
     for (;;) {
         const bool more = __any_sync(full, c.pr < end);
         if (!more && nclass == 0) break;
@@ -1491,7 +1493,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
         bool hit = false;
         if (c.pr < end) {
             hit = class_passes<float, 2, ANG>(p, c, sc, tau, kNegligibleF32, P);
-            pair_advance(p, c, st);
+            pair_advance(p.naxp, c, st);
         }
         auto put = [&](int slot) {
             cbuf[slot] = P.cen[0];
@@ -1641,8 +1643,8 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
     float *cbuf = buf + 3 * PV;  // the class queue
     int fill = 0;                // of the point queues kInt, kLarge, kSmall, 8 bits each; the same in every lane
     int nclass = 0;
-    PairCursor c = pair_cursor(p, first);
-    const PairStep st = pair_step(p, stride);
+    PairCursor c = pair_cursor(p.naxp, first);
+    const PairStep st = pair_step(p.naxp, stride);
     for (;;) {
         const bool more = __any_sync(full, c.pr < end);
         const bool drain = !more && nclass == 0;  // no class left: spread what is queued, and end
@@ -1653,7 +1655,7 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
             bool hit = false;
             if (c.pr < end) {
                 hit = class_passes<float, 3, ANG>(p, c, sc, tau, kNegligibleF32, P);
-                pair_advance(p, c, st);
+                pair_advance(p.naxp, c, st);
             }
             auto put = [&](int slot) {
 #pragma unroll
@@ -1724,6 +1726,205 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
             }
         }
         if (drain) break;
+    }
+}
+
+// ---- 2D FP64 grids in one tile: quads of mirrored classes
+//
+// The nodes are symmetric about 0 on every axis, so reflecting an axis maps a class {i, j} of that axis to
+// {N-1-i, N-1-j}, its centre to the opposite and its points to their mirror images, whose taps
+// are the same weights at the mirrored cells (u -> n/2 - u).  The classes of an orbit under the two
+// reflections therefore share their axis evaluations, as the four points of a quad do: four
+// evaluations (angle, map factor, w tap polynomials -- all of the FP64 arithmetic) serve up to 16
+// points, which leaves the spreading bound by its integer products and atomics instead of by the
+// FP64 pipe (1.7 operations per SM per clock).
+// Measured against points one by one: N = 64, M = 32, tol 1e-13 101 -> 44 ms, N = 40, M = 40, tol 1e-14
+// (logarithmic map) 26.3 -> 11.2 ms.  Then issue is 57% active, the FP64 pipe 42% and the shared
+// pipe 36% busy (N = 40, M = 8): latency of 16 warps, no single unit.
+//
+// An item is one quad m of one orbit; p.orb lists the axis orbits' representatives i + j <= N-1 (the
+// mirror image of i + j = N-1 is itself and its strength counts once).
+
+// Grid coordinate and fixed-point weights of one axis, out of line (one copy); the first tap.
+template <int W>
+__device__ __noinline__ int axis_eval_f64(const SpreadArgs &p, double v, FixW *out, double *m2)
+{
+    double mm;
+    const double x = grid_coord_f64(p.cd, v, p.r == 1, mm);
+    *m2 = mm;
+    double wt[W];
+    const int s = kernel_weights_f64<W>(x, wt);
+#pragma unroll
+    for (int a = 0; a < W; ++a) out[a] = fix_weight(wt[a]);
+    return s;
+}
+
+// One orbit: the geometry of its representative class, and per mirror image e (bit 0: axis 0 reflected,
+// bit 1: axis 1) the strength B x multiplicity x sum_o a a in grid units, or (angular kernels) the two
+// terms of the sum; 0 for mirror images that are negligible (class_passes).
+template <bool ANG>
+struct Orbit {
+    double cen[2], rad, x0[4], x1[4], dir[2];
+};
+
+template <bool ANG>
+__device__ __forceinline__ bool load_orbit(const SpreadArgs &p, int o0, int o1, double sc, double tau, double floor_q,
+                                           Orbit<ANG> &O)
+{
+    const int N = p.N;
+    const double *a = static_cast<const double *>(p.a), *vn = static_cast<const double *>(p.vnode);
+    const unsigned w0 = p.orb[o0], w1 = p.orb[o1];
+    const int i0 = w0 & 0xffffu, j0 = w0 >> 16, i1 = w1 & 0xffffu, j1 = w1 >> 16;
+    const double vi0 = vn[i0], vj0 = vn[j0], vi1 = vn[i1], vj1 = vn[j1];
+    const double d0 = vi0 - vj0, d1 = vi1 - vj1;
+    const double g = sqrt(d0 * d0 + d1 * d1);
+    const TypedConsts<double> &K = p.cd;
+    double B;
+    switch (p.fast_gamma) {
+    case 0: B = K.Bconst; break;
+    case 1: B = K.Bconst * g; break;
+    case 2: B = K.Bconst * sqrt(g); break;
+    default: B = K.Bconst * pow(g, K.gamma); break;
+    }
+    O.cen[0] = 0.5 * (vi0 + vj0);
+    O.cen[1] = 0.5 * (vi1 + vj1);
+    O.rad = 0.5 * g;
+    double U = K.Wang;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        const double R = fabs(O.cen[l]) + O.rad;
+        U *= (p.r == 1) ? (K.SS + R * R) * K.invS : K.S * cosh(R * K.invS);
+    }
+    if constexpr (ANG) {
+        const double ginv = g > 0.0 ? 1.0 / g : 0.0;
+        O.dir[0] = d0 * ginv;
+        O.dir[1] = d1 * ginv;
+    }
+    const double Bm = B * 2.0 * (i0 == j0 ? 0.5 : 1.0) * (i1 == j1 ? 0.5 : 1.0) * sc;
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int e0 = e & 1, e1 = e >> 1;
+        const int x0 = e0 ? N - 1 - i0 : i0, y0 = e0 ? N - 1 - j0 : j0;
+        const int x1 = e1 ? N - 1 - i1 : i1, y1 = e1 ? N - 1 - j1 : j1;
+        const double s0 = a[x0 * N + x1] * a[y0 * N + y1], s1 = a[y0 * N + x1] * a[x0 * N + y1];
+        const double sum = s0 + s1, sabs = fabs(s0) + fabs(s1);
+        bool keep = !((e0 && i0 + j0 == N - 1) || (e1 && i1 + j1 == N - 1));
+        // the screening threshold is in strengths, per pair sum B sabs
+        if (tau > 0.0 && B * sabs * U < tau) keep = false;
+        if ((ANG ? sabs : fabs(sum)) * Bm * U * K.wmax < floor_q) keep = false;
+        O.x0[e] = keep ? Bm * (ANG ? s0 : sum) : 0.0;
+        O.x1[e] = (ANG && keep) ? Bm * s1 : 0.0;
+        any = any || (keep && (ANG ? sabs : fabs(sum)) * Bm > 0.0);
+    }
+    return any;
+}
+
+// Quad m of an orbit.
+template <int W, bool ANG>
+__device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orbit<ANG> &O, int m, const WideTile &tile,
+                                                  int plane)
+{
+    const double *sig = static_cast<const double *>(p.sig);
+    const bool simple = p.simple_fold != 0;
+    const int nrow = (4 * m == p.M) ? 1 : 2, ncolumn = (m == 0) ? 1 : 2;  // 1: no mirror image
+    const double cs = sig[2 * m], sn = sig[2 * m + 1];
+    FixW fr[2][W], fc[2][W];  // local memory
+    double mr[2], mc[2];
+    int sr[2], cc[2];
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        if (k < nrow) sr[k] = axis_eval_f64<W>(p, O.cen[0] + (k ? -O.rad : O.rad) * cs, fr[k], &mr[k]);
+        if (k < ncolumn) {
+            const int s = axis_eval_f64<W>(p, O.cen[1] + (k ? -O.rad : O.rad) * sn, fc[k], &mc[k]);
+            cc[k] = min(max(s + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
+        }
+    }
+    double b0 = 1.0, b1 = 1.0;  // b_e(cos theta) of the points (+,+), (-,-) and (+,-), (-,+), unexchanged pair
+    if constexpr (ANG) {
+        const double a0 = O.dir[0] * cs, a1 = O.dir[1] * sn;
+        const double e0 = (a0 + a1) * (a0 + a1), e1 = (a0 - a1) * (a0 - a1);
+        b0 = b1 = p.cd.ang_even[p.nang_even - 1];
+        for (int k = p.nang_even - 2; k >= 0; --k) {
+            b0 = b0 * e0 + p.cd.ang_even[k];
+            b1 = b1 * e1 + p.cd.ang_even[k];
+        }
+    }
+    const double wm = static_cast<const double *>(p.wsig)[m];
+    int cl[W];
+#pragma unroll
+    for (int c = 0; c < W; ++c) cl[c] = c;
+#pragma unroll 1
+    for (int h = 0; h < 4; ++h) {  // column sets: coordinate t, mirrored (e1) or not
+        const int t = h >> 1, e1 = h & 1;
+        if (t >= ncolumn) break;
+        FixW fl[W];
+#pragma unroll
+        for (int c = 0; c < W; ++c) fl[c] = fc[t][e1 ? W - 1 - c : c];
+        const int cb = e1 ? p.ncol - W - cc[t] : cc[t];
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {  // row sets: coordinate s, mirrored (e0) or not
+            const int s = g >> 1, e0 = g & 1;
+            if (s >= nrow) break;
+            double q = O.x0[e0 + 2 * e1];
+            if constexpr (ANG) q = (s == t) ? q * b0 + O.x1[e0 + 2 * e1] * b1 : q * b1 + O.x1[e0 + 2 * e1] * b0;
+            q *= wm * mr[s] * mc[t];
+            if (q == 0.0) continue;
+            const WideScale k = wide_scale(q);
+#pragma unroll 1
+            for (int a = 0; a < W; ++a) {
+                int r = fold_cell(sr[s] + a, p.n, simple);
+                if (e0) r = p.nf - 1 - r;
+                const unsigned long long R2 = fix_mul(k.q2, fr[s][a]) << 1;
+                if (R2) wide_row<W>(tile, r * plane + cb, cl, R2, k, fl);
+            }
+        }
+    }
+}
+
+// The items it = first, first + stride, ... below end of one lane.  Items that are not negligible go
+// through the warp's queue of 32 item numbers (ids), so that 32 lanes spread 32 items.
+template <int W, bool ANG>
+__device__ __forceinline__ void spread_orbits(const SpreadArgs &p, long long first, long long end, long long stride,
+                                              double sc, double tau, double floor_q, const WideTile &tile, int plane,
+                                              unsigned *ids)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int queued = 0;  // the same in every lane
+    PairCursor c = pair_cursor(p.norb, first);
+    const PairStep st = pair_step(p.norb, stride);
+    for (;;) {
+        const bool more = __any_sync(full, c.pr < end);
+        if (!more && queued == 0) break;
+        bool hit = false;
+        // an item: quad m = c.t / norb (slowest, so that a warp's lanes mostly share it), orbits c.t % norb and c.i
+        const unsigned id = (unsigned)c.t * (unsigned)p.norb + (unsigned)c.i;
+        if (c.pr < end) {
+            Orbit<ANG> O;
+            hit = load_orbit<ANG>(p, c.t % p.norb, c.i, sc, tau, floor_q, O);
+            pair_advance(p.norb, c, st);
+        }
+        const unsigned mask = __ballot_sync(full, hit);
+        const int n = __popc(mask), rank = __popc(mask & ((1u << lane) - 1u)), room = 32 - queued;
+        if (hit && rank < room) ids[queued + rank] = id;
+        __syncwarp();
+        if (n < room && more) {
+            queued += n;
+            continue;
+        }
+        const bool valid = lane < min(queued + n, 32);
+        const unsigned mine = valid ? ids[lane] : 0u;
+        __syncwarp();
+        if (hit && rank >= room) ids[rank - room] = id;
+        queued = max(n - room, 0);
+        if (valid) {
+            const int t = (int)(mine / (unsigned)p.norb);
+            Orbit<ANG> O;
+            load_orbit<ANG>(p, t % p.norb, (int)(mine - (unsigned)t * (unsigned)p.norb), sc, tau, floor_q, O);
+            spread_orbit_quad<W, ANG>(p, O, t / p.norb, tile, plane);
+        }
+        __syncwarp();
     }
 }
 
@@ -1841,6 +2042,12 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
                       (threadIdx.x >> 5) * 32 * spread_queue_values(D, false);
         spread_pairs_queued<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
                                                           G.nrows, G.plane, buf);
+    } else if (D == 2 && p.queued) {
+        if constexpr (D == 2) {
+            unsigned *ids = reinterpret_cast<unsigned *>(smem_raw + tile_bytes(tile_cells, false)) +
+                            (threadIdx.x >> 5) * 32;
+            spread_orbits<W, ANG>(p, first, p.nitem, nthr, sc, tau, floor_q, tile, G.plane, ids);
+        }
     } else {
         spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
                                                    G.nrows, G.plane);
