@@ -331,6 +331,8 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.Wsig = cd.Wsig;
     sa.wmax_frac = 1.0 / cd.M;  // the sphere sets have equal weights
     sa.bound = nullptr;
+    sa.ub = nullptr;
+    sa.nub = 0;
     sa.tau = nullptr;  // the batched kernel reads Tcell directly
     sa.grid = b.grid + cd.grid_off;
     sa.simple_fold = (b.w <= cd.n / 2) ? 1 : 0;

@@ -136,9 +136,10 @@ struct pg_boltz_plan_s {
     float *a32 = nullptr;
     double *h = nullptr, *Qplus = nullptr, *Qlast = nullptr, *mom = nullptr;
     int *carry = nullptr;      // FP32 spreading: per-block carry counters
-    unsigned *orb = nullptr;   // FP64 2D spreading: axis orbits (SpreadArgs::orb)
+    unsigned *orb = nullptr;   // axis orbits of node pairs (SpreadArgs::orb, LossArgs::orb)
+    pgb::LossArgs largs{};     // loss by mirror images (nloss = 0: launch_loss)
     double *kpoly = nullptr;   // FP64 spreading: the kernel polynomial (kPolyCoefF64 doubles)
-    double *ub = nullptr;      // N^d per-node strength bounds
+    double *ub = nullptr;      // partial sums of the strength bound (per node, or LossArgs::nbound)
     double *bound = nullptr;   // scalar B >= sum_p |q_p| (follows the grid in one allocation)
     unsigned long long *grid = nullptr;  // folded grid, int64 fixed point
     double *tau = nullptr;     // scalar screening threshold (follows the bound)

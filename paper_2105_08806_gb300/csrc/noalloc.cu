@@ -90,7 +90,7 @@ PG_API int pg_boltz_project_noalloc(int d, int N, double S, int map_log, int Mp,
     int which = 0;
     for (int ax = 3 - d; ax < 3; ++ax) {
         double *dst = (ax == 2) ? ftilde_dev : bufs[which];
-        if (pgb::launch_axis_pass(cur, dims, ax, P, N + 1, dst, s) != cudaSuccess)
+        if (pgb::launch_axis_pass({cur, nullptr, dims, ax, N + 1, P, dst}, s) != cudaSuccess)
             return fail(PG_ERR_CUDA, "projection pass launch failed");
         dims.e[ax] = N + 1;
         cur = dst;

@@ -66,6 +66,9 @@ struct SpreadArgs {
     double Wsig;          // sum_m w_m
     double wmax_frac;     // max_m w_m / sum_m w_m: one point's share of a pair's strength bound
     const double *bound;  // device scalar B >= sum_p |q_p| (written by the loss kernel)
+    const double *ub;     // nub > 0: the partial sums of B / (1 + 1e-5) (LossArgs::ub); the kernel adds them up
+    int nub;              // and block 0 writes *bound.  0: *bound and *tau were written before
+    double *bound_out;    // = bound
     const double *tau;    // device scalar: node pairs whose strength bound is below it are skipped (0: none)
     unsigned long long *grid;  // nf^d folded grid, int64 fixed point in units of 2^-Eg
     int simple_fold;      // 1 when w <= n/2: unfolded indices lie in [-n/2, n] (no modulo needed)
@@ -215,13 +218,50 @@ struct Dims3 {
     int e[3];
 };
 
-// out = A contracted with `in` along axis `ax` (A is m x in.e[ax], row-major).
-cudaError_t launch_axis_pass(const double *in, Dims3 in_dims, int ax, const double *A, int m,
-                             double *out, cudaStream_t s);
+// out = A contracted along axis `ax` (A is m x dims.e[ax], row-major) with `in`, or with the int64
+// fixed-point array `fixed_in` (when not null).
+struct AxisPass {
+    const double *in;
+    const unsigned long long *fixed_in;
+    Dims3 dims;
+    int ax, m;
+    const double *A;
+    double *out;
+};
+cudaError_t launch_axis_pass(const AxisPass &P, cudaStream_t s);
+// Two independent passes in one launch; P0's fixed-point input is in units 2^-Eg (Eg from *B), times scale.
+cudaError_t launch_axis_pass_pair(const AxisPass &P0, const AxisPass &P1, const double *B, double scale, cudaStream_t s);
 // Last reconstruction pass along axis 2, then a_i = acc * prod_l scale[i_l];
-// writes a (FP64) and, if af != nullptr, a float copy.
+// writes a (FP64) and, if af != nullptr, a float copy; clears the nclear words at clear.
 cudaError_t launch_recon_last(const double *in, Dims3 in_dims, const double *A, int m,
-                              const double *scale, int d, double *a, float *af, cudaStream_t s);
+                              const double *scale, int d, double *a, float *af, unsigned long long *clear,
+                              long long nclear, cudaStream_t s);
+// The loss sums h_i and the strength bound by mirror images of the nodes (VHS kernels, and angular ones
+// in 2D, without screening; launch_loss otherwise).  f32: FP32 pair terms.
+struct LossArgs {
+    const double *a;        // N^d node values
+    const float *a32;
+    const double *v64;      // N node velocities
+    const float *v32, *v32lo;
+    int N, M;
+    int nloss;              // nodes with every index <= (N-1)/2, one block each
+    int nbound;             // blocks of the bound, each writing one partial sum to ub
+    const unsigned *orb;    // an axis' orbits of node pairs (SpreadArgs::orb)
+    int norb;
+    long long norbits;      // norb^d
+    const double *sig64;    // sphere set (angular kernels)
+    const float *sig32;
+    Angular ang;
+    double angmax, gamma;
+    int fast_gamma;
+    double Bw;
+    const double *inv_mu2;
+    double S;
+    int r;
+    double *h;              // N^d loss weights
+    double *ub;             // nbound partial sums of the strength bound B / (1 + 1e-5)
+};
+cudaError_t launch_loss_mirror(const LossArgs &L, int d, bool f32, cudaStream_t s);
 // Loss: h_i = a_i * Lsum_i * prod_l inv_mu2[i_l], Lsum_i = Bw * sum_j a_j B(|v_i - v_j|) A_ij,
 // A_ij = (1/Wsig) sum_m w_m b(cos theta_ijm) for an angular kernel (ang.n > 0; the sum over the
 // sphere set then runs per pair), 1 otherwise (Bw = Bconst Wsig);
@@ -250,9 +290,6 @@ __host__ __device__ inline int screen_bin(double u)
 // (an upper bound of the total strength of the pairs below tau), else *tau = 0.
 cudaError_t launch_bound_reduce(const double *ub, int n, const unsigned long long *hist, double eps, double *B,
                                 double *tau, cudaStream_t s);
-// First transform pass reading the int64 fixed-point grid (units 2^-Eg, Eg from *B), times scale.
-cudaError_t launch_axis_pass_fixed(const unsigned long long *in, Dims3 in_dims, int ax, const double *A,
-                                   int m, const double *B, double scale, double *out, cudaStream_t s);
 // Exact / FP32 value of the constant factors of an FP32 point strength: Bconst (the kernel's
 // constant), the common sphere weight w and 1/S per axis enter every strength as rounded FP32
 // constants, a common relative error that the transform of the FP32 grid divides out in FP64.

@@ -195,7 +195,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         }
     }
     // FP64 2D one-slab grids: quads of mirrored classes, numbered in 32 bits
-    const std::vector<unsigned> orbits = (!f32 && d == 2) ? axis_orbits(N) : std::vector<unsigned>();
+    const std::vector<unsigned> orbits = axis_orbits(N);
     const long long nitem = (long long)orbits.size() * (long long)orbits.size() * (M / 4 + 1);
     if (!f32 && d == 2 && p->nslab == 1 && nitem < (1ll << 32)) {
         if (ask_threads <= 0) {
@@ -232,7 +232,40 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         std::vector<double> kp(pgb::kPolyCoefF64, 0.0);
         kernel_poly(p->w, p->beta, kp.data());
         int rc2 = upload(p, &p->kpoly, kp);
-        if (rc2 || (p->queued && (rc2 = upload(p, &p->orb, orbits)))) return rc2;
+        if (rc2) return rc2;
+    }
+
+    int rc3 = upload(p, &p->orb, orbits);
+    if (rc3) return rc3;
+    // ---- loss by mirror images
+    if (!(p->screen_eps > 0.0) && !(ang && d == 3)) {
+        pgb::LossArgs &la = p->largs;
+        la.a = p->a64;
+        la.a32 = p->a32;
+        la.v64 = p->v64;
+        la.v32 = p->v32;
+        la.v32lo = p->v32lo;
+        la.N = N;
+        la.M = M;
+        la.nloss = (int)ipow((N + 1) / 2, d);
+        la.orb = p->orb;
+        la.norb = (int)orbits.size();
+        la.norbits = (long long)ipow((double)orbits.size(), d);
+        // at most two blocks per SM, each of a few orbits per thread; the ub array holds nnode sums
+        la.nbound = (int)std::max<long long>(1, std::min<long long>({(la.norbits + 511) / 512,
+                                                                     2ll * prop.multiProcessorCount, p->nnode}));
+        la.sig64 = p->sig64;
+        la.sig32 = p->sig32;
+        la.ang = p->ang;
+        la.angmax = p->angmax;
+        la.gamma = p->gamma;
+        la.fast_gamma = p->fast_gamma;
+        la.Bw = p->Bconst * p->Wsig;
+        la.inv_mu2 = p->inv_mu2;
+        la.S = p->S;
+        la.r = p->r;
+        la.h = p->h;
+        la.ub = p->ub;
     }
 
     // ---- spreading-kernel arguments
@@ -265,6 +298,9 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     // FP32 strengths carry Bconst, the (common) sphere weight and 1/S as rounded FP32 constants
     p->grid_scale_corr = f32 ? pgb::fp32_strength_correction(p->Bconst, sw[0], p->S, d) : 1.0;
     ka.bound = p->bound;
+    ka.bound_out = p->bound;
+    ka.ub = p->ub;
+    ka.nub = p->largs.nloss ? p->largs.nbound : 0;
     ka.tau = p->tau;
     ka.grid = p->grid;
     ka.simple_fold = (p->w <= p->n / 2) ? 1 : 0;
@@ -319,7 +355,7 @@ int leading_passes(pg_boltz_plan_t *p, const double *in, pgb::Dims3 &dims, const
     double *bufs[2] = {t1, t2};
     int which = 0;
     for (int ax = 3 - p->d; ax < 2; ++ax) {
-        int rc = cuda_check(pgb::launch_axis_pass(cur, dims, ax, A, m, bufs[which], p->stream), "axis pass");
+        int rc = cuda_check(pgb::launch_axis_pass({cur, nullptr, dims, ax, m, A, bufs[which]}, p->stream), "axis pass");
         if (rc) return rc;
         ++*launches;
         dims.e[ax] = m;
@@ -389,8 +425,8 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_ex(const pg_boltz_opts_t *opts)
     in.pairs = p->npairs;
     in.points = p->npairs * p->M;
     in.proj_nodes = p->Mp;
-    in.launches_per_collide = 3 + 3 * p->d;
-    in.kernels_per_collide = 2 + 3 * p->d;
+    in.launches_per_collide = 2 * p->d + 2 + (p->largs.nloss ? 0 : 1);
+    in.kernels_per_collide = in.launches_per_collide;
     in.device_bytes = p->device_bytes;
     return p;
 }
@@ -438,30 +474,32 @@ PG_API int pg_boltz_collide(pg_boltz_plan_t *p, const double *f_dev, double *Q_d
     pgb::Dims3 dims = dims_of(d, N + 1, N + 1, N + 1);
     const double *cur = nullptr;
     if ((rc = leading_passes(p, f_dev, dims, p->R, N, p->tA, p->tB, &cur, &launches))) return rc;
+    // (the last pass also clears the fixed-point grid, its bound and the screening histogram)
+    const long long clear = (long long)ipow(p->nf, d) + 2 + pgb::kScreenBins;
     if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, f32 ? p->a32 : nullptr,
-                                                p->stream), "reconstruct")))
+                                                p->grid, clear, p->stream), "reconstruct")))
         return rc;
     ++launches;
     mark(1);
-    // 2. clear the fixed-point grid and its bound; loss weights h_i = a_i L_i / mu_i^2 (Eq. Qminus,
-    //    inner sum over v_*, sigma) and the strength bound B >= sum_p |q_p|
-    const size_t grid_bytes = (size_t)ipow(p->nf, d) * 8;
-    if ((rc = cuda_check(cudaMemsetAsync(p->grid, 0, grid_bytes + 16 + pgb::kScreenBins * 8, p->stream),
-                         "memset grid")))
-        return rc;
-    ++launches;
-    if ((rc = cuda_check(pgb::launch_loss(p->a64, f32 ? p->a32 : nullptr, p->v64, f32 ? p->v32 : nullptr, p->v32lo, N,
-                                          d, p->M, p->sig64, p->wsig64, p->sig32, p->wsig32, p->ang, p->angmax,
-                                          p->Wsig, p->gamma, p->fast_gamma, p->Bconst * p->Wsig, p->inv_mu2, p->S, p->r, p->h, p->ub,
-                                          p->screen_eps > 0.0 ? p->hist : nullptr, p->stream),
-                         "loss")))
-        return rc;
-    ++launches;
-    if ((rc = cuda_check(pgb::launch_bound_reduce(p->ub, p->nnode, p->screen_eps > 0.0 ? p->hist : nullptr,
-                                                  p->screen_eps, p->bound, p->tau, p->stream),
-                         "bound")))
-        return rc;
-    ++launches;
+    // 2. loss weights h_i = a_i L_i / mu_i^2 (Eq. Qminus, inner sum over v_*, sigma) and the strength
+    //    bound B >= sum_p |q_p|
+    if (p->largs.nloss) {
+        if ((rc = cuda_check(pgb::launch_loss_mirror(p->largs, d, f32, p->stream), "loss"))) return rc;
+        ++launches;
+    } else {
+        if ((rc = cuda_check(pgb::launch_loss(p->a64, f32 ? p->a32 : nullptr, p->v64, f32 ? p->v32 : nullptr, p->v32lo,
+                                              N, d, p->M, p->sig64, p->wsig64, p->sig32, p->wsig32, p->ang, p->angmax,
+                                              p->Wsig, p->gamma, p->fast_gamma, p->Bconst * p->Wsig, p->inv_mu2, p->S,
+                                              p->r, p->h, p->ub, p->screen_eps > 0.0 ? p->hist : nullptr, p->stream),
+                             "loss")))
+            return rc;
+        ++launches;
+        if ((rc = cuda_check(pgb::launch_bound_reduce(p->ub, p->nnode, p->screen_eps > 0.0 ? p->hist : nullptr,
+                                                      p->screen_eps, p->bound, p->tau, p->stream),
+                             "bound")))
+            return rc;
+        ++launches;
+    }
     mark(2);
     // 3. spread the M N^(2d) post-collision points onto the folded grid   (Eq. num_fast_k, Eq. nufft)
     const pgb::SpreadArgs &sa = p->sargs;
@@ -472,26 +510,21 @@ PG_API int pg_boltz_collide(pg_boltz_plan_t *p, const double *f_dev, double *Q_d
     ++launches;
     mark(3);
     // 4. cosine transform + deconvolution of the grid (first pass converts from fixed point),
-    //    forward Chebyshev transform of the loss
-    pgb::Dims3 gd = dims_of(d, p->nf, p->nf, p->nf);
-    const int ax0 = 3 - d;
-    if ((rc = cuda_check(pgb::launch_axis_pass_fixed(p->grid, gd, ax0, p->Dm, N + 1, p->bound, p->grid_scale_corr,
-                                                     p->tA, p->stream),
-                         "transform pass")))
-        return rc;
-    ++launches;
-    gd.e[ax0] = N + 1;
-    const double *gcur = p->tA;
-    if (d == 3) {
-        if ((rc = cuda_check(pgb::launch_axis_pass(p->tA, gd, 1, p->Dm, N + 1, p->tB, p->stream), "transform pass")))
+    //    and the forward Chebyshev transform of the loss, pass by pass in one launch
+    pgb::Dims3 gd = dims_of(d, p->nf, p->nf, p->nf), hd = dims_of(d, N, N, N);
+    const double *gcur = nullptr, *hcur = p->h;
+    double *gbuf[2] = {p->tA, p->tB}, *hbuf[2] = {p->tC, p->tD};
+    for (int ax = 3 - d, k = 0; ax < 2; ++ax, ++k) {
+        const pgb::AxisPass pg{gcur, k ? nullptr : p->grid, gd, ax, N + 1, p->Dm, gbuf[k]};
+        const pgb::AxisPass ph{hcur, nullptr, hd, ax, N + 1, p->E, hbuf[k]};
+        if ((rc = cuda_check(pgb::launch_axis_pass_pair(pg, ph, p->bound, p->grid_scale_corr, p->stream),
+                             "transform pass")))
             return rc;
         ++launches;
-        gd.e[1] = N + 1;
-        gcur = p->tB;
+        gd.e[ax] = hd.e[ax] = N + 1;
+        gcur = gbuf[k];
+        hcur = hbuf[k];
     }
-    pgb::Dims3 hd = dims_of(d, N, N, N);
-    const double *hcur = nullptr;
-    if ((rc = leading_passes(p, p->h, hd, p->E, N + 1, p->tC, p->tD, &hcur, &launches))) return rc;
     // 5. Q = Q+ - Q-
     if ((rc = cuda_check(pgb::launch_final(gcur, gd, p->Dm, hcur, hd, p->E, N + 1, Q_dev, p->Qplus, p->Qlast, p->stream),
                          "final")))
@@ -501,7 +534,7 @@ PG_API int pg_boltz_collide(pg_boltz_plan_t *p, const double *f_dev, double *Q_d
     p->ev_recorded = p->timing;
     p->last_launches = launches;
     p->info.launches_per_collide = launches;
-    p->info.kernels_per_collide = launches - 1;  // one memset
+    p->info.kernels_per_collide = launches;
     p->have_q = true;
     return PG_OK;
 }
@@ -584,7 +617,7 @@ PG_API int pg_boltz_conservation(pg_boltz_plan_t *p, const double *f_dev, double
     pgb::Dims3 dims = dims_of(d, N + 1, N + 1, N + 1);
     const double *cur = nullptr;
     if ((rc = leading_passes(p, f_dev, dims, p->R, N, p->tA, p->tB, &cur, &launches))) return rc;
-    if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, nullptr, p->stream),
+    if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, nullptr, nullptr, 0, p->stream),
                          "reconstruct")))
         return rc;
     const int nout = 2 * (d + 2);
@@ -676,7 +709,7 @@ PG_API int pg_boltz_project(pg_boltz_plan_t *p, const double *fvals_dev, double 
     int which = 0;
     for (int ax = 3 - d; ax < 3; ++ax) {
         double *dst = (ax == 2) ? ftilde_dev : bufs[which];
-        int rc = cuda_check(pgb::launch_axis_pass(cur, dims, ax, p->Pm, N + 1, dst, p->stream), "projection pass");
+        int rc = cuda_check(pgb::launch_axis_pass({cur, nullptr, dims, ax, N + 1, p->Pm, dst}, p->stream), "projection pass");
         if (rc) return rc;
         dims.e[ax] = N + 1;
         cur = dst;

@@ -1959,6 +1959,28 @@ __device__ __forceinline__ void pair_schedule(const SpreadArgs &p, long long &fi
     first = (r * 1000003LL) % nthr;
 }
 
+// The strength bound B, from its partial sums when the loss kernel left those (the same order in
+// every block and for every block size; the factor covers FP32 rounding of the pair terms and of the
+// strengths in the FP32 kernels).  Every thread of the block calls it.
+__device__ __forceinline__ double strength_bound(const SpreadArgs &p)
+{
+    if (p.nub == 0) return *p.bound;
+    __shared__ double s_bound;
+    if (threadIdx.x < 32) {
+        double v = 0.0;
+        for (int k = threadIdx.x; k < p.nub; k += 32) v += p.ub[k];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (threadIdx.x == 0) {
+            v *= 1.0 + 1e-5;
+            s_bound = v;
+            if (blockIdx.x == 0) *p.bound_out = v;
+        }
+    }
+    __syncthreads();
+    return s_bound;
+}
+
 template <int D, int W, bool ANG>
 __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_constant__ SpreadArgs p)
 {
@@ -1971,8 +1993,8 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
         words[c] = 0;
         carry[c] = 0;
     }
+    const double Bnd = strength_bound(p);
     __syncthreads();
-    const double Bnd = *p.bound;
     const int Eg = global_exponent(Bnd);
     // Tile unit 2^-Et with Et = Eg - tile_bits(D) (2^-47 B or finer in 2D, 2^-53 B in 3D); kept
     // inside the float range for tiny inputs (a coarser unit there).
@@ -1980,7 +2002,7 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     const int shift = Eg - Et;
     const SplitTile tile{words, carry};
     const float sc = (float)ldexp(1.0, Et);
-    const float tau = (float)*p.tau;
+    const float tau = p.nub ? 0.0f : (float)*p.tau;
     long long first, nthr;
     pair_schedule(p, first, nthr);
     if (p.nslab > 1) {
@@ -2027,10 +2049,10 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
         tile.hi[c] = 0;
     }
     load_kernel_poly(p.kpoly);
+    const double Bnd = strength_bound(p);
     __syncthreads();
-    const double Bnd = *p.bound;
     const int Eg = global_exponent(Bnd);
-    const double tau = *p.tau;
+    const double tau = p.nub ? 0.0 : *p.tau;
     const double sc = ldexp(1.0, Eg);  // strengths in grid units
     // classes whose summed strength bounds stay below 2^-64 B are skipped (per-point bound below
     // floor_q, and at most nclass classes): 2^-3 grid units at most in all

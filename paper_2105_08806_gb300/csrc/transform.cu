@@ -34,19 +34,19 @@ __device__ __forceinline__ double split_sum(double v)
     return v;
 }
 
-__global__ void k_axis_pass(const double *__restrict__ in, Dims3 id, int ax,
-                            const double *__restrict__ A, int m, double *__restrict__ out)
+// out = (A contracted with `in` along axis ax) scale, by blocks block0 .. block0+nblk-1 of a grid.
+__device__ __forceinline__ void split_pass(const AxisPass &P, double scale, int block, int nblk)
 {
-    Dims3 od = id;
-    od.e[ax] = m;
+    Dims3 od = P.dims;
+    od.e[P.ax] = P.m;
     const long long total = (long long)od.e[0] * od.e[1] * od.e[2];
     const long long tlanes = total * kSplit;
-    const int len = id.e[ax];
-    const long long sax = stride_of(id, ax);
+    const int len = P.dims.e[P.ax];
+    const long long sax = stride_of(P.dims, P.ax);
     const int lane = threadIdx.x & 31;
     // every lane of a warp runs the same iterations (the shuffles need the whole warp)
-    for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt - lane < tlanes;
-         tt += (long long)gridDim.x * blockDim.x) {
+    for (long long tt = block * (long long)blockDim.x + threadIdx.x; tt - lane < tlanes;
+         tt += (long long)nblk * blockDim.x) {
         const long long o = tt / kSplit;
         const int g = (int)(tt % kSplit);
         double acc = 0.0;
@@ -56,38 +56,69 @@ __global__ void k_axis_pass(const double *__restrict__ in, Dims3 id, int ax,
             const long long t = o / od.e[2];
             oc[1] = (int)(t % od.e[1]);
             oc[0] = (int)(t / od.e[1]);
-            const int k = oc[ax];
-            oc[ax] = 0;
-            const long long base = ((long long)oc[0] * id.e[1] + oc[1]) * id.e[2] + oc[2];
-            const double *arow = A + (long long)k * len;
-            for (int s = g; s < len; s += kSplit) acc = fma(arow[s], in[base + s * sax], acc);
+            const int k = oc[P.ax];
+            oc[P.ax] = 0;
+            const long long base = ((long long)oc[0] * P.dims.e[1] + oc[1]) * P.dims.e[2] + oc[2];
+            const double *arow = P.A + (long long)k * len;
+            if (P.fixed_in) {
+                for (int s = g; s < len; s += kSplit)
+                    acc = fma(arow[s], (double)(long long)P.fixed_in[base + s * sax], acc);
+            } else {
+                for (int s = g; s < len; s += kSplit) acc = fma(arow[s], P.in[base + s * sax], acc);
+            }
         }
         acc = split_sum(acc);
-        if (tt < tlanes && g == 0) out[o] = acc;
+        if (tt < tlanes && g == 0) P.out[o] = acc * scale;
     }
 }
 
+__global__ void k_axis_pass(const __grid_constant__ AxisPass P) { split_pass(P, 1.0, blockIdx.x, gridDim.x); }
+
+// One pass of the spread grid's transform (blocks below nblk0; the first pass reads the int64
+// fixed-point grid: out = (A . in) 2^-Eg scale) and one of the loss's, side by side in one launch: the
+// two are independent, and each is a few microseconds that mostly wait on a launch and a serial chain.
+__global__ void k_axis_pass_pair(const __grid_constant__ AxisPass P0, const __grid_constant__ AxisPass P1, int nblk0,
+                                 const double *__restrict__ Bp, double scale)
+{
+    if ((int)blockIdx.x < nblk0)
+        split_pass(P0, P0.fixed_in ? ldexp(scale, -global_exponent(*Bp)) : 1.0, blockIdx.x, nblk0);
+    else
+        split_pass(P1, 1.0, blockIdx.x - nblk0, gridDim.x - nblk0);
+}
+
+// Last reconstruction pass (axis 2) and a_i = W_i mu_i^2 P_i; also clears the `nclear` words at
+// `clear` (the spread grid and its scalars, which nothing reads before the loss kernel), so that no
+// separate memset is launched.
 __global__ void k_recon_last(const double *__restrict__ in, Dims3 id, const double *__restrict__ A,
                              int m, const double *__restrict__ scale, int d, double *__restrict__ a,
-                             float *__restrict__ af)
+                             float *__restrict__ af, unsigned long long *__restrict__ clear, long long nclear)
 {
-    const long long total = (long long)id.e[0] * id.e[1] * m;
+    const long long nthr = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (long long k = tid; k < nclear; k += nthr) clear[k] = 0ull;
+    const long long total = (long long)id.e[0] * id.e[1] * m, tlanes = total * kSplit;
     const int len = id.e[2];
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < total;
-         o += (long long)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (long long tt = tid; tt - lane < tlanes; tt += nthr) {
+        const long long o = tt / kSplit;
+        const int g = (int)(tt % kSplit);
         const int o2 = (int)(o % m);
         const long long t = o / m;
         const int o1 = (int)(t % id.e[1]);
         const int o0 = (int)(t / id.e[1]);
-        const double *src = in + ((long long)o0 * id.e[1] + o1) * len;
-        const double *arow = A + (long long)o2 * len;
         double acc = 0.0;
-        for (int s = 0; s < len; ++s) acc = fma(arow[s], src[s], acc);
-        double sc = scale[o1] * scale[o2];
-        if (d == 3) sc *= scale[o0];
-        acc *= sc;
-        a[o] = acc;
-        if (af) af[o] = (float)acc;
+        if (tt < tlanes) {
+            const double *src = in + ((long long)o0 * id.e[1] + o1) * len;
+            const double *arow = A + (long long)o2 * len;
+            for (int s = g; s < len; s += kSplit) acc = fma(arow[s], src[s], acc);
+        }
+        acc = split_sum(acc);
+        if (tt < tlanes && g == 0) {
+            double sc = scale[o1] * scale[o2];
+            if (d == 3) sc *= scale[o0];
+            acc *= sc;
+            a[o] = acc;
+            if (af) af[o] = (float)acc;
+        }
     }
 }
 
@@ -271,6 +302,242 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const double *__restrict_
     }
 }
 
+// The loss sums and the strength bound by mirror images.
+//
+// The nodes are symmetric about 0 on every axis, so B(|v_i - v_j|) is the same for the 2^d mirror images
+// (i^e, j^e) of a pair (e: the axes reflected, i -> N-1-i): one block per node with i_l <= (N-1)/2 on
+// every axis evaluates B once for all of them and sums L of its 2^d mirror nodes.  The bound of the
+// spreading strengths (LossArgs::ub) is formed per class of node pairs and its mirror images instead of
+// per ordered pair (2^(2d) of them share B and the map factors): blocks nloss .. nloss+nbound-1.
+// With an angular factor (2D: the circle is symmetric in both axes) the mean of b over the sphere set
+// is the same for all of them, too, and only its even part survives the antipodal pairs.
+// The FP32 sums are those of k_loss: the product's FMA residual and a two-sum per term.
+// Measured, loss stage (with the bound's reduction before, which the spreading kernel now does):
+// 2D hard spheres N = 64 FP32 143 -> 43 us, FP64 1323 -> 252 us; N = 120 1294 -> 429 us; 3D VHS N = 24
+// 1212 -> 301 us; 2D angular N = 41, M = 22 408 -> 35 us.
+constexpr int kMirrorThreads = 128;
+
+// (1/Wsig) sum_m w_m b(dvec . sigma_m / g) for the uniform circle, by quarters.
+template <typename PT>
+__device__ __forceinline__ PT circle_mean(const LossArgs &L, const PT *sig, PT d0, PT d1, PT g)
+{
+    const PT ginv = g > PT(0) ? PT(1) / g : PT(0);
+    const int ne = (L.ang.n + 1) / 2;  // terms of the even part
+    PT acc = PT(0);
+    for (int m = 0; 4 * m <= L.M; ++m) {
+        const PT a0 = d0 * ginv * sig[2 * m], a1 = d1 * ginv * sig[2 * m + 1];
+        const PT c0 = (a0 + a1) * (a0 + a1), c1 = (a0 - a1) * (a0 - a1);
+        PT b0 = PT(L.ang.c[2 * (ne - 1)]), b1 = b0;
+        for (int t = ne - 2; t >= 0; --t) {
+            b0 = b0 * c0 + PT(L.ang.c[2 * t]);
+            b1 = b1 * c1 + PT(L.ang.c[2 * t]);
+        }
+        // 4 points of the quad, 2 where it has a zero sine or cosine
+        acc += ((m == 0 || 4 * m == L.M) ? PT(1) : PT(2)) * (b0 + b1);
+    }
+    return acc / PT(L.M);
+}
+
+template <typename PT>
+__device__ __forceinline__ PT vhs_factor(PT g2, PT g, int fast_gamma, PT gam)
+{
+    switch (fast_gamma) {
+    case 0: return PT(1);
+    case 1: return g;
+    case 2: return sqrt(g);
+    default: return (g2 > PT(0)) ? pow(g, gam) : PT(0);
+    }
+}
+
+template <typename PT, int D, bool ANG>
+__global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_constant__ LossArgs L)
+{
+    constexpr int E = 1 << D;
+    constexpr bool F32 = sizeof(PT) == 4;
+    __shared__ double part[kMirrorThreads / 32][E];
+    const int N = L.N;
+    const PT *vn, *av, *sig;
+    if constexpr (F32) {
+        vn = L.v32;
+        av = L.a32;
+        sig = L.sig32;
+    } else {
+        vn = L.v64;
+        av = L.a;
+        sig = L.sig64;
+    }
+    const PT gam = PT(L.gamma);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int)blockIdx.x >= L.nloss) {  // the strength bound
+        const PT S = PT(L.S), invS = PT(1) / S;
+        const int blk = blockIdx.x - L.nloss;
+        double acc = 0.0;
+        PT p = PT(0);
+        int np = 0;
+        for (long long o = blk * (long long)blockDim.x + threadIdx.x; o < L.norbits;
+             o += (long long)L.nbound * blockDim.x) {
+            int ni[D], nj[D];
+            long long t = o;
+            PT g2 = PT(0), cen[D], mult = PT(2);
+            bool self[D];
+#pragma unroll
+            for (int l = D - 1; l >= 0; --l) {
+                const unsigned w = L.orb[t % L.norb];
+                t /= L.norb;
+                ni[l] = w & 0xffffu;
+                nj[l] = w >> 16;
+                self[l] = ni[l] + nj[l] == N - 1;
+                if (ni[l] == nj[l]) mult *= PT(0.5);
+                const PT vi = vn[ni[l]], vj = vn[nj[l]];
+                g2 += (vi - vj) * (vi - vj);
+                cen[l] = PT(0.5) * (vi + vj);
+            }
+            const PT g = sqrt(g2);
+            PT u = mult * vhs_factor(g2, g, L.fast_gamma, gam);
+#pragma unroll
+            for (int l = 0; l < D; ++l) {
+                const PT R = fabs(cen[l]) + PT(0.5) * g;
+                u *= (L.r == 1) ? (S * S + R * R) * invS : S * cosh(R * invS);
+            }
+            PT sum = PT(0);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                bool skip = false;
+#pragma unroll
+                for (int l = 0; l < D; ++l) skip = skip || (((e >> l) & 1) && self[l]);
+                if (skip) continue;  // its own mirror image
+#pragma unroll
+                for (int x = 0; x < E / 2; ++x) {  // the ways to exchange axes 0 .. D-2
+                    int I = 0, J = 0;
+#pragma unroll
+                    for (int l = 0; l < D; ++l) {
+                        const int q = ((e >> l) & 1) ? N - 1 - ni[l] : ni[l];
+                        const int w = ((e >> l) & 1) ? N - 1 - nj[l] : nj[l];
+                        const bool ex = (x >> l) & 1;
+                        I = I * N + (ex ? w : q);
+                        J = J * N + (ex ? q : w);
+                    }
+                    sum += fabs(av[I] * av[J]);
+                }
+            }
+            p += u * sum;
+            if (++np == 64) {
+                acc += (double)p;
+                p = PT(0);
+                np = 0;
+            }
+        }
+        acc += (double)p;
+        const double tot = block_sum<kMirrorThreads>(acc);
+        if (threadIdx.x == 0) L.ub[blk] = tot * L.Bw * L.angmax;
+        return;
+    }
+    int xi[D];
+    {
+        const int nh = (N + 1) / 2;
+        int t = blockIdx.x;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            xi[l] = t % nh;
+            t /= nh;
+        }
+    }
+    PT vx[D], vxl[D];
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+        vx[l] = vn[xi[l]];
+        vxl[l] = F32 ? PT(L.v32lo[xi[l]]) : PT(0);
+    }
+    const int nnode = D == 2 ? N * N : N * N * N;
+    // node j = threadIdx.x + k blockDim.x: its axis indices (C order) advance by the step's digits
+    int jl[D], sl[D];
+    {
+        int t = threadIdx.x, u = blockDim.x;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            jl[l] = t % N;
+            t /= N;
+            sl[l] = u % N;
+            u /= N;
+        }
+    }
+    double acc[E];
+    float as[E], ac[E];  // FP32 plans: the sums as as + ac
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        acc[e] = 0.0;
+        as[e] = ac[e] = 0.0f;
+    }
+    for (int j = threadIdx.x; j < nnode; j += blockDim.x) {
+        PT g2 = PT(0), dv[D];
+        int idx[E];
+        idx[0] = j;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            dv[l] = vx[l] - vn[jl[l]];
+            if constexpr (F32) dv[l] += vxl[l] - PT(L.v32lo[jl[l]]);  // FP32 nodes: their rounding, too
+            g2 += dv[l] * dv[l];
+        }
+        int stride = 1;
+#pragma unroll
+        for (int l = D - 1, n = 1; l >= 0; --l, n *= 2) {
+            const int mir = (N - 1 - 2 * jl[l]) * stride;
+            stride *= N;
+#pragma unroll
+            for (int k = 0; k < n; ++k) idx[n + k] = idx[k] + mir;  // bit (D-1-l) of k's mask: axis l
+        }
+        const PT g = sqrt(g2);
+        PT B = vhs_factor(g2, g, L.fast_gamma, gam);
+        if constexpr (ANG) B *= circle_mean<PT>(L, sig, dv[0], dv[1], g);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const PT aj = av[idx[e]];
+            if constexpr (F32) {
+                const float pt = B * aj;
+                const float pe = fmaf(B, aj, -pt);
+                const float t = as[e] + pt;
+                const float bv = t - as[e];
+                ac[e] += ((as[e] - (t - bv)) + (pt - bv)) + pe;
+                as[e] = t;
+            } else {
+                acc[e] = fma(B, aj, acc[e]);
+            }
+        }
+        int carry = 0;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            jl[l] += sl[l] + carry;
+            carry = jl[l] >= N;
+            if (carry) jl[l] -= N;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        double v = acc[e] + ((double)as[e] + (double)ac[e]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) part[warp][e] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < E) {
+        const int e = threadIdx.x;  // bit k: axis D-1-k reflected
+        double tot = 0.0, sc = 1.0;
+#pragma unroll
+        for (int w = 0; w < kMirrorThreads / 32; ++w) tot += part[w][e];
+        int i = 0;
+        bool dup = false;
+#pragma unroll
+        for (int l = 0; l < D; ++l) {
+            const bool ref = (e >> (D - 1 - l)) & 1;
+            const int x = ref ? N - 1 - xi[l] : xi[l];
+            dup = dup || (ref && 2 * xi[l] == N - 1);
+            i = i * N + x;
+            sc *= L.inv_mu2[x];
+        }
+        if (!dup) L.h[i] = L.a[i] * L.Bw * tot * sc;
+    }
+}
+
 constexpr int kReduceThreads = 1024;
 
 // B = (1 + 1e-5) sum_i ub_i in a fixed order (deterministic); the factor covers FP32 rounding
@@ -298,41 +565,6 @@ __global__ void __launch_bounds__(kReduceThreads) k_bound_reduce(const double *_
             t = ldexp(1.0, k - kScreenOffset);
         }
         *tau = t;
-    }
-}
-
-// First transform pass over the int64 fixed-point grid: out = (A . in) 2^-Eg.
-__global__ void k_axis_pass_fixed(const unsigned long long *__restrict__ in, Dims3 id, int ax,
-                                  const double *__restrict__ A, int m, const double *__restrict__ Bp,
-                                  double scale, double *__restrict__ out)
-{
-    Dims3 od = id;
-    od.e[ax] = m;
-    const long long total = (long long)od.e[0] * od.e[1] * od.e[2];
-    const long long tlanes = total * kSplit;
-    const int len = id.e[ax];
-    const long long sax = stride_of(id, ax);
-    const double unit = ldexp(scale, -global_exponent(*Bp));
-    const int lane = threadIdx.x & 31;
-    for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt - lane < tlanes;
-         tt += (long long)gridDim.x * blockDim.x) {
-        const long long o = tt / kSplit;
-        const int g = (int)(tt % kSplit);
-        double acc = 0.0;
-        if (tt < tlanes) {
-            int oc[3];
-            oc[2] = (int)(o % od.e[2]);
-            const long long t = o / od.e[2];
-            oc[1] = (int)(t % od.e[1]);
-            oc[0] = (int)(t / od.e[1]);
-            const int k = oc[ax];
-            oc[ax] = 0;
-            const long long base = ((long long)oc[0] * id.e[1] + oc[1]) * id.e[2] + oc[2];
-            const double *arow = A + (long long)k * len;
-            for (int s = g; s < len; s += kSplit) acc = fma(arow[s], (double)(long long)in[base + s * sax], acc);
-        }
-        acc = split_sum(acc);
-        if (tt < tlanes && g == 0) out[o] = acc * unit;
     }
 }
 
@@ -525,21 +757,45 @@ int grid_for(long long total)
 
 }  // namespace
 
-cudaError_t launch_axis_pass(const double *in, Dims3 in_dims, int ax, const double *A, int m,
-                             double *out, cudaStream_t s)
+static int pass_blocks(const AxisPass &P)
 {
-    Dims3 od = in_dims;
-    od.e[ax] = m;
-    k_axis_pass<<<grid_for((long long)od.e[0] * od.e[1] * od.e[2] * kSplit), kThreads, 0, s>>>(in, in_dims,
-                                                                                              ax, A, m, out);
+    Dims3 od = P.dims;
+    od.e[P.ax] = P.m;
+    return grid_for((long long)od.e[0] * od.e[1] * od.e[2] * kSplit);
+}
+
+cudaError_t launch_axis_pass(const AxisPass &P, cudaStream_t s)
+{
+    k_axis_pass<<<pass_blocks(P), kThreads, 0, s>>>(P);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_axis_pass_pair(const AxisPass &P0, const AxisPass &P1, const double *B, double scale, cudaStream_t s)
+{
+    const int n0 = pass_blocks(P0), n1 = pass_blocks(P1);
+    k_axis_pass_pair<<<n0 + n1, kThreads, 0, s>>>(P0, P1, n0, B, scale);
     return cudaGetLastError();
 }
 
 cudaError_t launch_recon_last(const double *in, Dims3 in_dims, const double *A, int m,
-                              const double *scale, int d, double *a, float *af, cudaStream_t s)
+                              const double *scale, int d, double *a, float *af, unsigned long long *clear,
+                              long long nclear, cudaStream_t s)
 {
-    k_recon_last<<<grid_for((long long)in_dims.e[0] * in_dims.e[1] * m), kThreads, 0, s>>>(
-        in, in_dims, A, m, scale, d, a, af);
+    k_recon_last<<<grid_for((long long)in_dims.e[0] * in_dims.e[1] * m * kSplit), kThreads, 0, s>>>(
+        in, in_dims, A, m, scale, d, a, af, clear, nclear);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_loss_mirror(const LossArgs &L, int d, bool f32, cudaStream_t s)
+{
+    const int blocks = L.nloss + L.nbound;
+    const bool ang = L.ang.n > 0;
+    if (f32 && d == 2 && ang) k_loss_mirror<float, 2, true><<<blocks, kMirrorThreads, 0, s>>>(L);
+    else if (f32 && d == 2) k_loss_mirror<float, 2, false><<<blocks, kMirrorThreads, 0, s>>>(L);
+    else if (f32) k_loss_mirror<float, 3, false><<<blocks, kMirrorThreads, 0, s>>>(L);
+    else if (d == 2 && ang) k_loss_mirror<double, 2, true><<<blocks, kMirrorThreads, 0, s>>>(L);
+    else if (d == 2) k_loss_mirror<double, 2, false><<<blocks, kMirrorThreads, 0, s>>>(L);
+    else k_loss_mirror<double, 3, false><<<blocks, kMirrorThreads, 0, s>>>(L);
     return cudaGetLastError();
 }
 
@@ -571,16 +827,6 @@ cudaError_t launch_bound_reduce(const double *ub, int n, const unsigned long lon
                                 double *tau, cudaStream_t s)
 {
     k_bound_reduce<<<1, kReduceThreads, 0, s>>>(ub, n, hist, eps, B, tau);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_axis_pass_fixed(const unsigned long long *in, Dims3 in_dims, int ax, const double *A,
-                                   int m, const double *B, double scale, double *out, cudaStream_t s)
-{
-    Dims3 od = in_dims;
-    od.e[ax] = m;
-    k_axis_pass_fixed<<<grid_for((long long)od.e[0] * od.e[1] * od.e[2] * kSplit), kThreads, 0, s>>>(
-        in, in_dims, ax, A, m, B, scale, out);
     return cudaGetLastError();
 }
 
