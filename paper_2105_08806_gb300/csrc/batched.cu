@@ -313,6 +313,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.nnode = cd.nnode;
     sa.naxp = cd.naxp;
     sa.nclass = cd.nclass;
+    sa.nsplit = 1;
     sa.n = cd.n;
     sa.nf = cd.nf;
     sa.rows_per_slab = cd.nf;
@@ -435,7 +436,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
         if constexpr (F32) {
             float *buf = reinterpret_cast<float *>(smem_raw + b.queue_off) + warp * 32 * spread_queue_values(D, true);
             if constexpr (D == 2)
-                spread_quads<W, false, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
+                spread_quads<W, false, false, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
                                               plane, buf);
             else
                 spread_points3<W, false, false>(sa, first, p1, blockDim.x, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
@@ -898,7 +899,7 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
     const int accept_threads = pgb::accept_threads(d, f32);
     // the smallest block the plan makes: 128 threads, fewer where the largest tile leaves less room
     int min_threads = 128;
-    while (min_threads > 64 && batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
+    while (min_threads > 32 && batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
         min_threads -= 32;
     if (batch_smem(*B, min_threads) + B->static_smem > prop.sharedMemPerBlockOptin) {
         set_error(PG_ERR_ARG, "largest cell's folded grid (%d cells) does not fit shared memory", max_cells_tile);

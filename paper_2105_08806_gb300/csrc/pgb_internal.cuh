@@ -49,6 +49,7 @@ struct SpreadArgs {
     int nnode;            // N^d interior nodes
     int naxp;             // unordered pairs of node indices per axis, unordered_pairs(N)
     long long nclass;     // classes of node pairs that share their points, naxp^d
+    int nsplit;           // FP32 2D one-slab grids: shares that a class' quads are spread in (1: all at once)
     int n, nf;            // periodic grid size, folded cells per axis (n/2 + 1)
     int rows_per_slab;    // folded-grid rows (axis 0) held in shared memory by one block
     int nslab;            // number of slabs covering axis 0
@@ -132,11 +133,11 @@ __device__ __forceinline__ const TypedConsts<T> &kconst(const SpreadArgs &a)
 __host__ __device__ inline long long unordered_pairs(long long nnode) { return nnode * (nnode + 1) / 2; }
 
 // Values per slot of the spreading kernels' warp queues.  FP32 2D: a large or half quad (6) and a class
-// (4, angular kernels 8); 3D: three points by size (velocity and strength, 4 each) and a class (5,
+// (5, angular kernels 9); 3D: three points by size (velocity and strength, 4 each) and a class (5,
 // angular kernels 12).  FP64: a point, d coordinates and its strength.
 __host__ __device__ constexpr int spread_queue_values(int d, bool f32, bool ang = false)
 {
-    return !f32 ? d + 1 : d == 2 ? (ang ? 14 : 10) : (ang ? 24 : 17);
+    return !f32 ? d + 1 : d == 2 ? (ang ? 15 : 11) : (ang ? 24 : 17);
 }
 // Shared memory of the warp queues of a spreading block of `threads` threads: 32 slots per warp.
 __host__ __device__ constexpr size_t spread_queue_bytes(int threads, int d, bool f32, bool ang = false)

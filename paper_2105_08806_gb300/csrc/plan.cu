@@ -169,12 +169,20 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         p->spread_threads = std::max(128, std::min(max_threads, t));
     }
     if (p->nslab > 1 && ask_threads <= 0) p->spread_threads = slab_threads;  // the queues were sized for it
+    // FP32 2D: with fewer classes than threads, the classes' quads are cut into shares, so that there is
+    // an item per thread (2D N = 16, M = 8: 18,496 classes of 3 quads, spreading 41 -> 31 us).  With
+    // more classes (N = 32: 2.9 per thread) the repeated class tests cost what the fuller rounds gain.
+    int nsplit = 1;
+    if (f32 && p->nslab == 1 && d == 2) {
+        const long long want = (long long)prop.multiProcessorCount * max_threads;
+        nsplit = (int)std::max<long long>(1, std::min<long long>(M / 4 + 1, want / p->nclass));
+    }
     if (p->nslab == 1 && ask_threads <= 0) {
         // small plans: blocks no larger than it takes for every SM to have one (each thread then
         // owns one class; 1024-thread blocks would keep 18 of 152 SMs busy for 2D N = 16, whose
         // spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks of 1024 with a
         // point set per pair)
-        const long long per_block = (p->nclass + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
+        const long long per_block = (p->nclass * nsplit + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
         const int small = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
         p->spread_threads = std::min(p->spread_threads, small);
     }
@@ -216,7 +224,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     per_sm = std::max(per_sm, 1);
     long long blocks = (long long)prop.multiProcessorCount * per_sm;
     blocks = std::max<long long>(blocks / p->nslab, 1) * p->nslab;
-    const long long items = (!f32 && p->queued) ? nitem : p->nclass;
+    const long long items = (!f32 && p->queued) ? nitem : p->nclass * nsplit;
     const long long need = ((items + p->spread_threads - 1) / p->spread_threads) * p->nslab;
     blocks = std::min(blocks, need);
     p->spread_blocks = (int)blocks;
@@ -268,6 +276,8 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         la.ub = p->ub;
     }
 
+    if (!p->queued) nsplit = 1;  // (no queue: whole classes)
+
     // ---- spreading-kernel arguments
     pgb::SpreadArgs &ka = p->sargs;
     ka.d = d;
@@ -277,6 +287,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.nnode = p->nnode;
     ka.naxp = (int)pgb::unordered_pairs(N);
     ka.nclass = p->nclass;
+    ka.nsplit = nsplit;
     ka.n = p->n;
     ka.nf = p->nf;
     ka.rows_per_slab = p->rows_per_slab;

@@ -1279,10 +1279,17 @@ __device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float 
     }
 }
 
-// The points of one class per lane (every lane of the warp calls it; P.base = 0: none).  buf, count:
-// the warp's queue of large quads, 32 slots of kQuadValues floats, and its fill.
-template <int W, bool ANG>
-__device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const PairData<float, 2> &P, float qbase,
+// SPLIT (small plans): classes are spread in p.nsplit shares of their quads; share g takes
+// [share_start(g), share_start(g + 1)) of n.
+__device__ __forceinline__ int share_start(const SpreadArgs &p, int g, int n)
+{
+    return (int)((long long)g * n / p.nsplit);
+}
+
+// Share g of the quads of one class per lane (every lane of the warp calls it; P.base = 0: none).  buf,
+// count: the warp's queue of large quads, 32 slots of kQuadValues floats, and its fill.
+template <int W, bool ANG, bool SPLIT>
+__device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const PairData<float, 2> &P, float qbase, int g,
                                                    const SplitTile &tile, int nrows, int plane, float *buf, int &count)
 {
     const unsigned full = 0xffffffffu;
@@ -1290,10 +1297,17 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
     const TypedConsts<float> &K = p.cf;
     const bool alg = (p.r == 1);
     const bool simple = p.simple_fold != 0;
+    int m0 = 0, m1 = p.M / 4 + 1, steps = m1;
+    if constexpr (SPLIT) {
+        steps = (m1 + p.nsplit - 1) / p.nsplit;  // the largest share, so that the lanes stay together
+        m0 = share_start(p, g, m1);
+        m1 = share_start(p, g + 1, m1);
+    }
 #pragma unroll 1
-    for (int m = 0; 4 * m <= p.M; ++m) {
+    for (int k = 0; k < steps; ++k) {
+        const int m = SPLIT ? min(m0 + k, p.M / 4) : k;
         const bool one_row = (4 * m == p.M), one_col = (m == 0);  // no mirror image
-        const Quad Q = make_quad<ANG>(p, P, qbase, m);
+        const Quad Q = make_quad<ANG>(p, P, (!SPLIT || m0 + k < m1) ? qbase : 0.0f, m);
         const float qmax = fmaxf(fabsf(Q.q1), fabsf(Q.q2)) * fmaxf(Q.mr[0], Q.mr[1]) * fmaxf(Q.mc[0], Q.mc[1]);
         const bool large = qmax >= kIntLimitF32;
         const unsigned lmask = __ballot_sync(full, large);
@@ -1475,7 +1489,7 @@ __device__ __forceinline__ void spread_class_halves(const SpreadArgs &p, const P
 // that is negligible varies from lane to lane, and with every lane spreading its own the warp
 // waited for the lane with the most (about a third of the lanes' time on the headline workload).
 // buf: the warp's queues, 32 slots of spread_queue_values(2, true, ANG) floats.
-template <int W, bool ANG, bool SLAB>
+template <int W, bool ANG, bool SLAB, bool SPLIT>
 __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long first, long long end, long long stride,
                                              float sc, float tau, const SplitTile &tile, int row_lo, int nrows,
                                              int plane, float *buf)
@@ -1491,8 +1505,14 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
         if (!more && nclass == 0) break;
         PairData<float, 2> P;
         bool hit = false;
+        int share = 0;
         if (c.pr < end) {
-            hit = class_passes<float, 2, ANG>(p, c, sc, tau, kNegligibleF32, P);
+            PairCursor cc = c;
+            if constexpr (SPLIT) {  // the share is the slowest index
+                share = c.t / p.naxp;
+                cc.t = c.t - share * p.naxp;
+            }
+            hit = class_passes<float, 2, ANG>(p, cc, sc, tau, kNegligibleF32, P);
             pair_advance(p.naxp, c, st);
         }
         auto put = [&](int slot) {
@@ -1506,6 +1526,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
                 cbuf[192 + slot] = P.dir[0];
                 cbuf[224 + slot] = P.dir[1];
             }
+            if constexpr (SPLIT) cbuf[(ANG ? 256 : 128) + slot] = __int_as_float(share);
         };
         const unsigned mask = __ballot_sync(full, hit);
         const int n = __popc(mask), rank = __popc(mask & ((1u << lane) - 1u)), room = 32 - nclass;
@@ -1515,6 +1536,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
             const bool valid = lane < min(nclass + n, 32);
             PairData<float, 2> C;
             zero_pair<float, 2>(C);
+            int mine = 0;
             if (valid) {
                 C.cen[0] = cbuf[lane];
                 C.cen[1] = cbuf[32 + lane];
@@ -1526,12 +1548,13 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
                     C.dir[0] = cbuf[192 + lane];
                     C.dir[1] = cbuf[224 + lane];
                 }
+                if constexpr (SPLIT) mine = __float_as_int(cbuf[(ANG ? 256 : 128) + lane]);
             }
             __syncwarp();
             if (hit && rank >= room) put(rank - room);
             nclass = max(n - room, 0);
             if constexpr (SLAB) spread_class_halves<W, ANG>(p, C, C.base * sc, tile, row_lo, nrows, plane, buf, count);
-            else spread_class_quads<W, ANG>(p, C, C.base * sc, tile, nrows, plane, buf, count);
+            else spread_class_quads<W, ANG, SPLIT>(p, C, C.base * sc, mine, tile, nrows, plane, buf, count);
         } else {
             nclass += n;
         }
@@ -1981,7 +2004,7 @@ __device__ __forceinline__ double strength_bound(const SpreadArgs &p)
     return s_bound;
 }
 
-template <int D, int W, bool ANG>
+template <int D, int W, bool ANG, bool SPLIT>
 __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_constant__ SpreadArgs p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2009,14 +2032,15 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes((size_t)p.rows_per_slab * G.plane, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
         if constexpr (D == 2)
-            spread_quads<W, ANG, true>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
+            spread_quads<W, ANG, true, false>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
         else
             spread_points3<W, ANG, true>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
     } else if (p.queued) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes(G.ncell, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
         if constexpr (D == 2)
-            spread_quads<W, ANG, false>(p, first, p.nclass, nthr, sc, tau, tile, 0, G.nrows, G.plane, buf);
+            spread_quads<W, ANG, false, SPLIT>(p, first, SPLIT ? p.nclass * p.nsplit : p.nclass, nthr, sc, tau, tile, 0,
+                                               G.nrows, G.plane, buf);
         else
             spread_points3<W, ANG, false>(p, first, p.nclass, nthr, sc, tau, tile, 0, G.nrows, G.plane, buf);
     } else {
@@ -2084,7 +2108,9 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
 template <int D, int W, bool ANG>
 cudaError_t launch_f32(const SpreadArgs &a, int blocks, int threads, size_t smem, cudaStream_t s)
 {
-    auto kern = k_spread_f32<D, W, ANG>;
+    auto kern = k_spread_f32<D, W, ANG, false>;
+    if constexpr (D == 2)
+        if (a.nsplit > 1) kern = k_spread_f32<D, W, ANG, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks, threads, smem, s>>>(a);

@@ -374,16 +374,29 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
         double acc = 0.0;
         PT p = PT(0);
         int np = 0;
-        for (long long o = blk * (long long)blockDim.x + threadIdx.x; o < L.norbits;
-             o += (long long)L.nbound * blockDim.x) {
-            int ni[D], nj[D];
-            long long t = o;
-            PT g2 = PT(0), cen[D], mult = PT(2);
-            bool self[D];
+        const long long first = blk * (long long)blockDim.x + threadIdx.x, step = (long long)L.nbound * blockDim.x;
+        int ol[D], os[D];  // the orbit's axis orbits and the step's, digits in base norb (no division per orbit)
+        {
+            long long t = first, u = step;
 #pragma unroll
             for (int l = D - 1; l >= 0; --l) {
-                const unsigned w = L.orb[t % L.norb];
+                ol[l] = (int)(t % L.norb);
                 t /= L.norb;
+                os[l] = (int)(u % L.norb);
+                u /= L.norb;
+            }
+        }
+        for (long long o = first; o < L.norbits; o += step) {
+            int ni[D], nj[D];
+            PT g2 = PT(0), cen[D], mult = PT(2);
+            bool self[D];
+            int carry = 0;
+#pragma unroll
+            for (int l = D - 1; l >= 0; --l) {
+                const unsigned w = L.orb[ol[l]];
+                ol[l] += os[l] + carry;
+                carry = ol[l] >= L.norb;
+                if (carry) ol[l] -= L.norb;
                 ni[l] = w & 0xffffu;
                 nj[l] = w >> 16;
                 self[l] = ni[l] + nj[l] == N - 1;
