@@ -340,7 +340,7 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.nang_even = 0;  // batched cells use VHS kernels
     sa.angmax = 1.0;
     sa.cpad = tile_col_pad(b.w, b.d, f32);
-    sa.ncol = cd.nf + 2 * sa.cpad;
+    sa.ncol = tile_cols(cd.nf, b.w, b.d, f32);
     sa.kpoly = b.kpoly;
     sa.queued = 0;  // (FP64: no orbit items)
     sa.trim_q = b.trim_q;
@@ -800,7 +800,7 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         cd.grid_off = grid_off;
         grid_off += cells_tile;
         // block tile: the last axis padded with unfolded columns (see spread_impl.cuh)
-        const long long tile_cells = (long long)ipow(cd.nf, d - 1) * (cd.nf + 2 * pgb::tile_col_pad(B->w, d, f32));
+        const long long tile_cells = (long long)ipow(cd.nf, d - 1) * pgb::tile_cols(cd.nf, B->w, d, f32);
         max_cells_tile = std::max<int>(max_cells_tile, (int)tile_cells);
         cd.s_len = std::max<long long>(modes, (long long)(N + 1) * (long long)ipow(cd.nf, d - 1));
         cd.s_off = s_off;

@@ -73,8 +73,8 @@ struct SpreadArgs {
     const double *tau;    // device scalar: node pairs whose strength bound is below it are skipped (0: none)
     unsigned long long *grid;  // nf^d folded grid, int64 fixed point in units of 2^-Eg
     int simple_fold;      // 1 when w <= n/2: unfolded indices lie in [-n/2, n] (no modulo needed)
-    int cpad;             // unfolded padding columns on each side of the last axis in block tiles
-    int ncol;             // nf + 2 cpad: tile cells along the last axis
+    int cpad;             // unfolded padding columns before the last axis' columns in block tiles
+    int ncol;             // tile cells along the last axis (tile_cols)
     int tile_cells;       // cells of one block tile (rows_per_slab rows)
     int *carry;           // FP32: per-block carry counters, blocks x tile_cells (global memory)
     int queued;           // one-slab grids: 1 when the warps' queues follow the tile in shared memory (FP32:
@@ -151,12 +151,18 @@ __host__ __device__ inline size_t tile_bytes(size_t cells, bool f32)
     return (cells * (f32 ? 4 : 12) + 15) / 16 * 16;
 }
 
-// Padding columns of the block tiles' last axis for kernel width w: the unfolded support of a point
-// at grid coordinate x in [0, n/2] spans floor(x - w/2) + 1 .. floor(x + w/2), i.e. at most w/2
-// columns beyond either end; w/2 + 1 leave a margin for rounding of x.
-// FP64 3D tiles have none (N = 11, w = 14: 24 instead of 40 cells per line of the grid, so that it fits one
-// block instead of two slabs, both of which nearly every point reaches).
-__host__ __device__ inline int tile_col_pad(int w, int d, bool f32) { return (d == 3 && !f32) ? 0 : w / 2 + 1; }
+// Padding columns of the block tiles' last axis for kernel width w, before the grid's columns and after
+// them: the unfolded support of a point at grid coordinate x in [0, n/2] runs from floor(x - w/2) + 1 to
+// floor(x - w/2) + w, i.e. from -((w-1)/2) to n/2 + w/2.  FP64 2D tiles are symmetric (their mirrored
+// classes need it).  FP64 3D tiles have none (N = 11, w = 14: 24 instead of 38 cells per line of the
+// grid, so that it fits one block instead of two slabs, both of which nearly every point reaches).
+// (With one margin column more on each side FP32 3D tiles left room for 16 warps' queues instead of 20:
+// N = 24 52 -> 44 ms, N = 16 6.4 -> 6.0 ms.)
+__host__ __device__ inline int tile_col_pad(int w, int d, bool f32) { return f32 ? (w - 1) / 2 : d == 3 ? 0 : w / 2; }
+__host__ __device__ inline int tile_cols(int nf, int w, int d, bool f32)
+{
+    return nf + tile_col_pad(w, d, f32) + ((d == 3 && !f32) ? 0 : w / 2);
+}
 
 // FP32 block tiles count in units 2^-(Eg - tile_bits(d)), about 2^-47 B (2D) or 2^-53 B (3D) for the
 // strength bound B: each contribution is rounded to the tile unit once, and with w^3 contributions

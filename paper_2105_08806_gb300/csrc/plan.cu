@@ -115,7 +115,8 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "cudaGetDeviceProperties: %s", cudaGetErrorString(e));
     const size_t elem = (p->prec == PG_PREC_FP32) ? 4 : 12;  // 32-bit words per cell: FP32 one, FP64 three
     // block tiles: rows of (nf^(d-2) x ncol) cells, the last axis padded with unfolded columns (FP64 3D: not)
-    const int cpad = pgb::tile_col_pad(p->w, d, p->prec == PG_PREC_FP32), ncol = p->nf + 2 * cpad;
+    const int cpad = pgb::tile_col_pad(p->w, d, p->prec == PG_PREC_FP32);
+    const int ncol = pgb::tile_cols(p->nf, p->w, d, p->prec == PG_PREC_FP32);
     const size_t plane = (size_t)ipow(p->nf, d - 2) * ncol;
     const bool f32 = (p->prec == PG_PREC_FP32), ang = p->ang.n > 0;
     // leave room for the kernels' static shared memory (FP64: the kernel polynomial)
@@ -195,7 +196,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         if (ask_threads <= 0)
             while (p->spread_threads > 128 &&
                    p->spread_smem + pgb::spread_queue_bytes(p->spread_threads, d, true, ang) > max_smem)
-                p->spread_threads -= 128;
+                p->spread_threads -= 32;
         const size_t qq = pgb::spread_queue_bytes(p->spread_threads, d, true, ang);
         if (p->spread_smem + qq <= max_smem) {
             p->queued = 1;

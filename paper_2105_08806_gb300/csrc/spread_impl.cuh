@@ -764,8 +764,8 @@ __device__ __forceinline__ void make_point(const SpreadArgs &p, const PairData<T
 
 // Tile layout.  A block tile holds rows row_lo..row_lo+nrows-1 of axis 0 of the folded grid, and
 // along the last axis (but for FP64 3D tiles, whose three words per cell leave no room for it: cpad = 0,
-// ncol = nf, and a point's columns are folded once for its w^2 rows) it keeps the UNFOLDED columns u = -cpad..nf-1+cpad at u + cpad (ncol =
-// nf + 2 cpad cells): the w columns of a point are then consecutive, with no folding and no
+// ncol = nf, and a point's columns are folded once for its w^2 rows) it keeps the
+// UNFOLDED columns that points reach, u at u + cpad (ncol cells, tile_cols): the w columns of a point are then consecutive, with no folding and no
 // per-contribution index arithmetic.  The padding columns are folded onto their cells when the
 // tile is added to the global grid (tile_to_grid_cell).  2D cell (row, u): row ncol + u + cpad;
 // 3D cell (row, j, u): (row nf + j) ncol + u + cpad.
@@ -1371,10 +1371,29 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
     }
 }
 
+// The velocities v' on axis 0 whose points may reach the rows row_lo .. row_lo+nrows-1: a point at x
+// touches rows of [x - w/2, x + w/2] (and their mirror images beyond the grid's ends, which lie in the
+// first and last slabs), and x falls with v'.  A thousandth of a cell is added at both ends for the
+// rounding of x; a point that then misses the slab finds no row in it.  Two comparisons per point
+// and slab, where forming x and folding w rows took 85 instructions (3D VHS N = 24, three slabs: 55.7 -> 52.4 ms).
+struct SlabRange {
+    float lo, hi;
+};
+template <int W>
+__device__ __forceinline__ SlabRange slab_range(const SpreadArgs &p, int row_lo, int nrows)
+{
+    const double x0 = row_lo - 0.5 * W - 1e-3, x1 = row_lo + nrows - 1 + 0.5 * W + 1e-3;
+    auto velocity = [&](double x) {
+        const double z = x / p.grid_scale;
+        return (float)(p.r == 1 ? p.S * cos(z) / sin(z) : -p.S * log(tan(0.5 * z)));
+    };
+    const float inf = __int_as_float(0x7f800000);
+    return SlabRange{x1 >= 0.5 * p.n ? -inf : velocity(x1), x0 <= 0.0 ? inf : velocity(x0)};
+}
+
 // In a slabbed grid half of a quad's rows or more lie outside a block's slab, so there the quads are
-// queued by halves (N = 120, M = 8: spreading 5.44 -> 4.58 ms against a queue of single points): one
-// coordinate of axis 0 (cell X, fraction F) whose rows reach the slab, and the
-// two of axis 1 with the strengths of their points (0: no such point), kQuadValues values.
+// queued by halves (N = 120, M = 8: spreading 5.44 -> 4.58 ms against a queue of single points, 4.16 ms
+// with the slab's velocity range): one coordinate of axis 0 whose rows may reach the slab, and the two of axis 1 with the strengths of their points (0: no such point), kQuadValues values.
 
 // Add one point of a half quad: rows ra (-1: outside the slab) with factors pa, column factors col.
 template <int W, int KIND>
@@ -1414,8 +1433,9 @@ __device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const floa
     const int lane = threadIdx.x & 31;
     const TypedConsts<float> &K = p.cf;
     const bool simple = p.simple_fold != 0;
-    float t0;
-    const int s0 = first_tap_f32<W>(buf[lane], buf[32 + lane], t0);
+    float X, F, t0;
+    grid_coord_f32(K, buf[lane], p.r == 1, X, F);
+    const int s0 = first_tap_f32<W>(X, F, t0);
     float pa[W];
     int ra[W];
 #pragma unroll
@@ -1426,10 +1446,10 @@ __device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const floa
     }
 #pragma unroll 1
     for (int t = 0; t < 2; ++t) {
-        const float q = buf[(4 + t) * 32 + lane];
+        const float q = buf[(3 + t) * 32 + lane];
         if (!(fabsf(q) >= kNegligibleF32)) continue;
         QuadCols<W> col;
-        quad_cols<W>(p, buf[(2 + t) * 32 + lane], col);
+        quad_cols<W>(p, buf[(1 + t) * 32 + lane], col);
         if (fabsf(q) < kIntLimitF32) half_quad_point<W, kInt>(tile, ra, pa, col, q);
         else half_quad_point<W, kLarge>(tile, ra, pa, col, q);  // rare in grids of this size
     }
@@ -1440,7 +1460,7 @@ __device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const floa
 template <int W, bool ANG>
 __device__ __forceinline__ void spread_class_halves(const SpreadArgs &p, const PairData<float, 2> &P, float qbase,
                                                     const SplitTile &tile, int row_lo, int nrows, int plane,
-                                                    float *buf, int &count)
+                                                    SlabRange range, float *buf, int &count)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -1453,21 +1473,16 @@ __device__ __forceinline__ void spread_class_halves(const SpreadArgs &p, const P
             const float mr = s ? Q.mr[1] : Q.mr[0];
             const float qa = (s ? Q.q2 : Q.q1) * mr * Q.mc[0];
             const float qb = m ? (s ? Q.q1 : Q.q2) * mr * Q.mc[1] : 0.0f;
-            float X = 0.0f, F = 0.0f, t0;
-            bool hit = fmaxf(fabsf(qa), fabsf(qb)) >= kNegligibleF32;
-            if (hit) {
-                grid_coord_f32(p.cf, s ? Q.vr[1] : Q.vr[0], p.r == 1, X, F);
-                hit = rows_hit_from<W>(p, first_tap_f32<W>(X, F, t0), row_lo, nrows);
-            }
+            const float vr = s ? Q.vr[1] : Q.vr[0];
+            const bool hit = fmaxf(fabsf(qa), fabsf(qb)) >= kNegligibleF32 && vr >= range.lo && vr <= range.hi;
             const unsigned mask = __ballot_sync(full, hit);
             const int n = __popc(mask), rank = __popc(mask & ((1u << lane) - 1u)), room = 32 - count;
             auto put = [&](int slot) {
-                buf[slot] = X;
-                buf[32 + slot] = F;
-                buf[64 + slot] = Q.vc[0];
-                buf[96 + slot] = Q.vc[1];
-                buf[128 + slot] = qa;
-                buf[160 + slot] = qb;
+                buf[slot] = vr;
+                buf[32 + slot] = Q.vc[0];
+                buf[64 + slot] = Q.vc[1];
+                buf[96 + slot] = qa;
+                buf[128 + slot] = qb;
             };
             if (hit && rank < room) put(count + rank);
             if (n >= room) {
@@ -1497,6 +1512,8 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     float *cbuf = buf + 32 * kQuadValues;  // the class queue
+    SlabRange range{0.0f, 0.0f};
+    if constexpr (SLAB) range = slab_range<W>(p, row_lo, nrows);
     int count = 0, nclass = 0;             // queued (large or half) quads and classes, the same in every lane
     PairCursor c = pair_cursor(p.naxp, first);
     const PairStep st = pair_step(p.naxp, stride);
@@ -1553,7 +1570,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
             __syncwarp();
             if (hit && rank >= room) put(rank - room);
             nclass = max(n - room, 0);
-            if constexpr (SLAB) spread_class_halves<W, ANG>(p, C, C.base * sc, tile, row_lo, nrows, plane, buf, count);
+            if constexpr (SLAB) spread_class_halves<W, ANG>(p, C, C.base * sc, tile, row_lo, nrows, plane, range, buf, count);
             else spread_class_quads<W, ANG, SPLIT>(p, C, C.base * sc, mine, tile, nrows, plane, buf, count);
         } else {
             nclass += n;
@@ -1664,6 +1681,8 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     float *cbuf = buf + 3 * PV;  // the class queue
+    SlabRange range{0.0f, 0.0f};
+    if constexpr (SLAB) range = slab_range<W>(p, row_lo, nrows);
     int fill = 0;                // of the point queues kInt, kLarge, kSmall, 8 bits each; the same in every lane
     int nclass = 0;
     PairCursor c = pair_cursor(p.naxp, first);
@@ -1727,7 +1746,7 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
                 const float qa = fabsf(e.q());
                 if (qa >= kNegligibleF32) kind = qa >= kIntLimitF32 ? kLarge : qa < p.cf.trim_q ? kSmall : kInt;
                 if constexpr (SLAB)
-                    if (kind >= 0 && !e.template in_slab<W>(p, row_lo, nrows)) kind = -1;
+                    if (!(e.v[0] >= range.lo && e.v[0] <= range.hi)) kind = -1;
             }
 #pragma unroll 1
             for (int k = 0; k < 3; ++k) {
