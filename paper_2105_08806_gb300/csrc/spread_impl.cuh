@@ -1279,6 +1279,41 @@ __device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float 
     }
 }
 
+// One point of a quad, any strength, in little code: the rows in a loop and the taps as scaled integers
+// (spread_point_f32's kLarge, the same bits for points below 2^29 tile units as kInt).  Small plans run
+// every instruction a few times per warp, and what they wait for is mostly instruction fetch (2D Maxwell
+// N = 16: 5.3 of 12 warps); one such loop serves all their points in place of the unrolled code for the four
+// points of a quad and that of the large ones (spreading 33 -> 27 us).
+template <int W>
+__device__ __forceinline__ void spread_point_compact(const SpreadArgs &p, float v0, float v1, float q,
+                                                     const SplitTile &tile, int plane)
+{
+    const TypedConsts<float> &K = p.cf;
+    const bool alg = (p.r == 1), simple = p.simple_fold != 0;
+    int first[2];
+    float off[2];  // local memory
+#pragma unroll 1
+    for (int l = 0; l < 2; ++l) {
+        float X, F, t0;
+        grid_coord_f32(K, l ? v1 : v0, alg, X, F);
+        first[l] = first_tap_f32<W>(X, F, t0);
+        off[l] = t0;
+    }
+    const int cb = min(max(first[1] + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
+    int wi[W];
+#pragma unroll
+    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_f32(fmaf((float)c, 2.0f / W, off[1]), K.bl, 30.0f - K.bl));
+    const int sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
+    const float q4 = 4.0f * q * __int_as_float((127 - sc) << 23);
+#pragma unroll 1
+    for (int a = 0; a < W; ++a) {
+        const int rq = __float2int_rn(q4 * es_f32(fmaf((float)a, 2.0f / W, off[0]), K.bl, -K.bl));
+        const int line = fold_cell(first[0] + a, p.n, simple) * plane + cb;
+#pragma unroll
+        for (int c = 0; c < W; ++c) tile.add_scaled(line + c, mulhi_rn(rq, wi[c]), sc);
+    }
+}
+
 // SPLIT (small plans): classes are spread in p.nsplit shares of their quads; share g takes
 // [share_start(g), share_start(g + 1)) of n.
 __device__ __forceinline__ int share_start(const SpreadArgs &p, int g, int n)
@@ -1308,6 +1343,17 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
         const int m = SPLIT ? min(m0 + k, p.M / 4) : k;
         const bool one_row = (4 * m == p.M), one_col = (m == 0);  // no mirror image
         const Quad Q = make_quad<ANG>(p, P, (!SPLIT || m0 + k < m1) ? qbase : 0.0f, m);
+        if constexpr (SPLIT) {
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+                const int t = i >> 1, r = i & 1;
+                if ((t && one_col) || (r && one_row)) continue;
+                const float q = (r == t ? Q.q1 : Q.q2) * (r ? Q.mr[1] : Q.mr[0]) * (t ? Q.mc[1] : Q.mc[0]);
+                if (fabsf(q) >= kNegligibleF32)
+                    spread_point_compact<W>(p, r ? Q.vr[1] : Q.vr[0], t ? Q.vc[1] : Q.vc[0], q, tile, plane);
+            }
+            continue;
+        }
         const float qmax = fmaxf(fabsf(Q.q1), fabsf(Q.q2)) * fmaxf(Q.mr[0], Q.mr[1]) * fmaxf(Q.mc[0], Q.mc[1]);
         const bool large = qmax >= kIntLimitF32;
         const unsigned lmask = __ballot_sync(full, large);
@@ -1578,7 +1624,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
     }
     __syncwarp();
     if constexpr (SLAB) spread_half_quad<W>(p, buf, lane < count, tile, row_lo, nrows, plane);
-    else if (lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
+    else if (!SPLIT && lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
 }
 
 // ---- 3D FP32 grids
