@@ -2073,14 +2073,17 @@ template <int D, int W, bool ANG, bool SPLIT>
 __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_constant__ SpreadArgs p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_dependents();
     const SlabGeom G = slab_geometry(p, D);
     if (G.nrows <= 0) return;  // uniform over the block: an empty trailing slab does nothing
+    // (the tile and the carries are the block's own: no earlier kernel of this evaluation touches them)
     int *words = reinterpret_cast<int *>(smem_raw);
     int *carry = p.carry + (size_t)blockIdx.x * p.tile_cells;
     for (int c = threadIdx.x; c < G.ncell; c += blockDim.x) {
         words[c] = 0;
         carry[c] = 0;
     }
+    grid_wait();
     const double Bnd = strength_bound(p);
     __syncthreads();
     const int Eg = global_exponent(Bnd);
@@ -2126,6 +2129,7 @@ template <int D, int W, bool ANG>
 __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_constant__ SpreadArgs p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_dependents();
     const SlabGeom G = slab_geometry(p, D);
     if (G.nrows <= 0) return;  // uniform over the block
     // fraction, low and high words of rows_per_slab x plane cells each
@@ -2138,6 +2142,7 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
         tile.hi[c] = 0;
     }
     load_kernel_poly(p.kpoly);
+    grid_wait();
     const double Bnd = strength_bound(p);
     __syncthreads();
     const int Eg = global_exponent(Bnd);
@@ -2178,8 +2183,7 @@ cudaError_t launch_f32(const SpreadArgs &a, int blocks, int threads, size_t smem
         if (a.nsplit > 1) kern = k_spread_f32<D, W, ANG, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, blocks, threads, smem, s, a);
 }
 
 template <int D, int W, bool ANG>
@@ -2188,8 +2192,7 @@ cudaError_t launch_f64(const SpreadArgs &a, int blocks, int threads, size_t smem
     auto kern = k_spread_f64<D, W, ANG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, blocks, threads, smem, s, a);
 }
 
 // Compile-time dispatch on the kernel width w in [W, WMAX].  ANG: the angular-kernel variant

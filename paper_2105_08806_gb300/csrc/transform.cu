@@ -72,7 +72,11 @@ __device__ __forceinline__ void split_pass(const AxisPass &P, double scale, int 
     }
 }
 
-__global__ void k_axis_pass(const __grid_constant__ AxisPass P) { split_pass(P, 1.0, blockIdx.x, gridDim.x); }
+__global__ void k_axis_pass(const __grid_constant__ AxisPass P)
+{
+    launch_dependents();
+    split_pass(P, 1.0, blockIdx.x, gridDim.x);
+}
 
 // One pass of the spread grid's transform (blocks below nblk0; the first pass reads the int64
 // fixed-point grid: out = (A . in) 2^-Eg scale) and one of the loss's, side by side in one launch: the
@@ -80,6 +84,8 @@ __global__ void k_axis_pass(const __grid_constant__ AxisPass P) { split_pass(P, 
 __global__ void k_axis_pass_pair(const __grid_constant__ AxisPass P0, const __grid_constant__ AxisPass P1, int nblk0,
                                  const double *__restrict__ Bp, double scale)
 {
+    launch_dependents();
+    grid_wait();
     if ((int)blockIdx.x < nblk0)
         split_pass(P0, P0.fixed_in ? ldexp(scale, -global_exponent(*Bp)) : 1.0, blockIdx.x, nblk0);
     else
@@ -93,6 +99,8 @@ __global__ void k_recon_last(const double *__restrict__ in, Dims3 id, const doub
                              int m, const double *__restrict__ scale, int d, double *__restrict__ a,
                              float *__restrict__ af, unsigned long long *__restrict__ clear, long long nclear)
 {
+    launch_dependents();
+    grid_wait();
     const long long nthr = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     for (long long k = tid; k < nclear; k += nthr) clear[k] = 0ull;
     const long long total = (long long)id.e[0] * id.e[1] * m, tlanes = total * kSplit;
@@ -352,6 +360,8 @@ __device__ __forceinline__ PT vhs_factor(PT g2, PT g, int fast_gamma, PT gam)
 template <typename PT, int D, bool ANG>
 __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_constant__ LossArgs L)
 {
+    launch_dependents();
+    grid_wait();
     constexpr int E = 1 << D;
     constexpr bool F32 = sizeof(PT) == 4;
     __shared__ double part[kMirrorThreads / 32][E];
@@ -585,6 +595,7 @@ __global__ void k_final(const double *__restrict__ G, Dims3 gd, const double *__
                         const double *__restrict__ H, Dims3 hd, const double *__restrict__ E, int m,
                         double *__restrict__ Q, double *__restrict__ Qplus, double *__restrict__ Qcopy)
 {
+    grid_wait();
     const long long total = (long long)gd.e[0] * gd.e[1] * m;
     const long long tlanes = total * kSplit;
     const int lg = gd.e[2];
@@ -786,30 +797,26 @@ cudaError_t launch_axis_pass(const AxisPass &P, cudaStream_t s)
 cudaError_t launch_axis_pass_pair(const AxisPass &P0, const AxisPass &P1, const double *B, double scale, cudaStream_t s)
 {
     const int n0 = pass_blocks(P0), n1 = pass_blocks(P1);
-    k_axis_pass_pair<<<n0 + n1, kThreads, 0, s>>>(P0, P1, n0, B, scale);
-    return cudaGetLastError();
+    return launch_dependent(k_axis_pass_pair, n0 + n1, kThreads, 0, s, P0, P1, n0, B, scale);
 }
 
 cudaError_t launch_recon_last(const double *in, Dims3 in_dims, const double *A, int m,
                               const double *scale, int d, double *a, float *af, unsigned long long *clear,
                               long long nclear, cudaStream_t s)
 {
-    k_recon_last<<<grid_for((long long)in_dims.e[0] * in_dims.e[1] * m * kSplit), kThreads, 0, s>>>(
-        in, in_dims, A, m, scale, d, a, af, clear, nclear);
-    return cudaGetLastError();
+    return launch_dependent(k_recon_last, grid_for((long long)in_dims.e[0] * in_dims.e[1] * m * kSplit), kThreads, 0, s,
+                            in, in_dims, A, m, scale, d, a, af, clear, nclear);
 }
 
 cudaError_t launch_loss_mirror(const LossArgs &L, int d, bool f32, cudaStream_t s)
 {
     const int blocks = L.nloss + L.nbound;
     const bool ang = L.ang.n > 0;
-    if (f32 && d == 2 && ang) k_loss_mirror<float, 2, true><<<blocks, kMirrorThreads, 0, s>>>(L);
-    else if (f32 && d == 2) k_loss_mirror<float, 2, false><<<blocks, kMirrorThreads, 0, s>>>(L);
-    else if (f32) k_loss_mirror<float, 3, false><<<blocks, kMirrorThreads, 0, s>>>(L);
-    else if (d == 2 && ang) k_loss_mirror<double, 2, true><<<blocks, kMirrorThreads, 0, s>>>(L);
-    else if (d == 2) k_loss_mirror<double, 2, false><<<blocks, kMirrorThreads, 0, s>>>(L);
-    else k_loss_mirror<double, 3, false><<<blocks, kMirrorThreads, 0, s>>>(L);
-    return cudaGetLastError();
+    auto kern = k_loss_mirror<double, 3, false>;
+    if (f32 && d == 2) kern = ang ? k_loss_mirror<float, 2, true> : k_loss_mirror<float, 2, false>;
+    else if (f32) kern = k_loss_mirror<float, 3, false>;
+    else if (d == 2) kern = ang ? k_loss_mirror<double, 2, true> : k_loss_mirror<double, 2, false>;
+    return launch_dependent(kern, blocks, kMirrorThreads, 0, s, L);
 }
 
 cudaError_t launch_loss(const double *a, const float *a32, const double *vnode, const float *vnode32,
@@ -847,9 +854,8 @@ cudaError_t launch_final(const double *G, Dims3 g_dims, const double *D, const d
                          Dims3 h_dims, const double *E, int m, double *Q, double *Qplus,
                          double *Qcopy, cudaStream_t s)
 {
-    k_final<<<grid_for((long long)g_dims.e[0] * g_dims.e[1] * m * kSplit), kThreads, 0, s>>>(G, g_dims, D, H, h_dims,
-                                                                                            E, m, Q, Qplus, Qcopy);
-    return cudaGetLastError();
+    return launch_dependent(k_final, grid_for((long long)g_dims.e[0] * g_dims.e[1] * m * kSplit), kThreads, 0, s, G, g_dims,
+                            D, H, h_dims, E, m, Q, Qplus, Qcopy);
 }
 
 cudaError_t launch_axpy(const double *x, const double *k, double c, double *y, long long n, cudaStream_t s)
