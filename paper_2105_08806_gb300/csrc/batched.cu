@@ -336,7 +336,6 @@ __device__ __forceinline__ void cell_args(const BatchArgs &b, const CellDesc &cd
     sa.nub = 0;
     sa.tau = nullptr;  // the batched kernel reads Tcell directly
     sa.grid = b.grid + cd.grid_off;
-    sa.simple_fold = (b.w <= cd.n / 2) ? 1 : 0;
     sa.nang_even = 0;  // batched cells use VHS kernels
     sa.angmax = 1.0;
     sa.cpad = tile_col_pad(b.w, b.d, f32);

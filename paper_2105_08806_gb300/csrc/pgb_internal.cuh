@@ -72,7 +72,6 @@ struct SpreadArgs {
     double *bound_out;    // = bound
     const double *tau;    // device scalar: node pairs whose strength bound is below it are skipped (0: none)
     unsigned long long *grid;  // nf^d folded grid, int64 fixed point in units of 2^-Eg
-    int simple_fold;      // 1 when w <= n/2: unfolded indices lie in [-n/2, n] (no modulo needed)
     int cpad;             // unfolded padding columns before the last axis' columns in block tiles
     int ncol;             // tile cells along the last axis (tile_cols)
     int tile_cells;       // cells of one block tile (rows_per_slab rows)

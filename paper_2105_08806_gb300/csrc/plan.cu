@@ -315,7 +315,6 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.nub = p->largs.nloss ? p->largs.nbound : 0;
     ka.tau = p->tau;
     ka.grid = p->grid;
-    ka.simple_fold = (p->w <= p->n / 2) ? 1 : 0;
     ka.cpad = cpad;
     ka.ncol = ncol;
     ka.tile_cells = (int)tile_cells;

@@ -93,14 +93,14 @@ __device__ __forceinline__ int fold_index(int u, int n)
     return (g > (n >> 1)) ? n - g : g;
 }
 
-// Unfolded index u -> folded cell; `simple` when u is known to lie in [-n/2, n].
-__device__ __forceinline__ int fold_cell(int u, int n, bool simple)
+// Unfolded index u of a point's support -> folded cell: min(|u|, |n - |u||), which is fold(u) for |u| <= 3n/2.
+// A support reaches at most w/2 beyond [0, n/2], so |u| <= n/2 + w/2, and w <= 2n for every plan (n >= 8,
+// w <= 16): no modulo and no branch (a general path here, never taken but for the smallest grids, was
+// inlined at every tap row; with the guards of the inner taps, below, 1-4% of every FP32 evaluation).
+__device__ __forceinline__ int fold_cell(int u, int n)
 {
-    if (simple) {  // u in [-n/2, n]: fold(u) = min(|u|, n - |u|)
-        u = abs(u);
-        return min(u, n - u);
-    }
-    return fold_index(u, n);
+    u = abs(u);
+    return min(u, abs(n - u));
 }
 
 // Kernel weights psi(x_u - z) of one axis, u = s..s+w-1, in units where one grid cell is 1 and
@@ -270,6 +270,16 @@ __device__ __forceinline__ float es_f32(float t, float bl, float bias)
     const float e = fmaf(bl, om * rsqrt_approx(om), bias);
     return om > 0.0f ? ex2_approx(e) : 0.0f;
 }
+// The same at tap a of W (known when the loop over taps is unrolled): only the first and the last tap
+// can lie on the support's ends.
+template <int W>
+__device__ __forceinline__ float es_tap_f32(int a, float t0, float bl, float bias)
+{
+    const float t = fmaf((float)a, 2.0f / W, t0);
+    if (a == 0 || a == W - 1) return es_f32(t, bl, bias);
+    const float om = fmaf(-t, t, 1.0f);
+    return ex2_approx(fmaf(bl, om * rsqrt_approx(om), bias));
+}
 
 // First tap s = X + c0 of a point at X + F for kernel width W (s = floor(x - W/2) + 1) and the tap
 // offset t0 = (s - x) 2/W; tap a has t = t0 + a 2/W.
@@ -291,11 +301,10 @@ __device__ __forceinline__ void axis_weights_f32(const SpreadArgs &p, float X, f
     const int s = first_tap_f32<W>(X, F, t0);
     const float h2 = 2.0f / W;
     const float bl = p.cf.bl;
-    const bool simple = p.simple_fold != 0;
 #pragma unroll
     for (int a = 0; a < W; ++a) {
-        wt[a] = es_f32(fmaf((float)a, h2, t0), bl, -bl);
-        idx[a] = fold_cell(s + a, p.n, simple);
+        wt[a] = es_tap_f32<W>(a, t0, bl, -bl);
+        idx[a] = fold_cell(s + a, p.n);
     }
 }
 
@@ -806,7 +815,6 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     if (fabsf(q) < kNegligibleF32) return;  // every contribution rounds to zero
     const float bl = p.cf.bl;
     const float h2 = 2.0f / W;
-    const bool simple = p.simple_fold != 0;
     float t00, tl0;
     const int s0 = first_tap_f32<W>(pt.X[0], pt.F[0], t00);          // first row
     const int sl = first_tap_f32<W>(pt.X[D - 1], pt.F[D - 1], tl0);  // first column (unfolded)
@@ -828,7 +836,7 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     const float bias30 = 30.0f - bl;
     int wi[W];
 #pragma unroll
-    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_f32(fmaf((float)c, h2, tl0), bl, bias30));
+    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_tap_f32<W>(c, tl0, bl, bias30));
     auto run = [&](int line, int rq) {
         if constexpr (KIND == kLarge) {
 #pragma unroll
@@ -843,7 +851,7 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     if constexpr (D == 2) {
 #pragma unroll
         for (int a = 0; a < W; ++a) {
-            int r = fold_cell(s0 + a, p.n, simple);
+            int r = fold_cell(s0 + a, p.n);
             if constexpr (SLAB) {
                 r -= row_lo;
                 if ((unsigned)r >= (unsigned)nrows) continue;
@@ -853,7 +861,7 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     } else {
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            int r = fold_cell(s0 + a, p.n, simple);
+            int r = fold_cell(s0 + a, p.n);
             if constexpr (SLAB) {
                 r -= row_lo;
                 if ((unsigned)r >= (unsigned)nrows) continue;
@@ -870,10 +878,9 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
 template <int W>
 __device__ __forceinline__ bool rows_hit_from(const SpreadArgs &p, int s, int row_lo, int nrows)
 {
-    const bool simple = p.simple_fold != 0;
     bool hit = false;
 #pragma unroll
-    for (int a = 0; a < W; ++a) hit |= (unsigned)(fold_cell(s + a, p.n, simple) - row_lo) < (unsigned)nrows;
+    for (int a = 0; a < W; ++a) hit |= (unsigned)(fold_cell(s + a, p.n) - row_lo) < (unsigned)nrows;
     return hit;
 }
 
@@ -890,7 +897,6 @@ __device__ __forceinline__ void spread_point_f64(const SpreadArgs &p, const Poin
                                                  const WideTile &tile, int row_lo, int nrows, int plane)
 {
     if (pt.q == 0.0) return;
-    const bool simple = p.simple_fold != 0;
     if constexpr (SLAB) {
         if (!rows_hit_from<W>(p, (int)floor(pt.x[0] - 0.5 * W) + 1, row_lo, nrows)) return;
     }
@@ -906,19 +912,19 @@ __device__ __forceinline__ void spread_point_f64(const SpreadArgs &p, const Poin
         for (int c = 0; c < W; ++c) cl[c] = c;
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            const int r = fold_cell(s0 + a, p.n, simple) - row_lo;
+            const int r = fold_cell(s0 + a, p.n) - row_lo;
             if (SLAB && (unsigned)r >= (unsigned)nrows) continue;
             const unsigned long long R2 = fix_mul(k.q2, f0[a]) << 1;
             if (R2) wide_row<W>(tile, r * plane + cb, cl, R2, k, fl);
         }
     } else {
 #pragma unroll
-        for (int c = 0; c < W; ++c) cl[c] = fold_cell(sl + c, p.n, simple);
+        for (int c = 0; c < W; ++c) cl[c] = fold_cell(sl + c, p.n);
         FixW f1[W];
         const int s1 = axis_weights_f64<W>(pt.x[1], f1);
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            const int r = fold_cell(s0 + a, p.n, simple) - row_lo;
+            const int r = fold_cell(s0 + a, p.n) - row_lo;
             if (SLAB && (unsigned)r >= (unsigned)nrows) continue;
             const unsigned long long Ra2 = fix_mul(k.q2, f0[a]) << 1;
             if (!Ra2) continue;
@@ -926,7 +932,7 @@ __device__ __forceinline__ void spread_point_f64(const SpreadArgs &p, const Poin
 #pragma unroll 1
             for (int b = 0; b < W; ++b) {
                 const unsigned long long R2 = fix_mul(Ra2, f1[b]) << 1;
-                if (R2) wide_row<W>(tile, row + fold_cell(s1 + b, p.n, simple) * p.ncol, cl, R2, k, fl);
+                if (R2) wide_row<W>(tile, row + fold_cell(s1 + b, p.n) * p.ncol, cl, R2, k, fl);
             }
         }
     }
@@ -1255,7 +1261,7 @@ __device__ __forceinline__ void quad_cols(const SpreadArgs &p, float v, QuadCols
     c.cb = min(max(s + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
     const float bias30 = 30.0f - p.cf.bl;
 #pragma unroll
-    for (int k = 0; k < W; ++k) c.wi[k] = __float2int_rn(es_f32(fmaf((float)k, 2.0f / W, t0), p.cf.bl, bias30));
+    for (int k = 0; k < W; ++k) c.wi[k] = __float2int_rn(es_tap_f32<W>(k, t0, p.cf.bl, bias30));
 }
 
 // The large quad in slot `lane` of the queue: its points one by one.
@@ -1289,7 +1295,7 @@ __device__ __forceinline__ void spread_point_compact(const SpreadArgs &p, float 
                                                      const SplitTile &tile, int plane)
 {
     const TypedConsts<float> &K = p.cf;
-    const bool alg = (p.r == 1), simple = p.simple_fold != 0;
+    const bool alg = (p.r == 1);
     int first[2];
     float off[2];  // local memory
 #pragma unroll 1
@@ -1302,13 +1308,13 @@ __device__ __forceinline__ void spread_point_compact(const SpreadArgs &p, float 
     const int cb = min(max(first[1] + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
     int wi[W];
 #pragma unroll
-    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_f32(fmaf((float)c, 2.0f / W, off[1]), K.bl, 30.0f - K.bl));
+    for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_tap_f32<W>(c, off[1], K.bl, 30.0f - K.bl));
     const int sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
     const float q4 = 4.0f * q * __int_as_float((127 - sc) << 23);
 #pragma unroll 1
     for (int a = 0; a < W; ++a) {
         const int rq = __float2int_rn(q4 * es_f32(fmaf((float)a, 2.0f / W, off[0]), K.bl, -K.bl));
-        const int line = fold_cell(first[0] + a, p.n, simple) * plane + cb;
+        const int line = fold_cell(first[0] + a, p.n) * plane + cb;
 #pragma unroll
         for (int c = 0; c < W; ++c) tile.add_scaled(line + c, mulhi_rn(rq, wi[c]), sc);
     }
@@ -1331,7 +1337,6 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
     const int lane = threadIdx.x & 31;
     const TypedConsts<float> &K = p.cf;
     const bool alg = (p.r == 1);
-    const bool simple = p.simple_fold != 0;
     int m0 = 0, m1 = p.M / 4 + 1, steps = m1;
     if constexpr (SPLIT) {
         steps = (m1 + p.nsplit - 1) / p.nsplit;  // the largest share, so that the lanes stay together
@@ -1395,8 +1400,8 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
             int ra[W];
 #pragma unroll
             for (int k = 0; k < W; ++k) {
-                pa[k] = es_f32(fmaf((float)k, 2.0f / W, t0), K.bl, -K.bl);
-                ra[k] = fold_cell(s0 + k, p.n, simple) * plane;
+                pa[k] = es_tap_f32<W>(k, t0, K.bl, -K.bl);
+                ra[k] = fold_cell(s0 + k, p.n) * plane;
             }
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
@@ -1478,7 +1483,6 @@ __device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const floa
     if (!valid) return;
     const int lane = threadIdx.x & 31;
     const TypedConsts<float> &K = p.cf;
-    const bool simple = p.simple_fold != 0;
     float X, F, t0;
     grid_coord_f32(K, buf[lane], p.r == 1, X, F);
     const int s0 = first_tap_f32<W>(X, F, t0);
@@ -1486,8 +1490,8 @@ __device__ __forceinline__ void spread_half_quad(const SpreadArgs &p, const floa
     int ra[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-        pa[k] = es_f32(fmaf((float)k, 2.0f / W, t0), K.bl, -K.bl);
-        const int r = fold_cell(s0 + k, p.n, simple) - row_lo;
+        pa[k] = es_tap_f32<W>(k, t0, K.bl, -K.bl);
+        const int r = fold_cell(s0 + k, p.n) - row_lo;
         ra[k] = (unsigned)r < (unsigned)nrows ? r * plane : -1;
     }
 #pragma unroll 1
@@ -1645,7 +1649,7 @@ __device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *
 {
     if (!valid) return;
     const int lane = threadIdx.x & 31;
-    const bool alg = (p.r == 1), simple = p.simple_fold != 0;
+    const bool alg = (p.r == 1);
     const float bl = p.cf.bl, h2 = 2.0f / W;
     float X, F, t0, tl0, t1;
     grid_coord_f32(p.cf, buf[64 + lane], alg, X, F);
@@ -1659,9 +1663,9 @@ __device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *
     float w1[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-        wi[k] = __float2int_rn(es_f32(fmaf((float)k, h2, tl0), bl, 30.0f - bl));
-        w1[k] = es_f32(fmaf((float)k, h2, t1), bl, -bl);
-        c1[k] = fold_cell(s1 + k, p.n, simple) * p.ncol + cb;
+        wi[k] = __float2int_rn(es_tap_f32<W>(k, tl0, bl, 30.0f - bl));
+        w1[k] = es_tap_f32<W>(k, t1, bl, -bl);
+        c1[k] = fold_cell(s1 + k, p.n) * p.ncol + cb;
     }
     const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
     float q4 = 4.0f * q;
@@ -1673,7 +1677,7 @@ __device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *
     const int a0 = (kind == kSmall) ? 1 : 0;
 #pragma unroll 1
     for (int a = a0; a < W - a0; ++a) {
-        int r = fold_cell(s0 + a, p.n, simple);
+        int r = fold_cell(s0 + a, p.n);
         if constexpr (SLAB) {
             r -= row_lo;
             if ((unsigned)r >= (unsigned)nrows) continue;
@@ -1914,7 +1918,6 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
                                                   int plane)
 {
     const double *sig = static_cast<const double *>(p.sig);
-    const bool simple = p.simple_fold != 0;
     const int nrow = (4 * m == p.M) ? 1 : 2, ncolumn = (m == 0) ? 1 : 2;  // 1: no mirror image
     const double cs = sig[2 * m], sn = sig[2 * m + 1];
     FixW fr[2][W], fc[2][W];  // local memory
@@ -1961,7 +1964,7 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
             const WideScale k = wide_scale(q);
 #pragma unroll 1
             for (int a = 0; a < W; ++a) {
-                int r = fold_cell(sr[s] + a, p.n, simple);
+                int r = fold_cell(sr[s] + a, p.n);
                 if (e0) r = p.nf - 1 - r;
                 const unsigned long long R2 = fix_mul(k.q2, fr[s][a]) << 1;
                 if (R2) wide_row<W>(tile, r * plane + cb, cl, R2, k, fl);
