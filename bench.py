@@ -285,11 +285,11 @@ def errors_vs_oracle(Q, N, name):
 
 
 def spread_roofline(info, d, spread_ms, peaks):
-    """Shared-memory additions of the spreading kernel: w^d for each of the M N^d (N^d + 1)/2 points
-    of the unordered node pairs (the points the kernel skips exactly, whose contributions all round
-    to zero, included), per launch, over the launch's time; peak = the measured conflict-free
-    int32 shared-atomic rate of the whole GPU."""
-    adds = info["points"] * info["kernel_width"] ** d
+    """Shared-memory additions of the spreading kernel: w^d for each of the M (N (N + 1)/2)^d points of
+    the classes of node pairs that share their points (the points the kernel skips exactly, whose
+    contributions all round to zero, included), per launch, over the launch's time; peak = the
+    measured conflict-free int32 shared-atomic rate of the whole GPU."""
+    adds = info["M"] * (info["N"] * (info["N"] + 1) // 2) ** d * info["kernel_width"] ** d
     achieved = adds / (spread_ms * 1e-3)
     return {"bound": "alu", "achieved": achieved / 1e9, "peak": peaks["shared_atomics_free"] / 1e9,
             "unit": "G shared-memory additions/s", "frac": achieved / peaks["shared_atomics_free"],
@@ -609,7 +609,7 @@ def run_ours(args):
         r.pop("_wall_s", None)
     r32 = h["fp32"]
     roof = dict(r32["roofline"])
-    roof["kernel"] = f"k_spread_f32<{h['d']},{r32['kernel_width']},0>"
+    roof["kernel"] = f"k_spread_f32<{h['d']},{r32['kernel_width']},0,0>"
     same_kernel = PROFILED_TRAFFIC["source_sha16"] == kernel_source_sha16() and head == HEADLINE
     roof["traffic"] = PROFILED_TRAFFIC["bytes"] if same_kernel else None
     res = {

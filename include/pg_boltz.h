@@ -100,12 +100,13 @@ typedef struct {
     int slabs;             /* shared-memory slabs of the folded grid along axis 1           */
     int spread_blocks, spread_threads;
     size_t spread_smem_bytes;
-    long long points;      /* non-uniform points spread per evaluation, M x pairs            */
-    long long pairs;       /* node pairs spread per evaluation: each unordered pair {i, j} of
-                              the N^d interior nodes once, N^d (N^d + 1) / 2 (the orders (i, j)
-                              and (j, i) add the same points with the same strength)          */
+    long long points;      /* non-uniform points of one evaluation, M x pairs                */
+    long long pairs;       /* unordered node pairs {i, j} of the N^d interior nodes,
+                              N^d (N^d + 1) / 2.  (Pairs that share their points -- exchanged
+                              components on some axes -- are spread as one: M (N (N + 1)/2)^d
+                              points are spread.)                                             */
     int proj_nodes;
-    int launches_per_collide; /* kernels + memsets enqueued by one pg_boltz_collide          */
+    int launches_per_collide; /* kernels enqueued by one pg_boltz_collide (batched: and memsets) */
     size_t device_bytes;   /* device memory owned by the plan                               */
     int kernels_per_collide; /* kernel launches (memsets excluded) of one collide              */
 } pg_boltz_info_t;
@@ -275,7 +276,7 @@ int pg_boltz_batched_use_graph(pg_boltz_plan_t *plan, int enable);
  * Autotuner of a batched plan's persistent spreading launch (no counterpart in the paper, which
  * evaluates one operator at a time): runs pg_boltz_collide_batched's launch sequence on the
  * caller's f_packed_dev / Q_packed_dev (Q is overwritten), first for threads per block in
- * {128, 256, 512, 1024} and every blocks-per-SM count the kernel's occupancy allows (FP32 plans:
+ * {128, 256, 512} and every blocks-per-SM count the kernel's occupancy allows (FP32 plans:
  * at most the block count the plan sized its carry counters for), then at the fastest shape for
  * work items of 2^15, 2^16, ..., 2^19 points (the node-pair ranges the blocks take from the
  * global counter); `trials` timed runs each after one warm-up.  Keeps the fastest shape and item

@@ -80,12 +80,22 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     std::vector<float> spf(sp.begin(), sp.end()), swf(sw.begin(), sw.end());
 
     int rc;
+    // one allocation for the node and sphere tables in FP64, one for those in FP32
+    std::vector<double> t64;
+    std::vector<float> t32;
+    for (const std::vector<double> *v : {&nt.scale_a, &nt.inv_mu2, &nt.v, &sp, &sw})
+        t64.insert(t64.end(), v->begin(), v->end());
+    for (const std::vector<float> *v : {&vf, &vflo, &spf, &swf}) t32.insert(t32.end(), v->begin(), v->end());
     if ((rc = upload(p, &p->R, nt.R)) || (rc = upload(p, &p->E, nt.E)) || (rc = upload(p, &p->Dm, D)) ||
-        (rc = upload(p, &p->Pm, P)) || (rc = upload(p, &p->scale_a, nt.scale_a)) ||
-        (rc = upload(p, &p->inv_mu2, nt.inv_mu2)) || (rc = upload(p, &p->v64, nt.v)) ||
-        (rc = upload(p, &p->v32, vf)) || (rc = upload(p, &p->v32lo, vflo)) || (rc = upload(p, &p->sig64, sp)) ||
-        (rc = upload(p, &p->wsig64, sw)) || (rc = upload(p, &p->sig32, spf)) || (rc = upload(p, &p->wsig32, swf)))
+        (rc = upload(p, &p->Pm, P)) || (rc = upload(p, &p->scale_a, t64)) || (rc = upload(p, &p->v32, t32)))
         return rc;
+    p->inv_mu2 = p->scale_a + N;
+    p->v64 = p->inv_mu2 + N;
+    p->sig64 = p->v64 + N;
+    p->wsig64 = p->sig64 + sp.size();
+    p->v32lo = p->v32 + N;
+    p->sig32 = p->v32lo + N;
+    p->wsig32 = p->sig32 + spf.size();
 
     // ---- workspace
     const long long modes = (long long)ipow(N + 1, d);

@@ -30,7 +30,7 @@
 //    words (WideTile: native 32-bit atomics, the next word's only when a carry or a high part
 //    needs it).  The kernel weights are FP64; per point, a row factor R = round(q psi_a 2^(Eg+s))
 //    with a per-point scale s that keeps R below 2^62 (3D: then round(R psi_b) in integers) is
-//    formed once per row, and each contribution is round(R psi_c) from a 61-bit fixed-point psi_c
+//    formed once per row, and each contribution is round(R psi_c) from a 63-bit fixed-point psi_c
 //    by four 32 x 32-bit integer products, so no FP64 operation runs per cell (the FP64 pipe of
 //    this GPU runs at about 1/70 of the FP32 rate) and each contribution keeps about 2^-61 of its
 //    size plus 2^-32 grid units.  At the end each cell rounds to the grid unit once per block.
@@ -44,16 +44,17 @@
 //    are several times slower than 32-bit ones.)  Points below 2^29 tile units -- nearly all of
 //    them -- form their contributions in integers: the row factor 4 q psi_a (psi_b) and the column
 //    factor 2^30 psi_c are rounded once per row and column, and a contribution is the rounded high
-//    word of their 64-bit product (one integer multiply-add).  At the end each block adds
+//    word of their 64-bit product (one integer multiply-add); larger points do the same on a coarser
+//    unit of their own.  At the end each block adds
 //    word + 2^32 carry (scaled by 2^tile_bits(d)) to the global grid.  Each contribution is rounded
 //    to the tile unit (at most about one unit); all later additions are exact.
 //
-// Negligible pairs: in the FP32 kernels a pair whose strength bound keeps every one of its points
+// Negligible classes: in the FP32 kernels a class whose strength bound keeps every one of its points
 // below 0.1 tile unit adds exactly zero (every contribution rounds to zero), so it is skipped, and
-// so are such points one by one; the FP64 kernels skip pairs whose summed bounds stay below
-// 2^-64 B (2^-3 grid units in all).  Each lane searches ahead for its
-// next pair that is not negligible, so that the lanes of a warp spread real pairs together (with
-// the node sets of the workloads here, 25-75% of all pairs lie in the tails of f and are skipped).
+// so are such points one by one; the FP64 kernels skip classes whose summed bounds stay below
+// 2^-64 B (2^-3 grid units in all).  The FP32 kernels and the FP64 2D kernel queue the classes (items)
+// that are not negligible per warp, so that its lanes spread together (with the node sets of the
+// workloads here, up to 70% of all classes lie in the tails of f and are skipped).
 #pragma once
 
 #include <climits>
@@ -1021,138 +1022,36 @@ __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long firs
     }
 }
 
-// ---- slabbed grids: warp point queues
+// ---- slabbed FP64 grids: warp point queues
 //
 // When the folded grid is split into slabs along axis 0, a point adds to a block's slab only
 // if one of its w axis-0 rows lies there, and with a few slabs most points of a warp miss it:
 // spreading them where they are generated would leave most lanes idle while the others add.
 // Instead each warp appends the points that hit its slab to a queue of 32 entries in shared
-// memory (slot-major) and spreads a full queue with all 32 lanes, one point per lane.
-
-// Whether any of the w axis-0 rows of a point lies in the slab (the rows of the point's spreading).
-template <typename T, int D, int W>
-__device__ __forceinline__ bool rows_hit(const SpreadArgs &p, const Point<T, D> &pt, int row_lo, int nrows)
-{
-    int s;
-    if constexpr (sizeof(T) == 4) {
-        float t0;
-        s = first_tap_f32<W>(pt.X[0], pt.F[0], t0);
-    } else {
-        s = (int)floor(pt.x[0] - 0.5 * W) + 1;
-    }
-    return rows_hit_from<W>(p, s, row_lo, nrows);
-}
-
-// What a warp queue holds for one point.  LATE (FP32): the post-collision velocity v'[D] and the
-// strength q; the grid coordinates are formed after the queue, only for the points that go there (in a
-// slabbed grid axis 0's once more: 45 instructions of the thousand that a 3D point takes, for two
-// words less per slot).  Otherwise (FP64) the point itself, x[D] and q.
-// Slot layout: value k of slot j at buf[32 k + j].
-template <typename T, int D, bool LATE, bool SLAB>
-struct QEntry {
-    Point<T, D> pt;
-    __device__ __forceinline__ T q() const { return pt.q; }
-    __device__ __forceinline__ void put(T *buf, int slot) const
-    {
-#pragma unroll
-        for (int l = 0; l < D; ++l) {
-            if constexpr (sizeof(T) == 4) {
-                buf[l * 32 + slot] = pt.X[l];
-                buf[(D + l) * 32 + slot] = pt.F[l];
-            } else {
-                buf[l * 32 + slot] = pt.x[l];
-            }
-        }
-        buf[(sizeof(T) == 4 ? 2 * D : D) * 32 + slot] = pt.q;
-    }
-    __device__ __forceinline__ void get(const T *buf, int slot)
-    {
-#pragma unroll
-        for (int l = 0; l < D; ++l) {
-            if constexpr (sizeof(T) == 4) {
-                pt.X[l] = buf[l * 32 + slot];
-                pt.F[l] = buf[(D + l) * 32 + slot];
-            } else {
-                pt.x[l] = buf[l * 32 + slot];
-            }
-        }
-        pt.q = buf[(sizeof(T) == 4 ? 2 * D : D) * 32 + slot];
-    }
-    template <bool ANG>
-    __device__ __forceinline__ void make(const SpreadArgs &p, const PairData<T, D> &P, T qbase, int m)
-    {
-        make_point<T, D, ANG>(p, P, qbase, m, pt);
-    }
-    template <int W>
-    __device__ __forceinline__ bool in_slab(const SpreadArgs &p, int row_lo, int nrows)
-    {
-        return rows_hit<T, D, W>(p, pt, row_lo, nrows);
-    }
-    __device__ __forceinline__ void point(const SpreadArgs &, Point<T, D> &out) const { out = pt; }
-};
-template <int D, bool SLAB>
-struct QEntry<float, D, true, SLAB> {
-    float v[D], qv;
-    __device__ __forceinline__ float q() const { return qv; }
-    __device__ __forceinline__ void put(float *buf, int slot) const
-    {
-#pragma unroll
-        for (int l = 0; l < D; ++l) buf[l * 32 + slot] = v[l];
-        buf[D * 32 + slot] = qv;
-    }
-    __device__ __forceinline__ void get(const float *buf, int slot)
-    {
-#pragma unroll
-        for (int l = 0; l < D; ++l) v[l] = buf[l * 32 + slot];
-        qv = buf[D * 32 + slot];
-    }
-    template <bool ANG>
-    __device__ __forceinline__ void make(const SpreadArgs &p, const PairData<float, D> &P, float qbase, int m)
-    {
-        qv = point_velocity_f32<D, ANG>(p, P, qbase, m, v);
-    }
-    // slabs: whether one of the point's rows lies in the slab
-    template <int W>
-    __device__ __forceinline__ bool in_slab(const SpreadArgs &p, int row_lo, int nrows)
-    {
-        float X0, F0, t0;
-        grid_coord_f32(kconst<float>(p), v[0], p.r == 1, X0, F0);
-        return rows_hit_from<W>(p, first_tap_f32<W>(X0, F0, t0), row_lo, nrows);
-    }
-    // the same point make_point forms (same velocity, strength and coordinates)
-    __device__ __forceinline__ void point(const SpreadArgs &p, Point<float, D> &out) const
-    {
-#pragma unroll
-        for (int l = 0; l < D; ++l) grid_coord_f32(kconst<float>(p), v[l], p.r == 1, out.X[l], out.F[l]);
-        out.q = qv;
-    }
-};
+// memory (value k of slot j at buf[32 k + j]) and spreads a full queue with all 32 lanes, one point
+// per lane.
 
 // Spread queue slot `lane` (when valid) with the whole warp.
-template <typename T, int D, int W, typename Tile, bool SLAB, bool LATE>
-__device__ __forceinline__ void queue_spread(const SpreadArgs &p, const T *buf, int lane, bool valid,
-                                             const Tile &tile, int row_lo, int nrows, int plane)
+template <int D, int W>
+__device__ __forceinline__ void queue_spread(const SpreadArgs &p, const double *buf, int lane, bool valid,
+                                             const WideTile &tile, int row_lo, int nrows, int plane)
 {
     if (!valid) return;
-    QEntry<T, D, LATE, SLAB> e;
-    e.get(buf, lane);
-    Point<T, D> pt;
-    e.point(p, pt);
-    spread_point_body<T, D, W, Tile, SLAB>(p, pt, tile, row_lo, nrows, plane);
+    Point<double, D> pt;
+#pragma unroll
+    for (int l = 0; l < D; ++l) pt.x[l] = buf[l * 32 + lane];
+    pt.q = buf[D * 32 + lane];
+    spread_point_f64<D, W, true>(p, pt, tile, row_lo, nrows, plane);
 }
 
-// The pairs pr = first, first + nthr, ... below end of one thread, spread through the warp's
-// queue `buf` (spread_queue_values x 32 values) into one slab (SLAB) or a tile that
-// holds every row.  Points below floor_q (they add exactly zero) are not queued, so that every
-// lane spreads a real point; FP32 points queue their velocity and strength and form their grid
-// coordinates after the queue (QEntry; with slabs, all but axis 0's).  Every loop condition is
-// uniform over the warp.
-template <typename T, int D, int W, typename Tile, bool ANG, bool SLAB = true>
+// The classes pr = first, first + nthr, ... below end of one thread, spread through the warp's
+// queue `buf` (spread_queue_values x 32 values) into one slab.  Points below floor_q are not queued.
+// Every loop condition is uniform over the warp.
+template <int D, int W, bool ANG>
 __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long long first, long long end,
-                                                    long long nthr, T sc, T tau, T floor_q, const Tile &tile,
-                                                    int row_lo, int nrows, int plane, T *buf)
+                                                    long long nthr, double sc, double tau, double floor_q,
+                                                    const WideTile &tile, int row_lo, int nrows, int plane, double *buf)
 {
-    constexpr bool LATE = (sizeof(T) == 4);
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -1160,27 +1059,31 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
     PairCursor c = pair_cursor(p.naxp, first);
     const PairStep st = pair_step(p.naxp, nthr);
     for (;;) {
-        PairData<T, D> P;
-        const bool ok = next_pair<T, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
+        PairData<double, D> P;
+        const bool ok = next_pair<double, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
         if (!__any_sync(full, ok)) break;
-        const T qbase = ok ? P.base * sc : T(0);
+        const double qbase = ok ? P.base * sc : 0.0;
         for (int m = 0; m < p.M; ++m) {
-            QEntry<T, D, LATE, SLAB> e;
+            Point<double, D> pt;
             bool hit = false;
             if (ok) {
-                e.template make<ANG>(p, P, qbase, m);
-                // points below floor_q add exactly zero and are not queued
-                hit = fabs(e.q()) >= floor_q;
-                if constexpr (SLAB) hit = hit && e.template in_slab<W>(p, row_lo, nrows);
+                make_point<double, D, ANG>(p, P, qbase, m, pt);
+                hit = fabs(pt.q) >= floor_q &&
+                      rows_hit_from<W>(p, (int)floor(pt.x[0] - 0.5 * W) + 1, row_lo, nrows);
             }
             const unsigned mask = __ballot_sync(full, hit);
             const int n = __popc(mask), rank = __popc(mask & lt), room = 32 - count;
-            if (hit && rank < room) e.put(buf, count + rank);
+            auto put = [&](int slot) {
+#pragma unroll
+                for (int l = 0; l < D; ++l) buf[l * 32 + slot] = pt.x[l];
+                buf[D * 32 + slot] = pt.q;
+            };
+            if (hit && rank < room) put(count + rank);
             if (n >= room) {  // full: spread 32 points, then queue the rest
                 __syncwarp();
-                queue_spread<T, D, W, Tile, SLAB, LATE>(p, buf, lane, true, tile, row_lo, nrows, plane);
+                queue_spread<D, W>(p, buf, lane, true, tile, row_lo, nrows, plane);
                 __syncwarp();
-                if (hit && rank >= room) e.put(buf, rank - room);
+                if (hit && rank >= room) put(rank - room);
                 count = n - room;
             } else {
                 count += n;
@@ -1189,7 +1092,7 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
         if (ok) pair_advance(p.naxp, c, st);
     }
     __syncwarp();
-    queue_spread<T, D, W, Tile, SLAB, LATE>(p, buf, lane, lane < count, tile, row_lo, nrows, plane);
+    queue_spread<D, W>(p, buf, lane, lane < count, tile, row_lo, nrows, plane);
 }
 
 // ---- 2D FP32 grids in one tile: quads
@@ -1789,29 +1692,34 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
         const float qbase = C.base * sc;
 #pragma unroll 1
         for (int m = 0; m < (drain ? 1 : p.M); ++m) {
-            QEntry<float, 3, true, SLAB> e;
+            float v[3], q = 0.0f;
             int kind = -1;
             if (!drain) {
-                e.template make<ANG>(p, C, qbase, m);
-                const float qa = fabsf(e.q());
+                q = point_velocity_f32<3, ANG>(p, C, qbase, m, v);
+                const float qa = fabsf(q);
                 if (qa >= kNegligibleF32) kind = qa >= kIntLimitF32 ? kLarge : qa < p.cf.trim_q ? kSmall : kInt;
                 if constexpr (SLAB)
-                    if (!(e.v[0] >= range.lo && e.v[0] <= range.hi)) kind = -1;
+                    if (!(v[0] >= range.lo && v[0] <= range.hi)) kind = -1;
             }
 #pragma unroll 1
             for (int k = 0; k < 3; ++k) {
                 const unsigned km = __ballot_sync(full, kind == k);
                 const int cnt = (fill >> (8 * k)) & 255;
                 if (!km && !(drain && cnt)) continue;
-                float *q = buf + k * PV;
+                float *const pq = buf + k * PV;
+                auto put = [&](int slot) {
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) pq[l * 32 + slot] = v[l];
+                    pq[96 + slot] = q;
+                };
                 const int kn = __popc(km), kr = __popc(km & lt), kroom = 32 - cnt;
-                if (kind == k && kr < kroom) e.put(q, cnt + kr);
+                if (kind == k && kr < kroom) put(cnt + kr);
                 int now = cnt + kn;
                 if (kn >= kroom || drain) {
                     __syncwarp();
-                    queue3_spread<W, SLAB>(p, q, k, !drain || lane < cnt, tile, row_lo, nrows, plane);
+                    queue3_spread<W, SLAB>(p, pq, k, !drain || lane < cnt, tile, row_lo, nrows, plane);
                     __syncwarp();
-                    if (kind == k && kr >= kroom) e.put(q, kr - kroom);
+                    if (kind == k && kr >= kroom) put(kr - kroom);
                     now = max(kn - kroom, 0);
                 }
                 fill += (now - cnt) << (8 * k);
@@ -2159,8 +2067,8 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
     if (p.nslab > 1) {
         double *buf = reinterpret_cast<double *>(smem_raw + tile_bytes(tile_cells, false)) +
                       (threadIdx.x >> 5) * 32 * spread_queue_values(D, false);
-        spread_pairs_queued<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
-                                                          G.nrows, G.plane, buf);
+        spread_pairs_queued<D, W, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo, G.nrows, G.plane,
+                                       buf);
     } else if (D == 2 && p.queued) {
         if constexpr (D == 2) {
             unsigned *ids = reinterpret_cast<unsigned *>(smem_raw + tile_bytes(tile_cells, false)) +
