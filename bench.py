@@ -48,7 +48,7 @@ HEADLINE = "2d-hard-spheres"
 # DRAM bytes (read + write) of one launch of the FP32 spreading kernel on the headline workload,
 # from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum), valid only while the code
 # of the kernel's sources (comments aside) hashes to source_sha16 (reported as null otherwise).
-PROFILED_TRAFFIC = {"kernel": "k_spread_f32<2,6,0>", "bytes": 292608, "source_sha16": "1662833d363ae60e"}
+PROFILED_TRAFFIC = {"kernel": "k_spread_f32<2,6,0,0>", "bytes": 275200, "source_sha16": "2268a65a636c92a9"}
 KERNEL_SOURCES = ("spread_impl.cuh", "spread_f32_2d.cu", "pgb_internal.cuh")
 
 
@@ -374,7 +374,7 @@ def measure_config(name, args, dev, stream, timer, peaks, world):
         row["norm_Q_over_norm_gain"] = float(np.linalg.norm(q64)) / mom64["norm_gain"]
         row["speedup_fp32_vs_fp64"] = mean64 / mean32
     else:
-        row["fp64"] = {"skipped": "not timed by default: one FP64 evaluation takes about 77 s here "
+        row["fp64"] = {"skipped": "not timed by default: one FP64 evaluation takes about 9.2 s here "
                                   "(--fp64-steps 1 times it)" if (d == 3 and N > 16 and args.fp64_steps < 0)
                        else "--no-fp64-3d or --fp64-steps 0"}
         row["norm_Q_over_norm_gain"] = float(np.linalg.norm(q32)) / mom32["norm_gain"]
