@@ -133,7 +133,10 @@ __device__ __forceinline__ const TypedConsts<T> &kconst(const SpreadArgs &a)
 // every block of its predecessor has called launch_dependents() (or ended), so that its launch and
 // set-up overlap the predecessor's run; grid_wait() then waits until the predecessor has completed and
 // its writes are visible.  Every such kernel calls grid_wait() before it touches what an earlier
-// kernel writes or reads; the first kernel of an evaluation is launched in the ordinary way.  Without
+// kernel writes or reads; the first kernel of an evaluation is launched in the ordinary way.  In these
+// kernels only the plan's constants may be const __restrict__: what an earlier kernel of the evaluation
+// writes changes while they run, so the compiler must neither read it through the non-coherent path nor
+// move its loads across grid_wait(), which orders only memory that other pointers may reach.  Without
 // the launch attribute both calls do nothing.  2D Maxwell N = 16: 56.4 -> 49.5 us.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -82,7 +82,7 @@ __global__ void k_axis_pass(const __grid_constant__ AxisPass P)
 // fixed-point grid: out = (A . in) 2^-Eg scale) and one of the loss's, side by side in one launch: the
 // two are independent, and each is a few microseconds that mostly wait on a launch and a serial chain.
 __global__ void k_axis_pass_pair(const __grid_constant__ AxisPass P0, const __grid_constant__ AxisPass P1, int nblk0,
-                                 const double *__restrict__ Bp, double scale)
+                                 const double *Bp, double scale)
 {
     launch_dependents();
     grid_wait();
@@ -95,9 +95,9 @@ __global__ void k_axis_pass_pair(const __grid_constant__ AxisPass P0, const __gr
 // Last reconstruction pass (axis 2) and a_i = W_i mu_i^2 P_i; also clears the `nclear` words at
 // `clear` (the spread grid and its scalars, which nothing reads before the loss kernel), so that no
 // separate memset is launched.
-__global__ void k_recon_last(const double *__restrict__ in, Dims3 id, const double *__restrict__ A,
-                             int m, const double *__restrict__ scale, int d, double *__restrict__ a,
-                             float *__restrict__ af, unsigned long long *__restrict__ clear, long long nclear)
+__global__ void k_recon_last(const double *in, Dims3 id, const double *__restrict__ A, int m,
+                             const double *__restrict__ scale, int d, double *a, float *af,
+                             unsigned long long *clear, long long nclear)
 {
     launch_dependents();
     grid_wait();
@@ -591,9 +591,8 @@ __global__ void __launch_bounds__(kReduceThreads) k_bound_reduce(const double *_
     }
 }
 
-__global__ void k_final(const double *__restrict__ G, Dims3 gd, const double *__restrict__ D,
-                        const double *__restrict__ H, Dims3 hd, const double *__restrict__ E, int m,
-                        double *__restrict__ Q, double *__restrict__ Qplus, double *__restrict__ Qcopy)
+__global__ void k_final(const double *G, Dims3 gd, const double *__restrict__ D, const double *H, Dims3 hd,
+                        const double *__restrict__ E, int m, double *Q, double *Qplus, double *Qcopy)
 {
     grid_wait();
     const long long total = (long long)gd.e[0] * gd.e[1] * m;
