@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
     __shared__ CellDesc s_cd;
     constexpr bool F32 = (sizeof(T) == 4);
     int cur = -1, ncell = 0, plane = 0, Eg = 0, shift = 0;
-    T sc = T(0), tau = T(0), floor_q = T(0);
+    T sc = T(0), pre = T(1), tau = T(0), floor_q = T(0);
     // the current cell's spreading arguments live in shared memory: kept in registers they cost
     // 30-odd registers per thread (fewer resident warps, or spills under a 1024-thread bound)
     __shared__ SpreadArgs s_sa;
@@ -408,10 +408,12 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
             ncell = plane * s_cd.nf;
             const double Bc = b.Bcell[cell];
             Eg = global_exponent(Bc);
-            const int Et = F32 ? min(Eg - tile_bits(D), 120) : Eg;
+            const int K = F32 ? product_scale(Eg) : 0;
+            const int Et = F32 ? min(Eg - tile_bits(D), 120 + K) : Eg;
             shift = Eg - Et;
-            sc = T(ldexp(1.0, Et));  // strengths in tile units (FP64: grid units, Et = Eg)
-            tau = T(b.Tcell[cell]);
+            pre = T(ldexp(1.0, K));
+            sc = T(ldexp(1.0, Et - K));  // strengths in tile units (FP64: grid units, Et = Eg)
+            tau = T(ldexp(b.Tcell[cell], K));
             // negligible points: FP32 points below 0.1 tile unit add exactly zero; FP64 pairs whose
             // summed bounds stay below 2^-64 B are skipped
             floor_q = F32 ? T(spread_detail::kNegligibleF32)
@@ -440,13 +442,13 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
         if constexpr (F32) {
             float *buf = reinterpret_cast<float *>(smem_raw + b.queue_off) + warp * 32 * spread_queue_values(D, true);
             if constexpr (D == 2)
-                spread_quads<W, false, false, false>(sa, first, pend, nwarp, sc, tau, SplitTile{lo, carry}, 0,
+                spread_quads<W, false, false, false>(sa, first, pend, nwarp, sc, pre, tau, SplitTile{lo, carry}, 0,
                                                      s_cd.nf, plane, buf);
             else
-                spread_points3<W, false, false>(sa, first, pend, nwarp, sc, tau, SplitTile{lo, carry}, 0, s_cd.nf,
+                spread_points3<W, false, false>(sa, first, pend, nwarp, sc, pre, tau, SplitTile{lo, carry}, 0, s_cd.nf,
                                                 plane, buf);
         } else
-            spread_pairs<T, D, W, WideTile, false>(sa, first, pend, nwarp, sc, tau, floor_q, wt, 0,
+            spread_pairs<T, D, W, WideTile, false>(sa, first, pend, nwarp, sc, pre, tau, floor_q, wt, 0,
                                                       s_cd.nf, plane);
         __syncthreads();
     }

@@ -211,6 +211,17 @@ __host__ __device__ inline int global_exponent(double B)
     return 60 - ilogb(B);
 }
 
+// The FP32 kernels form the products a_i a_j of node values, and so the strengths, times 2^K with
+// K = product_scale(Eg), about -log2 B: B bounds their sum, so they and the sums over a class stay away
+// from both ends of FP32's range for every amplitude at which the node values themselves fit it (a power
+// of two: no rounding changes).  K is kept within +-100, so that 2^K a_i does not leave the range in its turn.
+// Without it the class sums overflowed from amplitudes of 1e19 on, and products underflowed below 1e-14.
+__host__ __device__ inline int product_scale(int Eg)
+{
+    const int e = Eg - 60;
+    return e > 100 ? 100 : e < -100 ? -100 : e;
+}
+
 // Screening of negligible node pairs: the loss kernel counts the pair bounds per binary
 // exponent (kScreenBins bins, bin k holds bounds in [2^(k - kScreenOffset), 2^(k+1 - kScreenOffset)),
 // the first and last bins also everything below / above).

@@ -94,6 +94,9 @@ __device__ __forceinline__ int fold_index(int u, int n)
     return (g > (n >> 1)) ? n - g : g;
 }
 
+// 2^e as a float, 0 below the normal range (e <= 127).
+__device__ __forceinline__ float exp2_int(int e) { return __int_as_float(max(e + 127, 0) << 23); }
+
 // Unfolded index u of a point's support -> folded cell: min(|u|, |n - |u||), which is fold(u) for |u| <= 3n/2.
 // A support reaches at most w/2 beyond [0, n/2], so |u| <= n/2 + w/2, and w <= 2n for every plan (n >= 8,
 // w <= 16): no modulo and no branch (a general path here, never taken but for the smallest grids, was
@@ -397,9 +400,10 @@ __device__ __forceinline__ void pair_advance(int naxp, PairCursor &c, const Pair
 // axis pair of a plan: N <= 512), so the truncation is the exact quotient.
 __device__ __forceinline__ int axis_pair_row(int p, float invN) { return __float2int_rz(((float)p + 0.5f) * invN); }
 
-// Load the class at cursor c; false when its strength is zero.  ANG: angular kernels.
+// Load the class at cursor c; false when its strength is zero.  ANG: angular kernels.  FP32: strengths are
+// formed times `pre` (product_scale).
 template <typename T, int D, bool ANG = false>
-__device__ __forceinline__ bool load_pair(const SpreadArgs &p, const PairCursor &c, PairData<T, D> &P)
+__device__ __forceinline__ bool load_pair(const SpreadArgs &p, const PairCursor &c, T pre, PairData<T, D> &P)
 {
     constexpr int NO = 1 << (D - 1);
     const int N = p.N;
@@ -434,7 +438,7 @@ __device__ __forceinline__ bool load_pair(const SpreadArgs &p, const PairCursor 
             I = I * N + (ex ? nj[l] : ni[l]);
             J = J * N + (ex ? ni[l] : nj[l]);
         }
-        x[o] = acoef[I] * acoef[J];
+        x[o] = (sizeof(T) == 4 ? acoef[I] * pre : acoef[I]) * acoef[J];
         sum += x[o];
         sabs += fabs(x[o]);
     }
@@ -958,12 +962,13 @@ __device__ __forceinline__ void spread_point_body(const SpreadArgs &p, const Poi
 // Load the class at cursor c; whether it is not negligible: non-zero strength, not below the
 // screening threshold tau (0: no screening; the sum of its pairs' bounds is compared, so every pair
 // skipped is below tau), and a bound Ut >= floor_q on every point's |q| in tile units.  On success
-// P.base is multiplied by the class' multiplicity.
+// P.base is multiplied by the class' multiplicity.  sc: tile units per strength as load_pair forms it (so
+// tau, too, is in those units).
 template <typename T, int D, bool ANG>
-__device__ __forceinline__ bool class_passes(const SpreadArgs &p, const PairCursor &c, T sc, T tau, T floor_q,
-                                             PairData<T, D> &P)
+__device__ __forceinline__ bool class_passes(const SpreadArgs &p, const PairCursor &c, T sc, T pre, T tau,
+                                             T floor_q, PairData<T, D> &P)
 {
-    if (!load_pair<T, D, ANG>(p, c, P)) return false;
+    if (!load_pair<T, D, ANG>(p, c, pre, P)) return false;
     const T U = pair_bound<T, D>(p, P);
     if (tau > T(0) && P.sabs * U < tau) return false;
     if ((ANG ? P.sabs : fabs(P.base)) * U * P.mult * sc * kconst<T>(p).wmax < floor_q) return false;
@@ -975,10 +980,10 @@ __device__ __forceinline__ bool class_passes(const SpreadArgs &p, const PairCurs
 // negligible (class_passes); false when none is left.
 template <typename T, int D, bool ANG>
 __device__ __forceinline__ bool next_pair(const SpreadArgs &p, PairCursor &c, long long end, const PairStep &st, T sc,
-                                          T tau, T floor_q, PairData<T, D> &P)
+                                          T pre, T tau, T floor_q, PairData<T, D> &P)
 {
     for (; c.pr < end; pair_advance(p.naxp, c, st))
-        if (class_passes<T, D, ANG>(p, c, sc, tau, floor_q, P)) return true;
+        if (class_passes<T, D, ANG>(p, c, sc, pre, tau, floor_q, P)) return true;
     return false;
 }
 
@@ -1003,13 +1008,14 @@ __device__ __forceinline__ void zero_pair(PairData<T, D> &P)
 // every row.  Every lane of the warp runs every point step (the loop conditions are uniform).
 template <typename T, int D, int W, typename Tile, bool ANG>
 __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long first, long long end, long long stride,
-                                             T sc, T tau, T floor_q, const Tile &tile, int row_lo, int nrows, int plane)
+                                             T sc, T pre, T tau, T floor_q, const Tile &tile, int row_lo, int nrows,
+                                             int plane)
 {
     PairCursor c = pair_cursor(p.naxp, first);
     const PairStep st = pair_step(p.naxp, stride);
     for (;;) {
         PairData<T, D> P;
-        const bool ok = next_pair<T, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
+        const bool ok = next_pair<T, D, ANG>(p, c, end, st, sc, pre, tau, floor_q, P);
         if (!__any_sync(0xffffffffu, ok)) break;
         if (!ok) zero_pair<T, D>(P);
         const T qbase = P.base * sc;
@@ -1060,7 +1066,7 @@ __device__ __forceinline__ void spread_pairs_queued(const SpreadArgs &p, long lo
     const PairStep st = pair_step(p.naxp, nthr);
     for (;;) {
         PairData<double, D> P;
-        const bool ok = next_pair<double, D, ANG>(p, c, end, st, sc, tau, floor_q, P);
+        const bool ok = next_pair<double, D, ANG>(p, c, end, st, sc, 1.0, tau, floor_q, P);
         if (!__any_sync(full, ok)) break;
         const double qbase = ok ? P.base * sc : 0.0;
         for (int m = 0; m < p.M; ++m) {
@@ -1459,8 +1465,8 @@ __device__ __forceinline__ void spread_class_halves(const SpreadArgs &p, const P
 // buf: the warp's queues, 32 slots of spread_queue_values(2, true, ANG) floats.
 template <int W, bool ANG, bool SLAB, bool SPLIT>
 __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long first, long long end, long long stride,
-                                             float sc, float tau, const SplitTile &tile, int row_lo, int nrows,
-                                             int plane, float *buf)
+                                             float sc, float pre, float tau, const SplitTile &tile, int row_lo,
+                                             int nrows, int plane, float *buf)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -1482,7 +1488,7 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
                 share = c.t / p.naxp;
                 cc.t = c.t - share * p.naxp;
             }
-            hit = class_passes<float, 2, ANG>(p, cc, sc, tau, kNegligibleF32, P);
+            hit = class_passes<float, 2, ANG>(p, cc, sc, pre, tau, kNegligibleF32, P);
             pair_advance(p.naxp, c, st);
         }
         auto put = [&](int slot) {
@@ -1626,8 +1632,8 @@ __device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *
 
 template <int W, bool ANG, bool SLAB>
 __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long first, long long end, long long stride,
-                                               float sc, float tau, const SplitTile &tile, int row_lo, int nrows,
-                                               int plane, float *buf)
+                                               float sc, float pre, float tau, const SplitTile &tile, int row_lo,
+                                               int nrows, int plane, float *buf)
 {
     constexpr int PV = 32 * 4;  // values of a point queue: velocity and strength
     const unsigned full = 0xffffffffu;
@@ -1649,7 +1655,7 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
             PairData<float, 3> P;
             bool hit = false;
             if (c.pr < end) {
-                hit = class_passes<float, 3, ANG>(p, c, sc, tau, kNegligibleF32, P);
+                hit = class_passes<float, 3, ANG>(p, c, sc, pre, tau, kNegligibleF32, P);
                 pair_advance(p.naxp, c, st);
             }
             auto put = [&](int slot) {
@@ -1998,32 +2004,33 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     const double Bnd = strength_bound(p);
     __syncthreads();
     const int Eg = global_exponent(Bnd);
-    // Tile unit 2^-Et with Et = Eg - tile_bits(D) (2^-47 B or finer in 2D, 2^-53 B in 3D); kept
-    // inside the float range for tiny inputs (a coarser unit there).
-    const int Et = min(Eg - tile_bits(D), 120);
+    // Tile unit 2^-Et with Et = Eg - tile_bits(D) (2^-47 B or finer in 2D, 2^-53 B in 3D); a coarser
+    // unit for inputs so small that sc would leave the float range.
+    const int K = product_scale(Eg);
+    const int Et = min(Eg - tile_bits(D), 120 + K);
     const int shift = Eg - Et;
     const SplitTile tile{words, carry};
-    const float sc = (float)ldexp(1.0, Et);
-    const float tau = p.nub ? 0.0f : (float)*p.tau;
+    const float pre = exp2_int(K), sc = exp2_int(Et - K);
+    const float tau = p.nub ? 0.0f : (float)ldexp(*p.tau, K);
     long long first, nthr;
     pair_schedule(p, first, nthr);
     if (p.nslab > 1) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes((size_t)p.rows_per_slab * G.plane, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
         if constexpr (D == 2)
-            spread_quads<W, ANG, true, false>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
+            spread_quads<W, ANG, true, false>(p, first, p.nclass, nthr, sc, pre, tau, tile, G.row_lo, G.nrows, G.plane, buf);
         else
-            spread_points3<W, ANG, true>(p, first, p.nclass, nthr, sc, tau, tile, G.row_lo, G.nrows, G.plane, buf);
+            spread_points3<W, ANG, true>(p, first, p.nclass, nthr, sc, pre, tau, tile, G.row_lo, G.nrows, G.plane, buf);
     } else if (p.queued) {
         float *buf = reinterpret_cast<float *>(smem_raw + tile_bytes(G.ncell, true)) +
                      (threadIdx.x >> 5) * 32 * spread_queue_values(D, true, ANG);
         if constexpr (D == 2)
-            spread_quads<W, ANG, false, SPLIT>(p, first, SPLIT ? p.nclass * p.nsplit : p.nclass, nthr, sc, tau, tile, 0,
+            spread_quads<W, ANG, false, SPLIT>(p, first, SPLIT ? p.nclass * p.nsplit : p.nclass, nthr, sc, pre, tau, tile, 0,
                                                G.nrows, G.plane, buf);
         else
-            spread_points3<W, ANG, false>(p, first, p.nclass, nthr, sc, tau, tile, 0, G.nrows, G.plane, buf);
+            spread_points3<W, ANG, false>(p, first, p.nclass, nthr, sc, pre, tau, tile, 0, G.nrows, G.plane, buf);
     } else {
-        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, tau, kNegligibleF32, tile, G.row_lo,
+        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, pre, tau, kNegligibleF32, tile, G.row_lo,
                                                    G.nrows, G.plane);
     }
     __syncthreads();
@@ -2076,7 +2083,7 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
             spread_orbits<W, ANG>(p, first, p.nitem, nthr, sc, tau, floor_q, tile, G.plane, ids);
         }
     } else {
-        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, tau, floor_q, tile, G.row_lo,
+        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, 1.0, tau, floor_q, tile, G.row_lo,
                                                    G.nrows, G.plane);
     }
     __syncthreads();

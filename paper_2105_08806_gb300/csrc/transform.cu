@@ -7,6 +7,7 @@
 //  - the final pass that forms Q = Q+ - Q- (Section 4.2),
 //  - mass / energy diagnostics from the identities of Section 3.3.
 // All arrays are C-order three-axis arrays (2D arrays carry a leading axis of 1).
+#include <cfloat>
 #include <cuda_runtime.h>
 
 #include "pgb_internal.cuh"
@@ -357,6 +358,97 @@ __device__ __forceinline__ PT vhs_factor(PT g2, PT g, int fast_gamma, PT gam)
     }
 }
 
+// This thread's share of block blk's part of the strength bound (over Bw angmax): the sums of |a_i a_j| over a
+// class and its mirror images in AT, times the class' factor in PT.  In FP32 a class' sum (at most 32 terms of
+// rounded values), its factor and a partial sum of 64 classes are each rounded by at most 2e-6, 1e-6 and 4e-6: the
+// margin of 1e-5 that the spreading kernel adds covers them together.  (The nodes' own rounding moves |v_i - v_j| of
+// neighbours by more, but the box |c| + rad exceeds their points by far more than that; and the int64 grid holds
+// four times the B 2^Eg < 2^61 that it is scaled for.)
+template <typename PT, typename AT, int D>
+__device__ __forceinline__ double mirror_bound(const LossArgs &L, const PT *vn, const PT *av, int blk)
+{
+    constexpr int E = 1 << D;
+    const int N = L.N;
+    const PT gam = PT(L.gamma), S = PT(L.S), invS = PT(1) / S;
+    double acc = 0.0;
+    AT p = AT(0);
+    int np = 0;
+    const long long first = blk * (long long)blockDim.x + threadIdx.x, step = (long long)L.nbound * blockDim.x;
+    int ol[D], os[D];  // the orbit's axis orbits and the step's, digits in base norb (no division per orbit)
+    {
+        long long t = first, u = step;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            ol[l] = (int)(t % L.norb);
+            t /= L.norb;
+            os[l] = (int)(u % L.norb);
+            u /= L.norb;
+        }
+    }
+    for (long long o = first; o < L.norbits; o += step) {
+        int ni[D], nj[D];
+        PT g2 = PT(0), cen[D], mult = PT(2);
+        bool self[D];
+        int carry = 0;
+#pragma unroll
+        for (int l = D - 1; l >= 0; --l) {
+            const unsigned w = L.orb[ol[l]];
+            ol[l] += os[l] + carry;
+            carry = ol[l] >= L.norb;
+            if (carry) ol[l] -= L.norb;
+            ni[l] = w & 0xffffu;
+            nj[l] = w >> 16;
+            self[l] = ni[l] + nj[l] == N - 1;
+            if (ni[l] == nj[l]) mult *= PT(0.5);
+            const PT vi = vn[ni[l]], vj = vn[nj[l]];
+            g2 += (vi - vj) * (vi - vj);
+            cen[l] = PT(0.5) * (vi + vj);
+        }
+        const PT g = sqrt(g2);
+        PT u = mult * vhs_factor(g2, g, L.fast_gamma, gam);
+#pragma unroll
+        for (int l = 0; l < D; ++l) {
+            const PT R = fabs(cen[l]) + PT(0.5) * g;
+            u *= (L.r == 1) ? (S * S + R * R) * invS : S * cosh(R * invS);
+        }
+        AT sum = AT(0);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            bool skip = false;
+#pragma unroll
+            for (int l = 0; l < D; ++l) skip = skip || (((e >> l) & 1) && self[l]);
+            if (skip) continue;  // its own mirror image
+#pragma unroll
+            for (int x = 0; x < E / 2; ++x) {  // the ways to exchange axes 0 .. D-2
+                int I = 0, J = 0;
+#pragma unroll
+                for (int l = 0; l < D; ++l) {
+                    const int q = ((e >> l) & 1) ? N - 1 - ni[l] : ni[l];
+                    const int w = ((e >> l) & 1) ? N - 1 - nj[l] : nj[l];
+                    const bool ex = (x >> l) & 1;
+                    I = I * N + (ex ? w : q);
+                    J = J * N + (ex ? q : w);
+                }
+                sum += fabs(AT(av[I]) * AT(av[J]));
+            }
+        }
+        p += AT(u) * sum;
+        if (++np == 64) {
+            acc += (double)p;
+            p = AT(0);
+            np = 0;
+        }
+    }
+    return acc + (double)p;
+}
+
+// The same with the sums in FP64, out of line: FP32 plans whose FP32 sums left the range.
+template <int D>
+__device__ __noinline__ double mirror_bound_wide(const LossArgs &L, int blk)
+{
+    return mirror_bound<float, double, D>(L, L.v32, L.a32, blk);
+}
+
 template <typename PT, int D, bool ANG>
 __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_constant__ LossArgs L)
 {
@@ -379,79 +471,15 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
     const PT gam = PT(L.gamma);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if ((int)blockIdx.x >= L.nloss) {  // the strength bound
-        const PT S = PT(L.S), invS = PT(1) / S;
         const int blk = blockIdx.x - L.nloss;
-        double acc = 0.0;
-        PT p = PT(0);
-        int np = 0;
-        const long long first = blk * (long long)blockDim.x + threadIdx.x, step = (long long)L.nbound * blockDim.x;
-        int ol[D], os[D];  // the orbit's axis orbits and the step's, digits in base norb (no division per orbit)
-        {
-            long long t = first, u = step;
-#pragma unroll
-            for (int l = D - 1; l >= 0; --l) {
-                ol[l] = (int)(t % L.norb);
-                t /= L.norb;
-                os[l] = (int)(u % L.norb);
-                u /= L.norb;
-            }
+        double tot = block_sum<kMirrorThreads>(mirror_bound<PT, PT, D>(L, vn, av, blk));
+        if constexpr (F32) {
+            // FP32 sums overflow from amplitudes of about 1e19 on; below 1e-24 what underflowed may
+            // matter (at most 1e7 products per block, each 1e-45 off, times the class' factor).  The
+            // test costs an evaluation about 0.3 us (2D Maxwell N = 16: 49.9 -> 50.2 us).
+            const bool out = threadIdx.x == 0 && !(tot >= 1e-24 && tot <= DBL_MAX);
+            if (__syncthreads_or(out)) tot = block_sum<kMirrorThreads>(mirror_bound_wide<D>(L, blk));
         }
-        for (long long o = first; o < L.norbits; o += step) {
-            int ni[D], nj[D];
-            PT g2 = PT(0), cen[D], mult = PT(2);
-            bool self[D];
-            int carry = 0;
-#pragma unroll
-            for (int l = D - 1; l >= 0; --l) {
-                const unsigned w = L.orb[ol[l]];
-                ol[l] += os[l] + carry;
-                carry = ol[l] >= L.norb;
-                if (carry) ol[l] -= L.norb;
-                ni[l] = w & 0xffffu;
-                nj[l] = w >> 16;
-                self[l] = ni[l] + nj[l] == N - 1;
-                if (ni[l] == nj[l]) mult *= PT(0.5);
-                const PT vi = vn[ni[l]], vj = vn[nj[l]];
-                g2 += (vi - vj) * (vi - vj);
-                cen[l] = PT(0.5) * (vi + vj);
-            }
-            const PT g = sqrt(g2);
-            PT u = mult * vhs_factor(g2, g, L.fast_gamma, gam);
-#pragma unroll
-            for (int l = 0; l < D; ++l) {
-                const PT R = fabs(cen[l]) + PT(0.5) * g;
-                u *= (L.r == 1) ? (S * S + R * R) * invS : S * cosh(R * invS);
-            }
-            PT sum = PT(0);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                bool skip = false;
-#pragma unroll
-                for (int l = 0; l < D; ++l) skip = skip || (((e >> l) & 1) && self[l]);
-                if (skip) continue;  // its own mirror image
-#pragma unroll
-                for (int x = 0; x < E / 2; ++x) {  // the ways to exchange axes 0 .. D-2
-                    int I = 0, J = 0;
-#pragma unroll
-                    for (int l = 0; l < D; ++l) {
-                        const int q = ((e >> l) & 1) ? N - 1 - ni[l] : ni[l];
-                        const int w = ((e >> l) & 1) ? N - 1 - nj[l] : nj[l];
-                        const bool ex = (x >> l) & 1;
-                        I = I * N + (ex ? w : q);
-                        J = J * N + (ex ? q : w);
-                    }
-                    sum += fabs(av[I] * av[J]);
-                }
-            }
-            p += u * sum;
-            if (++np == 64) {
-                acc += (double)p;
-                p = PT(0);
-                np = 0;
-            }
-        }
-        acc += (double)p;
-        const double tot = block_sum<kMirrorThreads>(acc);
         if (threadIdx.x == 0) L.ub[blk] = tot * L.Bw * L.angmax;
         return;
     }
