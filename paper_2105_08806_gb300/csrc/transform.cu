@@ -320,7 +320,8 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const double *__restrict_
 // per ordered pair (2^(2d) of them share B and the map factors): blocks nloss .. nloss+nbound-1.
 // With an angular factor (2D: the circle is symmetric in both axes) the mean of b over the sphere set
 // is the same for all of them, too, and only its even part survives the antipodal pairs.
-// The FP32 sums are those of k_loss: the product's FMA residual and a two-sum per term.
+// The sums are those of k_loss: FP32 plans add the FP32 coefficients' products as float pairs (the product's
+// FMA residual and a two-sum per term), angular ones FP32 pair terms times the FP64 coefficients in FP64.
 // Measured, loss stage (with the bound's reduction before, which the spreading kernel now does):
 // 2D hard spheres N = 64 FP32 143 -> 43 us, FP64 1323 -> 252 us; N = 120 1294 -> 429 us; 3D VHS N = 24
 // 1212 -> 301 us; 2D angular N = 41, M = 22 408 -> 35 us.
@@ -542,8 +543,8 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
         if constexpr (ANG) B *= circle_mean<PT>(L, sig, dv[0], dv[1], g);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const PT aj = av[idx[e]];
-            if constexpr (F32) {
+            if constexpr (F32 && !ANG) {
+                const float aj = av[idx[e]];
                 const float pt = B * aj;
                 const float pe = fmaf(B, aj, -pt);
                 const float t = as[e] + pt;
@@ -551,7 +552,7 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
                 ac[e] += ((as[e] - (t - bv)) + (pt - bv)) + pe;
                 as[e] = t;
             } else {
-                acc[e] = fma(B, aj, acc[e]);
+                acc[e] = fma((double)B, L.a[idx[e]], acc[e]);
             }
         }
         int carry = 0;
