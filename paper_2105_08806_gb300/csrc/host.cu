@@ -222,10 +222,15 @@ NodeTables node_tables(int N, double S, int r)
     const double wnode = kPi / (N + 1);
     for (int i = 0; i < N; ++i) {
         const double phi = kPi * (i + 1) / (N + 1);
-        const double mu2 = ipow(std::sin(phi), 1 + r) / S;
+        // The nodes of the upper half are the exact mirror images of those of the lower half, which the
+        // kernels' classes of mirrored node pairs rely on.  Evaluated at phi > pi/2 they would not be: the
+        // rounding of phi moves sin(phi) by up to 1e-14 of itself near pi.
+        const int low = std::min(i, N - 1 - i);
+        const double phl = kPi * (low + 1) / (N + 1);
+        const double mu2 = ipow(std::sin(phl), 1 + r) / S;
         t.scale_a[i] = wnode * mu2;
         t.inv_mu2[i] = 1.0 / mu2;
-        t.v[i] = map_v(phi, S, r);
+        t.v[i] = (2 * i == N - 1) ? 0.0 : (i == low) ? map_v(phl, S, r) : -map_v(phl, S, r);
         for (int k = 0; k <= N; ++k) {
             const double tk = std::cos(k * (kPi - phi)) / std::sqrt(k == 0 ? kPi : 0.5 * kPi);
             t.R[(size_t)i * (N + 1) + k] = tk;
