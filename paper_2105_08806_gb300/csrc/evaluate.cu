@@ -8,12 +8,17 @@
 // One thread per point.  The sum over the last axis is cut into chunks of at most 32 coefficients
 // whose T_k(x_l) a thread keeps in registers; for every row of coefficients (the leading axes' modes) a
 // chunk is one FMA per coefficient -- every thread of a warp reads the same coefficient, a broadcast
-// load -- and the row's product of leading T_k comes from a running recurrence.
+// load -- and the rows go through a Clenshaw recurrence per leading axis.  Both run from the highest mode
+// down, so that the small terms are added first: the error on smooth densities is that of a Clenshaw
+// recurrence on every axis (2.8e-16 of the values at N = 48, logarithmic map, where sums from the lowest mode up
+// left 4.4e-16).
 //
-// The FP64 pipe bounds it (two operations per SM and cycle on this GPU): a nested Clenshaw recurrence
-// takes two operations per coefficient, this form one and a few per row.  Blocks of one warp, so that
-// the points spread evenly over the SMs.  200 x 200 points at N = 48, 2D: 705 -> 248 us (one FMA per
-// coefficient at the measured 5.3e11/s: 182 us).
+// The FP64 pipe bounds it (two operations per SM and cycle on this GPU): Clenshaw recurrences
+// on every axis take two operations per coefficient, this form one and two per row.  Blocks of one warp, so that
+// the points spread evenly over the SMs, and registers for 12 of them per SM, so that a row's loads are all in
+// flight at once (with the compiler's own choice few points were slower: N = 120, one point 0.68 ms instead of
+// 0.61).  200 x 200 points at N = 48, 2D: 705 us with recurrences on every axis, 237 us so (one FMA per coefficient at the
+// measured 5.3e11/s: 182 us).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -51,11 +56,27 @@ __device__ void map_point(double v, double S, int r, double &xi, double &mu4)
     }
 }
 
+// sum_k a_k T_k(x) / sqrt(c_k), k = 0..N, of coefficients that next() gives from a_N down to a_0:
+// sum_{k>=1} a_k T_k(x) = x b_1 - b_2 with b_k = a_k + 2 x b_{k+1} - b_{k+2}.
+template <typename F>
+__device__ __forceinline__ double clenshaw(int N, double x, F next)
+{
+    const double two_x = 2.0 * x;
+    double b1 = 0.0, b2 = 0.0;
+    for (int k = N; k > 0; --k) {
+        const double t = fma(two_x, b1, next() - b2);
+        b2 = b1;
+        b1 = t;
+    }
+    const double a0 = next();
+    return kSqrt2OverPi * fma(x, b1, -b2) + kInvSqrtPi * a0;
+}
+
 constexpr int kEvalThreads = 32;
 
 // C: coefficients of the last axis per chunk.
 template <int D, int C>
-__global__ void __launch_bounds__(kEvalThreads) k_evaluate(int N, double S, int r, const double *__restrict__ u,
+__global__ void __launch_bounds__(kEvalThreads, 12) k_evaluate(int N, double S, int r, const double *__restrict__ u,
                                                            long long npts, const double *__restrict__ pts,
                                                            double *__restrict__ out)
 {
@@ -70,63 +91,47 @@ __global__ void __launch_bounds__(kEvalThreads) k_evaluate(int N, double S, int 
         }
         double total = 0.0;
         double ta = kInvSqrtPi, tb = kSqrt2OverPi * x[D - 1];  // the last axis' T_k/sqrt(c_k) and T_{k+1}/sqrt(c_{k+1})
-        for (int c0 = 0; c0 <= N; c0 += C) {
+        for (int done = 0; done <= N; done += C) {
+            // the last chunk ends with the row: coefficients that were added before are multiplied by 0
+            const int c0 = min(done, N + 1 - C);
             double T[C];
 #pragma unroll
             for (int k = 0; k < C; ++k) {
-                T[k] = (c0 + k <= N) ? ta : 0.0;
+                T[k] = 0.0;
+                if (c0 + k < done) continue;
+                T[k] = ta;
                 // T_{k+2} = 2 x T_{k+1} - T_k, with T_0 in the scale of the others
                 const double prev = (c0 + k == 0) ? kSqrt2OverPi : ta;
                 ta = tb;
                 tb = fma(2.0 * x[D - 1], tb, -prev);
             }
-            const int last = N - c0;  // coefficients past it are multiplied by 0 (the row's last is read)
             auto row = [&](const double *q) {
                 double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-                for (int k = 0; k < C; ++k) {
-                    const double c = __ldg(q + min(k, last));
+                for (int k = C - 1; k >= 0; --k) {
+                    const double c = __ldg(q + k);
                     if (k & 1) s1 = fma(c, T[k], s1);
                     else s0 = fma(c, T[k], s0);
                 }
                 return s0 + s1;
             };
-            const double *q = u + c0;
-            double acc = 0.0, a0 = kInvSqrtPi, b0 = kSqrt2OverPi * x[0];
-            for (int k0 = 0; k0 <= N; ++k0) {
-                double in;
-                if constexpr (D == 2) {
-                    in = row(q);
-                    q += N + 1;
-                } else {
-                    in = 0.0;
-                    double a1 = kInvSqrtPi, b1 = kSqrt2OverPi * x[1];
-                    for (int k1 = 0; k1 <= N; ++k1) {
-                        in = fma(a1, row(q), in);
-                        q += N + 1;
-                        const double prev = k1 == 0 ? kSqrt2OverPi : a1;
-                        a1 = b1;
-                        b1 = fma(2.0 * x[1], b1, -prev);
-                    }
-                }
-                acc = fma(a0, in, acc);
-                const double prev = k0 == 0 ? kSqrt2OverPi : a0;
-                a0 = b0;
-                b0 = fma(2.0 * x[0], b0, -prev);
-            }
-            total += acc;
+            // rows of the leading axes' modes, from the last one down
+            const double *q = u + c0 + (D == 3 ? (size_t)(N + 1) * (N + 1) * (N + 1) : (size_t)(N + 1) * (N + 1));
+            auto next_row = [&]() { return row(q -= N + 1); };
+            if constexpr (D == 2) total += clenshaw(N, x[0], next_row);
+            else total += clenshaw(N, x[0], [&]() { return clenshaw(N, x[1], next_row); });
         }
         out[p] = w * total;
     }
 }
 
-// Dispatch on the chunk size (even, 4 .. 32).
+// Dispatch on the chunk size, 3 .. 32.
 template <int D, int C>
 void launch_evaluate(int c, int blocks, cudaStream_t s, int N, double S, int r, const double *u, long long npts,
                      const double *pts, double *out)
 {
     if (c == C) k_evaluate<D, C><<<blocks, kEvalThreads, 0, s>>>(N, S, r, u, npts, pts, out);
-    else if constexpr (C < 32) launch_evaluate<D, C + 2>(c, blocks, s, N, S, r, u, npts, pts, out);
+    else if constexpr (C < 32) launch_evaluate<D, C + 1>(c, blocks, s, N, S, r, u, npts, pts, out);
 }
 
 }  // namespace
@@ -141,12 +146,12 @@ PG_API int pg_boltz_evaluate(pg_boltz_plan_t *p, const double *coef_dev, long lo
     if (!coef_dev || !pts_dev || !out_dev) return set_error(PG_ERR_ARG, "NULL device pointer");
     DeviceGuard guard(p->device);
     if (!guard.ok) return set_error(PG_ERR_CUDA, "cannot select the plan's device");
-    // as few chunks of the last axis as 32 registers' worth allows, of even size (a little padding)
-    const int chunks = (p->N + 32) / 32, C = std::max(4, ((p->N + chunks) / chunks + 1) / 2 * 2);
+    // as few chunks of the last axis as 32 values in registers allow
+    const int chunks = (p->N + 32) / 32, C = (p->N + chunks) / chunks;
     const int blocks = (int)std::min<long long>((npts + kEvalThreads - 1) / kEvalThreads, 1 << 20);
     if (p->d == 2)
-        launch_evaluate<2, 4>(C, blocks, p->stream, p->N, p->S, p->r, coef_dev, npts, pts_dev, out_dev);
+        launch_evaluate<2, 3>(C, blocks, p->stream, p->N, p->S, p->r, coef_dev, npts, pts_dev, out_dev);
     else
-        launch_evaluate<3, 4>(C, blocks, p->stream, p->N, p->S, p->r, coef_dev, npts, pts_dev, out_dev);
+        launch_evaluate<3, 3>(C, blocks, p->stream, p->N, p->S, p->r, coef_dev, npts, pts_dev, out_dev);
     return cuda_check(cudaGetLastError(), "evaluation kernel");
 }
