@@ -270,6 +270,132 @@ pgb::Dims3 dims_of(int d, int a, int b, int c)
     return x;
 }
 
+int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
+{
+    const int d = in.d, N = in.N, nf = in.nf;
+    const bool f32 = in.f32;
+    const size_t elem = f32 ? 4 : 12;  // 32-bit words per cell: FP32 one, FP64 three
+    // block tiles: rows of (nf^(d-2) x tile_cols) cells, the last axis padded with unfolded columns (FP64 3D: not)
+    const size_t plane = (size_t)ipow(nf, d - 2) * pgb::tile_cols(nf, in.w, d, f32);
+    // leave room for the kernels' static shared memory (FP64: the kernel polynomial)
+    // (and 16 bytes for rounding the tile up to 16 bytes)
+    const size_t max_smem = in.smem_block - 1024 - 16 - (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
+    const int max_threads = f32 ? pgb::kMaxThreadsF32 : pgb::kMaxThreadsF64;
+    const int accept_threads = pgb::accept_threads(d, f32);
+    if (in.ask_threads > accept_threads || (in.ask_threads > 0 && in.ask_threads % 32))
+        return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
+    int ask_threads = std::min(in.ask_threads, max_threads);  // <= 0: chosen here
+    const long long nclass = (long long)ipow((double)pgb::unordered_pairs(N), d);
+    auto queue_bytes = [&](int threads) { return pgb::spread_queue_bytes(threads, d, f32, in.ang); };
+    // threads whose queues fit beside a tile
+    auto room = [&](size_t tile) { return tile < max_smem ? 32 * (int)((max_smem - tile) / queue_bytes(32)) : 0; };
+    // small one-slab plans: blocks no larger than it takes for every SM to have one (each thread then owns
+    // one item; 2D Maxwell N = 16: spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks
+    // of 1024 with a point set per pair)
+    auto small_block = [&](long long items) {
+        const long long per_block = (items + in.sms - 1) / in.sms;
+        return (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
+    };
+    // FP32 2D: with fewer classes than threads, the classes' quads are cut into shares, so that there is
+    // an item per thread (2D N = 16, M = 8: 18,496 classes of 3 quads, spreading 41 -> 31 us).  With
+    // more classes (N = 32: 2.9 per thread) the repeated class tests cost what the fuller rounds gain.
+    int nsplit = 1;
+    if (f32 && d == 2)
+        nsplit = (int)std::max<long long>(1, std::min<long long>(in.M / 4 + 1, (long long)in.sms * max_threads / nclass));
+
+    int rows_fit = (int)std::min<size_t>(nf, max_smem / (plane * elem));
+    const size_t whole = pgb::tile_bytes((size_t)nf * plane, f32);
+    if (rows_fit == nf && f32 && ask_threads <= 0) {
+        // A grid that nearly fills one block leaves room for the queues of a few warps only; two slabs, which
+        // generate every point twice, are then faster.  One slab (its threads) against two, ms:
+        //   2D w = 6, M = 8:   N = 114 (320) 3.28 / 3.54   N = 115 (256) 3.60 / 3.47   N = 116 (160) 5.22 / 3.52
+        //   2D w = 6, M = 32:  N = 114 (320) 8.78 / 9.28   N = 115 (256) 9.29 / 8.96
+        //   2D w = 8, M = 8:   N = 113 (384) 3.90 / 4.75   N = 114 (288) 4.73 / 4.51
+        //   2D angular, M = 8: N = 112 (352) 3.45 / 3.91   N = 113 (288) 4.22 / 4.17
+        //   3D w = 6:          N = 16 angular (512) 6.91 / 8.03   N = 17 (256) 3.04 / 2.36
+        //   3D w = 8, sigma = 1.5: N = 22 (352) 11.1 / 11.0
+        // (One slab spread point by point without queues, 640 threads: 3.15 at N = 115 and 3.79 at N = 117 where two
+        // slabs take 3.47 and 3.78 ms, but 10.4 against 9.9 at M = 32, 9.98 against 8.84 angular and 4.6 against 2.4 in 3D.)
+        if (room(whole) < std::min(small_block(nclass * nsplit), d == 3 ? 384 : 320)) rows_fit = nf - 1;
+    }
+    size_t qbytes = 0;
+    if (rows_fit < nf) {
+        // slabbed grid: the warps' queues (one block per SM) share the block's shared memory with the slab.
+        // FP32: at least 384 threads, and as many as the fewest slabs that leave room for those allow
+        // (a point is generated once per slab and its rows straddle two now and then)
+        auto fit = [&](int thr) {
+            qbytes = queue_bytes(thr);
+            return (max_smem > qbytes) ? (int)std::min<size_t>(nf, (max_smem - qbytes) / (plane * elem)) : 0;
+        };
+        rows_fit = fit((ask_threads > 0) ? ask_threads : f32 ? 384 : max_threads);
+        if (rows_fit < 1 && f32) {  // a plane that leaves little room
+            ask_threads = (ask_threads > 0) ? std::min(ask_threads, 128) : 128;
+            rows_fit = fit(ask_threads);
+        }
+    }
+    if (rows_fit < 1) return set_error(PG_ERR_ARG, "folded grid plane of %zu cells does not fit shared memory", plane);
+    out.nslab = (nf + rows_fit - 1) / rows_fit;
+    out.rows_per_slab = (nf + out.nslab - 1) / out.nslab;
+    out.nslab = (nf + out.rows_per_slab - 1) / out.rows_per_slab;  // no empty trailing slab
+    out.tile_cells = (long long)out.rows_per_slab * (long long)plane;
+    const size_t tile = pgb::tile_bytes((size_t)out.tile_cells, f32);
+    out.smem = tile;
+    out.queued = 0;
+    out.nsplit = 1;
+    out.nitem = 0;
+    long long items = nclass;
+    // FP32: one block per SM (measured fastest; more, smaller blocks multiply the tile clears and flushes)
+    int per_sm = 1;
+    if (out.nslab > 1) {
+        out.threads = ask_threads > 0 ? ask_threads : f32 ? std::min(max_threads, room(tile)) : max_threads;
+        out.smem += queue_bytes(out.threads);
+        if (ask_threads > 0 || !f32)
+            per_sm = (int)(in.smem_sm / (out.smem + 1024 + in.smem_reserved));
+    } else if (f32) {
+        // the warps' queues follow the tile (2D: large quads; 3D: the points that add something)
+        out.threads = ask_threads > 0 ? ask_threads : std::min(small_block(nclass * nsplit), room(whole));
+        if (ask_threads > 0) per_sm = (int)(in.smem_sm / (tile + 1024 + in.smem_reserved));
+        out.queued = room(whole) >= out.threads;  // (block sizes asked for may not fit: point by point, whole classes)
+        if (out.queued) {
+            out.smem += queue_bytes(out.threads);
+            out.nsplit = nsplit;
+            items = nclass * nsplit;
+        }
+    } else {
+        // about 1024 resident threads per SM, small plans fewer
+        per_sm = std::max(1, (int)(in.smem_sm / (tile + 1024 + in.smem_reserved)));
+        out.threads = ask_threads > 0 ? ask_threads
+                                      : std::min(std::max(128, std::min(max_threads, (1024 / per_sm) / 32 * 32)),
+                                                 small_block(nclass));
+        // 2D: quads of mirrored classes, numbered in 32 bits, 4 bytes of queue per thread
+        const long long norb = (long long)axis_orbits(N).size(), nitem = norb * norb * (in.M / 4 + 1);
+        if (d == 2 && nitem < (1ll << 32)) {
+            int threads = ask_threads > 0 ? ask_threads : small_block(nitem);
+            if (ask_threads <= 0)
+                while (threads > 128 && tile + (size_t)threads * 4 > max_smem) threads -= 128;
+            if (tile + (size_t)threads * 4 <= max_smem) {
+                out.queued = 1;
+                out.threads = threads;
+                out.smem += (size_t)threads * 4;
+                out.nitem = items = nitem;
+                if (ask_threads <= 0) per_sm = 1;
+            }
+        }
+    }
+    per_sm = std::min(per_sm, in.sm_threads / out.threads);
+    if (in.ask_per_sm > 0) per_sm = std::min(per_sm, in.ask_per_sm);
+    per_sm = std::max(per_sm, 1);
+    long long blocks = (long long)in.sms * per_sm;
+    blocks = std::max<long long>(blocks / out.nslab, 1) * out.nslab;
+    blocks = std::min(blocks, ((items + out.threads - 1) / out.threads) * out.nslab);
+    out.blocks = (int)blocks;
+    // the pair schedule permutes thread starts by a multiplier prime to every smaller count
+    if ((blocks / out.nslab) * out.threads >= 1000003)
+        return set_error(PG_ERR_ARG, "spreading launch of %lld threads per slab exceeds the pair schedule's range",
+                         (blocks / out.nslab) * out.threads);
+    return PG_OK;
+}
+
 int dev_alloc(pg_boltz_plan_t *p, void **ptr, size_t bytes)
 {
     *ptr = nullptr;

@@ -83,6 +83,23 @@ std::vector<double> transform_matrix(int N, int n, int w, double beta);
 
 pgb::Dims3 dims_of(int d, int a, int b, int c);
 
+// A plan's spreading launch from its sizes, its options and the device's limits alone.
+struct SpreadShapeIn {
+    int d, N, M, nf, w;
+    bool f32, ang;
+    int ask_threads, ask_per_sm;  // pg_boltz_opts_t::spread_threads, spread_blocks_per_sm (<= 0: automatic)
+    size_t smem_block, smem_sm, smem_reserved;  // shared memory: per block (opt-in), per SM, reserved per block
+    int sms, sm_threads;
+};
+struct SpreadShape {
+    int nslab, rows_per_slab;  // slabs of the folded grid along axis 0
+    int threads, blocks;
+    size_t smem;               // dynamic shared memory of a block
+    int queued, nsplit;        // SpreadArgs
+    long long nitem, tile_cells;
+};
+int spread_shape(const SpreadShapeIn &in, SpreadShape &out);
+
 }  // namespace pgbh
 
 struct BatchState;

@@ -114,7 +114,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         (rc = dev_alloc(p, (void **)&p->rk, 5 * modes * 8)) ||
         (rc = dev_alloc(p, (void **)&p->mom, 16 * 8)))
         return rc;
-    // one allocation: [grid | B | tau | screening histogram], cleared by one memset per call
+    // one allocation: [grid | B | tau | screening histogram], cleared by each reconstruction's last pass
     p->bound = reinterpret_cast<double *>(p->grid + grid_cells);
     p->tau = p->bound + 1;
     p->hist = reinterpret_cast<unsigned long long *>(p->tau + 1);
@@ -123,127 +123,21 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, p->device);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "cudaGetDeviceProperties: %s", cudaGetErrorString(e));
-    const size_t elem = (p->prec == PG_PREC_FP32) ? 4 : 12;  // 32-bit words per cell: FP32 one, FP64 three
-    // block tiles: rows of (nf^(d-2) x ncol) cells, the last axis padded with unfolded columns (FP64 3D: not)
-    const int cpad = pgb::tile_col_pad(p->w, d, p->prec == PG_PREC_FP32);
-    const int ncol = pgb::tile_cols(p->nf, p->w, d, p->prec == PG_PREC_FP32);
-    const size_t plane = (size_t)ipow(p->nf, d - 2) * ncol;
     const bool f32 = (p->prec == PG_PREC_FP32), ang = p->ang.n > 0;
-    // leave room for the kernels' static shared memory (FP64: the kernel polynomial)
-    // (and 16 bytes for rounding the tile up to 16 bytes)
-    const size_t max_smem = prop.sharedMemPerBlockOptin - 1024 - 16 - (f32 ? 0 : sizeof(double) * pgb::kPolyCoefF64);
-    const int max_threads = f32 ? pgb::kMaxThreadsF32 : pgb::kMaxThreadsF64;
-    const int accept_threads = pgb::accept_threads(d, f32);
-    if (o.spread_threads > accept_threads || (o.spread_threads > 0 && o.spread_threads % 32))
-        return set_error(PG_ERR_ARG, "spread_threads must be a multiple of 32 and <= %d", accept_threads);
-    int ask_threads = std::min(o.spread_threads, max_threads);  // <= 0: chosen here
-    int rows_fit = (int)std::min<size_t>(p->nf, max_smem / (plane * elem));
-    size_t qbytes = 0;
-    if (rows_fit < p->nf) {
-        // slabbed grid: the warps' queues (one block per SM) share the block's shared memory with the slab.
-        // FP32: at least 384 threads, and as many as the fewest slabs that leave room for those allow
-        // (a point is generated once per slab and its rows straddle two now and then)
-        auto fit = [&](int thr) {
-            qbytes = pgb::spread_queue_bytes(thr, d, f32, ang);
-            return (max_smem > qbytes) ? (int)std::min<size_t>(p->nf, (max_smem - qbytes) / (plane * elem)) : 0;
-        };
-        rows_fit = fit((ask_threads > 0) ? ask_threads : f32 ? 384 : max_threads);
-        if (rows_fit < 1 && f32) {  // a plane that leaves little room
-            ask_threads = (ask_threads > 0) ? std::min(ask_threads, 128) : 128;
-            rows_fit = fit(ask_threads);
-        }
-    }
-    if (rows_fit < 1) return set_error(PG_ERR_ARG, "folded grid plane of %zu cells does not fit shared memory", plane);
-    p->nslab = (p->nf + rows_fit - 1) / rows_fit;
-    p->rows_per_slab = (p->nf + p->nslab - 1) / p->nslab;
-    p->nslab = (p->nf + p->rows_per_slab - 1) / p->rows_per_slab;  // no empty trailing slab
-    const size_t tile_bytes = pgb::tile_bytes((size_t)p->rows_per_slab * plane, f32);
-    int slab_threads = max_threads;  // threads whose queues fit beside a slab
-    if (p->nslab > 1 && f32 && ask_threads <= 0) {
-        const int warps = (int)((max_smem - tile_bytes) / pgb::spread_queue_bytes(32, d, f32, ang));
-        slab_threads = std::min(max_threads, 32 * warps);
-        qbytes = pgb::spread_queue_bytes(slab_threads, d, f32, ang);
-    }
-    p->spread_smem = tile_bytes + (p->nslab > 1 ? qbytes : 0);
-    int per_sm = (int)(prop.sharedMemPerMultiprocessor / (p->spread_smem + 1024 + prop.reservedSharedMemPerBlock));
-    per_sm = std::max(per_sm, 1);
-    if (ask_threads > 0) {
-        p->spread_threads = ask_threads;
-    } else if (f32) {
-        // FP32: one block per SM (measured fastest; more, smaller blocks multiply the tile
-        // clears and flushes)
-        p->spread_threads = max_threads;
-        per_sm = 1;
-    } else {
-        // about 1024 resident threads per SM
-        int t = (1024 / per_sm) / 32 * 32;
-        p->spread_threads = std::max(128, std::min(max_threads, t));
-    }
-    if (p->nslab > 1 && ask_threads <= 0) p->spread_threads = slab_threads;  // the queues were sized for it
-    // FP32 2D: with fewer classes than threads, the classes' quads are cut into shares, so that there is
-    // an item per thread (2D N = 16, M = 8: 18,496 classes of 3 quads, spreading 41 -> 31 us).  With
-    // more classes (N = 32: 2.9 per thread) the repeated class tests cost what the fuller rounds gain.
-    int nsplit = 1;
-    if (f32 && p->nslab == 1 && d == 2) {
-        const long long want = (long long)prop.multiProcessorCount * max_threads;
-        nsplit = (int)std::max<long long>(1, std::min<long long>(M / 4 + 1, want / p->nclass));
-    }
-    if (p->nslab == 1 && ask_threads <= 0) {
-        // small plans: blocks no larger than it takes for every SM to have one (each thread then
-        // owns one class; 1024-thread blocks would keep 18 of 152 SMs busy for 2D N = 16, whose
-        // spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks of 1024 with a
-        // point set per pair)
-        const long long per_block = (p->nclass * nsplit + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
-        const int small = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
-        p->spread_threads = std::min(p->spread_threads, small);
-    }
-    if (p->nslab > 1 && pgb::spread_queue_bytes(p->spread_threads, d, f32, ang) > qbytes)
-        return set_error(PG_ERR_STATE, "internal: point queues larger than reserved");
-    // FP32 one-slab grids: the warps' queues follow the tile (2D: large quads; 3D: the points that add
-    // something) when they fit beside it, with fewer threads if need be
-    p->queued = 0;
-    if (f32 && p->nslab == 1) {
-        if (ask_threads <= 0)
-            while (p->spread_threads > 128 &&
-                   p->spread_smem + pgb::spread_queue_bytes(p->spread_threads, d, true, ang) > max_smem)
-                p->spread_threads -= 32;
-        const size_t qq = pgb::spread_queue_bytes(p->spread_threads, d, true, ang);
-        if (p->spread_smem + qq <= max_smem) {
-            p->queued = 1;
-            p->spread_smem += qq;
-        }
-    }
-    // FP64 2D one-slab grids: quads of mirrored classes, numbered in 32 bits
+    SpreadShape sh;
+    int rc1 = spread_shape({d, N, M, p->nf, p->w, f32, ang, o.spread_threads, o.spread_blocks_per_sm,
+                            prop.sharedMemPerBlockOptin, prop.sharedMemPerMultiprocessor,
+                            prop.reservedSharedMemPerBlock, prop.multiProcessorCount, prop.maxThreadsPerMultiProcessor},
+                           sh);
+    if (rc1) return rc1;
+    p->nslab = sh.nslab;
+    p->rows_per_slab = sh.rows_per_slab;
+    p->spread_threads = sh.threads;
+    p->spread_blocks = sh.blocks;
+    p->spread_smem = sh.smem;
+    p->queued = sh.queued;
     const std::vector<unsigned> orbits = axis_orbits(N);
-    const long long nitem = (long long)orbits.size() * (long long)orbits.size() * (M / 4 + 1);
-    if (!f32 && d == 2 && p->nslab == 1 && nitem < (1ll << 32)) {
-        if (ask_threads <= 0) {
-            const long long per_block = (nitem + prop.multiProcessorCount - 1) / prop.multiProcessorCount;
-            p->spread_threads = (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);
-            while (p->spread_threads > 128 && p->spread_smem + (size_t)p->spread_threads * 4 > max_smem)
-                p->spread_threads -= 128;
-            per_sm = 1;
-        }
-        const size_t qq = (size_t)p->spread_threads * 4;
-        if (p->spread_smem + qq <= max_smem) {
-            p->queued = 1;
-            p->spread_smem += qq;
-        }
-    }
-    per_sm = std::min(per_sm, prop.maxThreadsPerMultiProcessor / p->spread_threads);
-    if (o.spread_blocks_per_sm > 0) per_sm = std::min(per_sm, o.spread_blocks_per_sm);
-    per_sm = std::max(per_sm, 1);
-    long long blocks = (long long)prop.multiProcessorCount * per_sm;
-    blocks = std::max<long long>(blocks / p->nslab, 1) * p->nslab;
-    const long long items = (!f32 && p->queued) ? nitem : p->nclass * nsplit;
-    const long long need = ((items + p->spread_threads - 1) / p->spread_threads) * p->nslab;
-    blocks = std::min(blocks, need);
-    p->spread_blocks = (int)blocks;
-    // the pair schedule permutes thread starts by a multiplier prime to every smaller count
-    if ((blocks / p->nslab) * p->spread_threads >= 1000003)
-        return set_error(PG_ERR_ARG, "spreading launch of %lld threads per slab exceeds the pair schedule's range",
-                         (blocks / p->nslab) * p->spread_threads);
-    const long long tile_cells = (long long)p->rows_per_slab * (long long)plane;
+    const long long blocks = sh.blocks, tile_cells = sh.tile_cells;
     if (f32) {  // per-block carry counters of the FP32 tiles (global memory, cleared by each block)
         int rc2 = dev_alloc(p, (void **)&p->carry, (size_t)blocks * tile_cells * sizeof(int));
         if (rc2) return rc2;
@@ -287,8 +181,6 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         la.ub = p->ub;
     }
 
-    if (!p->queued) nsplit = 1;  // (no queue: whole classes)
-
     // ---- spreading-kernel arguments
     pgb::SpreadArgs &ka = p->sargs;
     ka.d = d;
@@ -298,7 +190,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.nnode = p->nnode;
     ka.naxp = (int)pgb::unordered_pairs(N);
     ka.nclass = p->nclass;
-    ka.nsplit = nsplit;
+    ka.nsplit = sh.nsplit;
     ka.n = p->n;
     ka.nf = p->nf;
     ka.rows_per_slab = p->rows_per_slab;
@@ -325,14 +217,14 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     ka.nub = p->largs.nloss ? p->largs.nbound : 0;
     ka.tau = p->tau;
     ka.grid = p->grid;
-    ka.cpad = cpad;
-    ka.ncol = ncol;
+    ka.cpad = pgb::tile_col_pad(p->w, d, f32);
+    ka.ncol = pgb::tile_cols(p->nf, p->w, d, f32);
     ka.tile_cells = (int)tile_cells;
     ka.carry = p->carry;
     ka.queued = p->queued;
     ka.orb = p->orb;
     ka.norb = (int)orbits.size();
-    ka.nitem = nitem;
+    ka.nitem = sh.nitem;
     ka.nang_even = p->ang.n ? (p->ang.n + 1) / 2 : 0;
     for (int k = 0; k < ka.nang_even; ++k) ka.ang_even[k] = p->ang.c[2 * k];
     ka.angmax = p->angmax;

@@ -1,19 +1,12 @@
 """Host tables of the plan (host.cu: node_tables), printed by a small program linked with the library's host
 object: the nodes are exactly symmetric about 0, as the kernels' mirror images of node pairs take
 them to be, and accurate in the tails, against phi_i = pi i/(N+1) evaluated in extended precision."""
-import os
-import subprocess
-
 import numpy as np
 import pytest
 
-from paper_2105_08806_gb300 import build as B
+from _host_program import host_program
 
 PROGRAM = """
-#include <cstdio>
-#include <cstdlib>
-#include "host.cuh"
-void pg_free_batch(BatchState *) {}
 int main(int argc, char **argv)
 {
     for (int a = 1; a + 2 < argc; a += 3) {
@@ -27,17 +20,8 @@ int main(int argc, char **argv)
 
 @pytest.fixture(scope="module")
 def tables(tmp_path_factory):
-    B.build()
-    d = tmp_path_factory.mktemp("host")
-    src, exe = str(d / "tables.cu"), str(d / "tables")
-    open(src, "w").write(PROGRAM)
-    subprocess.run([B.nvcc(), *B.ARCH, "-std=c++17", "-I", B.CSRC, "-I", os.path.join(B.ROOT, "include"), "-o", exe, src,
-                    os.path.join(B.BUILD, "host.o")], check=True, capture_output=True)
-
-    def run(args):
-        out = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout
-        return [np.array([float.fromhex(x) for x in line.split()]).reshape(-1, 3).T for line in out.splitlines()]
-    return run
+    run = host_program(tmp_path_factory.mktemp("tables"), PROGRAM)
+    return lambda args: [np.array([float.fromhex(x) for x in line.split()]).reshape(-1, 3).T for line in run(args)]
 
 
 def test_nodes_are_exactly_symmetric_and_accurate(tables):
