@@ -150,7 +150,7 @@ struct pg_boltz_plan_s {
     // workspace
     double *tA = nullptr, *tB = nullptr, *tC = nullptr, *tD = nullptr;
     double *a64 = nullptr;
-    float *a32 = nullptr;
+    float *a32 = nullptr, *a32lo = nullptr;  // a32lo: 2D angular FP32 plans (LossArgs)
     double *h = nullptr, *Qplus = nullptr, *Qlast = nullptr, *mom = nullptr;
     int *carry = nullptr;      // FP32 spreading: per-block carry counters
     unsigned *orb = nullptr;   // axis orbits of node pairs (SpreadArgs::orb, LossArgs::orb)

@@ -281,15 +281,16 @@ cudaError_t launch_axis_pass(const AxisPass &P, cudaStream_t s);
 // Two independent passes in one launch; P0's fixed-point input is in units 2^-Eg (Eg from *B), times scale.
 cudaError_t launch_axis_pass_pair(const AxisPass &P0, const AxisPass &P1, const double *B, double scale, cudaStream_t s);
 // Last reconstruction pass along axis 2, then a_i = acc * prod_l scale[i_l];
-// writes a (FP64) and, if af != nullptr, a float copy; clears the nclear words at clear.
+// writes a (FP64) and, if af != nullptr, a float copy and, if alo != nullptr, what it leaves of a (a float);
+// clears the nclear words at clear.
 cudaError_t launch_recon_last(const double *in, Dims3 in_dims, const double *A, int m,
-                              const double *scale, int d, double *a, float *af, unsigned long long *clear,
+                              const double *scale, int d, double *a, float *af, float *alo, unsigned long long *clear,
                               long long nclear, cudaStream_t s);
 // The loss sums h_i and the strength bound by mirror images of the nodes (VHS kernels, and angular ones
 // in 2D, without screening; launch_loss otherwise).  f32: FP32 pair terms.
 struct LossArgs {
     const double *a;        // N^d node values
-    const float *a32;
+    const float *a32, *a32lo;  // FP32 plans: a as a32 + a32lo (a32lo: 2D angular ones)
     const double *v64;      // N node velocities
     const float *v32, *v32lo;
     int N, M;

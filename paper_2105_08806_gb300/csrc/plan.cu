@@ -103,10 +103,11 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
     const long long mpd1 = (long long)ipow(Mp, d - 1);
     const long long big = std::max({modes, (long long)(N + 1) * nfd1, (long long)(N + 1) * mpd1});
     const long long grid_cells = nfd1 * p->nf;
+    const bool two_term = p->prec == PG_PREC_FP32 && p->ang.n > 0 && d == 2;
     if ((rc = dev_alloc(p, (void **)&p->tA, big * 8)) || (rc = dev_alloc(p, (void **)&p->tB, big * 8)) ||
         (rc = dev_alloc(p, (void **)&p->tC, modes * 8)) || (rc = dev_alloc(p, (void **)&p->tD, modes * 8)) ||
         (rc = dev_alloc(p, (void **)&p->a64, (size_t)p->nnode * 8)) ||
-        (rc = dev_alloc(p, (void **)&p->a32, (size_t)p->nnode * 4)) ||
+        (rc = dev_alloc(p, (void **)&p->a32, (size_t)p->nnode * (two_term ? 8 : 4))) ||
         (rc = dev_alloc(p, (void **)&p->h, (size_t)p->nnode * 8)) ||
         (rc = dev_alloc(p, (void **)&p->grid, grid_cells * 8 + 16 + pgb::kScreenBins * 8)) ||
         (rc = dev_alloc(p, (void **)&p->ub, (size_t)p->nnode * 8)) ||
@@ -114,6 +115,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         (rc = dev_alloc(p, (void **)&p->rk, 5 * modes * 8)) ||
         (rc = dev_alloc(p, (void **)&p->mom, 16 * 8)))
         return rc;
+    if (two_term) p->a32lo = p->a32 + p->nnode;
     // one allocation: [grid | B | tau | screening histogram], cleared by each reconstruction's last pass
     p->bound = reinterpret_cast<double *>(p->grid + grid_cells);
     p->tau = p->bound + 1;
@@ -155,6 +157,7 @@ int build_plan(pg_boltz_plan_t *p, const pg_boltz_opts_t &o)
         pgb::LossArgs &la = p->largs;
         la.a = p->a64;
         la.a32 = p->a32;
+        la.a32lo = p->a32lo;
         la.v64 = p->v64;
         la.v32 = p->v32;
         la.v32lo = p->v32lo;
@@ -390,7 +393,7 @@ PG_API int pg_boltz_collide(pg_boltz_plan_t *p, const double *f_dev, double *Q_d
     // (the last pass also clears the fixed-point grid, its bound and the screening histogram)
     const long long clear = (long long)ipow(p->nf, d) + 2 + pgb::kScreenBins;
     if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, f32 ? p->a32 : nullptr,
-                                                p->grid, clear, p->stream), "reconstruct")))
+                                                p->a32lo, p->grid, clear, p->stream), "reconstruct")))
         return rc;
     ++launches;
     mark(1);
@@ -530,7 +533,8 @@ PG_API int pg_boltz_conservation(pg_boltz_plan_t *p, const double *f_dev, double
     pgb::Dims3 dims = dims_of(d, N + 1, N + 1, N + 1);
     const double *cur = nullptr;
     if ((rc = leading_passes(p, f_dev, dims, p->R, N, p->tA, p->tB, &cur, &launches))) return rc;
-    if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, nullptr, nullptr, 0, p->stream),
+    if ((rc = cuda_check(pgb::launch_recon_last(cur, dims, p->R, N, p->scale_a, d, p->a64, nullptr, nullptr, nullptr, 0,
+                                                p->stream),
                          "reconstruct")))
         return rc;
     const int nout = 2 * (d + 2);

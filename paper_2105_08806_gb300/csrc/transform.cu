@@ -97,7 +97,7 @@ __global__ void k_axis_pass_pair(const __grid_constant__ AxisPass P0, const __gr
 // `clear` (the spread grid and its scalars, which nothing reads before the loss kernel), so that no
 // separate memset is launched.
 __global__ void k_recon_last(const double *in, Dims3 id, const double *__restrict__ A, int m,
-                             const double *__restrict__ scale, int d, double *a, float *af,
+                             const double *__restrict__ scale, int d, double *a, float *af, float *alo,
                              unsigned long long *clear, long long nclear)
 {
     launch_dependents();
@@ -127,6 +127,7 @@ __global__ void k_recon_last(const double *in, Dims3 id, const double *__restric
             acc *= sc;
             a[o] = acc;
             if (af) af[o] = (float)acc;
+            if (alo) alo[o] = (float)(acc - (double)(float)acc);
         }
     }
 }
@@ -320,8 +321,10 @@ __global__ void __launch_bounds__(kLossThreads) k_loss(const double *__restrict_
 // per ordered pair (2^(2d) of them share B and the map factors): blocks nloss .. nloss+nbound-1.
 // With an angular factor (2D: the circle is symmetric in both axes) the mean of b over the sphere set
 // is the same for all of them, too, and only its even part survives the antipodal pairs.
-// The sums are those of k_loss: FP32 plans add the FP32 coefficients' products as float pairs (the product's
-// FMA residual and a two-sum per term), angular ones FP32 pair terms times the FP64 coefficients in FP64.
+// FP32 plans add the FP32 coefficients' products as float pairs, as k_loss does (the product's FMA residual and a
+// two-sum per term), angular ones with the coefficients in two terms: k_loss sums those in FP64, which took
+// half of this stage at N = 100 (2D angular, M = 8: evaluation 1.42 ms, 1.60 with FP64 sums), while two terms and a
+// pair keep 2^-48 of each term, whose factor B b carries 2^-24 anyway.
 // Measured, loss stage (with the bound's reduction before, which the spreading kernel now does):
 // 2D hard spheres N = 64 FP32 143 -> 43 us, FP64 1323 -> 252 us; N = 120 1294 -> 429 us; 3D VHS N = 24
 // 1212 -> 301 us; 2D angular N = 41, M = 22 408 -> 35 us.
@@ -543,10 +546,11 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
         if constexpr (ANG) B *= circle_mean<PT>(L, sig, dv[0], dv[1], g);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            if constexpr (F32 && !ANG) {
+            if constexpr (F32) {
                 const float aj = av[idx[e]];
                 const float pt = B * aj;
-                const float pe = fmaf(B, aj, -pt);
+                float pe = fmaf(B, aj, -pt);
+                if constexpr (ANG) pe = fmaf(B, L.a32lo[idx[e]], pe);
                 const float t = as[e] + pt;
                 const float bv = t - as[e];
                 ac[e] += ((as[e] - (t - bv)) + (pt - bv)) + pe;
@@ -829,11 +833,11 @@ cudaError_t launch_axis_pass_pair(const AxisPass &P0, const AxisPass &P1, const 
 }
 
 cudaError_t launch_recon_last(const double *in, Dims3 in_dims, const double *A, int m,
-                              const double *scale, int d, double *a, float *af, unsigned long long *clear,
+                              const double *scale, int d, double *a, float *af, float *alo, unsigned long long *clear,
                               long long nclear, cudaStream_t s)
 {
     return launch_dependent(k_recon_last, grid_for((long long)in_dims.e[0] * in_dims.e[1] * m * kSplit), kThreads, 0, s,
-                            in, in_dims, A, m, scale, d, a, af, clear, nclear);
+                            in, in_dims, A, m, scale, d, a, af, alo, clear, nclear);
 }
 
 cudaError_t launch_loss_mirror(const LossArgs &L, int d, bool f32, cudaStream_t s)

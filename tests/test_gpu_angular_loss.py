@@ -1,6 +1,6 @@
-"""The loss sums of 2D angular FP32 plans take the FP64 node values and are summed in FP64.  With
+"""The loss sums of 2D angular FP32 plans keep the FP64 node values (in two FP32 terms).  With
 b = 1 and gamma = 0 every pair term is exactly a_j, so the loss's total mass, the gain's less Q's, is that of the
-FP64 plan to FP64 rounding (below 1e-12 of the gain's mass; values rounded to FP32 leave 1e-10)."""
+FP64 plan to rounding (2^-48 of a term: below 1e-12 of the gain's mass; values rounded to FP32 leave 1e-10)."""
 import numpy as np
 import pytest
 
