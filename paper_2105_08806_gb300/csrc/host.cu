@@ -368,8 +368,19 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
                                       : std::min(std::max(128, std::min(max_threads, (1024 / per_sm) / 32 * 32)),
                                                  small_block(nclass));
         // 2D: quads of mirrored classes, numbered in 32 bits, 4 bytes of queue per thread
-        const long long norb = (long long)axis_orbits(N).size(), nitem = norb * norb * (in.M / 4 + 1);
-        if (d == 2 && nitem < (1ll << 32)) {
+        const long long norb = (long long)axis_orbits(N).size();
+        long long nitem = norb * norb * (in.M / 4 + 1);
+        const long long all = (long long)in.sms * max_threads;
+        // (two sphere points, and classes for two thirds of the threads at most: a class' two points at once are
+        // faster, w = 14 N = 16 131 us, by quads 177; N = 20 197 / 332)
+        if (d == 2 && nitem < (1ll << 32) && (in.M > 2 || nclass > all * 2 / 3)) {
+            // With fewer items than threads the launch waits for the 16 points that a thread adds one after the
+            // other: shares of 4 points, or of 1, which evaluate the axes 3 or 8 times as often.  us, whole / 4 / 16
+            // shares: N = 8, M = 6, w = 14 276 / - / 84; N = 12, M = 8, w = 10 185 / 140 / 171; N = 14, M = 6, w = 14 274 / 212 / 231;
+            // logarithmic map, w = 10: N = 15, M = 14 239 / 200, M = 22 (4 shares are 1.3 per thread) 301 / 361.  (M = 4: 8
+            // points in series; N = 14, w = 14 189 / 212 / 207.)
+            const int share = 16 * nitem <= all * 3 / 4 ? 16 : (in.M > 4 && 4 * nitem <= all) ? 4 : 1;
+            nitem *= share;
             int threads = ask_threads > 0 ? ask_threads : small_block(nitem);
             if (ask_threads <= 0)
                 while (threads > 128 && tile + (size_t)threads * 4 > max_smem) threads -= 128;
@@ -378,6 +389,7 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
                 out.threads = threads;
                 out.smem += (size_t)threads * 4;
                 out.nitem = items = nitem;
+                out.nsplit = share;
                 if (ask_threads <= 0) per_sm = 1;
             }
         }

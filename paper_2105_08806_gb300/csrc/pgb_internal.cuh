@@ -49,7 +49,7 @@ struct SpreadArgs {
     int nnode;            // N^d interior nodes
     int naxp;             // unordered pairs of node indices per axis, unordered_pairs(N)
     long long nclass;     // classes of node pairs that share their points, naxp^d
-    int nsplit;           // FP32 2D one-slab grids: shares that a class' quads are spread in (1: all at once)
+    int nsplit;           // one-slab 2D grids, shares: FP32: of a class' quads; FP64: of a quad's points (1: all at once)
     int n, nf;            // periodic grid size, folded cells per axis (n/2 + 1)
     int rows_per_slab;    // folded-grid rows (axis 0) held in shared memory by one block
     int nslab;            // number of slabs covering axis 0
@@ -81,7 +81,7 @@ struct SpreadArgs {
                           // warp, and the fields below are set)
     const unsigned *orb;  // FP64 2D: the axis orbits' representative node pairs, i + 65536 j
     int norb;             // their number
-    long long nitem;      // quads of all orbits, (M/4 + 1) norb^2
+    long long nitem;      // quads of all orbits, (M/4 + 1) norb^2, times nsplit
     // angular kernel: a spread pair stands for both orders, whose cos theta differ in sign, so
     // the gain needs the even part b_e(c) = (b(c) + b(-c))/2 = sum_k ang_even[k] c^(2k) only
     int nang_even;        // terms of ang_even; 0: VHS kernel (no angular factor)

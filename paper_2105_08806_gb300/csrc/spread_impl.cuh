@@ -1748,7 +1748,7 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
 // (logarithmic map) 26.3 -> 11.2 ms.  Then issue is 57% active, the FP64 pipe 42% and the shared
 // pipe 36% busy (N = 40, M = 8): latency of 16 warps, no single unit.
 //
-// An item is one quad m of one orbit; p.orb lists the axis orbits' representatives i + j <= N-1 (the
+// An item is one quad m of one orbit (small plans: a share of it); p.orb lists the axis orbits' representatives i + j <= N-1 (the
 // mirror image of i + j = N-1 is itself and its strength counts once).
 
 // Grid coordinate and fixed-point weights of one axis, out of line (one copy); the first tap.
@@ -1826,10 +1826,37 @@ __device__ __forceinline__ bool load_orbit(const SpreadArgs &p, int o0, int o1, 
     return any;
 }
 
-// Quad m of an orbit.
-template <int W, bool ANG>
-__device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orbit<ANG> &O, int m, const WideTile &tile,
-                                                  int plane)
+// The point sets of a quad: column sets h0 .. h1-1 (coordinate h >> 1, mirrored if h is odd) times row sets
+// g0 .. g1-1.  Small plans cut the quads into shares (SpreadArgs::nsplit: 4, one column set each, or 16,
+// one point set each), so that a thread adds 4 points or 1 in series instead of 16.
+struct QuadShare {
+    int h0, h1, g0, g1;
+};
+template <bool SPLIT>
+__device__ __forceinline__ QuadShare quad_share(const SpreadArgs &p, int share)
+{
+    if (!SPLIT) return QuadShare{0, 4, 0, 4};
+    if (p.nsplit == 4) return QuadShare{share, share + 1, 0, 4};
+    return QuadShare{share >> 2, (share >> 2) + 1, share & 3, (share & 3) + 1};
+}
+
+// Whether share H of quad m of an orbit whose mirror images have strengths holds a point of one of them.
+template <bool ANG>
+__device__ __forceinline__ bool share_holds(const Orbit<ANG> &O, const QuadShare &H)
+{
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const bool in = (H.h1 - H.h0 > 1 || (H.h0 & 1) == (e >> 1)) && (H.g1 - H.g0 > 1 || (H.g0 & 1) == (e & 1));
+        any = any || (in && (O.x0[e] != 0.0 || (ANG && O.x1[e] != 0.0)));
+    }
+    return any;
+}
+
+// Share H of quad m of an orbit.
+template <int W, bool ANG, bool SPLIT>
+__device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orbit<ANG> &O, int m, const QuadShare &H,
+                                                  const WideTile &tile, int plane)
 {
     const double *sig = static_cast<const double *>(p.sig);
     const int nrow = (4 * m == p.M) ? 1 : 2, ncolumn = (m == 0) ? 1 : 2;  // 1: no mirror image
@@ -1839,8 +1866,8 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
     int sr[2], cc[2];
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
-        if (k < nrow) sr[k] = axis_eval_f64<W>(p, O.cen[0] + (k ? -O.rad : O.rad) * cs, fr[k], &mr[k]);
-        if (k < ncolumn) {
+        if (k < nrow && 2 * k < H.g1 && 2 * k + 1 >= H.g0) sr[k] = axis_eval_f64<W>(p, O.cen[0] + (k ? -O.rad : O.rad) * cs, fr[k], &mr[k]);
+        if (k < ncolumn && 2 * k < H.h1 && 2 * k + 1 >= H.h0) {
             const int s = axis_eval_f64<W>(p, O.cen[1] + (k ? -O.rad : O.rad) * sn, fc[k], &mc[k]);
             cc[k] = min(max(s + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
         }
@@ -1860,7 +1887,7 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
 #pragma unroll
     for (int c = 0; c < W; ++c) cl[c] = c;
 #pragma unroll 1
-    for (int h = 0; h < 4; ++h) {  // column sets: coordinate t, mirrored (e1) or not
+    for (int h = H.h0; h < H.h1; ++h) {  // column sets: coordinate t, mirrored (e1) or not
         const int t = h >> 1, e1 = h & 1;
         if (t >= ncolumn) break;
         FixW fl[W];
@@ -1868,7 +1895,7 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
         for (int c = 0; c < W; ++c) fl[c] = fc[t][e1 ? W - 1 - c : c];
         const int cb = e1 ? p.ncol - W - cc[t] : cc[t];
 #pragma unroll 1
-        for (int g = 0; g < 4; ++g) {  // row sets: coordinate s, mirrored (e0) or not
+        for (int g = H.g0; g < H.g1; ++g) {  // row sets: coordinate s, mirrored (e0) or not
             const int s = g >> 1, e0 = g & 1;
             if (s >= nrow) break;
             double q = O.x0[e0 + 2 * e1];
@@ -1889,7 +1916,7 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
 
 // The items it = first, first + stride, ... below end of one lane.  Items that are not negligible go
 // through the warp's queue of 32 item numbers (ids), so that 32 lanes spread 32 items.
-template <int W, bool ANG>
+template <int W, bool ANG, bool SPLIT>
 __device__ __forceinline__ void spread_orbits(const SpreadArgs &p, long long first, long long end, long long stride,
                                               double sc, double tau, double floor_q, const WideTile &tile, int plane,
                                               unsigned *ids)
@@ -1903,11 +1930,20 @@ __device__ __forceinline__ void spread_orbits(const SpreadArgs &p, long long fir
         const bool more = __any_sync(full, c.pr < end);
         if (!more && queued == 0) break;
         bool hit = false;
-        // an item: quad m = c.t / norb (slowest, so that a warp's lanes mostly share it), orbits c.t % norb and c.i
+        // an item: quad and share, m nsplit + share = c.t / norb (slowest, so that a warp's lanes mostly share it),
+        // orbits c.t % norb and c.i
         const unsigned id = (unsigned)c.t * (unsigned)p.norb + (unsigned)c.i;
         if (c.pr < end) {
             Orbit<ANG> O;
-            hit = load_orbit<ANG>(p, c.t % p.norb, c.i, sc, tau, floor_q, O);
+            if constexpr (SPLIT) {
+                const int k = c.t / p.norb, m = k / p.nsplit;
+                const QuadShare H = quad_share<true>(p, k % p.nsplit);
+                // (no mirror image of a zero sine or cosine)
+                hit = !(m == 0 && H.h0 > 1) && !(4 * m == p.M && H.g0 > 1) &&
+                      load_orbit<ANG>(p, c.t % p.norb, c.i, sc, tau, floor_q, O) && share_holds<ANG>(O, H);
+            } else {
+                hit = load_orbit<ANG>(p, c.t % p.norb, c.i, sc, tau, floor_q, O);
+            }
             pair_advance(p.norb, c, st);
         }
         const unsigned mask = __ballot_sync(full, hit);
@@ -1927,7 +1963,11 @@ __device__ __forceinline__ void spread_orbits(const SpreadArgs &p, long long fir
             const int t = (int)(mine / (unsigned)p.norb);
             Orbit<ANG> O;
             load_orbit<ANG>(p, t % p.norb, (int)(mine - (unsigned)t * (unsigned)p.norb), sc, tau, floor_q, O);
-            spread_orbit_quad<W, ANG>(p, O, t / p.norb, tile, plane);
+            const int k = t / p.norb;
+            if constexpr (SPLIT)
+                spread_orbit_quad<W, ANG, true>(p, O, k / p.nsplit, quad_share<true>(p, k % p.nsplit), tile, plane);
+            else
+                spread_orbit_quad<W, ANG, false>(p, O, k, quad_share<false>(p, 0), tile, plane);
         }
         __syncwarp();
     }
@@ -2043,7 +2083,7 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
     }
 }
 
-template <int D, int W, bool ANG>
+template <int D, int W, bool ANG, bool SPLIT>
 __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_constant__ SpreadArgs p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2080,7 +2120,7 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
         if constexpr (D == 2) {
             unsigned *ids = reinterpret_cast<unsigned *>(smem_raw + tile_bytes(tile_cells, false)) +
                             (threadIdx.x >> 5) * 32;
-            spread_orbits<W, ANG>(p, first, p.nitem, nthr, sc, tau, floor_q, tile, G.plane, ids);
+            spread_orbits<W, ANG, SPLIT>(p, first, p.nitem, nthr, sc, tau, floor_q, tile, G.plane, ids);
         }
     } else {
         spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, 1.0, tau, floor_q, tile, G.row_lo,
@@ -2107,7 +2147,9 @@ cudaError_t launch_f32(const SpreadArgs &a, int blocks, int threads, size_t smem
 template <int D, int W, bool ANG>
 cudaError_t launch_f64(const SpreadArgs &a, int blocks, int threads, size_t smem, cudaStream_t s)
 {
-    auto kern = k_spread_f64<D, W, ANG>;
+    auto kern = k_spread_f64<D, W, ANG, false>;
+    if constexpr (D == 2)
+        if (a.nsplit > 1) kern = k_spread_f64<D, W, ANG, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_dependent(kern, blocks, threads, smem, s, a);

@@ -69,3 +69,18 @@ def test_fp32_blocks_keep_their_warps(shapes):
             continue
         assert s["queued"] or s["nslab"] > 1, (p, s)
         assert s["threads"] >= least, (p, s)
+
+
+def test_fp64_2d_small_plans_share_their_quads(shapes):
+    """A thread adds the 16 points of an orbit's quad one after the other only where there are quads for a quarter
+    of the GPU's threads; below that they are cut into 4 shares or 16 (one point each; 8 points at M = 4: 16 or none)."""
+    plans = [(2, N, M, w, 2.0, 0, ang, 0, 0) for N in range(2, 65) for M in (2, 4, 6, 12, 32) for w in (6, 10, 14) for ang in (0, 1)]
+    for p, s in zip(plans, shapes(plans)):
+        N, M = p[1:3]
+        norb = sum(1 for i in range(N) for j in range(i, N) if i + j <= N - 1)
+        if not s["queued"]:
+            assert M == 2 and s["nsplit"] == 1 and (N * (N + 1) // 2) ** 2 <= 152 * 512 * 2 // 3, (p, s)
+            continue
+        quads = norb ** 2 * (M // 4 + 1)
+        assert s["nitem"] == quads * s["nsplit"] and s["nsplit"] in (1, 4, 16), (p, s)
+        assert s["nsplit"] > 1 or (4 if M > 4 else 24) * quads > 152 * 512, (p, s)
