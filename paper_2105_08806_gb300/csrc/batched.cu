@@ -620,7 +620,6 @@ void pg_free_batch(BatchState *b)
 
 namespace {
 
-constexpr long long kItemPoints = 1 << 17;     // points per work item (default)
 constexpr long long kItemPointsMin = 1 << 15;  // the autotuner's work-item sizes: 2^15 .. 2^19
 constexpr long long kItemPointsMax = 1 << 19;
 
@@ -824,8 +823,14 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         return nullptr;
     }
     B->item_capacity = (int)capacity;
-    B->item_points = kItemPoints;
-    split_items(cells, kItemPoints, &item_cell);
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
+        set_error(PG_ERR_CUDA, "cudaDeviceGetAttribute failed");
+        free_plan(p);
+        return nullptr;
+    }
+    B->item_points = default_item_points(d, split_items(cells, kItemPoints, nullptr), sms);
+    split_items(cells, B->item_points, &item_cell);
     B->nitems = (int)item_cell.size();
     B->grid_cells = grid_off;
     std::vector<float> v32(v64.begin(), v64.end()), sig32(sig64.begin(), sig64.end()), wsig32(wsig64.begin(), wsig64.end());

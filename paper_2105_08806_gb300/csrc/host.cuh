@@ -83,6 +83,17 @@ std::vector<double> transform_matrix(int N, int n, int w, double beta);
 
 pgb::Dims3 dims_of(int d, int a, int b, int c);
 
+// Points per work item of a batched plan, before tuning, for cells that make `items` items of kItemPoints points.  A
+// class stands for 2 node pairs in 2D and 4 in 3D, so that kItemPoints points of classes make that many fewer items
+// than of pairs: with less than two per SM the items are cut to as many as of pairs.  4 cells, ms whole / cut: 2D (N = 16
+// and 24) FP64 30.4 / 16.8, FP32 2.90 / 2.18; 3D (N = 6 .. 10) FP64 60.3 / 17.9, FP32 5.80 / 2.64.  With many items the whole ones are
+// faster (768 2D cells 28.2 / 28.7, 64 of N = 48 and 96 140.6 / 144.8).
+constexpr long long kItemPoints = 1 << 17;
+inline long long default_item_points(int d, long long items, int sms)
+{
+    return items < 2ll * sms ? kItemPoints >> (d - 1) : kItemPoints;
+}
+
 // A plan's spreading launch from its sizes, its options and the device's limits alone.
 struct SpreadShapeIn {
     int d, N, M, nf, w;
