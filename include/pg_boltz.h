@@ -275,9 +275,10 @@ int pg_boltz_batched_use_graph(pg_boltz_plan_t *plan, int enable);
 /*
  * Autotuner of a batched plan's persistent spreading launch (no counterpart in the paper, which
  * evaluates one operator at a time): runs pg_boltz_collide_batched's launch sequence on the
- * caller's f_packed_dev / Q_packed_dev (Q is overwritten), first for threads per block in
- * {128, 256, 512} and every blocks-per-SM count the kernel's occupancy allows (FP32 plans:
- * at most the block count the plan sized its carry counters for), then at the fastest shape for
+ * caller's f_packed_dev / Q_packed_dev (Q is overwritten), first for the plan's current launch shape,
+ * the one it started with, and threads per block in {128, 256, 512} with every blocks-per-SM count
+ * the kernel's occupancy allows (FP32 plans: at most the block count the plan sized its carry
+ * counters for), then at the fastest shape for
  * work items of 2^15, 2^16, ..., 2^19 points (the node-pair ranges the blocks take from the
  * global counter); `trials` timed runs each after one warm-up.  Keeps the fastest shape and item
  * size for later calls (the next call captures a new graph).  The results do not depend on

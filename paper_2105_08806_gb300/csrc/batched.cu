@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -587,6 +588,7 @@ struct BatchState {
     long long points = 0, pairs = 0, grid_cells = 0;
     int nitems = 0;
     int spread_blocks = 0, spread_threads = 0;
+    int start_blocks = 0, start_threads = 0;  // the shape before tuning
     size_t spread_smem = 0;
     size_t tile_smem = 0;    // dynamic shared memory of the largest cell tile (16-byte multiple)
     size_t static_smem = 0;  // the spreading kernel's static shared memory
@@ -944,6 +946,8 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
     per_sm = std::min(per_sm, std::max(1, prop.maxThreadsPerMultiProcessor / B->spread_threads));
     per_sm = std::min(per_sm, std::max(1, (int)(prop.sharedMemPerMultiprocessor / (B->spread_smem + per_block_extra))));
     B->spread_blocks = prop.multiProcessorCount * per_sm;
+    B->start_threads = B->spread_threads;
+    B->start_blocks = B->spread_blocks;
     a.carry = nullptr;
     a.carry_stride = max_cells_tile;
     B->carry_blocks = B->spread_blocks;
@@ -1061,10 +1065,9 @@ PG_API int pg_boltz_batched_use_graph(pg_boltz_plan_t *p, int enable)
     return PG_OK;
 }
 
-// Time a set of launch shapes of the persistent spreading kernel on the caller's data and keep the
-// fastest: threads per block in {128, 256, 512, 1024} (within the kernel's bound) and every
-// blocks-per-SM count the kernel's occupancy allows, up to the blocks the carry counters were
-// sized for.  Each shape: one launch sequence to warm up, then the best of `trials` timed ones.
+// Time a set of launch shapes of the persistent spreading kernel on the caller's data and keep the fastest
+// (tune_shapes; at most the blocks that the carry counters were sized for), then the work-item sizes at that
+// shape.  Each: one launch sequence to warm up, then the best of `trials` timed ones.
 namespace {
 
 // Re-split the cells into work items of about item_points points and upload the new item table
@@ -1132,26 +1135,26 @@ PG_API int pg_boltz_batched_autotune(pg_boltz_plan_t *p, const double *f_dev, do
         return r;
     };
     // 1. launch shapes at the current work-item size
-    int best_threads = best0_threads, best_blocks = best0_blocks;
-    double best_ms = 1e300;
-    for (int threads = 128; threads <= max_threads && rc == PG_OK; threads *= 2) {
+    auto occupancy = [&](int threads) {
         int occ = 0;
         const size_t smem = batch_smem(B, threads);
-        if (smem + B.static_smem > prop.sharedMemPerBlockOptin) continue;
-        if (pgb::batch_spread_occupancy(f32, B.d, B.w, threads, smem, &occ) != cudaSuccess || occ < 1) continue;
-        for (int per_sm = 1; per_sm <= occ && rc == PG_OK; ++per_sm) {
-            const int blocks = prop.multiProcessorCount * per_sm;
-            if (f32 && blocks > B.carry_blocks) break;  // no carry counters for more blocks
-            B.spread_threads = threads;
-            B.spread_blocks = blocks;
-            B.spread_smem = smem;
-            double ms_best = 1e300;
-            rc = time_config(ms_best);
-            if (rc == PG_OK && ms_best < best_ms) {
-                best_ms = ms_best;
-                best_threads = threads;
-                best_blocks = blocks;
-            }
+        if (smem + B.static_smem > prop.sharedMemPerBlockOptin) return 0;
+        return pgb::batch_spread_occupancy(f32, B.d, B.w, threads, smem, &occ) == cudaSuccess ? occ : 0;
+    };
+    int best_threads = best0_threads, best_blocks = best0_blocks;
+    double best_ms = 1e300;
+    for (const LaunchShape &s : tune_shapes({best0_threads, best0_blocks}, {B.start_threads, B.start_blocks},
+                                            prop.multiProcessorCount, max_threads,
+                                            f32 ? B.carry_blocks : LLONG_MAX, occupancy)) {
+        B.spread_threads = s.threads;
+        B.spread_blocks = s.blocks;
+        B.spread_smem = batch_smem(B, s.threads);
+        double ms_best = 1e300;
+        if ((rc = time_config(ms_best))) break;
+        if (ms_best < best_ms) {
+            best_ms = ms_best;
+            best_threads = s.threads;
+            best_blocks = s.blocks;
         }
     }
     // 2. work-item sizes at the best shape

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <vector>
 
@@ -92,6 +93,30 @@ constexpr long long kItemPoints = 1 << 17;
 inline long long default_item_points(int d, long long items, int sms)
 {
     return items < 2ll * sms ? kItemPoints >> (d - 1) : kItemPoints;
+}
+
+// Launch shapes that the batched autotuner times: the plan's current one first, so that tuning never makes a plan
+// slower; the one it started with; and 128, 256 and 512 threads in every number of blocks per SM that occupancy(threads)
+// (0: does not fit) and max_blocks allow.
+struct LaunchShape {
+    int threads, blocks;
+    bool operator==(const LaunchShape &o) const { return threads == o.threads && blocks == o.blocks; }
+};
+template <typename F>
+std::vector<LaunchShape> tune_shapes(LaunchShape now, LaunchShape start, int sms, int max_threads, long long max_blocks,
+                                     F occupancy)
+{
+    std::vector<LaunchShape> out{now};
+    auto add = [&](LaunchShape s) {
+        for (const LaunchShape &o : out)
+            if (o == s) return;
+        out.push_back(s);
+    };
+    add(start);
+    for (int threads = 128; threads <= std::min(max_threads, 512); threads *= 2)
+        for (int per_sm = 1, occ = occupancy(threads); per_sm <= occ && (long long)sms * per_sm <= max_blocks; ++per_sm)
+            add({threads, sms * per_sm});
+    return out;
 }
 
 // A plan's spreading launch from its sizes, its options and the device's limits alone.
