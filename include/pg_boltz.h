@@ -74,7 +74,11 @@ typedef struct {
     int sphere;          /* PG_SPHERE_*                                                  */
     double upsampfac;    /* grid oversampling sigma, 0 -> 2.0, range [1.5, 4]             */
     int proj_nodes;      /* Chebyshev-Gauss nodes per axis for pg_boltz_project, 0 -> 4(N+1) */
-    int spread_threads;  /* threads per spreading block, 0 -> automatic                  */
+    int spread_threads;  /* threads per spreading block, a multiple of 32 up to 1024 (FP32), 256
+                            (FP64, 2D) or 512 (FP64, 3D); 0 -> automatic.  Launches may have fewer
+                            (pg_boltz_info): FP32 kernels at most 640, and no more than what their
+                            queues leave room for beside the grid in shared memory.  Batched FP32
+                            plans refuse a block whose 2 d + 1 floats per thread do not fit.   */
     int spread_blocks_per_sm; /* spreading blocks per SM, 0 -> automatic                 */
     int screen;          /* 1: skip the node pairs with the smallest strength bounds, as many
                             as keep their summed bound below 0.05 tol B (B >= the sum of all

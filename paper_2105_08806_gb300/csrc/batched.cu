@@ -927,22 +927,16 @@ PG_API pg_boltz_plan_t *pg_boltz_plan_batched_ex(const pg_boltz_opts_t *opts, in
         free_plan(p);
         return nullptr;
     }
-    B->spread_threads = (o.spread_threads > 0) ? std::min(o.spread_threads, max_threads)
-                                                : std::max(min_threads, std::min(max_threads, (1024 / per_sm) / 32 * 32));
-    // fewer threads where the queues would not fit beside the tile (a block size that was asked for
-    // shrinks only when 20 bytes of queue per thread fit)
-    if (o.spread_threads <= 0 ||
-        B->tile_smem + (size_t)o.spread_threads * 20 + B->static_smem <= prop.sharedMemPerBlockOptin)
-        while (B->spread_threads > 32 &&
-               batch_smem(*B, B->spread_threads) + B->static_smem > prop.sharedMemPerBlockOptin)
-            B->spread_threads -= 32;
-    B->spread_smem = batch_smem(*B, B->spread_threads);
-    if (B->spread_smem + B->static_smem > prop.sharedMemPerBlockOptin) {
+    B->spread_threads = batch_block_threads(d, f32, o.spread_threads,
+                                            std::max(min_threads, std::min(max_threads, (1024 / per_sm) / 32 * 32)),
+                                            B->tile_smem, prop.sharedMemPerBlockOptin - B->static_smem);
+    if (!B->spread_threads) {
         set_error(PG_ERR_ARG, "largest cell's folded grid (%d cells) and the queues of %d threads do not fit "
-                  "shared memory", max_cells_tile, B->spread_threads);
+                  "shared memory", max_cells_tile, o.spread_threads);
         free_plan(p);
         return nullptr;
     }
+    B->spread_smem = batch_smem(*B, B->spread_threads);
     per_sm = std::min(per_sm, std::max(1, prop.maxThreadsPerMultiProcessor / B->spread_threads));
     per_sm = std::min(per_sm, std::max(1, (int)(prop.sharedMemPerMultiprocessor / (B->spread_smem + per_block_extra))));
     B->spread_blocks = prop.multiProcessorCount * per_sm;

@@ -270,6 +270,16 @@ pgb::Dims3 dims_of(int d, int a, int b, int c)
     return x;
 }
 
+int batch_block_threads(int d, bool f32, int ask, int automatic, size_t tile, size_t limit)
+{
+    const int max_threads = f32 ? pgb::kBatchThreadsF32 : pgb::kMaxThreadsF64;
+    auto need = [&](int threads) { return tile + (f32 ? pgb::spread_queue_bytes(threads, d, true) : 0); };
+    if (ask > 0 && f32 && tile + (size_t)ask * 4 * (2 * d + 1) > limit) return 0;
+    int threads = ask > 0 ? std::min(ask, max_threads) : automatic;
+    while (threads > 32 && need(threads) > limit) threads -= 32;
+    return need(threads) <= limit ? threads : 0;
+}
+
 int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
 {
     const int d = in.d, N = in.N, nf = in.nf;
@@ -328,9 +338,12 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
             return (max_smem > qbytes) ? (int)std::min<size_t>(nf, (max_smem - qbytes) / (plane * elem)) : 0;
         };
         rows_fit = fit((ask_threads > 0) ? ask_threads : f32 ? 384 : max_threads);
-        if (rows_fit < 1 && f32) {  // a plane that leaves little room
+        if (rows_fit < 1 && f32) {
+            // a plane that leaves little room: the block that still fits, at worst one warp with half of the kilobyte
+            // left for static shared memory (the FP32 kernels have 16 bytes)
             ask_threads = (ask_threads > 0) ? std::min(ask_threads, 128) : 128;
-            rows_fit = fit(ask_threads);
+            while ((rows_fit = fit(ask_threads)) < 1 && ask_threads > 32) ask_threads -= 32;
+            if (rows_fit < 1 && queue_bytes(32) + plane * elem <= max_smem + 512) rows_fit = 1;
         }
     }
     if (rows_fit < 1) return set_error(PG_ERR_ARG, "folded grid plane of %zu cells does not fit shared memory", plane);

@@ -95,6 +95,11 @@ inline long long default_item_points(int d, long long items, int sms)
     return items < 2ll * sms ? kItemPoints >> (d - 1) : kItemPoints;
 }
 
+// Threads of a batched plan's spreading block for a largest tile of `tile` bytes in `limit` bytes of dynamic shared memory:
+// `ask` (> 0: pg_boltz_opts_t::spread_threads) or `automatic`, less where the warps' queues do not fit beside the
+// tile; 0: refused.  A block size that is asked for is refused when 2 d + 1 floats per thread do not fit, whatever the queues take.
+int batch_block_threads(int d, bool f32, int ask, int automatic, size_t tile, size_t limit);
+
 // Launch shapes that the batched autotuner times: the plan's current one first, so that tuning never makes a plan
 // slower; the one it started with; and 128, 256 and 512 threads in every number of blocks per SM that occupancy(threads)
 // (0: does not fit) and max_blocks allow.

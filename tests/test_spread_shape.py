@@ -84,3 +84,50 @@ def test_fp64_2d_small_plans_share_their_quads(shapes):
         quads = norb ** 2 * (M // 4 + 1)
         assert s["nitem"] == quads * s["nsplit"] and s["nsplit"] in (1, 4, 16), (p, s)
         assert s["nsplit"] > 1 or (4 if M > 4 else 24) * quads > 152 * 512, (p, s)
+
+
+def _accepted_before(d, w, nf, f32, threads):
+    """Whether a plan with points spread one by one through queues of 2 d + 1 floats (FP64: d + 1 doubles) per thread, with
+    a margin column more on both sides of the last axis (and padded FP64 3D tiles), found room for a row of the grid."""
+    room = LIMITS[0] - 1024 - 16 - (0 if f32 else 8 * 136)
+    plane = nf ** (d - 2) * (nf + 2 * (w // 2 + 1)) * (4 if f32 else 12)
+    queue = threads * (4 * (2 * d + 1) if f32 else 8 * (d + 1))
+    return nf * plane <= room or queue + plane <= room
+
+
+@pytest.mark.parametrize("threads", [32, 64, 96, 128, 256, 1024])
+def test_no_block_size_is_refused_that_was_not_before(shapes, threads):
+    """3D FP32 grids whose planes all but fill the block: the queues per thread grew, the block shrinks instead."""
+    plans = [(3, N, 4, w, sigma, 1, ang, threads, 0) for w in range(2, 11) for sigma in (1.5, 2.0, 4.0) for ang in (0, 1)
+             for N in range(2, 129)]
+    for p, s in zip(plans, shapes(plans)):
+        if _accepted_before(3, p[3], s["nf"], True, threads):
+            assert s["rc"] == 0 and s["threads"] <= threads and s["smem"] <= LIMITS[0] - 512, (p, s)
+
+
+BATCH = """
+int main()
+{
+    int d, f32, ask, automatic;
+    long long tile, limit;
+    while (scanf("%d %d %d %d %lld %lld", &d, &f32, &ask, &automatic, &tile, &limit) == 6)
+        printf("%d\\n", pgbh::batch_block_threads(d, f32 != 0, ask, automatic, tile, limit));
+}
+"""
+
+
+def test_batched_blocks_that_are_asked_for(tmp_path):
+    """Refused exactly when 2 d + 1 floats per thread do not fit beside the tile (FP64: when the tile does not); otherwise
+    the largest block up to the one asked for whose queues fit."""
+    run, limit = host_program(tmp_path, BATCH), 230000
+    cases = [(d, f32, ask, 128, limit - left, limit) for d in (2, 3) for f32 in (0, 1) for ask in (32, 96, 256, 512, 1024)
+             for left in (0, 1000, 2000, 3000, 6000, 12000, 13000, 24000, 28000, 40000)]
+    out = run(stdin="".join("%d %d %d %d %d %d\n" % c for c in cases))
+    for (d, f32, ask, _, tile, _), got in zip(cases, map(int, out)):
+        left = limit - tile
+        if not f32:
+            assert got == min(ask, 512)
+            continue
+        per = {2: 44, 3: 68}[d]
+        fits = min(ask, 640, left // (32 * per) * 32)
+        assert got == (fits if ask * 4 * (2 * d + 1) <= left else 0), (d, ask, left, got)
