@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
     int cur = -1, ncell = 0, plane = 0, Eg = 0, shift = 0;
     T sc = T(0), pre = T(1), tau = T(0), floor_q = T(0);
     // the current cell's spreading arguments live in shared memory: kept in registers they cost
-    // 30-odd registers per thread (fewer resident warps, or spills under a 1024-thread bound)
+    // 30-odd registers per thread (spills under the kernel's thread bound)
     __shared__ SpreadArgs s_sa;
     SpreadArgs &sa = s_sa;
     if constexpr (!F32) load_kernel_poly(b.kpoly);  // the same kernel polynomial for every cell
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(max_threads_of<T, D>(), 1) k_batch_spread(cons
                 spread_points3<W, false, false>(sa, first, pend, nwarp, sc, pre, tau, SplitTile{lo, carry}, 0, s_cd.nf,
                                                 plane, buf);
         } else
-            spread_pairs<T, D, W, WideTile, false>(sa, first, pend, nwarp, sc, pre, tau, floor_q, wt, 0,
+            spread_pairs<T, D, W, WideTile, false>(sa, first, pend, nwarp, sc, pre, tau, floor_q, wt,
                                                       s_cd.nf, plane);
         __syncthreads();
     }

@@ -300,8 +300,7 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
     // threads whose queues fit beside a tile
     auto room = [&](size_t tile) { return tile < max_smem ? 32 * (int)((max_smem - tile) / queue_bytes(32)) : 0; };
     // small one-slab plans: blocks no larger than it takes for every SM to have one (each thread then owns
-    // one item; 2D Maxwell N = 16: spreading takes 55 us in 145 blocks of 128 threads, 74 us in 33 blocks
-    // of 1024 with a point set per pair)
+    // one item; 2D Maxwell N = 16 has one for each of 145 blocks of 384)
     auto small_block = [&](long long items) {
         const long long per_block = (items + in.sms - 1) / in.sms;
         return (int)std::min<long long>((std::max<long long>(per_block, 64) + 31) / 32 * 32, max_threads);

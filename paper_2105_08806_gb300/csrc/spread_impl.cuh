@@ -303,7 +303,6 @@ __device__ __forceinline__ void axis_weights_f32(const SpreadArgs &p, float X, f
 {
     float t0;
     const int s = first_tap_f32<W>(X, F, t0);
-    const float h2 = 2.0f / W;
     const float bl = p.cf.bl;
 #pragma unroll
     for (int a = 0; a < W; ++a) {
@@ -615,7 +614,9 @@ __device__ __forceinline__ unsigned long long fix_mul(unsigned long long R2, Fix
 
 // The scale of a point of strength q (grid units 2^-Eg): its contributions are formed in units
 // 2^-(Eg+s) with s = 60 - ilogb|q|, at most 32 (the fraction word's resolution) and at least 0, so that
-// |q| 2^s < 2^61.
+// |q| 2^s < 2^61.  Points below 2^28 grid units thus have their row factors rounded to 2^-32 units, as their
+// contributions are (at s = 94, 2^-61 of the point, the factors alone would be finer): an error that can at
+// most double one that the sum of a cell, rounded to whole grid units per block, exceeds a millionfold.
 struct WideScale {
     int s;
     unsigned long long q2;    // round(|q| 2^(s+1))
@@ -802,19 +803,24 @@ __device__ __forceinline__ int mulhi_rn(int a, int b)
     return (int)(((long long)a * (long long)b + 0x80000000LL) >> 32);
 }
 
+// Large points: the factor q4 of a point of strength q scaled by 2^-sc, which leaves |q| 2^-sc in [2^28, 2^29).
+__device__ __forceinline__ float scale_large(float q4, float q, int &sc)
+{
+    sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
+    return q4 * __int_as_float((127 - sc) << 23);
+}
+
 // Add the w^d contributions q psi_a psi_b psi_c of one FP32 point to the block tile: the column
 // factors 2^30 psi_c and, per row, 4 q psi_a (psi_b) are rounded to integers, and a contribution is
 // mulhi_rn of the two (at most about one tile unit of rounding).  kLarge: the same with q 2^-s in
 // [2^28, 2^29) for the point's own s, i.e. rounded to 2^s tile units, 2^-28 of the point's strength
 // (an FP32 product is rounded to 2^-24 of the contribution, which is more over a point's taps; and
 // the float path that formed it took twice the instructions: 768 batched cells, where points of 2^29
-// units are common, 43.9 -> 33.2 ms).
-// SLAB: the tile holds a slab of the grid's rows and rows outside it are skipped; otherwise it holds
-// every row (row_lo = 0, nrows = n/2 + 1).  3D points loop over their axis-0 rows (computing that
+// units are common, 43.9 -> 33.2 ms).  The tile holds every row of the grid.  3D points loop over their axis-0 rows (computing that
 // row's kernel value in the loop) so that the unrolled code stays small.
-template <int D, int W, int KIND, bool SLAB>
+template <int D, int W, int KIND>
 __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Point<float, D> &pt,
-                                                 const SplitTile &tile, int row_lo, int nrows, int plane)
+                                                 const SplitTile &tile, int plane)
 {
     const float q = pt.q;
     if (fabsf(q) < kNegligibleF32) return;  // every contribution rounds to zero
@@ -834,10 +840,7 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
     float q4 = 4.0f * q;
     int sc = 0;
-    if constexpr (KIND == kLarge) {
-        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
-        q4 *= __int_as_float((127 - sc) << 23);  // 2^-sc
-    }
+    if constexpr (KIND == kLarge) q4 = scale_large(q4, q, sc);
     const float bias30 = 30.0f - bl;
     int wi[W];
 #pragma unroll
@@ -856,21 +859,13 @@ __device__ __forceinline__ void spread_point_f32(const SpreadArgs &p, const Poin
     if constexpr (D == 2) {
 #pragma unroll
         for (int a = 0; a < W; ++a) {
-            int r = fold_cell(s0 + a, p.n);
-            if constexpr (SLAB) {
-                r -= row_lo;
-                if ((unsigned)r >= (unsigned)nrows) continue;
-            }
+            const int r = fold_cell(s0 + a, p.n);
             run(r * plane + cb, __float2int_rn(q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl)));
         }
     } else {
 #pragma unroll 1
         for (int a = 0; a < W; ++a) {
-            int r = fold_cell(s0 + a, p.n);
-            if constexpr (SLAB) {
-                r -= row_lo;
-                if ((unsigned)r >= (unsigned)nrows) continue;
-            }
+            const int r = fold_cell(s0 + a, p.n);
             const float qa = q4 * es_f32(fmaf((float)a, h2, t00), bl, -bl);
             const int row = r * plane;
 #pragma unroll
@@ -947,15 +942,15 @@ __device__ __forceinline__ void spread_point_f64(const SpreadArgs &p, const Poin
 // integer products for points below 2^29 tile units, chosen per lane (a point's contributions must
 // not depend on its warp-mates: bitwise reproducibility across launch shapes; points of 2^29 tile
 // units or more are rare); a lane whose point is below kNegligibleF32 idles.
-template <typename T, int D, int W, typename Tile, bool SLAB>
+template <typename T, int D, int W, typename Tile>
 __device__ __forceinline__ void spread_point_body(const SpreadArgs &p, const Point<T, D> &pt, const Tile &tile,
-                                                  int row_lo, int nrows, int plane)
+                                                  int nrows, int plane)
 {
     if constexpr (sizeof(T) == 4) {
-        if (fabsf(pt.q) < kIntLimitF32) spread_point_f32<D, W, kInt, SLAB>(p, pt, tile, row_lo, nrows, plane);
-        else spread_point_f32<D, W, kLarge, SLAB>(p, pt, tile, row_lo, nrows, plane);
+        if (fabsf(pt.q) < kIntLimitF32) spread_point_f32<D, W, kInt>(p, pt, tile, plane);
+        else spread_point_f32<D, W, kLarge>(p, pt, tile, plane);
     } else {
-        spread_point_f64<D, W, SLAB>(p, pt, tile, row_lo, nrows, plane);
+        spread_point_f64<D, W, false>(p, pt, tile, 0, nrows, plane);
     }
 }
 
@@ -1008,8 +1003,7 @@ __device__ __forceinline__ void zero_pair(PairData<T, D> &P)
 // every row.  Every lane of the warp runs every point step (the loop conditions are uniform).
 template <typename T, int D, int W, typename Tile, bool ANG>
 __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long first, long long end, long long stride,
-                                             T sc, T pre, T tau, T floor_q, const Tile &tile, int row_lo, int nrows,
-                                             int plane)
+                                             T sc, T pre, T tau, T floor_q, const Tile &tile, int nrows, int plane)
 {
     PairCursor c = pair_cursor(p.naxp, first);
     const PairStep st = pair_step(p.naxp, stride);
@@ -1022,7 +1016,7 @@ __device__ __forceinline__ void spread_pairs(const SpreadArgs &p, long long firs
         for (int m = 0; m < p.M; ++m) {
             Point<T, D> pt;
             make_point<T, D, ANG>(p, P, qbase, m, pt);
-            spread_point_body<T, D, W, Tile, false>(p, pt, tile, row_lo, nrows, plane);
+            spread_point_body<T, D, W, Tile>(p, pt, tile, nrows, plane);
         }
         if (ok) pair_advance(p.naxp, c, st);
     }
@@ -1175,8 +1169,7 @@ __device__ __forceinline__ void quad_cols(const SpreadArgs &p, float v, QuadCols
 
 // The large quad in slot `lane` of the queue: its points one by one.
 template <int W>
-__device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float *buf, const SplitTile &tile, int nrows,
-                                               int plane)
+__device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float *buf, const SplitTile &tile, int plane)
 {
     const int lane = threadIdx.x & 31;
     const bool alg = (p.r == 1);
@@ -1190,7 +1183,7 @@ __device__ __noinline__ void spread_large_quad(const SpreadArgs &p, const float 
                axis_m2_f32(p.cf, v1, alg);
         grid_coord_f32(p.cf, v0, alg, pt.X[0], pt.F[0]);
         grid_coord_f32(p.cf, v1, alg, pt.X[1], pt.F[1]);
-        spread_point_f32<2, W, kLarge, false>(p, pt, tile, 0, nrows, plane);
+        spread_point_f32<2, W, kLarge>(p, pt, tile, plane);
     }
 }
 
@@ -1218,8 +1211,8 @@ __device__ __forceinline__ void spread_point_compact(const SpreadArgs &p, float 
     int wi[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) wi[c] = __float2int_rn(es_tap_f32<W>(c, off[1], K.bl, 30.0f - K.bl));
-    const int sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
-    const float q4 = 4.0f * q * __int_as_float((127 - sc) << 23);
+    int sc;
+    const float q4 = scale_large(4.0f * q, q, sc);
 #pragma unroll 1
     for (int a = 0; a < W; ++a) {
         const int rq = __float2int_rn(q4 * es_f32(fmaf((float)a, 2.0f / W, off[0]), K.bl, -K.bl));
@@ -1240,7 +1233,7 @@ __device__ __forceinline__ int share_start(const SpreadArgs &p, int g, int n)
 // count: the warp's queue of large quads, 32 slots of kQuadValues floats, and its fill.
 template <int W, bool ANG, bool SPLIT>
 __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const PairData<float, 2> &P, float qbase, int g,
-                                                   const SplitTile &tile, int nrows, int plane, float *buf, int &count)
+                                                   const SplitTile &tile, int plane, float *buf, int &count)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -1285,7 +1278,7 @@ __device__ __forceinline__ void spread_class_quads(const SpreadArgs &p, const Pa
             if (large && rank < room) put(count + rank);
             if (n >= room) {
                 __syncwarp();
-                spread_large_quad<W>(p, buf, tile, nrows, plane);
+                spread_large_quad<W>(p, buf, tile, plane);
                 __syncwarp();
                 if (large && rank >= room) put(rank - room);
                 count = n - room;
@@ -1363,10 +1356,7 @@ __device__ __forceinline__ void half_quad_point(const SplitTile &tile, const int
     const int sg = q < 0.0f ? -1 : 1;
     float q4 = 4.0f * q;
     int sc = 0;
-    if constexpr (KIND == kLarge) {  // as spread_point_f32
-        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
-        q4 *= __int_as_float((127 - sc) << 23);
-    }
+    if constexpr (KIND == kLarge) q4 = scale_large(q4, q, sc);
 #pragma unroll
     for (int k = 0; k < W; ++k) {
         if (ra[k] < 0) continue;
@@ -1530,14 +1520,14 @@ __device__ __forceinline__ void spread_quads(const SpreadArgs &p, long long firs
             if (hit && rank >= room) put(rank - room);
             nclass = max(n - room, 0);
             if constexpr (SLAB) spread_class_halves<W, ANG>(p, C, C.base * sc, tile, row_lo, nrows, plane, range, buf, count);
-            else spread_class_quads<W, ANG, SPLIT>(p, C, C.base * sc, mine, tile, nrows, plane, buf, count);
+            else spread_class_quads<W, ANG, SPLIT>(p, C, C.base * sc, mine, tile, plane, buf, count);
         } else {
             nclass += n;
         }
     }
     __syncwarp();
     if constexpr (SLAB) spread_half_quad<W>(p, buf, lane < count, tile, row_lo, nrows, plane);
-    else if (!SPLIT && lane < count) spread_large_quad<W>(p, buf, tile, nrows, plane);
+    else if (!SPLIT && lane < count) spread_large_quad<W>(p, buf, tile, plane);
 }
 
 // ---- 3D FP32 grids
@@ -1579,10 +1569,7 @@ __device__ __forceinline__ void queue3_spread(const SpreadArgs &p, const float *
     const int sg = q < 0.0f ? -1 : 1;  // the sign of every contribution (or zero)
     float q4 = 4.0f * q;
     int sc = 0;
-    if (kind == kLarge) {  // as spread_point_f32
-        sc = min(max(((__float_as_int(q) >> 23) & 255) - 127 - 28, 0), 31);
-        q4 *= __int_as_float((127 - sc) << 23);
-    }
+    if (kind == kLarge) q4 = scale_large(q4, q, sc);
     const int a0 = (kind == kSmall) ? 1 : 0;
 #pragma unroll 1
     for (int a = a0; a < W - a0; ++a) {
@@ -2070,8 +2057,8 @@ __global__ void __launch_bounds__(kMaxThreadsF32) k_spread_f32(const __grid_cons
         else
             spread_points3<W, ANG, false>(p, first, p.nclass, nthr, sc, pre, tau, tile, 0, G.nrows, G.plane, buf);
     } else {
-        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, pre, tau, kNegligibleF32, tile, G.row_lo,
-                                                   G.nrows, G.plane);
+        spread_pairs<float, D, W, SplitTile, ANG>(p, first, p.nclass, nthr, sc, pre, tau, kNegligibleF32, tile, G.nrows,
+                                                   G.plane);
     }
     __syncthreads();
     for (int c = threadIdx.x; c < G.ncell; c += blockDim.x) {
@@ -2123,8 +2110,8 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1) k_spread_f64(const __grid_c
             spread_orbits<W, ANG, SPLIT>(p, first, p.nitem, nthr, sc, tau, floor_q, tile, G.plane, ids);
         }
     } else {
-        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, 1.0, tau, floor_q, tile, G.row_lo,
-                                                   G.nrows, G.plane);
+        spread_pairs<double, D, W, WideTile, ANG>(p, first, p.nclass, nthr, sc, 1.0, tau, floor_q, tile, G.nrows,
+                                                   G.plane);
     }
     __syncthreads();
     for (int c = threadIdx.x; c < G.ncell; c += blockDim.x) {
