@@ -17,8 +17,8 @@
 // on every axis take two operations per coefficient, this form one and two per row.  Blocks of one warp, so that
 // the points spread evenly over the SMs, and registers for 12 of them per SM, so that a row's loads are all in
 // flight at once (with the compiler's own choice few points were slower: N = 120, one point 0.68 ms instead of
-// 0.61).  200 x 200 points at N = 48, 2D: 705 us with recurrences on every axis, 237 us so (one FMA per coefficient at the
-// measured 5.3e11/s: 182 us).
+// 0.61).  200 x 200 points at N = 48, 2D: 705 us with recurrences on every axis, 237 us so (one FMA per
+// coefficient at the measured 5.3e11/s: 182 us).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -324,7 +324,8 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
         //   3D w = 6:          N = 16 angular (512) 6.91 / 8.03   N = 17 (256) 3.04 / 2.36
         //   3D w = 8, sigma = 1.5: N = 22 (352) 11.1 / 11.0
         // (One slab spread point by point without queues, 640 threads: 3.15 at N = 115 and 3.79 at N = 117 where two
-        // slabs take 3.47 and 3.78 ms, but 10.4 against 9.9 at M = 32, 9.98 against 8.84 angular and 4.6 against 2.4 in 3D.)
+        // slabs take 3.47 and 3.78 ms, but N = 117 10.4 against 9.9 at M = 32, 9.98 against 8.84 angular, and 3D N = 17
+        // 4.6 against 2.4.)
         if (room(whole) < std::min(small_block(nclass * nsplit), d == 3 ? 384 : 320)) rows_fit = nf - 1;
     }
     size_t qbytes = 0;
@@ -388,9 +389,9 @@ int spread_shape(const SpreadShapeIn &in, SpreadShape &out)
         if (d == 2 && nitem < (1ll << 32) && (in.M > 2 || nclass > all * 2 / 3)) {
             // With fewer items than threads the launch waits for the 16 points that a thread adds one after the
             // other: shares of 4 points, or of 1, which evaluate the axes 3 or 8 times as often.  us, whole / 4 / 16
-            // shares: N = 8, M = 6, w = 14 276 / - / 84; N = 12, M = 8, w = 10 185 / 140 / 171; N = 14, M = 6, w = 14 274 / 212 / 231;
-            // logarithmic map, w = 10: N = 15, M = 14 239 / 200, M = 22 (4 shares are 1.3 per thread) 301 / 361.  (M = 4: 8
-            // points in series; N = 14, w = 14 189 / 212 / 207.)
+            // shares: N = 8, M = 6, w = 14 276 / - / 84; N = 12, M = 8, w = 10 185 / 140 / 171; N = 14, M = 6, w = 14
+            // 274 / 212 / 231; logarithmic map, w = 10: N = 15, M = 14 239 / 200, M = 22 (4 shares are 1.3 per
+            // thread) 301 / 361.  (M = 4: 8 points in series; N = 14, w = 14 189 / 212 / 207.)
             const int share = 16 * nitem <= all * 3 / 4 ? 16 : (in.M > 4 && 4 * nitem <= all) ? 4 : 1;
             nitem *= share;
             int threads = ask_threads > 0 ? ask_threads : small_block(nitem);

@@ -85,19 +85,20 @@ std::vector<double> transform_matrix(int N, int n, int w, double beta);
 pgb::Dims3 dims_of(int d, int a, int b, int c);
 
 // Points per work item of a batched plan, before tuning, for cells that make `items` items of kItemPoints points.  A
-// class stands for 2 node pairs in 2D and 4 in 3D, so that kItemPoints points of classes make that many fewer items
-// than of pairs: with less than two per SM the items are cut to as many as of pairs.  4 cells, ms whole / cut: 2D (N = 16
-// and 24) FP64 30.4 / 16.8, FP32 2.90 / 2.18; 3D (N = 6 .. 10) FP64 60.3 / 17.9, FP32 5.80 / 2.64.  With many items the whole ones are
-// faster (768 2D cells 28.2 / 28.7, 64 of N = 48 and 96 140.6 / 144.8).
+// class stands for 2 node pairs in 2D and 4 in 3D, so that kItemPoints points of classes make that many fewer
+// items than of pairs: with less than two per SM the items are cut to as many as of pairs.  4 cells, ms whole / cut:
+// 2D (N = 16 and 24) FP64 30.4 / 16.8, FP32 2.90 / 2.18; 3D (N = 6 .. 10) FP64 60.3 / 17.9, FP32 5.80 / 2.64.  With many
+// items the whole ones are faster (768 2D cells 28.2 / 28.7, 64 of N = 48 and 96 140.6 / 144.8).
 constexpr long long kItemPoints = 1 << 17;
 inline long long default_item_points(int d, long long items, int sms)
 {
     return items < 2ll * sms ? kItemPoints >> (d - 1) : kItemPoints;
 }
 
-// Threads of a batched plan's spreading block for a largest tile of `tile` bytes in `limit` bytes of dynamic shared memory:
-// `ask` (> 0: pg_boltz_opts_t::spread_threads) or `automatic`, less where the warps' queues do not fit beside the
-// tile; 0: refused.  A block size that is asked for is refused when 2 d + 1 floats per thread do not fit, whatever the queues take.
+// Threads of a batched plan's spreading block for a largest tile of `tile` bytes in `limit` bytes of dynamic shared
+// memory: `ask` (> 0: pg_boltz_opts_t::spread_threads) or `automatic`, less where the warps' queues do not fit
+// beside the tile; 0: refused.  A block size that is asked for is refused when 2 d + 1 floats per thread do not
+// fit, whatever the queues take.
 int batch_block_threads(int d, bool f32, int ask, int automatic, size_t tile, size_t limit);
 
 // Launch shapes that the batched autotuner times: the plan's current one first, so that tuning never makes a plan

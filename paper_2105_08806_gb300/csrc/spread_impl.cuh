@@ -1346,7 +1346,8 @@ __device__ __forceinline__ SlabRange slab_range(const SpreadArgs &p, int row_lo,
 
 // In a slabbed grid half of a quad's rows or more lie outside a block's slab, so there the quads are
 // queued by halves (N = 120, M = 8: spreading 5.44 -> 4.58 ms against a queue of single points, 4.16 ms
-// with the slab's velocity range): one coordinate of axis 0 whose rows may reach the slab, and the two of axis 1 with the strengths of their points (0: no such point), kQuadValues values.
+// with the slab's velocity range): one coordinate of axis 0 whose rows may reach the slab, and the two of
+// axis 1 with the strengths of their points (0: no such point), kQuadValues values.
 
 // Add one point of a half quad: rows ra (-1: outside the slab) with factors pa, column factors col.
 template <int W, int KIND>
@@ -1735,7 +1736,8 @@ __device__ __forceinline__ void spread_points3(const SpreadArgs &p, long long fi
 // (logarithmic map) 26.3 -> 11.2 ms.  Then issue is 57% active, the FP64 pipe 42% and the shared
 // pipe 36% busy (N = 40, M = 8): latency of 16 warps, no single unit.
 //
-// An item is one quad m of one orbit (small plans: a share of it); p.orb lists the axis orbits' representatives i + j <= N-1 (the
+// An item is one quad m of one orbit (small plans: a share of it); p.orb lists the axis orbits'
+// representatives i + j <= N-1 (the
 // mirror image of i + j = N-1 is itself and its strength counts once).
 
 // Grid coordinate and fixed-point weights of one axis, out of line (one copy); the first tap.
@@ -1853,7 +1855,8 @@ __device__ __forceinline__ void spread_orbit_quad(const SpreadArgs &p, const Orb
     int sr[2], cc[2];
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
-        if (k < nrow && 2 * k < H.g1 && 2 * k + 1 >= H.g0) sr[k] = axis_eval_f64<W>(p, O.cen[0] + (k ? -O.rad : O.rad) * cs, fr[k], &mr[k]);
+        if (k < nrow && 2 * k < H.g1 && 2 * k + 1 >= H.g0)
+            sr[k] = axis_eval_f64<W>(p, O.cen[0] + (k ? -O.rad : O.rad) * cs, fr[k], &mr[k]);
         if (k < ncolumn && 2 * k < H.h1 && 2 * k + 1 >= H.h0) {
             const int s = axis_eval_f64<W>(p, O.cen[1] + (k ? -O.rad : O.rad) * sn, fc[k], &mc[k]);
             cc[k] = min(max(s + p.cpad, 0), p.ncol - W);  // clamped: x lies in [0, n/2]
