@@ -446,11 +446,15 @@ __device__ __forceinline__ double mirror_bound(const LossArgs &L, const PT *vn, 
     return acc + (double)p;
 }
 
-// The same with the sums in FP64, out of line: FP32 plans whose FP32 sums left the range.
+// Block blk's part of the bound with the sums in FP64: FP32 plans whose FP32 sums left the range.  FP32 sums
+// overflow from amplitudes of about 1e19 on; below 1e-24 what underflowed may matter (at most 1e7 products per
+// block, each 1e-45 off, times the class' factor).  Out of line with its reduction and its store, so that the usual path
+// keeps its registers (56 instead of 64; loss stage at N = 64 43 -> 40 us).
 template <int D>
-__device__ __noinline__ double mirror_bound_wide(const LossArgs &L, int blk)
+__device__ __noinline__ void mirror_bound_wide(const LossArgs &L, int blk)
 {
-    return mirror_bound<float, double, D>(L, L.v32, L.a32, blk);
+    const double tot = block_sum<kMirrorThreads>(mirror_bound<float, double, D>(L, L.v32, L.a32, blk));
+    if (threadIdx.x == 0) L.ub[blk] = tot * L.Bw * L.angmax;
 }
 
 template <typename PT, int D, bool ANG>
@@ -476,15 +480,12 @@ __global__ void __launch_bounds__(kMirrorThreads) k_loss_mirror(const __grid_con
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if ((int)blockIdx.x >= L.nloss) {  // the strength bound
         const int blk = blockIdx.x - L.nloss;
-        double tot = block_sum<kMirrorThreads>(mirror_bound<PT, PT, D>(L, vn, av, blk));
-        if constexpr (F32) {
-            // FP32 sums overflow from amplitudes of about 1e19 on; below 1e-24 what underflowed may
-            // matter (at most 1e7 products per block, each 1e-45 off, times the class' factor).  The
-            // test costs an evaluation about 0.3 us (2D Maxwell N = 16: 49.9 -> 50.2 us).
-            const bool out = threadIdx.x == 0 && !(tot >= 1e-24 && tot <= DBL_MAX);
-            if (__syncthreads_or(out)) tot = block_sum<kMirrorThreads>(mirror_bound_wide<D>(L, blk));
-        }
+        const double tot = block_sum<kMirrorThreads>(mirror_bound<PT, PT, D>(L, vn, av, blk));
         if (threadIdx.x == 0) L.ub[blk] = tot * L.Bw * L.angmax;
+        if constexpr (F32) {
+            const bool out = threadIdx.x == 0 && !(tot >= 1e-24 && tot <= DBL_MAX);
+            if (__syncthreads_or(out)) mirror_bound_wide<D>(L, blk);
+        }
         return;
     }
     int xi[D];
